@@ -163,30 +163,35 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
             }
         }
     } else if (warp == 5) {
-        if (lane == 0) {                                                // ---- MMA issuer
+        {                                                               // ---- MMA issuer (one elected lane of a converged warp)
+            const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             constexpr uint32_t idesc = idesc_bf16(false, kTok);
             bool ok = true;
             #pragma unroll 1
             for (int i = 0; i < n_st && ok; ++i) {
                 const int st = i % kStages;
-                if (!mbar_wait(full(st), (i / kStages) & 1)) { ok = false; break; }
+                if (!mbar_wait_warp(full(st), (i / kStages) & 1)) { ok = false; break; }
                 tc_fence_after();
-                if (i == 0) SPARROW_STAMP(2);                           // first tile landed
+                if (i == 0 && lane == 0) SPARROW_STAMP(2);                           // first tile landed
                 const int boxes = min(kBoxes, n_kt - i * kBoxes);
                 const uint32_t base = smem_u32(sm + st * kStageBytes);
-                for (int bx = 0; bx < boxes; ++bx) {
-                    const uint64_t wd = smem_desc(base + bx * kWBytes, 16, 1024);
-                    const uint64_t xd = smem_desc(base + kBoxes * kWBytes + bx * kXBytes, 16, 1024);
-                    #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)
-                        mma_ss(tmem, wd + (uint64_t)((ks * 32) >> 4), xd + (uint64_t)((ks * 32) >> 4), idesc,
-                               (i > 0 || bx > 0 || ks > 0) ? 1u : 0u);
+                if (elect_one()) {
+                    for (int bx = 0; bx < boxes; ++bx) {
+                        const uint64_t wd = smem_desc(base + bx * kWBytes, 16, 1024);
+                        const uint64_t xd = smem_desc(base + kBoxes * kWBytes + bx * kXBytes, 16, 1024);
+                        #pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_ss(tmem_u, wd + (uint64_t)((ks * 32) >> 4), xd + (uint64_t)((ks * 32) >> 4), idesc,
+                                   (i > 0 || bx > 0 || ks > 0) ? 1u : 0u);
+                    }
+                    tc_commit(empty(st));
                 }
-                tc_commit(empty(st));
+                __syncwarp();
             }
-            tc_commit(done);
-            SPARROW_STAMP(3);                                           // last MMA issued
-            if (!ok) { atomicOr(args.status, timeout_bits(kSiteMma)); *abort_flag = 1; }
+            if (elect_one()) tc_commit(done);
+            __syncwarp();
+            if (lane == 0) SPARROW_STAMP(3);                            // last MMA issued
+            if (!ok && lane == 0) { atomicOr(args.status, timeout_bits(kSiteMma)); *abort_flag = 1; }
         }
     } else {
         // ---- epilogue warps, part 1: thread = one output feature (TMEM lane), 64 token columns.

@@ -131,15 +131,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
-// Same for a whole warp, with a warp-uniform result.  One lane polls (32 lanes hammering the same
-// barrier word serialise and cost hundreds of cycles per wait); the shuffle carries the verdict to
-// the others and orders their later accesses behind the observation.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity)
-{
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity) ? 1 : 0;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
-}
+// Same for a whole warp.  Every lane polls, so that the warp stays converged and no shuffle stands
+// between the phase flip and the next instruction: a wait-issue-commit round of eight tensor-core
+// instructions takes 616 cycles like this, 672 with one lane polling and issuing, 815 with one lane
+// polling, a shuffle, and an elected lane issuing.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) { return mbar_wait(bar, parity); }
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, uint32_t bar)
 {
     asm volatile(
@@ -165,6 +161,16 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
 }
 // barrier among the 256 softmax threads only (id 1; id 0 is __syncthreads)
 __device__ __forceinline__ void softmax_bar_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// One lane of a converged warp.  The tensor-core instructions take their descriptors from uniform
+// registers, which the compiler only uses behind elect.sync in a warp whose control flow stays
+// converged.  Behind `if (lane == 0)` every tcgen05.mma first moves its operands over: 93 to 104
+// cycles per 128 x 128 x 16 instruction, against the pipe's own 64 (one CTA per SM).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
 // D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
 {
@@ -408,8 +414,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_k) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_v) : "memory");
         for (int i = 0; i < 3; ++i) { mbar_init(B.k_full(i), 1); mbar_init(B.k_empty(i), 1); mbar_init(B.v_full(i), 1); mbar_init(B.v_empty(i), 1); }
-        // one row block: a P block comes from all 256 softmax threads; two: from the block's own warpgroup
-        for (int i = 0; i < 4; ++i) { mbar_init(B.s_full(i), 1); mbar_init(B.p_full(i), NB == 1 ? 256 : 128); }
+        // one row block: a P block comes from all eight softmax warps; two: from the block's own four
+        for (int i = 0; i < 4; ++i) { mbar_init(B.s_full(i), 1); mbar_init(B.p_full(i), NB == 1 ? 8 : 4); }
         for (int i = 0; i < 4; ++i) { mbar_init(B.o_done(0, i), 1); mbar_init(B.o_done(1, i), 1); }
         mbar_init(B.q_full(), 1);
         mbar_init(B.fin(), 1);
@@ -478,13 +484,15 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
     } else if (warp == kMmaWarp) {
         // ================= MMA issuer =================
-        if (lane == 0) {
+        // the whole warp walks the jobs, converged; one elected lane issues (see elect_one)
+        {
+            const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             // descriptors differ from job to job only in their 14-bit address field
             const uint64_t q_desc0 = smem_desc(smem_u32(q_sm), 16, 1024);
             const uint64_t k_desc0 = smem_desc(smem_u32(kv_sm), 16, 1024);
             const uint64_t v_desc0 = smem_desc(smem_u32(kv_sm) + 2 * kSubTileBytes, kSubTileBytes, 1024);
-            bool ok = mbar_wait(B.q_full(), 0);
-            SPARROW_STAMP(2);                                           // Q landed
+            bool ok = mbar_wait_warp(B.q_full(), 0);
+            if (lane == 0) SPARROW_STAMP(2);                                           // Q landed
             if constexpr (NB == 2) {
                 // Two row blocks, each with its own softmax warpgroup.  Job n = (key tile j = n / 2,
                 // block b = n % 2).  Block b owns TMEM columns [128 b, 128 b + 128) for its scores,
@@ -497,35 +505,41 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 auto issue_qk2 = [&](int m) -> bool {
                     const int j = m >> 1, b = m & 1, st = j % NS;
                     if (b == 0) {                                             // first use of this K tile
-                        if (!mbar_wait(B.k_full(st), (j / NS) & 1)) return false;
+                        if (!mbar_wait_warp(B.k_full(st), (j / NS) & 1)) return false;
                         tc_fence_after();
-                        if (j == 0) SPARROW_STAMP(3);                   // first K tile landed
+                        if (j == 0 && lane == 0) SPARROW_STAMP(3);                   // first K tile landed
                     }
                     const uint64_t qd = q_desc0 + (uint64_t)((b * kQBlockBytes) >> 4);
                     const uint64_t kd = k_desc0 + (uint64_t)((st * kStageBytes) >> 4);
-                    #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
-                        const uint32_t off = ((ks >> 2) * kSubTileBytes + (ks & 3) * 32) >> 4;
-                        mma_ss(tmem + b * 128, qd + off, kd + off, idesc_qk, ks > 0);
+                    if (elect_one()) {
+                        #pragma unroll
+                        for (int ks = 0; ks < 8; ++ks) {
+                            const uint32_t off = ((ks >> 2) * kSubTileBytes + (ks & 3) * 32) >> 4;
+                            mma_ss(tmem_u + b * 128, qd + off, kd + off, idesc_qk, ks > 0);
+                        }
+                        tc_commit(B.s_full(b));
+                        if (b == 1) tc_commit(B.k_empty(st));                 // last use of the tile
                     }
-                    tc_commit(B.s_full(b));
-                    if (b == 1) tc_commit(B.k_empty(st));                     // last use of the tile
+                    __syncwarp();
                     return true;
                 };
                 for (int m = 0; m < 2 && m < n_jobs && ok; ++m) ok = issue_qk2(m);
                 #pragma unroll 1
                 for (int n = 0; n < n_jobs && ok; ++n) {
                     const int j = n >> 1, b = n & 1, st = j % NS;
-                    if (b == 0 && !mbar_wait(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
-                    if (!mbar_wait(B.p_full(b), j & 1)) { ok = false; break; }
+                    if (b == 0 && !mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
+                    if (!mbar_wait_warp(B.p_full(b), j & 1)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
-                    #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_ts(tmem + 256 + b * 128, tmem + b * 128 + 64 + kk * 8, vd + (uint64_t)((kk * 2048) >> 4),
-                               idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
-                    tc_commit(B.o_done(b, j));
-                    if (b == 1) tc_commit(B.v_empty(st));
+                    if (elect_one()) {
+                        #pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            mma_ts(tmem_u + 256 + b * 128, tmem_u + b * 128 + 64 + kk * 8, vd + (uint64_t)((kk * 2048) >> 4),
+                                   idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+                        tc_commit(B.o_done(b, j));
+                        if (b == 1) tc_commit(B.v_empty(st));
+                    }
+                    __syncwarp();
                     if (n + 2 < n_jobs) ok = issue_qk2(n + 2);                // this block's next scores
                 }
             } else {
@@ -535,40 +549,46 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             auto issue_qk = [&](int m) -> bool {
                 const int j = m / NB, blk = m % NB, sb = m % NSB, st = j % NS;
                 if (blk == 0) {                                           // first use of this K tile
-                    if (!mbar_wait(B.k_full(st), (j / NS) & 1)) return false;
+                    if (!mbar_wait_warp(B.k_full(st), (j / NS) & 1)) return false;
                     tc_fence_after();
-                    if (j == 0) SPARROW_STAMP(3);                       // first K tile landed
+                    if (j == 0 && lane == 0) SPARROW_STAMP(3);                       // first K tile landed
                 }
                 const uint64_t qd = q_desc0 + (uint64_t)((blk * kQBlockBytes) >> 4);
                 const uint64_t kd = k_desc0 + (uint64_t)((st * kStageBytes) >> 4);
-                #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t off = ((ks >> 2) * kSubTileBytes + (ks & 3) * 32) >> 4;
-                    mma_ss(tmem + sb * 128, qd + off, kd + off, idesc_qk, ks > 0);
+                if (elect_one()) {
+                    #pragma unroll
+                    for (int ks = 0; ks < 8; ++ks) {
+                        const uint32_t off = ((ks >> 2) * kSubTileBytes + (ks & 3) * 32) >> 4;
+                        mma_ss(tmem_u + sb * 128, qd + off, kd + off, idesc_qk, ks > 0);
+                    }
+                    tc_commit(B.s_full(sb));
+                    if (blk == NB - 1) tc_commit(B.k_empty(st));          // last use of the tile
                 }
-                tc_commit(B.s_full(sb));
-                if (blk == NB - 1) tc_commit(B.k_empty(st));              // last use of the tile
+                __syncwarp();
                 return true;
             };
             for (int m = 0; m < NSB && m < n_jobs && ok; ++m) ok = issue_qk(m);
             #pragma unroll 1
             for (int n = 0; n < n_jobs && ok; ++n) {
                 const int j = n / NB, blk = n % NB, sb = n % NSB, st = j % NS;
-                if (blk == 0 && !mbar_wait(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
-                if (!mbar_wait(B.p_full(sb), (n / NSB) & 1)) { ok = false; break; }
+                if (blk == 0 && !mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
+                if (!mbar_wait_warp(B.p_full(sb), (n / NSB) & 1)) { ok = false; break; }
                 tc_fence_after();
                 const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
-                #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)
-                    mma_ts(tmem + kOCol + blk * 128, tmem + sb * 128 + kk * 8, vd + (uint64_t)((kk * 2048) >> 4),
-                           idesc_pv, (n >= NB || kk > 0) ? 1u : 0u);
-                tc_commit(B.o_done(blk, j));
-                if (blk == NB - 1) tc_commit(B.v_empty(st));
+                if (elect_one()) {
+                    #pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)
+                        mma_ts(tmem_u + kOCol + blk * 128, tmem_u + sb * 128 + kk * 8, vd + (uint64_t)((kk * 2048) >> 4),
+                               idesc_pv, (n >= NB || kk > 0) ? 1u : 0u);
+                    tc_commit(B.o_done(blk, j));
+                    if (blk == NB - 1) tc_commit(B.v_empty(st));
+                }
+                __syncwarp();
                 if (n + NSB < n_jobs) ok = issue_qk(n + NSB);             // its S block was job n's
             }
             }
-            SPARROW_STAMP(4);                                           // last product issued
-            if (!ok) { atomicOr(args.status, timeout_bits(kSiteMma)); *abort_flag = 1; }
+            if (lane == 0) SPARROW_STAMP(4);                            // last product issued
+            if (!ok && lane == 0) { atomicOr(args.status, timeout_bits(kSiteMma)); *abort_flag = 1; }
         }
     } else if (warp == kGateWarp) {
         if (lane == 0 && sync.enabled) {
@@ -710,7 +730,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 my_l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
                 tmem_wait_st();                                            // this job's P is in TMEM
                 tc_fence_before();
-                mbar_arrive(B.p_full(blk));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(B.p_full(blk));
             }
         } else {
         // The scores of a job are requested from TMEM at the end of the job before it, ahead of the
@@ -828,7 +849,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 }
                 tmem_wait_st();                                            // this job's P is in TMEM
                 tc_fence_before();
-                mbar_arrive(B.p_full(sb));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(B.p_full(sb));
                 if (!ok) break;
             }
         }
