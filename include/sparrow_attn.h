@@ -462,7 +462,8 @@ sparrow_status sparrow_last_device_status(sparrow_ctx* ctx, void* stream);
  * (0 before the first call).  Bits 0..2: malformed tree, bad anchor, timeout.  A wait that gave up
  * also sets bit 8 + site: 0 TMA producer, 1 MMA issuer, 2 softmax warps, 3 / 4 the waits in front
  * of a CTA's first global write (same / other call parity), 5 finisher waiting for the call's
- * pieces, 6 finisher waiting for the previous call, 7 finisher's bulk copies, 8 the debug wait.
+ * pieces, 6 finisher waiting for the previous call, 7 finisher's bulk copies, 8 the debug wait,
+ * 9 the partial sums of the temperature-1 acceptance.
  * For diagnosis only. */
 uint32_t sparrow_debug_status_word(const sparrow_ctx* ctx);
 

@@ -60,6 +60,7 @@ struct sparrow_ctx {
     size_t part_offset;                      // first byte of the split-KV partials in the workspace
     int part_buffers;                        // 2: alternate by call parity (fused mode); 1: stream-ordered calls only
     std::atomic<long long> launches;
+    int max_sample_cluster;                  // CTAs per cluster of the temperature-1 acceptance kernel the device takes
     bool use_pdl;
     bool log_plans;                          // SPARROW_LOG=1 when the context was created: one line per call on stderr
     bool overlap_single_calls;               // sparrow_set_call_overlap()
@@ -81,6 +82,7 @@ struct sparrow_ctx {
 
 namespace {
 
+constexpr int kMaxStaticDevices = 16;       // devices with per-process state (the static scratch, queried limits)
 constexpr size_t kStatusBytes = 1024;      // word 0: sticky status; words 16, 17: finisher counters
 constexpr size_t kFinDoneOffset = 64;
 constexpr size_t kArrivalsOffset = 128;     // words 32..35: arrival words of the four call slots
@@ -524,6 +526,40 @@ __global__ void early_trigger_copy_kernel(const uint4* src, uint4* dst, size_t n
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += (size_t)gridDim.x * blockDim.x) dst[i] = src[i];
 }
 
+// Largest cluster the temperature-1 acceptance kernel can be launched with on the current device: 16
+// CTAs where the device has room for such a cluster, else the portable 8.
+int query_sample_cluster_limit()
+{
+    if (cudaFuncSetAttribute(sample::accept_sample_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return 8;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(sample::kMaxCluster);
+    cfg.blockDim = dim3(sample::kThreads);
+    cfg.dynamicSmemBytes = sample::kMaxResident * sizeof(uint2);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = sample::kMaxCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, sample::accept_sample_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 8; }
+    return n > 0 ? sample::kMaxCluster : 8;
+}
+
+// The same, asked once per device and process (a property of the device).
+int sample_cluster_limit(int device)
+{
+    static std::atomic<int> known[kMaxStaticDevices];
+    if (device < 0 || device >= kMaxStaticDevices) return query_sample_cluster_limit();
+    int n = known[device].load();
+    if (n == 0) { n = query_sample_cluster_limit(); known[device].store(n); }
+    return n;
+}
+
 struct DeviceGuard {
     int prev = -1;
     bool ok = true;
@@ -643,9 +679,11 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
         return SPARROW_ERR_SHAPE;
     int count = 0;
     if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count) { cudaGetLastError(); return SPARROW_ERR_CUDA; }
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return SPARROW_ERR_CUDA;
-    if (prop.major != 10) return SPARROW_ERR_ARCH;
+    int major = 0, n_sm = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+        return SPARROW_ERR_CUDA;
+    if (major != 10) return SPARROW_ERR_ARCH;
     DeviceGuard guard(device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     if (cudaFuncSetAttribute(gather::split_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -655,6 +693,9 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
                              tc::smem_bytes(1, 3)) != cudaSuccess ||
         cudaFuncSetAttribute(tc::verify_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc::smem_bytes(2, 2)) != cudaSuccess)
+        return SPARROW_ERR_CUDA;
+    if (cudaFuncSetAttribute(sample::accept_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             sample::kMaxResident * (int)sizeof(uint2)) != cudaSuccess)
         return SPARROW_ERR_CUDA;
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
@@ -667,13 +708,14 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
     c->encode = reinterpret_cast<TensorMapEncodeFn>(fn);
     c->layout = *L;
     c->device = device;
-    c->n_sm = prop.multiProcessorCount;
+    c->n_sm = n_sm;
     c->plan_policy = SPARROW_PLAN_BALANCED;
     c->ws = nullptr;
     c->ws_bytes = 0;
     c->part_offset = fixed_bytes(*L);
     c->part_buffers = 2;
     c->launches.store(0);
+    c->max_sample_cluster = sample_cluster_limit(device);
     const char* e = std::getenv("SPARROW_NO_PDL");
     // more SMs than the list of possibly-resident calls can hold: calls never start early
     c->use_pdl = !(e && e[0] == '1') && c->n_sm < kRecentCalls;
@@ -781,7 +823,6 @@ sparrow_status sparrow_verify_attn_window(sparrow_ctx* c, const void* q, const v
 static __device__ __align__(256) unsigned char g_static_scratch[SPARROW_STATIC_SCRATCH_BYTES];
 
 namespace {
-constexpr int kMaxStaticDevices = 16;
 struct StaticSlot {
     bool ready;
     sparrow_ctx ctx;
@@ -1161,10 +1202,29 @@ sparrow_status sparrow_accept_sample(sparrow_ctx* c, const int32_t* draft_tokens
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     other_kernel_enqueued();
-    sample::accept_sample_kernel<<<c->layout.batch, sample::kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        draft_tokens, parents, p_target, p_draft, u_node, u_bonus, T, vocab, path_out, n_accept_out, bonus_out,
-        reinterpret_cast<unsigned*>(c->ws));
-    if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
+    // CTAs per sequence: more of them until a CTA's slice of the vocabulary is too small to be worth the
+    // exchange of sums (0.9 us a step), or until the batch's clusters no longer run all at once
+    int n_cta = 1;
+    while (n_cta < c->max_sample_cluster && vocab >= 2 * n_cta * sample::kMinSlice && 2 * n_cta * c->layout.batch <= c->n_sm) n_cta *= 2;
+    const int per_cta = (vocab + n_cta - 1) / n_cta;
+    const int resident = per_cta < sample::kMaxResident ? per_cta : sample::kMaxResident;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(c->layout.batch * n_cta));
+    cfg.blockDim = dim3(sample::kThreads);
+    cfg.dynamicSmemBytes = (size_t)resident * sizeof(uint2);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)n_cta;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, sample::accept_sample_kernel, draft_tokens, parents, p_target, p_draft, u_node, u_bonus, T, vocab, n_cta,
+                           resident, path_out, n_accept_out, bonus_out, reinterpret_cast<unsigned*>(c->ws)) != cudaSuccess) {
+        cudaGetLastError();
+        return SPARROW_ERR_CUDA;
+    }
     c->launches.fetch_add(1);
     return SPARROW_OK;
 }

@@ -50,7 +50,7 @@ constexpr unsigned kStatTimeout = 4u;
 // A wait that gives up also sets bit (8 + site) of the status word, so that the raw word tells which wait it was.
 __host__ __device__ constexpr unsigned timeout_bits(int site) { return kStatTimeout | (1u << (8 + site)); }
 enum WaitSite { kSiteProducer = 0, kSiteMma = 1, kSiteSoftmax = 2, kSiteWriteSame = 3, kSiteWriteOther = 4,
-                kSiteArrivals = 5, kSiteFinOther = 6, kSiteFinCopies = 7, kSiteDebug = 8 };
+                kSiteArrivals = 5, kSiteFinOther = 6, kSiteFinCopies = 7, kSiteDebug = 8, kSiteSample = 9 };
 
 // The GQA group's g query heads x T draft tokens are packed into 128-row blocks of p = 128 / g
 // tokens: block i holds tokens [p i, p i + p), row r of a block is (token p i + r / g, head r % g),

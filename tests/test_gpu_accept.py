@@ -181,3 +181,33 @@ def test_accept_sample_edge_cases():
     with pytest.raises(B.SparrowError):
         B.sparrow_accept_sample(ctx, d([[0]]), d([[-1]]), torch.from_numpy(p).to(DEV), torch.from_numpy(q).to(DEV),
                                 _u32(np.zeros((1, 1), np.uint64)), _u32(np.zeros((1, 2), np.uint64)), 0, 1, path, n_acc, bonus)
+
+
+@pytest.mark.parametrize("batch,T,vocab,sharp,scale", [
+    (1, 8, 8191, 0.5, 1.0),          # one CTA per sequence, the largest slice before a cluster of two
+    (2, 8, 8192, 0.5, 1.0),          # clusters of two
+    (1, 12, 40001, 0.2, 1.0),        # flat rows: several rejections per level, residuals replaced in place
+    (1, 12, 40001, 0.2, 1.5),        # rows that do not sum to one: residuals recomputed from the history
+    (1, 6, 163841, 0.5, 1.0),        # one entry more than the threads fetch ahead
+    (1, 4, 409601, 0.5, 1.0),        # one entry more than stays in shared memory
+    (9, 5, 70001, 0.5, 1.0),         # a batch that leaves room for clusters of sixteen
+    (10, 5, 70001, 0.5, 1.0),        # ... and of eight
+])
+def test_accept_sample_slices(batch, T, vocab, sharp, scale):
+    """Vocabulary sizes and batches at the edges of the kernel's split over a cluster's CTAs.  Integer
+    results: bit-exact."""
+    tok, par, p, q, u_node, u_bonus = _sampling_problem(9700 + vocab + batch, batch, T, vocab, sharp)
+    p, q = np.minimum(p * scale, 1.0).astype(np.float32), np.minimum(q * scale, 1.0).astype(np.float32)
+    ctx = B.Context(batch, 128, W.HKV * 128 * W.D, 128 * W.D, W.SCALE)
+    d = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32, device=DEV)
+    path = torch.full((batch, T), 99, dtype=torch.int32, device=DEV)
+    n_acc = torch.full((batch,), 99, dtype=torch.int32, device=DEV)
+    bonus = torch.full((batch,), 99, dtype=torch.int32, device=DEV)
+    B.sparrow_accept_sample(ctx, d(tok), d(par), torch.from_numpy(p).to(DEV), torch.from_numpy(q).to(DEV),
+                            _u32(u_node), _u32(u_bonus), vocab, T, path, n_acc, bonus)
+    torch.cuda.synchronize()
+    assert ctx.last_device_status() == 0
+    for b in range(batch):
+        ref_path, ref_bonus = oracle.sample_accept(tok[b], par[b], p[b], q[b], u_node[b], u_bonus[b])
+        assert path[b].tolist() == ref_path + [-1] * (T - len(ref_path))
+        assert int(n_acc[b]) == len(ref_path) and int(bonus[b]) == ref_bonus
