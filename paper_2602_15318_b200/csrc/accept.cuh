@@ -19,6 +19,8 @@ accept_greedy_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __
                      const int32_t* __restrict__ target_next, int batch, int T, int32_t* __restrict__ path,
                      int32_t* __restrict__ n_accept, int32_t* __restrict__ bonus, unsigned* status)
 {
+    let_dependents_launch();
+    wait_for_predecessors();
     const int b = threadIdx.x;
     if (b >= batch) return;
     const int32_t* tok = draft_tokens + (size_t)b * T;
@@ -64,6 +66,8 @@ struct KeepArgs {
 __global__ void __launch_bounds__(256)
 keep_accepted_rows_kernel(const __grid_constant__ KeepArgs a)
 {
+    let_dependents_launch();
+    wait_for_predecessors();
     extern __shared__ uint4 rows_sm[];                       // [2][T][16] chunks of 16 bytes
     const int b = blockIdx.x / a.n_kv_heads, h = blockIdx.x % a.n_kv_heads;
     int n = a.n_accept[b];

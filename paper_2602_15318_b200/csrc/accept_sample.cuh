@@ -169,6 +169,8 @@ accept_sample_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __
                      const uint32_t* __restrict__ u_node, const uint32_t* __restrict__ u_bonus, int T, int V, int n_cta, int resident,
                      int32_t* __restrict__ path, int32_t* __restrict__ n_accept, int32_t* __restrict__ bonus, unsigned* status)
 {
+    let_dependents_launch();
+    wait_for_predecessors();
     extern __shared__ uint2 row_s[];                   // the first `resident` entries of this CTA's slice: (P, Q) fixed point
     __shared__ Shared sh;
     const int b = blockIdx.x / n_cta, tid = threadIdx.x;

@@ -64,6 +64,7 @@ struct sparrow_ctx {
     bool use_pdl;
     bool log_plans;                          // SPARROW_LOG=1 when the context was created: one line per call on stderr
     bool overlap_single_calls;               // sparrow_set_call_overlap()
+    bool in_batch;                           // the call being enqueued belongs to a sparrow_verify_attn_batch()
     bool chain_next;                         // the call being enqueued directly follows this context's previous fused call
     // Host mirror of the ordering counters in the workspace (see SyncArgs): call sequence number
     // of the fused calls and, per call parity, the cumulative number of finishers launched so far.
@@ -241,10 +242,10 @@ int policy_target(int n_sm, int policy)
     }
 }
 
-// Calls that cannot overlap others always get one wave over all SMs.
-int plan_target(const sparrow_ctx* c, bool overlaps)
+// Calls that share the GPU with no other call get one wave over all SMs.
+int plan_target(const sparrow_ctx* c, bool may_share)
 {
-    return overlaps ? policy_target(c->n_sm, c->plan_policy) : c->n_sm;
+    return may_share ? policy_target(c->n_sm, c->plan_policy) : c->n_sm;
 }
 
 constexpr int kCallRanges = 7;
@@ -321,7 +322,7 @@ void note_fused_launch(sparrow_ctx* c, const CallRanges& cr, bool launched_early
 
 // `after_previous`: the call's final results must wait for the previous fused call as a whole (its
 // outputs overlap that call's memory); otherwise they only wait for the calls before that one.
-SyncArgs next_sync(const sparrow_ctx* c, const SplitPlan& p, bool overlaps, bool after_previous)
+SyncArgs next_sync(const sparrow_ctx* c, const SplitPlan& p, bool overlaps, bool after_previous, bool may_share)
 {
     SyncArgs sy;
     const int parity = (int)(c->seq & 1u);
@@ -335,11 +336,12 @@ SyncArgs next_sync(const sparrow_ctx* c, const SplitPlan& p, bool overlaps, bool
         if (p.seq[b].n_splits > 1) n_arrive += p.n_kv_heads * p.n_groups * p.seq[b].n_splits;
     sy.n_arrive = n_arrive;
     // Finishers wait, holding their SM, until the call's last piece is in: few of them where later
-    // calls should move in beside this one, all CTAs under the one-wave latency policy.
-    const bool all_finish = overlaps && c->plan_policy == SPARROW_PLAN_LATENCY;
+    // calls should move in beside this one, all CTAs where none can or under the latency policy.
+    const bool all_finish = overlaps && (!may_share || c->plan_policy == SPARROW_PLAN_LATENCY);
     sy.n_fin = n_arrive == 0 ? 0 : ((all_finish || p.n_items < kFinisherCtas) ? p.n_items : kFinisherCtas);
     sy.fin_wait_same = c->fin_total[parity];
     sy.fin_wait_other = after_previous ? c->fin_total[parity ^ 1] : c->fin_before_last[parity ^ 1];
+    sy.wait_first = 0;
     sy.call = c->seq;
     return sy;
 }
@@ -358,8 +360,45 @@ std::atomic<sparrow_ctx*> g_last_fused_ctx{nullptr};
 // verification call takes a plain launch behind it.
 inline void other_kernel_enqueued() { g_last_fused_ctx.store(nullptr); }
 
-sparrow_status launch_combine(sparrow_ctx* c, const SplitPlan& plan, const SyncArgs& sy, void* out, float* lse, cudaStream_t st,
-                              bool programmatic = false)
+// Programmatic launches are kept out of captured streams (measured slower in a replay) and can be
+// switched off for the context.
+bool programmatic_launch(const sparrow_ctx* c, cudaStream_t st) { return call_overlaps(c, st, true); }
+
+// Launches a kernel that orders itself behind its predecessor (wait_for_predecessors() in front of its
+// first global access): its launch and set-up overlap the predecessor's end.  Back to back, per call,
+// plain launch -> this: Eq. 1 projection 16.4 -> 13.9 us, verification of 2,048 keys 14.8 -> 12.6, of 26,112
+// keys 24.8 -> 22.5, gather + combine 12.3 -> 11.5.  cluster > 0: that many CTAs per
+// thread-block cluster (stated even when it is one: st.async to the own CTA is an illegal instruction in a
+// launch without cluster dimensions).
+template <class... KArgs, class... Args>
+sparrow_status launch_behind(sparrow_ctx* c, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                             unsigned cluster, const Args&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    unsigned n = 0;
+    if (programmatic_launch(c, st)) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 0) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    if (cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...) != cudaSuccess) { cudaGetLastError(); return SPARROW_ERR_CUDA; }
+    c->launches.fetch_add(1);
+    return SPARROW_OK;
+}
+
+sparrow_status launch_combine(sparrow_ctx* c, const SplitPlan& plan, const SyncArgs& sy, void* out, float* lse, cudaStream_t st)
 {
     CombineArgs ca;
     ca.o_part = o_part_ptr(c, sy.parity);
@@ -369,24 +408,12 @@ sparrow_status launch_combine(sparrow_ctx* c, const SplitPlan& plan, const SyncA
     const int rows = plan.batch * plan.n_kv_heads * plan.M;
     int ctas = (rows + combine::kWarps - 1) / combine::kWarps;
     if (ctas > 8 * c->n_sm) ctas = 8 * c->n_sm;
-    cudaLaunchConfig_t cfg;
-    std::memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(combine::kWarps * 32);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = programmatic ? 1 : 0;       // its CTAs become resident while the split-KV pass runs and wait for it
-    if (cudaLaunchKernelEx(&cfg, combine::combine_kernel, plan, ca) != cudaSuccess) { cudaGetLastError(); return SPARROW_ERR_CUDA; }
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, combine::combine_kernel, (unsigned)ctas, combine::kWarps * 32, 0, st, 0, plan, ca);
 }
 
 sparrow_status launch_split_gather(sparrow_ctx* c, const SplitPlan& plan, const SyncArgs& sy, const void* q, const void* k, const void* v,
                                    const int32_t* parents, const int32_t* anchor_idx, int n_anchor, int window,
-                                   void* out, float* lse, cudaStream_t st, bool early_dependents = false, int tree_nodes = 0)
+                                   void* out, float* lse, cudaStream_t st, int tree_nodes = 0)
 {
     SplitArgs a;
     a.q = static_cast<const __nv_bfloat16*>(q);
@@ -406,12 +433,8 @@ sparrow_status launch_split_gather(sparrow_ctx* c, const SplitPlan& plan, const 
     a.out = static_cast<__nv_bfloat16*>(out);
     a.lse = lse;
     a.status = reinterpret_cast<unsigned*>(c->ws);
-    a.early_dependents = early_dependents ? 1 : 0;
     other_kernel_enqueued();
-    gather::split_gather_kernel<<<plan.n_items, gather::kThreads, gather::kSmemBytes, st>>>(plan, a);
-    if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, gather::split_gather_kernel, (unsigned)plan.n_items, gather::kThreads, gather::kSmemBytes, st, 0, plan, a);
 }
 
 // Cached tensor maps.  tag == 0: one K or V buffer, dims (128 dims, capacity rows, KV heads,
@@ -467,8 +490,7 @@ void clear_tensor_maps(sparrow_ctx* c)
 }
 
 sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const SyncArgs& sy, const void* q, const void* k, const void* v,
-                                const int32_t* parents, const int32_t* first_visible, void* out, float* lse, cudaStream_t st,
-                                bool start_early)
+                                const int32_t* parents, const int32_t* first_visible, void* out, float* lse, cudaStream_t st)
 {
     CUtensorMap mq, mk, mv;
     if (!tensor_map_for(c, q, plan.batch * plan.T, &mq) || !tensor_map_for(c, k, 0, &mk) || !tensor_map_for(c, v, 0, &mv))
@@ -493,10 +515,10 @@ sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const Syn
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    // A call may start early behind the kernel launched directly before it in the stream only
-    // where the caller of this function has made sure that that kernel is this context's previous
-    // call; every other launch takes plain stream order.
-    cfg.numAttrs = start_early ? 1 : 0;
+    // Programmatic: an early start (only where verify_call() has made sure that the kernel directly
+    // before is this context's previous call), or, with wait_first, stream order with the launch and
+    // the set-up overlapping the predecessor's end.
+    cfg.numAttrs = sy.enabled ? 1 : 0;
     const cudaError_t e = nb == 1 ? cudaLaunchKernelEx(&cfg, tc::verify_tc_kernel<1>, a, sy, plan, mq, mk, mv)
                                   : cudaLaunchKernelEx(&cfg, tc::verify_tc_kernel<2>, a, sy, plan, mq, mk, mv);
     if (e != cudaSuccess) return SPARROW_ERR_CUDA;
@@ -609,31 +631,33 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     // nothing about another context's writes; nothing else can sit in between for the calls after
     // the first of sparrow_verify_attn_batch(), or once the caller has vouched for the stream with
     // sparrow_set_call_overlap()), and where it reads nothing that a call which may still be
-    // running writes.  Every other launch takes plain stream order.  A captured call is two plain
+    // running writes.  Every other launch takes stream order.  A captured call is two plain
     // launches: the split-KV pass and the combine kernel.
     const CallRanges cr = call_ranges(c, q, k, v, parents, T_tree, T, first_visible, out, lse);
     const bool protocol = call_overlaps(c, st, true);                // not capturing, programmatic launch on
     const bool same_ctx_before = g_last_fused_ctx.exchange(c) == c;
     const bool early = protocol && same_ctx_before && (c->chain_next || c->overlap_single_calls) &&
                        !inputs_touch_recent_outputs(c, cr);
+    const bool may_share = protocol;
     SplitPlan plan;
     const int group = layout_group(c->layout);
-    sparrow_status s = make_plan(plan_target(c, protocol), c->layout.batch, c->layout.n_kv_heads, group, n_keys, T,
+    sparrow_status s = make_plan(plan_target(c, may_share), c->layout.batch, c->layout.n_kv_heads, group, n_keys, T,
                                  blocks_per_group_tc(T, group), &plan, kMinPieceKeys, key0);
     if (s != SPARROW_OK) return s;
     plan.T_tree = T_tree;
     for (int b = 0; b < c->layout.batch; ++b) plan.seq[b].kv_len = kv_len[b];
     if ((s = check_ws(c, plan)) != SPARROW_OK) return s;
-    const SyncArgs sy = next_sync(c, plan, protocol, outputs_touch_previous(c, cr));
+    SyncArgs sy = next_sync(c, plan, protocol, outputs_touch_previous(c, cr), may_share);
+    sy.wait_first = protocol && !early;
     if (c->log_plans) {
         std::fprintf(stderr, "[sparrow] verify call %u: T %d of %d nodes, %d row block(s) x %d group(s), %d items (target %d), %s, %s;",
-                     c->seq, T, T_tree, plan.blocks_per_group, plan.n_groups, plan.n_items, plan_target(c, protocol),
-                     protocol ? "counter protocol" : "stream-ordered", early ? "starts early" : "plain launch");
+                     c->seq, T, T_tree, plan.blocks_per_group, plan.n_groups, plan.n_items, plan_target(c, may_share),
+                     protocol ? "counter protocol" : "stream-ordered", early ? "starts early" : "stream order");
         for (int b = 0; b < plan.batch; ++b)
             std::fprintf(stderr, " seq %d: keys [%d, %d) in %d piece(s)", b, plan.seq[b].key0, plan.seq[b].n_keys, plan.seq[b].n_splits);
         std::fprintf(stderr, "; %d finisher(s)\n", sy.n_fin);
     }
-    if ((s = launch_verify_tc(c, plan, sy, q, k, v, parents, first_visible, out, lse, st, early)) != SPARROW_OK) return s;
+    if ((s = launch_verify_tc(c, plan, sy, q, k, v, parents, first_visible, out, lse, st)) != SPARROW_OK) return s;
     if (protocol) {
         advance_sync(c, plan, sy);
         std::memcpy(c->prev_ranges, cr.r, sizeof(cr.r));
@@ -722,7 +746,7 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
     c->overlap_single_calls = false;
     const char* lg = std::getenv("SPARROW_LOG");
     c->log_plans = lg && lg[0] == '1';
-    c->chain_next = false;
+    c->chain_next = c->in_batch = false;
     c->n_recent = c->recent_head = 0;
     c->seq = 0;
     c->fin_total[0] = c->fin_total[1] = 0;
@@ -899,7 +923,7 @@ sparrow_status sparrow_verify_attn_static(const sparrow_layout* L, const void* q
         c->launches.store(0);
         c->use_pdl = false;
         c->overlap_single_calls = false;
-        c->chain_next = false;
+        c->chain_next = c->in_batch = false;
         c->n_recent = c->recent_head = 0;
         c->seq = 0;
         c->fin_total[0] = c->fin_total[1] = 0;
@@ -931,8 +955,9 @@ sparrow_status sparrow_verify_attn_batch(sparrow_ctx* c, const sparrow_verify_ca
         const sparrow_verify_call& k = calls[i];
         // from the second call on, the kernel directly before this one in the stream is the previous call's
         c->chain_next = i > 0;
+        c->in_batch = true;
         const sparrow_status s = sparrow_verify_attn(c, k.q, k.k_cache, k.v_cache, k.kv_len, k.parents, k.T, k.out, k.lse, stream);
-        c->chain_next = false;
+        c->chain_next = c->in_batch = false;
         if (s != SPARROW_OK) return s;
     }
     return SPARROW_OK;
@@ -959,15 +984,10 @@ sparrow_status anchor_call(sparrow_ctx* c, const void* q, const void* k, const v
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const SyncArgs sy = next_sync(c, plan, false, true);
-    // the two kernels of the call are chained programmatically unless the stream is being captured
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
-    const bool chained = c->use_pdl && cap == cudaStreamCaptureStatusNone;
-    if ((s = launch_split_gather(c, plan, sy, q, k, v, parents, anchor_idx, n_anchor, window, out, lse, st, chained,
-                                 tree_nodes)) != SPARROW_OK)
+    const SyncArgs sy = next_sync(c, plan, false, true, false);
+    if ((s = launch_split_gather(c, plan, sy, q, k, v, parents, anchor_idx, n_anchor, window, out, lse, st, tree_nodes)) != SPARROW_OK)
         return s;
-    return launch_combine(c, plan, sy, out, lse, st, chained);
+    return launch_combine(c, plan, sy, out, lse, st);
 }
 }  // namespace
 
@@ -1023,10 +1043,7 @@ sparrow_status sparrow_kv_append(sparrow_ctx* c, const void* k_new, const void* 
     if (!guard.ok) return SPARROW_ERR_CUDA;
     const long long threads = (long long)L.batch * L.n_kv_heads * T * 16;
     other_kernel_enqueued();
-    move_rows_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, move_rows_kernel, (unsigned)((threads + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream), 0, a);
 }
 
 sparrow_status sparrow_compact_anchors(sparrow_ctx* c, const void* k, const void* v, const int32_t* anchor_idx,
@@ -1062,10 +1079,7 @@ sparrow_status sparrow_compact_anchors(sparrow_ctx* c, const void* k, const void
     long long blocks = (threads + 255) / 256;
     if (blocks > 8LL * c->n_sm) blocks = 8LL * c->n_sm;
     other_kernel_enqueued();
-    move_rows_kernel<<<(unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, move_rows_kernel, (unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream), 0, a);
 }
 
 sparrow_status sparrow_window_first_visible(const int32_t* anchor_idx, int32_t n_anchor, int32_t window, int32_t T_tree,
@@ -1098,11 +1112,8 @@ sparrow_status sparrow_window_first_visible_device(sparrow_ctx* c, const int32_t
     if (!guard.ok) return SPARROW_ERR_CUDA;
     const int n = c->layout.batch * T_new;
     other_kernel_enqueued();
-    window_bounds_kernel<<<(n + 127) / 128, 128, 0, static_cast<cudaStream_t>(stream)>>>(anchor_idx, n_anchor, window, T_tree, T_new,
-                                                                                         c->layout.batch, first_visible);
-    if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, window_bounds_kernel, (unsigned)((n + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream), 0, anchor_idx, n_anchor, window, T_tree,
+                         T_new, c->layout.batch, first_visible);
 }
 
 // K-range slices per feature tile: about one work item per SM, never more slices than K tiles.
@@ -1156,21 +1167,9 @@ sparrow_status sparrow_hsr_fuse(sparrow_ctx* c, const void* e, const void* h, co
     a.n_slices = n_slices;
     a.k_tiles = 2 * d / hsr::kKTile;
     other_kernel_enqueued();
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((d_out / hsr::kFeat) * n_slices));
-    cfg.blockDim = dim3(hsr::kThreadsHsr);
-    cfg.dynamicSmemBytes = hsr::kSmemBytes;
-    cfg.stream = static_cast<cudaStream_t>(stream);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;              // the slices of a feature tile share a cluster
-    attr[0].val.clusterDim.x = (unsigned)n_slices;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, hsr::hsr_fuse_kernel, a, mw, me, mh) != cudaSuccess) { cudaGetLastError(); return SPARROW_ERR_CUDA; }
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    // (the slices of a feature tile share a cluster)
+    return launch_behind(c, hsr::hsr_fuse_kernel, (unsigned)((d_out / hsr::kFeat) * n_slices), hsr::kThreadsHsr, hsr::kSmemBytes,
+                         static_cast<cudaStream_t>(stream), (unsigned)n_slices, a, mw, me, mh);
 }
 
 sparrow_status sparrow_accept_greedy(sparrow_ctx* c, const int32_t* draft_tokens, const int32_t* parents,
@@ -1183,12 +1182,8 @@ sparrow_status sparrow_accept_greedy(sparrow_ctx* c, const int32_t* draft_tokens
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     other_kernel_enqueued();
-    accept_greedy_kernel<<<1, kMaxBatch, 0, static_cast<cudaStream_t>(stream)>>>(
-        draft_tokens, parents, target_next, c->layout.batch, T, path_out, n_accept_out, bonus_out,
-        reinterpret_cast<unsigned*>(c->ws));
-    if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, accept_greedy_kernel, 1, kMaxBatch, 0, static_cast<cudaStream_t>(stream), 0, draft_tokens, parents, target_next, c->layout.batch, T,
+                         path_out, n_accept_out, bonus_out, reinterpret_cast<unsigned*>(c->ws));
 }
 
 sparrow_status sparrow_accept_sample(sparrow_ctx* c, const int32_t* draft_tokens, const int32_t* parents, const float* p_target,
@@ -1208,25 +1203,10 @@ sparrow_status sparrow_accept_sample(sparrow_ctx* c, const int32_t* draft_tokens
     while (n_cta < c->max_sample_cluster && vocab >= 2 * n_cta * sample::kMinSlice && 2 * n_cta * c->layout.batch <= c->n_sm) n_cta *= 2;
     const int per_cta = (vocab + n_cta - 1) / n_cta;
     const int resident = per_cta < sample::kMaxResident ? per_cta : sample::kMaxResident;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(c->layout.batch * n_cta));
-    cfg.blockDim = dim3(sample::kThreads);
-    cfg.dynamicSmemBytes = (size_t)resident * sizeof(uint2);
-    cfg.stream = static_cast<cudaStream_t>(stream);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)n_cta;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, sample::accept_sample_kernel, draft_tokens, parents, p_target, p_draft, u_node, u_bonus, T, vocab, n_cta,
-                           resident, path_out, n_accept_out, bonus_out, reinterpret_cast<unsigned*>(c->ws)) != cudaSuccess) {
-        cudaGetLastError();
-        return SPARROW_ERR_CUDA;
-    }
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, sample::accept_sample_kernel, (unsigned)(c->layout.batch * n_cta), sample::kThreads,
+                         (size_t)resident * sizeof(uint2), static_cast<cudaStream_t>(stream), (unsigned)n_cta, draft_tokens, parents, p_target,
+                         p_draft, u_node, u_bonus, T, vocab, n_cta, resident, path_out, n_accept_out, bonus_out,
+                         reinterpret_cast<unsigned*>(c->ws));
 }
 
 sparrow_status sparrow_kv_keep_accepted(sparrow_ctx* c, void* k_cache, void* v_cache, const int32_t* kv_len,
@@ -1253,10 +1233,7 @@ sparrow_status sparrow_kv_keep_accepted(sparrow_ctx* c, void* k_cache, void* v_c
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     other_kernel_enqueued();
-    keep_accepted_rows_kernel<<<L.batch * L.n_kv_heads, 256, (size_t)2 * T * 256, static_cast<cudaStream_t>(stream)>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
-    c->launches.fetch_add(1);
-    return SPARROW_OK;
+    return launch_behind(c, keep_accepted_rows_kernel, (unsigned)(L.batch * L.n_kv_heads), 256, (size_t)2 * T * 256, static_cast<cudaStream_t>(stream), 0, a);
 }
 
 sparrow_status sparrow_verify_step_host(sparrow_ctx* c, const void* q_host, const void* k_new_host,
@@ -1321,9 +1298,8 @@ sparrow_status sparrow_verify_step_host(sparrow_ctx* c, const void* q_host, cons
         ia.n_parents = L.batch * T;
         const long long work = (long long)(new_bytes / 16) + ia.q_chunks + ia.n_parents;
         other_kernel_enqueued();
-        ingest_step_kernel<<<(unsigned)((work + 255) / 256), 256, 0, st>>>(ia);
-        if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
-        c->launches.fetch_add(1);
+        const sparrow_status is = launch_behind(c, ingest_step_kernel, (unsigned)((work + 255) / 256), 256, 0, st, 0, ia);
+        if (is != SPARROW_OK) return is;
         const sparrow_status s = sparrow_verify_attn(c, q_dev, k_cache, v_cache, kv_len, par_dev, T, out_view,
                                                      static_cast<float*>(lse_view), stream);
         if (s != SPARROW_OK) return s;

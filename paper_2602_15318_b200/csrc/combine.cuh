@@ -147,7 +147,8 @@ combine_kernel(const __grid_constant__ SplitPlan plan, const __grid_constant__ C
 {
     // Launched programmatically behind the split-KV kernel it may start early: wait for that grid
     // to complete (with its writes visible).  Without a programmatic dependency this returns at once.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    let_dependents_launch();
+    wait_for_predecessors();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rows_total = plan.batch * plan.n_kv_heads * plan.M;
     for (int row_id = blockIdx.x * kWarps + warp; row_id < rows_total; row_id += gridDim.x * kWarps) {

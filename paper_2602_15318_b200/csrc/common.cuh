@@ -94,8 +94,8 @@ constexpr int kPartRowHalves = 136;
 
 // Overlapped mode: ordering between the CTAs of one call and between consecutive calls.
 //
-// The split-KV kernel is launched with programmatic stream serialisation and never waits for the
-// previous grid as a whole, so the next call's CTAs start (and read their inputs) while the
+// A call that starts early is launched with programmatic stream serialisation and does not wait for the
+// previous grid as a whole (but for CTA 0, which does before it leaves), so the next call's CTAs start (and read their inputs) while the
 // previous call is still finishing.  What must be ordered goes through counters in the workspace,
 // released / acquired at GPU scope.  Partial buffers are double-buffered by the parity of the call
 // number n, arrival words rotate over n modulo 4.
@@ -127,6 +127,7 @@ struct SyncArgs {
     int32_t n_fin;           // finisher CTAs of this call (0 when no unit has several pieces)
     uint32_t fin_wait_same;
     uint32_t fin_wait_other;
+    int32_t wait_first;      // launched with programmatic stream serialisation but ordered behind its predecessor: wait before the first global access
     uint32_t call;           // running number of the context's fused calls (the timeline build files its stamps under it)
 };
 
@@ -166,6 +167,14 @@ __device__ __forceinline__ void publish_counter(unsigned* addr)
 {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(addr) : "memory");
 }
+
+// Launch overlap between kernels in stream order.  A kernel launched with programmatic stream
+// serialisation starts while its predecessor is finishing, and wait_for_predecessors() holds it, in front
+// of its first access to global memory, until the predecessor has completed with its writes visible.
+// Every kernel of this library either waits like that or (early-started verification calls) does so
+// before its grid ends, so completion of the predecessor implies completion of everything before it.
+__device__ __forceinline__ void wait_for_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 struct Item {
     int b, kvh, group, split, key_begin, key_end;

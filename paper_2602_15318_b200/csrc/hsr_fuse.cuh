@@ -137,6 +137,7 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
         mbar_init(done, 1);
         *abort_flag = 0;
         fence_barrier_init();
+        wait_for_predecessors();
         for (int i = 0; i < n_st && i < kStages; ++i) issue(i);
     }
     if (warp == 5) {
@@ -147,6 +148,7 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    let_dependents_launch();
     if (tid == 0) SPARROW_STAMP(1);                                     // set-up done
 
     const int feat_local = (warp & 3) * 32 + lane;

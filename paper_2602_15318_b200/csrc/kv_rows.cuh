@@ -53,6 +53,8 @@ __device__ __forceinline__ void move_row_chunk(const RowMoveArgs& a, long long i
 __global__ void __launch_bounds__(256)
 move_rows_kernel(const __grid_constant__ RowMoveArgs a)
 {
+    let_dependents_launch();
+    wait_for_predecessors();
     const long long total = (long long)a.batch * a.n_kv_heads * a.n_rows * 16;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
         move_row_chunk(a, i);
@@ -74,6 +76,8 @@ struct IngestArgs {
 __global__ void __launch_bounds__(256)
 ingest_step_kernel(const __grid_constant__ IngestArgs a)
 {
+    let_dependents_launch();
+    wait_for_predecessors();
     const long long row_chunks = (long long)a.rows.batch * a.rows.n_kv_heads * a.rows.n_rows * 16;
     const long long total = row_chunks + a.q_chunks + a.n_parents;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {

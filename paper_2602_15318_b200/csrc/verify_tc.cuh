@@ -422,8 +422,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         *abort_flag = 0;
         *write_ok = sync.enabled ? 0u : 1u;
         fence_barrier_init();
+        if (sync.wait_first) wait_for_predecessors();
         // Q first (the first S = Q K^T needs it and it is small), then K and V tiles in the order
-        // they are consumed.  Nothing here depends on the previous kernel in the stream.
+        // they are consumed.
         mbar_expect_tx(B.q_full(), (uint32_t)(NB * 2 * 64 * qg * tpb * 2));   // two boxes of 64 dims x g heads x p tokens per block
         #pragma unroll
         for (int blk = 0; blk < NB; ++blk) {
@@ -440,6 +441,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     }
     if (warp == 0) {
         const int Tt = plan.T_tree;
+        if (sync.wait_first) wait_for_predecessors();
         if (it.key_end > kv_len) {                   // this piece reaches the draft block: it needs the tree
             const int32_t* par_g = args.parents + (size_t)it.b * Tt;
             if (lane < Tt) par_s[lane] = __ldg(par_g + lane);
@@ -465,7 +467,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 0) SPARROW_STAMP(1);                             // set-up done
-    if (sync.enabled) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // (behind the wait above: a dependent that starts early may rely on everything before this call)
+    if (sync.enabled) let_dependents_launch();
 
     if (warp == kProducerWarp) {
         // ================= TMA producer =================
@@ -1132,6 +1135,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);
         __syncthreads();
     }
+    // an early-started call must not complete before its predecessors (see wait_for_predecessors)
+    if (sync.enabled && !sync.wait_first && blockIdx.x == 0 && threadIdx.x == 0) wait_for_predecessors();
     if (threadIdx.x == 0) SPARROW_STAMP(11);                            // leaving
     if (warp == kMmaWarp) {
         tc_fence_after();

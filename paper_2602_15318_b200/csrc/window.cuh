@@ -23,6 +23,8 @@ __host__ __device__ __forceinline__ int first_anchor_above(const int32_t* anchor
 __global__ void window_bounds_kernel(const int32_t* __restrict__ anchor_idx, int n_anchor, int window, int T_tree, int T_new,
                                      int batch, int32_t* __restrict__ first_visible)
 {
+    let_dependents_launch();
+    wait_for_predecessors();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= batch * T_new) return;
     const int b = i / T_new, t = i - b * T_new;
