@@ -92,8 +92,9 @@ sparrow_status sparrow_destroy(sparrow_ctx* ctx);
  *   THROUGHPUT  about n_sm / 7 items: longest pieces, several calls resident at once; best when
  *               many independent calls are queued back to back (one per layer or per request).
  * Results differ between policies only by the rounding order of the split-KV merge.  Calls that
- * cannot overlap (graph capture, SPARROW_NO_PDL, sparrow_anchor_attn, sparrow_verify_attn_static)
- * always use one wave over all SMs. */
+ * share the GPU with no other call of the context (single calls without sparrow_set_call_overlap(), graph
+ * capture, SPARROW_NO_PDL, sparrow_anchor_attn, sparrow_verify_attn_static) always use one wave
+ * over all SMs. */
 typedef enum {
     SPARROW_PLAN_LATENCY    = 0,
     SPARROW_PLAN_BALANCED   = 1,
@@ -136,8 +137,9 @@ sparrow_status sparrow_set_workspace(sparrow_ctx* ctx, void* dev_ptr, size_t byt
  * One kernel per call: a split-KV pass over ~one work item per SM whose last CTAs merge the
  * pieces by log-sum-exp.
  *
- * Ordering.  By default a call is an ordinary launch: it starts after everything enqueued before
- * it on `stream` has finished.  Where the library knows that the kernel directly before a call in
+ * Ordering.  By default a call is ordered by the stream: it touches no memory before everything
+ * enqueued before it on `stream` has finished (its launch and set-up may overlap the end of the kernel
+ * directly before it, as those of every kernel of this library).  Where the library knows that the kernel directly before a call in
  * the stream is this context's previous verification call, the call starts early (programmatic
  * stream serialisation): it reads q / k_cache / v_cache / parents while that call is still
  * finishing, and several calls can be resident at once.  That is the case

@@ -638,7 +638,12 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     const bool same_ctx_before = g_last_fused_ctx.exchange(c) == c;
     const bool early = protocol && same_ctx_before && (c->chain_next || c->overlap_single_calls) &&
                        !inputs_touch_recent_outputs(c, cr);
-    const bool may_share = protocol;
+    // Can another call of this context run beside this one?  Only inside a batch, or with the opt-in for
+    // single calls.  A call that has the GPU to itself is cut into one wave whatever the policy: measured
+    // single calls, balanced policy's 55 items -> 148 items: 33.0 -> 24.8 us (26,112 keys, T = 16), 52.6 ->
+    // 32.2 (three sequences of 9,001 keys and fewer, T = 23, 8 KV heads), 105 -> 50 (six of 9,000, T = 30),
+    // 16.5 -> 14.8 (2,048 keys, T = 8), no size slower.
+    const bool may_share = protocol && (c->in_batch || c->overlap_single_calls);
     SplitPlan plan;
     const int group = layout_group(c->layout);
     sparrow_status s = make_plan(plan_target(c, may_share), c->layout.batch, c->layout.n_kv_heads, group, n_keys, T,
