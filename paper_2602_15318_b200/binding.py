@@ -1,4 +1,5 @@
-"""ctypes binding of libsparrow_attn: argument marshalling only.
+"""Binding of libsparrow_attn: argument marshalling only -- in C (`_pycall`) for the calls of a decoder's
+step, through ctypes for the rest.
 
 Every step of the attention path runs in the library's CUDA kernels; torch is used here for device
 memory and streams.  The functions carry the C ABI's names and argument order.  There is no CPU
@@ -111,6 +112,45 @@ def _chk(status: int, what: str):
         raise SparrowError(status, what)
 
 
+# C arguments of the calls that go through _pycall: c context, t tensor, i int32, l / L (optional) list of
+# ints -> int32 array, s stream.
+_SIGNATURES = {
+    "sparrow_verify_attn": "ctttltitts",
+    "sparrow_verify_attn_window": "ctttltiitLtts",
+    "sparrow_window_first_visible_device": "ctiiiits",
+    "sparrow_anchor_attn": "cttttiiitts",
+    "sparrow_anchor_attn_tree": "cttttiitiitts",
+    "sparrow_kv_append": "cttttlis",
+    "sparrow_compact_anchors": "ctttittiis",
+    "sparrow_hsr_fuse": "cttttiiits",
+    "sparrow_accept_greedy": "ctttittts",
+    "sparrow_accept_sample": "cttttttiittts",
+    "sparrow_kv_keep_accepted": "cttlttis",
+    "sparrow_verify_step_host": "ctttttltitts",
+}
+
+
+class _Calls:
+    """The library's functions bound through _pycall, loaded at the first use of one."""
+
+    def __getattr__(self, name):
+        if name not in _SIGNATURES:
+            raise AttributeError(name)
+        L = lib()
+        try:
+            from . import _pycall
+        except ImportError as e:
+            raise RuntimeError("the _pycall extension is not built: run `python -m paper_2602_15318_b200.build`") from e
+        torch.cuda.current_stream()                       # brings torch's CUDA state up
+        _pycall.set_stream_functions(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        for fn, sig in _SIGNATURES.items():
+            setattr(self, fn, _pycall.bind(ctypes.cast(getattr(L, fn), ctypes.c_void_p).value, sig, fn, _chk))
+        return self.__dict__[name]
+
+
+_calls = _Calls()
+
+
 def _ptr(t) -> Optional[int]:
     if t is None:
         return None
@@ -119,7 +159,8 @@ def _ptr(t) -> Optional[int]:
 
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream or None
+        torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream or None
     return stream or None
@@ -141,6 +182,7 @@ class Context:
         self.handle = ctypes.c_void_p()
         _chk(lib().sparrow_create(ctypes.byref(self.handle), ctypes.byref(self.layout), device),
              "sparrow_create")
+        self.address = self.handle.value
         self.workspace = None
         if allocate_workspace:
             n = self.workspace_bytes(max_T)
@@ -185,6 +227,7 @@ class Context:
         if self.handle:
             lib().sparrow_destroy(self.handle)
             self.handle = ctypes.c_void_p()
+            self.address = 0
 
     def __del__(self):
         try:
@@ -197,9 +240,7 @@ def sparrow_verify_attn(ctx: Context, q, k_cache, v_cache, kv_len: Sequence[int]
                         out, lse, stream=None):
     """q/out: CUDA bf16 [B,T,Hq,128]; caches: CUDA bf16; kv_len: host ints; parents: CUDA int32
     [B,T]; lse: CUDA fp32 [B,Hq,T]."""
-    kl = _i32_array(kv_len)
-    _chk(lib().sparrow_verify_attn(ctx.handle, _ptr(q), _ptr(k_cache), _ptr(v_cache), kl, _ptr(parents),
-                                   T, _ptr(out), _ptr(lse), _stream_handle(stream)), "sparrow_verify_attn")
+    _calls.sparrow_verify_attn(ctx, q, k_cache, v_cache, kv_len, parents, T, out, lse, stream)
 
 
 def sparrow_verify_attn_window(ctx: Context, q, k_cache, v_cache, kv_len: Sequence[int], parents, T_tree: int,
@@ -207,11 +248,8 @@ def sparrow_verify_attn_window(ctx: Context, q, k_cache, v_cache, kv_len: Sequen
                                stream=None):
     """Verification kernel on a compacted anchored cache: queries = the last T_new of T_tree draft
     nodes; first_visible: CUDA int32 [B,T_new] or None; first_visible_min: host ints or None."""
-    kl = _i32_array(kv_len)
-    fm = _i32_array(first_visible_min) if first_visible_min is not None else None
-    _chk(lib().sparrow_verify_attn_window(ctx.handle, _ptr(q), _ptr(k_cache), _ptr(v_cache), kl, _ptr(parents),
-                                          T_tree, T_new, _ptr(first_visible), fm, _ptr(out), _ptr(lse),
-                                          _stream_handle(stream)), "sparrow_verify_attn_window")
+    _calls.sparrow_verify_attn_window(ctx, q, k_cache, v_cache, kv_len, parents, T_tree, T_new, first_visible, first_visible_min, out, lse,
+                                      stream)
 
 
 def sparrow_window_first_visible(anchor_idx: Sequence[int], window: int, T_tree: int, T_new: int):
@@ -226,9 +264,7 @@ def sparrow_window_first_visible(anchor_idx: Sequence[int], window: int, T_tree:
 
 def sparrow_window_first_visible_device(ctx: Context, anchor_idx, n_anchor: int, window: int, T_tree: int, T_new: int,
                                         first_visible, stream=None):
-    _chk(lib().sparrow_window_first_visible_device(ctx.handle, _ptr(anchor_idx), n_anchor, window, T_tree, T_new,
-                                                   _ptr(first_visible), _stream_handle(stream)),
-         "sparrow_window_first_visible_device")
+    _calls.sparrow_window_first_visible_device(ctx, anchor_idx, n_anchor, window, T_tree, T_new, first_visible, stream)
 
 
 def sparrow_verify_attn_static(layout: Layout, q, k_cache, v_cache, kv_len: Sequence[int], parents, T: int,
@@ -273,36 +309,26 @@ def sparrow_verify_attn_batch(ctx: Context, batch: VerifyBatch, n_calls: Optiona
 
 def sparrow_anchor_attn(ctx: Context, q, k, v, anchor_idx, n_anchor: int, window: int, T: int, out, lse,
                         stream=None):
-    _chk(lib().sparrow_anchor_attn(ctx.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(anchor_idx), n_anchor,
-                                   window, T, _ptr(out), _ptr(lse), _stream_handle(stream)),
-         "sparrow_anchor_attn")
+    _calls.sparrow_anchor_attn(ctx, q, k, v, anchor_idx, n_anchor, window, T, out, lse, stream)
 
 
 def sparrow_anchor_attn_tree(ctx: Context, q, k, v, anchor_idx, n_anchor: int, window: int, parents, T_tree: int,
                              T_new: int, out, lse, stream=None):
-    _chk(lib().sparrow_anchor_attn_tree(ctx.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(anchor_idx), n_anchor,
-                                        window, _ptr(parents), T_tree, T_new, _ptr(out), _ptr(lse),
-                                        _stream_handle(stream)),
-         "sparrow_anchor_attn_tree")
+    _calls.sparrow_anchor_attn_tree(ctx, q, k, v, anchor_idx, n_anchor, window, parents, T_tree, T_new, out, lse, stream)
 
 
 def sparrow_kv_append(ctx: Context, k_new, v_new, k_cache, v_cache, kv_len: Sequence[int], T: int, stream=None):
-    _chk(lib().sparrow_kv_append(ctx.handle, _ptr(k_new), _ptr(v_new), _ptr(k_cache), _ptr(v_cache),
-                                 _i32_array(kv_len), T, _stream_handle(stream)), "sparrow_kv_append")
+    _calls.sparrow_kv_append(ctx, k_new, v_new, k_cache, v_cache, kv_len, T, stream)
 
 
 def sparrow_compact_anchors(ctx: Context, k, v, anchor_idx, n_anchor: int, k_compact, v_compact,
                             compact_capacity: int, dst_row: int = 0, stream=None):
-    _chk(lib().sparrow_compact_anchors(ctx.handle, _ptr(k), _ptr(v), _ptr(anchor_idx), n_anchor, _ptr(k_compact),
-                                       _ptr(v_compact), compact_capacity, dst_row, _stream_handle(stream)),
-         "sparrow_compact_anchors")
+    _calls.sparrow_compact_anchors(ctx, k, v, anchor_idx, n_anchor, k_compact, v_compact, compact_capacity, dst_row, stream)
 
 
 def sparrow_accept_greedy(ctx: Context, draft_tokens, parents, target_next, T: int, path_out, n_accept_out,
                           bonus_out, stream=None):
-    _chk(lib().sparrow_accept_greedy(ctx.handle, _ptr(draft_tokens), _ptr(parents), _ptr(target_next), T,
-                                     _ptr(path_out), _ptr(n_accept_out), _ptr(bonus_out), _stream_handle(stream)),
-         "sparrow_accept_greedy")
+    _calls.sparrow_accept_greedy(ctx, draft_tokens, parents, target_next, T, path_out, n_accept_out, bonus_out, stream)
 
 
 def sparrow_hsr_fuse(ctx: Context, e, h, w, bias, z, stream=None):
@@ -310,34 +336,26 @@ def sparrow_hsr_fuse(ctx: Context, e, h, w, bias, z, stream=None):
     [d_out] or None; z: CUDA bf16 [M, d_out]."""
     M, d = e.shape
     d_out = w.shape[0]
-    _chk(lib().sparrow_hsr_fuse(ctx.handle, _ptr(e), _ptr(h), _ptr(w), _ptr(bias), M, d, d_out, _ptr(z),
-                                _stream_handle(stream)),
-         "sparrow_hsr_fuse")
+    _calls.sparrow_hsr_fuse(ctx, e, h, w, bias, M, d, d_out, z, stream)
 
 
 def sparrow_accept_sample(ctx: Context, draft_tokens, parents, p_target, p_draft, u_node, u_bonus, vocab: int, T: int,
                           path_out, n_accept_out, bonus_out, stream=None):
     """Temperature-1 acceptance.  p_target / p_draft: CUDA fp32 [B, T+1, vocab]; u_node: CUDA int32
     [B, T] and u_bonus: CUDA int32 [B, T+1] holding the bit patterns of 32-bit unsigned uniforms."""
-    _chk(lib().sparrow_accept_sample(ctx.handle, _ptr(draft_tokens), _ptr(parents), _ptr(p_target), _ptr(p_draft),
-                                     _ptr(u_node), _ptr(u_bonus), vocab, T, _ptr(path_out), _ptr(n_accept_out),
-                                     _ptr(bonus_out), _stream_handle(stream)), "sparrow_accept_sample")
+    _calls.sparrow_accept_sample(ctx, draft_tokens, parents, p_target, p_draft, u_node, u_bonus, vocab, T, path_out, n_accept_out, bonus_out,
+                                 stream)
 
 
 def sparrow_kv_keep_accepted(ctx: Context, k_cache, v_cache, kv_len: Sequence[int], path, n_accept, T: int,
                              stream=None):
-    _chk(lib().sparrow_kv_keep_accepted(ctx.handle, _ptr(k_cache), _ptr(v_cache), _i32_array(kv_len), _ptr(path),
-                                        _ptr(n_accept), T, _stream_handle(stream)), "sparrow_kv_keep_accepted")
+    _calls.sparrow_kv_keep_accepted(ctx, k_cache, v_cache, kv_len, path, n_accept, T, stream)
 
 
 def sparrow_verify_step_host(ctx: Context, q_host, k_new_host, v_new_host, k_cache, v_cache,
                              kv_len: Sequence[int], parents_host, T: int, out_host, lse_host, stream=None):
     """Host tensors (ideally pinned) in and out; the caches stay on the device."""
-    kl = _i32_array(kv_len)
-    _chk(lib().sparrow_verify_step_host(ctx.handle, _ptr(q_host), _ptr(k_new_host), _ptr(v_new_host),
-                                        _ptr(k_cache), _ptr(v_cache), kl, _ptr(parents_host), T,
-                                        _ptr(out_host), _ptr(lse_host), _stream_handle(stream)),
-         "sparrow_verify_step_host")
+    _calls.sparrow_verify_step_host(ctx, q_host, k_new_host, v_new_host, k_cache, v_cache, kv_len, parents_host, T, out_host, lse_host, stream)
 
 
 def sparrow_build_ancestor_masks(parents: Sequence[int]):

@@ -1,12 +1,16 @@
-"""Builds libsparrow_attn.so (C ABI, sm_100a only) in-tree with nvcc."""
+"""Builds libsparrow_attn.so (C ABI, sm_100a only; nvcc) and _pycall.so (the Python binding's argument
+marshalling; gcc) in-tree."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsparrow_attn.so")
+PYCALL = os.path.join(HERE, "_pycall.so")
+PYCALL_SOURCE = os.path.join(CSRC, "pycall.c")
 SOURCES = [os.path.join(CSRC, "api.cu")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC"]
@@ -27,7 +31,15 @@ def nvcc() -> str:
     return "nvcc"
 
 
+def build_pycall(force: bool = False) -> str:
+    if force or not os.path.exists(PYCALL) or os.path.getmtime(PYCALL) < os.path.getmtime(PYCALL_SOURCE):
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], "-o", PYCALL,
+                        PYCALL_SOURCE], check=True)
+    return PYCALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_pycall(force)
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source():
         return LIB
     cmd = [nvcc()] + NVCC_FLAGS + ["-I" + os.path.join(ROOT, "include"), "-I" + CSRC, "-o", LIB] + SOURCES
