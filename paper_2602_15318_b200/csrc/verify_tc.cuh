@@ -18,15 +18,24 @@
 //                        stored back with tcgen05.st.
 //                        One row block (T <= 18): the two threads with the same lane (warps w and
 //                        w + 4) share a row, warpgroup g taking key columns [64 g, 64 g + 64) of every
-//                        job.  They keep the same reference maximum: one barrier with an OR reduction
-//                        per job tells whether any row's maximum grew by more than 2^8; only then the
-//                        halves' maxima meet in shared memory and O is rescaled in TMEM.  Each
-//                        thread sums its own columns; the halves' sums meet once, in the epilogue.
+//                        tile, with its P over its own scores.  They keep the same reference maximum:
+//                        one barrier with an OR reduction per tile tells whether any row's maximum grew
+//                        by more than 2^8; only then the halves' maxima meet in shared memory and O is
+//                        rescaled in TMEM.  Each thread sums its own columns; the halves' sums meet
+//                        once, in the epilogue.
 //                        Two row blocks: warpgroup g owns block g, one thread per row and all 128
 //                        keys of a tile, and works through its block's tiles on its own (no
 //                        barrier between the warpgroups); per block the chain is scores -> softmax
 //                        -> O += P V -> next scores, and the two chains interleave on the tensor
-//                        pipe and the exponential unit.
+//                        pipe and the exponential unit.  P is handed over in two halves, the first
+//                        half's product running beside the exponentials of the second.
+//                        The loops are rolled around 64 scores: what a tile costs beyond its
+//                        exponentials (1,024 cycles a block) is mostly instruction supply and hand-over
+//                        latency.  Two blocks, 36 tokens, cycles per tile: 3,900 with both passes unrolled
+//                        over 128 scores, 3,480 like this; sixteen softmax warps (a warpgroup per half row)
+//                        3,500; 64-key steps with their own N = 64 products slower (the 64-column product
+//                        takes 48 cycles instead of 32).  Long streams of calls run at the power limit
+//                        (1,000 W, 1.5 GHz) whatever the loop looks like.
 //   warp 10, one thread  gatekeeper (overlapped mode): waits, beside the main loop, for the counters
 //                        that allow this CTA's first global write.
 //
@@ -198,6 +207,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v)
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
+{
+    uint32_t* r = reinterpret_cast<uint32_t*>(v);
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r)
@@ -534,15 +553,25 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     if (!mbar_wait_warp(B.p_full(b), j & 1)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
-                    if (elect_one()) {
-                        #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)
-                            mma_ts(tmem_u + 256 + b * 128, tmem_u + b * 128 + 64 + kk * 8, vd + (uint64_t)((kk * 2048) >> 4),
-                                   idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
-                        tc_commit(B.o_done(b, j));
-                        if (b == 1) tc_commit(B.v_empty(st));
+                    #pragma unroll
+                    for (int half = 0; half < 2; ++half) {                    // keys 64-127, then 0-63, as their P arrives
+                        if (half == 1) {
+                            if (!mbar_wait_warp(B.p_full(2 + b), j & 1)) { ok = false; break; }
+                            tc_fence_after();
+                        }
+                        if (elect_one()) {
+                            #pragma unroll
+                            for (int kk = 4 - half * 4; kk < 8 - half * 4; ++kk)
+                                mma_ts(tmem_u + 256 + b * 128, tmem_u + b * 128 + 64 + kk * 8, vd + (uint64_t)((kk * 2048) >> 4),
+                                       idesc_pv, (j > 0 || half > 0 || kk > 4) ? 1u : 0u);
+                            if (half == 1) {
+                                tc_commit(B.o_done(b, j));
+                                if (b == 1) tc_commit(B.v_empty(st));
+                            }
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
+                    if (!ok) break;
                     if (n + 2 < n_jobs) ok = issue_qk2(n + 2);                // this block's next scores
                 }
             } else {
@@ -581,7 +610,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 if (elect_one()) {
                     #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
-                        mma_ts(tmem_u + kOCol + blk * 128, tmem_u + sb * 128 + kk * 8, vd + (uint64_t)((kk * 2048) >> 4),
+                        mma_ts(tmem_u + kOCol + blk * 128, tmem_u + sb * 128 + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)((kk * 2048) >> 4),
                                idesc_pv, (n >= NB || kk > 0) ? 1u : 0u);
                     tc_commit(B.o_done(blk, j));
                     if (blk == NB - 1) tc_commit(B.v_empty(st));
@@ -631,6 +660,24 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
         bool ok = true;
 
+        // visibility word, for the 64 keys that start at key j0, of a row with ancestor word `anc_row` and lower
+        // window bound `lo` (which never exceeds kv_len): the prefix columns, then the ancestor word shifted to the
+        // draft block's column, cut at the end of the key range and left of the window
+        auto vis_word = [&](int j0, unsigned long long anc_row, int lo) -> unsigned long long {
+            const int d0 = kv_len - j0;                                 // column of draft token 0 (any sign)
+            const int nval = it.key_end - j0;                           // valid columns (may be <= 0)
+            unsigned long long vis;
+            if (d0 >= 64) vis = ~0ull;
+            else if (d0 > 0) vis = ((1ull << d0) - 1ull) | (anc_row << d0);
+            else if (d0 > -64) vis = anc_row >> (-d0);
+            else vis = 0ull;
+            if (nval <= 0) vis = 0ull;
+            else if (nval < 64) vis &= (1ull << nval) - 1ull;
+            const int cut = lo - j0;
+            if (cut >= 64) vis = 0ull;
+            else if (cut > 0) vis &= ~((1ull << cut) - 1ull);
+            return vis;
+        };
         float my_m = -INFINITY, my_l = 0.f;       // two row blocks: the state of this warpgroup's own block
         if constexpr (NB == 2) {
             // ---- two row blocks: warpgroup g owns block g, one thread per query row, and works
@@ -642,54 +689,52 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const int my_lo = wg ? lo_row[NB - 1] : lo_row[0];
             const bool my_ok = wg ? row_ok[NB - 1] : row_ok[0];
             const uint32_t s_addr = lane_addr + blk * 128;
-            // visibility word of this row for the 64 keys that start at key j0
-            auto vis_word = [&](int j0) -> unsigned long long {
-                if (!(j0 + 64 > it.key_end || j0 + 64 > kv_len || j0 < my_lo)) return ~0ull;
-                const int d0 = kv_len - j0;                                 // column of draft token 0 (any sign)
-                const int nval = it.key_end - j0;                           // valid columns (may be <= 0)
-                unsigned long long vis;
-                if (d0 >= 64) vis = ~0ull;
-                else if (d0 > 0) vis = ((1ull << d0) - 1ull) | (my_anc << d0);
-                else if (d0 > -64) vis = my_anc >> (-d0);
-                else vis = 0ull;
-                if (nval <= 0) vis = 0ull;
-                else if (nval < 64) vis &= (1ull << nval) - 1ull;
-                const int cut = my_lo - j0;
-                if (cut >= 64) vis = 0ull;
-                else if (cut > 0) vis &= ~((1ull << cut) - 1ull);
-                return vis;
-            };
-            float x0[32], x1[32];
+            // tiles whose every key is visible to this row: [j_head, j_tail)
+            const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
+            const int j_head = my_lo > it.key_begin ? (my_lo - it.key_begin + kTile - 1) / kTile : 0;
+            // (visibility masks are applied in TMEM, by a pass of their own over the few tiles that need one)
             #pragma unroll 1
             for (int j = 0; j < n_tiles && ok; ++j) {
-                const int st = j % NS;
                 const int tile0 = it.key_begin + j * kTile;
                 if (!mbar_wait_warp(B.s_full(blk), j & 1)) { ok = false; break; }
                 tc_fence_after();
-                // first pass over the row's 128 scores, 64 at a time: the maximum.  The upper 64 stay
-                // in registers; the lower 64 are fetched again for the second pass.
-                tmem_ld32(s_addr, x0);
-                tmem_ld32(s_addr + 32, x1);
-                const unsigned long long vis_lo = vis_word(tile0), vis_hi = vis_word(tile0 + 64);
                 // V rows past the end of the sequence may hold anything: zero them so 0 * x stays 0
                 // (once per tile, by the threads of the first block, thread r taking key row r)
                 if (blk == 0 && tile0 + kTile > n_keys_seq && tile0 + row_local >= n_keys_seq) {
+                    const int st = j % NS;
                     mbar_wait(B.v_full(st), (j / NS) & 1);
                     unsigned char* vrow = kv_sm + st * kStageBytes + 2 * kSubTileBytes + row_local * 128;
-                    #pragma unroll
+                    #pragma unroll 1
                     for (int c = 0; c < 8; ++c) {
                         *reinterpret_cast<uint4*>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
                         *reinterpret_cast<uint4*>(vrow + kSubTileBytes + c * 16) = make_uint4(0, 0, 0, 0);
                     }
                     fence_proxy_async();
                 }
+                __syncwarp();
+                if (__any_sync(0xffffffffu, j >= j_tail || j < j_head)) {  // the tile crosses a visibility boundary of some row
+                    const unsigned long long lo = vis_word(tile0, my_anc, my_lo), hi = vis_word(tile0 + 64, my_anc, my_lo);
+                    #pragma unroll 1
+                    for (int ch = 0; ch < 4; ++ch) {                       // 32 keys at a time, where any row has one to hide
+                        const uint32_t vis = (uint32_t)((ch & 2 ? hi : lo) >> (32 * (ch & 1)));
+                        if (!__any_sync(0xffffffffu, vis != ~0u)) continue;
+                        float x[32];
+                        tmem_ld32(s_addr + 32 * ch, x);
+                        tmem_wait_ld();
+                        mask_chunk(x, vis);
+                        tmem_st32(s_addr + 32 * ch, reinterpret_cast<uint32_t*>(x));
+                    }
+                    tmem_wait_st();
+                }
+                // first pass over the row's 128 scores, 64 at a time: the maximum
+                float x0[32], x1[32];
+                tmem_ld32(s_addr, x0);
+                tmem_ld32(s_addr + 32, x1);
                 tmem_wait_ld();
-                if (vis_lo != ~0ull) { mask_chunk(x0, (uint32_t)vis_lo); mask_chunk(x1, (uint32_t)(vis_lo >> 32)); }
                 float mx = fmaxf(chunk_max(x0), chunk_max(x1));
                 tmem_ld32(s_addr + 64, x0);
                 tmem_ld32(s_addr + 96, x1);
                 tmem_wait_ld();
-                if (vis_hi != ~0ull) { mask_chunk(x0, (uint32_t)vis_hi); mask_chunk(x1, (uint32_t)(vis_hi >> 32)); }
                 mx = fmaxf(mx, fmaxf(chunk_max(x0), chunk_max(x1)));
                 // lazy reference maximum, per row; the accumulator is rescaled by the whole warp (the
                 // TMEM accesses are warp-wide) whenever one of its rows moved
@@ -706,158 +751,127 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                         tc_fence_after();
                         const uint32_t o_addr = lane_addr + kOCol + blk * 128;
                         #pragma unroll 1
-                        for (int ch = 0; ch < 4; ++ch) {
-                            float o[32];
-                            tmem_ld32(o_addr + ch * 32, o);
+                        for (int ch = 0; ch < 8; ++ch) {
+                            float o[16];
+                            tmem_ld16(o_addr + ch * 16, o);
                             tmem_wait_ld();
                             #pragma unroll
-                            for (int c = 0; c < 32; ++c) o[c] *= alpha;
-                            tmem_st32(o_addr + ch * 32, reinterpret_cast<uint32_t*>(o));
+                            for (int c = 0; c < 16; ++c) o[c] *= alpha;
+                            tmem_st16(o_addr + ch * 16, reinterpret_cast<uint32_t*>(o));
                         }
-                        tmem_wait_st();
                     }
                 }
-                // second pass: p = 2^(s c2 - m c2), row sum from the unrounded p, P (bf16) over the upper
-                // half of the score block -- first the upper 64 keys (their scores are in registers and
-                // their columns are the ones P overwrites), then the lower 64, fetched again
+                // second pass: p = 2^(s c2 - m c2), row sum from the unrounded p, P (bf16) over the upper half
+                // of the score block -- first the upper 64 keys (their scores are in registers and their
+                // columns are the ones P overwrites), then the lower 64, fetched again.  The upper keys'
+                // half of O += P V runs beside the exponentials of the lower ones.
                 const float mc = (my_m == -INFINITY) ? 0.f : my_m * c2;
                 float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-                exp_chunk(x0, c2, mc, sum4, s_addr + 64 + 32);
-                exp_chunk(x1, c2, mc, sum4, s_addr + 64 + 48);
-                tmem_ld32(s_addr, x0);
-                tmem_ld32(s_addr + 32, x1);
-                tmem_wait_ld();
-                if (vis_lo != ~0ull) { mask_chunk(x0, (uint32_t)vis_lo); mask_chunk(x1, (uint32_t)(vis_lo >> 32)); }
-                exp_chunk(x0, c2, mc, sum4, s_addr + 64);
-                exp_chunk(x1, c2, mc, sum4, s_addr + 64 + 16);
+                #pragma unroll 1
+                for (int half = 1; half >= 0; --half) {
+                    if (half == 0) {
+                        tmem_ld32(s_addr, x0);
+                        tmem_ld32(s_addr + 32, x1);
+                        tmem_wait_ld();
+                    }
+                    exp_chunk(x0, c2, mc, sum4, s_addr + 64 + 32 * half);
+                    exp_chunk(x1, c2, mc, sum4, s_addr + 80 + 32 * half);
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(B.p_full(2 * (1 - half) + blk));
+                }
                 my_l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-                tmem_wait_st();                                            // this job's P is in TMEM
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(B.p_full(blk));
             }
         } else {
-        // The scores of a job are requested from TMEM at the end of the job before it, ahead of the
-        // wait for that job's P stores, so the two latencies overlap; whether those scores are there
-        // is probed before the exponentials and only waited for if the probe said no.
+        // One row block: the two warpgroups split a tile's 128 keys; thread = one row, 64 keys.  The scores
+        // of a tile are requested from TMEM at the end of the tile before it, ahead of the wait for that
+        // tile's P stores, so the two latencies overlap.
+        const int sb_wg = 64 * wg;
         float x0[32], x1[32];
-        if (n_jobs > 0) {
+        if (n_tiles > 0) {
             ok = mbar_wait_warp(B.s_full(0), 0);
             tc_fence_after();
-            if (ok) { tmem_ld32(lane_addr + 64 * wg, x0); tmem_ld32(lane_addr + 64 * wg + 32, x1); }
+            if (ok) { tmem_ld32(lane_addr + sb_wg, x0); tmem_ld32(lane_addr + sb_wg + 32, x1); }
         }
-
+        // tiles whose every key is visible to the row: [j_head, j_tail)
+        const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
+        const int j_head = lo_row[0] > it.key_begin ? (lo_row[0] - it.key_begin + kTile - 1) / kTile : 0;
         #pragma unroll 1
         for (int j = 0; j < n_tiles && ok; ++j) {
-            const int st = j % NS;
-            const int tile0 = it.key_begin + j * kTile;          // first key of the tile
-            const int j0 = tile0 + 64 * wg;                       // first key of this thread's columns
-            #pragma unroll
-            for (int blk = 0; blk < NB; ++blk) {
-                const int n = j * NB + blk, sb = n % NSB;
-                // Visibility word of this row for the thread's 64 columns (all ones away from the
-                // draft block and the end of the key range).
-                const bool boundary = j0 + 64 > it.key_end || j0 + 64 > kv_len || j0 < lo_row[blk];
-                unsigned long long vis = ~0ull;
-                if (boundary) {
-                    // prefix columns, then the ancestor word shifted to the draft block's column, cut
-                    // at the end of the key range
-                    const int d0 = kv_len - j0;                             // column of draft token 0 (any sign)
-                    const int nval = it.key_end - j0;                       // valid columns (may be <= 0)
-                    if (d0 >= 64) vis = ~0ull;
-                    else if (d0 > 0) vis = ((1ull << d0) - 1ull) | (anc[blk] << d0);
-                    else if (d0 > -64) vis = anc[blk] >> (-d0);
-                    else vis = 0ull;
-                    if (nval <= 0) vis = 0ull;
-                    else if (nval < 64) vis &= (1ull << nval) - 1ull;
-                    // prefix keys left of the row's window (the bound never exceeds kv_len, so
-                    // the draft block's columns are not touched)
-                    const int cut = lo_row[blk] - j0;
-                    if (cut >= 64) vis = 0ull;
-                    else if (cut > 0) vis &= ~((1ull << cut) - 1ull);
-                }
+            const int sb = j % NSB;
+            const uint32_t x_addr = lane_addr + sb * 128 + sb_wg;           // this thread's scores, then its P
+            tmem_wait_ld();
+            if (j >= j_tail || j < j_head) {
+                const int tile0 = it.key_begin + j * kTile;          // first key of the tile
                 // V rows past the end of the sequence may hold anything: zero them so 0 * x stays 0
-                // (once per tile, by the threads of the first half, thread r taking key row r).
-                if (blk == 0 && wg == 0 && tile0 + kTile > n_keys_seq && tile0 + row_local >= n_keys_seq) {
+                // (once per tile, by the first warpgroup, thread r taking key row r)
+                if (wg == 0 && tile0 + row_local >= n_keys_seq) {
+                    const int st = j % NS;
                     mbar_wait(B.v_full(st), (j / NS) & 1);
                     unsigned char* vrow = kv_sm + st * kStageBytes + 2 * kSubTileBytes + row_local * 128;
-                    #pragma unroll
+                    #pragma unroll 1
                     for (int c = 0; c < 8; ++c) {
                         *reinterpret_cast<uint4*>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
                         *reinterpret_cast<uint4*>(vrow + kSubTileBytes + c * 16) = make_uint4(0, 0, 0, 0);
                     }
                     fence_proxy_async();
                 }
-                tmem_wait_ld();
-                if (boundary) { mask_chunk(x0, (uint32_t)vis); mask_chunk(x1, (uint32_t)(vis >> 32)); }
-                const float mx = fmaxf(chunk_max(x0), chunk_max(x1));
-
-                // Rows of padding hold whatever the Q box left there: they never force a rescale.  The
-                // barrier also orders both halves' score loads before anyone's P stores (P aliases S).
-                const bool need = row_ok[blk] && (mx > m_ref[blk] + thr || (m_ref[blk] == -INFINITY && mx > -INFINITY));
-                if (softmax_bar_or(need)) {
-                    // some row's maximum moved: the two halves of every row agree on the new reference
-                    xch[wg * 128 + row_local] = need ? mx : -INFINITY;
-                    softmax_bar_sync();
-                    const float cand = fmaxf(need ? mx : -INFINITY, xch[(wg ^ 1) * 128 + row_local]);
-                    float alpha = 1.f;
-                    if (cand > -INFINITY) {
-                        alpha = (m_ref[blk] == -INFINITY) ? 0.f : ex2((m_ref[blk] - cand) * c2);
-                        m_ref[blk] = cand;
-                        l_run[blk] *= alpha;
-                    }
-                    if (j > 0 && __any_sync(0xffffffffu, cand > -INFINITY)) {     // O holds earlier tiles: rescale this half of it
-                        // every earlier tile's product has been added (they complete in order)
-                        if (!mbar_wait_warp(B.o_done(blk, j - 1), ((j - 1) >> 2) & 1)) { ok = false; break; }
-                        tc_fence_after();
-                        const uint32_t o_addr = lane_addr + kOCol + blk * 128 + 64 * wg;
-                        #pragma unroll 1
-                        for (int ch = 0; ch < 2; ++ch) {
-                            float o[32];
-                            tmem_ld32(o_addr + ch * 32, o);
-                            tmem_wait_ld();
-                            #pragma unroll
-                            for (int c = 0; c < 32; ++c) o[c] *= alpha;
-                            tmem_st32(o_addr + ch * 32, reinterpret_cast<uint32_t*>(o));
-                        }
-                        tmem_wait_st();
-                    }
-                }
-
-                // are the next job's scores there already?  (asked now, used after the exponentials)
-                const bool has_next = n + 1 < n_jobs;
-                const int sb_next = (n + 1) % NSB;
-                const uint32_t par_next = (uint32_t)((n + 1) / NSB) & 1u;
-                uint32_t next_ready = 0;
-                if (has_next && lane == 0) next_ready = mbar_test_wait(B.s_full(sb_next), par_next) ? 1u : 0u;
-
-                // p = 2^(s c2 - m c2), row sum from the unrounded p, P (bf16) over the S block: this
-                // thread's 64 keys land on columns [32 wg, 32 wg + 32) of the block.
-                const float mc = (m_ref[blk] == -INFINITY) ? 0.f : m_ref[blk] * c2;
-                float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-                const uint32_t p_addr = lane_addr + sb * 128 + 32 * wg;
-                exp_chunk(x0, c2, mc, sum4, p_addr);
-                exp_chunk(x1, c2, mc, sum4, p_addr + 16);
-                l_run[blk] += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-
-                if (has_next) {                                            // request the next job's scores
-                    if (__shfl_sync(0xffffffffu, next_ready, 0) == 0u && !mbar_wait_warp(B.s_full(sb_next), par_next)) {
-                        ok = false;
-                    } else {
-                        tc_fence_after();
-                        const uint32_t s_next = lane_addr + sb_next * 128 + 64 * wg;
-                        tmem_ld32(s_next, x0);
-                        tmem_ld32(s_next + 32, x1);
-                    }
-                }
-                tmem_wait_st();                                            // this job's P is in TMEM
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(B.p_full(sb));
-                if (!ok) break;
+                const unsigned long long vis = vis_word(tile0 + sb_wg, anc[0], lo_row[0]);
+                mask_chunk(x0, (uint32_t)vis);
+                mask_chunk(x1, (uint32_t)(vis >> 32));
             }
+            const float mx = fmaxf(chunk_max(x0), chunk_max(x1));
+            // Rows of padding hold whatever the Q box left there: they never force a rescale.
+            const bool need = row_ok[0] && (mx > m_ref[0] + thr || (m_ref[0] == -INFINITY && mx > -INFINITY));
+            if (softmax_bar_or(need)) {
+                // some row's maximum moved: the two halves of every row agree on the new reference
+                xch[wg * 128 + row_local] = need ? mx : -INFINITY;
+                softmax_bar_sync();
+                const float cand = fmaxf(need ? mx : -INFINITY, xch[(wg ^ 1) * 128 + row_local]);
+                float alpha = 1.f;
+                if (cand > -INFINITY) {
+                    alpha = (m_ref[0] == -INFINITY) ? 0.f : ex2((m_ref[0] - cand) * c2);
+                    m_ref[0] = cand;
+                    l_run[0] *= alpha;
+                }
+                if (j > 0 && __any_sync(0xffffffffu, cand > -INFINITY)) {     // O holds earlier tiles: rescale this half of it
+                    // every earlier tile's product has been added (they complete in order)
+                    if (!mbar_wait_warp(B.o_done(0, j - 1), ((j - 1) >> 2) & 1)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t o_addr = lane_addr + kOCol + sb_wg;
+                    #pragma unroll 1
+                    for (int ch = 0; ch < 4; ++ch) {
+                        float o[16];
+                        tmem_ld16(o_addr + ch * 16, o);
+                        tmem_wait_ld();
+                        #pragma unroll
+                        for (int c = 0; c < 16; ++c) o[c] *= alpha;
+                        tmem_st16(o_addr + ch * 16, reinterpret_cast<uint32_t*>(o));
+                    }
+                }
+            }
+            // p = 2^(s c2 - m c2), row sum from the unrounded p, P (bf16) over this thread's own scores
+            const float mc = (m_ref[0] == -INFINITY) ? 0.f : m_ref[0] * c2;
+            float sum4[4] = {0.f, 0.f, 0.f, 0.f};
+            exp_chunk(x0, c2, mc, sum4, x_addr);
+            exp_chunk(x1, c2, mc, sum4, x_addr + 16);
+            l_run[0] += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
+            if (j + 1 < n_tiles) {                                     // request the next tile's scores
+                if (!mbar_wait_warp(B.s_full((j + 1) % NSB), (uint32_t)((j + 1) / NSB) & 1u)) {
+                    ok = false;
+                } else {
+                    tc_fence_after();
+                    const uint32_t s_next = lane_addr + ((j + 1) % NSB) * 128 + sb_wg;
+                    tmem_ld32(s_next, x0);
+                    tmem_ld32(s_next + 32, x1);
+                }
+            }
+            tmem_wait_st();                                            // this tile's P is in TMEM
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(B.p_full(sb));
         }
-
         }
         // ---- epilogue: normalised partial output + natural-log LSE -------------------------------
         if (tid == 0) SPARROW_STAMP(5);                                 // softmax loop left
