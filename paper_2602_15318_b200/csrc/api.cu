@@ -528,8 +528,12 @@ sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const Syn
 
 __global__ void ancestor_masks_kernel(const int32_t* parents, int T, unsigned long long* masks, unsigned* status)
 {
-    const int i = threadIdx.x;
-    if (i < T) masks[i] = ancestor_word(parents, T, i, status);
+    __shared__ int32_t par_s[kMaxT];
+    __shared__ unsigned long long anc_s[kMaxT];
+    for (int i = threadIdx.x; i < T; i += 32) par_s[i] = parents[i];
+    __syncwarp();
+    build_ancestor_words(par_s, anc_s, T, status);
+    for (int i = threadIdx.x; i < T; i += 32) masks[i] = anc_s[i];
 }
 
 // One thread waits (bounded) on a finisher counter; see sparrow_debug_wait_counter().
@@ -1371,7 +1375,7 @@ sparrow_status sparrow_debug_ancestor_masks_device(sparrow_ctx* c, const int32_t
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     other_kernel_enqueued();
-    ancestor_masks_kernel<<<1, kMaxT, 0, static_cast<cudaStream_t>(stream)>>>(
+    ancestor_masks_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(
         parents_dev, T, reinterpret_cast<unsigned long long*>(masks_dev), reinterpret_cast<unsigned*>(c->ws));
     if (cudaGetLastError() != cudaSuccess) return SPARROW_ERR_CUDA;
     c->launches.fetch_add(1);

@@ -211,25 +211,41 @@ __device__ __forceinline__ Item decode_item(const SplitPlan& p, int item)
     return it;
 }
 
-// Ancestor word of draft node i: bit a set iff a == i or a is an ancestor of i.  Walks the parent
-// chain (at most T steps, so a malformed array cannot loop).  A parent outside [-1, node) is
-// treated as "root" and reported.
-__device__ __forceinline__ unsigned long long ancestor_word(const int32_t* __restrict__ parents,
-                                                            int T, int i, unsigned* status)
+// Ancestor words of a draft tree, built by one warp: anc[i] has bit a set iff a == i or a is an
+// ancestor of i.  On entry jump[i] (shared memory, T <= 64 entries) is the parent of node i; it is used
+// up.  A parent outside [-1, node) is treated as "root" and reported.  Pointer doubling: after round
+// r a word covers 2^r generations, so six rounds do for any tree (a walk from every node to its root is
+// a chain of up to 64 dependent reads: 4.5 us on the critical path of a 40-node chain, 0.3 us like this).
+__device__ __forceinline__ void build_ancestor_words(int32_t* jump, unsigned long long* anc, int T, unsigned* status)
 {
-    unsigned long long m = 1ull << i;
-    int node = i;
-    for (int step = 0; step < T; ++step) {
-        const int p = parents[node];
-        if (p == -1) break;
-        if (p < -1 || p >= node) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < T; i += 32) {
+        const int p = jump[i];
+        if (p < -1 || p >= i) {
             if (status) atomicOr(status, kStatTree);
-            break;
+            jump[i] = -1;
         }
-        m |= 1ull << p;
-        node = p;
+        anc[i] = 1ull << i;
     }
-    return m;
+    __syncwarp();
+    #pragma unroll 1
+    for (int reach = 1; reach < T; reach <<= 1) {
+        unsigned long long more[2];
+        int next[2];
+        #pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = lane + 32 * k, p = i < T ? jump[i] : -1;
+            more[k] = p >= 0 ? anc[p] : 0ull;
+            next[k] = p >= 0 ? jump[p] : -1;
+        }
+        __syncwarp();
+        #pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = lane + 32 * k;
+            if (i < T) { anc[i] |= more[k]; jump[i] = next[k]; }
+        }
+        __syncwarp();
+    }
 }
 
 }  // namespace sparrow

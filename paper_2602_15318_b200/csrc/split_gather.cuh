@@ -157,8 +157,6 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
 
     // ---- prologue: masks / query positions, packed Q block -> registers --------------------
     const int tree_nodes = anchored ? args.tree_nodes : 0;
-    // The parent array is staged in shared memory first: the walk up the tree is a chain of
-    // dependent reads, one memory round trip each if it went to global memory.
     __shared__ int32_t par_s[kMaxT];
     const int n_par = anchored ? tree_nodes : T;
     if (tid < n_par) par_s[tid] = __ldg(args.parents + (size_t)it.b * n_par + tid);
@@ -168,7 +166,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
         qpos_s[tid] = p;
     }
     __syncthreads();
-    if (tid < n_par) anc_s[tid] = ancestor_word(par_s, n_par, tid, args.status);
+    if (warp == 0) build_ancestor_words(par_s, anc_s, n_par, args.status);
     {
         constexpr int kChunksPerThread = kRows * 16 / kThreads;      // 8: all loads first, then the stores
         uint4 val[kChunksPerThread];

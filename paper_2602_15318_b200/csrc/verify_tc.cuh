@@ -36,8 +36,9 @@
 //                        3,500; 64-key steps with their own N = 64 products slower (the 64-column product
 //                        takes 48 cycles instead of 32).  Long streams of calls run at the power limit
 //                        (1,000 W, 1.5 GHz) whatever the loop looks like.
-//   warp 10, one thread  gatekeeper (overlapped mode): waits, beside the main loop, for the counters
-//                        that allow this CTA's first global write.
+//   warp 10              gatekeeper: fills the tables of ancestor words and window bounds, then one
+//                        thread waits (overlapped mode), beside the main loop, for the counters that
+//                        allow this CTA's first global write.
 //
 // With one row block there are three S blocks and one O accumulator, with two row blocks one S
 // block and one accumulator per block.
@@ -170,6 +171,9 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
 }
 // barrier among the 256 softmax threads only (id 1; id 0 is __syncthreads)
 __device__ __forceinline__ void softmax_bar_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// The gatekeeper warp has filled the tables that the 256 softmax threads read (id 3).
+__device__ __forceinline__ void tables_ready_arrive() { asm volatile("bar.arrive 3, 288;" ::: "memory"); }
+__device__ __forceinline__ void tables_ready_sync() { asm volatile("bar.sync 3, 288;" ::: "memory"); }
 // One lane of a converged warp.  The tensor-core instructions take their descriptors from uniform
 // registers, which the compiler only uses behind elect.sync in a warp whose control flow stays
 // converged.  Behind `if (lane == 0)` every tcgen05.mma first moves its operands over: 93 to 104
@@ -458,29 +462,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (warp == 0) {
-        const int Tt = plan.T_tree;
-        if (sync.wait_first) wait_for_predecessors();
-        if (it.key_end > kv_len) {                   // this piece reaches the draft block: it needs the tree
-            const int32_t* par_g = args.parents + (size_t)it.b * Tt;
-            if (lane < Tt) par_s[lane] = __ldg(par_g + lane);
-            if (lane + 32 < Tt) par_s[lane + 32] = __ldg(par_g + lane + 32);
-            __syncwarp();
-            for (int i = lane; i < Tt; i += 32) anc_s[i] = ancestor_word(par_s, Tt, i, args.status);
-            __syncwarp();
-        }
-        // Lower window bound of every query token, clamped to what this call streams: a bound
-        // left of the first streamed key cannot be honoured (the keys in between were not planned)
-        // and is reported.
-        for (int t = lane; t < T; t += 32) {
-            int lo = args.first_visible ? __ldg(args.first_visible + (size_t)it.b * T + t) : 0;
-            if (lo < plan.seq[it.b].key0) {
-                if (args.first_visible) atomicOr(args.status, kStatAnchor);
-                lo = plan.seq[it.b].key0;
-            }
-            par_s[t] = lo < kv_len ? lo : kv_len;
-        }
-    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -623,6 +604,29 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             if (!ok && lane == 0) { atomicOr(args.status, timeout_bits(kSiteMma)); *abort_flag = 1; }
         }
     } else if (warp == kGateWarp) {
+        // The tree and the window bounds, beside the first loads; the softmax warps wait for them at a barrier.
+        {
+            const int Tt = plan.T_tree;
+            if (sync.wait_first) wait_for_predecessors();
+            if (it.key_end > kv_len) {                   // this piece reaches the draft block: it needs the tree
+                const int32_t* par_g = args.parents + (size_t)it.b * Tt;
+                for (int i = lane; i < Tt; i += 32) par_s[i] = __ldg(par_g + i);
+                __syncwarp();
+                build_ancestor_words(par_s, anc_s, Tt, args.status);
+            }
+            // Lower window bound of every query token, clamped to what this call streams: a bound
+            // left of the first streamed key cannot be honoured (the keys in between were not planned)
+            // and is reported.
+            for (int t = lane; t < T; t += 32) {
+                int lo = args.first_visible ? __ldg(args.first_visible + (size_t)it.b * T + t) : 0;
+                if (lo < plan.seq[it.b].key0) {
+                    if (args.first_visible) atomicOr(args.status, kStatAnchor);
+                    lo = plan.seq[it.b].key0;
+                }
+                par_s[t] = lo < kv_len ? lo : kv_len;
+            }
+            tables_ready_arrive();
+        }
         if (lane == 0 && sync.enabled) {
             // Overlapped mode: whoever read this parity's partial buffer two calls ago must be done
             // before this CTA's first global write, and final results may only follow every earlier
@@ -639,6 +643,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
     } else if (warp < 8) {
         // ================= softmax =================
+        tables_ready_sync();                             // ancestor words and window bounds are in shared memory
         const int wg = warp >> 2;                        // key-column half this thread takes
         const int row_local = (warp & 3) * 32 + lane;    // TMEM lane = row inside the 128-row block
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -984,150 +989,152 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             if (!direct) fence_proxy_async_global();
             softmax_bar_sync();                                        // every global store of this CTA has been issued
             if (tid == 0) SPARROW_STAMP(7);                            // partial rows stored
-            if (tid == 0) {
-                if (!direct) publish_counter(arrive_word);
-                if (merges) {
-                    // every partial of the call in place, and (overlapped mode) the previous call's final results written
-                    // (both words are polled in one loop: the second is usually there already)
-                    bool have_all = false, prev_done = false;
-                    #pragma unroll 1
-                    for (uint32_t i = 0; i < kCounterPolls && !(have_all && prev_done); ++i) {
-                        if (!have_all) have_all = ld_acquire(arrive_word) == (unsigned)sync.n_arrive;
-                        if (!prev_done) prev_done = (int32_t)(ld_acquire(sync.fin_done + (sync.parity ^ 1)) - sync.fin_wait_other) >= 0;
-                        if (!(have_all && prev_done)) __nanosleep(i < 256 ? 20 : 200);
-                    }
-                    SPARROW_STAMP(8);                                   // all arrivals seen
-                    if (!have_all) atomicOr(args.status, timeout_bits(kSiteArrivals));
-                    else if (!prev_done) atomicOr(args.status, timeout_bits(kSiteFinOther));
-                    SPARROW_STAMP(9);                                   // previous call's finishers seen
-                    *fin_go = (have_all && prev_done) ? 1 : 0;
-                }
-            }
+            if (tid == 0 && !direct) publish_counter(arrive_word);
             if (merges) {
-                softmax_bar_sync();
-                if (*fin_go) {
-                    // 16 R G threads merge R rows at a time.  The rows' pieces are first brought into the
-                    // (idle) K/V ring by bulk copies, [piece][row][272 bytes], one copy per piece and
-                    // block touched -- far fewer and larger requests than per-thread loads.  (The pieces
-                    // were written with ordinary stores and the copies read through the async proxy: the
-                    // writers issued the proxy fence, before they published their piece.)
-                    // Thread (row i, 16-byte chunk c, piece group g) then folds pieces g, g + G, ... of its
-                    // row into a running (max, sum, weighted output); the groups' results meet in shared
-                    // memory (the Q blocks, idle by now).
-                    constexpr int kRowBytes = kPartRowHalves * 2;               // 272
-                    float* red = reinterpret_cast<float*>(q_sm);                // [256][10]: 8 outputs, sum, max
-                    int ubase = 0, phase = 0;
-                    bool fin_ok = true;
-                    #pragma unroll 1
-                    for (int b = 0; b < plan.batch; ++b) {
-                        const int ns = plan.seq[b].n_splits;
-                        if (ns == 1) continue;
-                        // rows per pass: a power of two, no more than this finisher has, than fit the ring
-                        // with all their pieces, or than 16
-                        int R = 1;
-                        while (R < 16 && R < chunk) R <<= 1;
-                        while (R > 1 && R * ns * kRowBytes > NS * kStageBytes) R >>= 1;
-                        const int G = 16 / R;                                   // piece groups
-                        const int c16 = tid & 15, grp_p = (tid >> 4) % G, row_i = tid / (16 * G);
-                        const size_t piece_pitch = (size_t)plan.part_rows * kPartRowHalves;      // halves between pieces
-                        #pragma unroll 1
-                        for (int u = 0; u < plan.n_kv_heads * plan.n_groups; ++u) {
-                            const int kvh = u / plan.n_groups, grp = u - kvh * plan.n_groups;
-                            const int tok0 = grp * NB * tpb;                        // first token of this row group
-                            const int list_len = qg * min(NB * tpb, T - tok0);  // its valid rows
-                            const int row_begin = max(my_begin, ubase) - ubase, row_end = min(my_end, ubase + list_len) - ubase;
-                            ubase += list_len;
-                            if (row_begin >= row_end) continue;                    // (the same in every thread of the CTA)
-                            const size_t item0 = (size_t)plan.seq[b].item_begin + (size_t)u * ns;
+                // 16 R G threads merge R rows at a time.  The rows' pieces are first brought into the
+                // (idle) K/V ring by bulk copies, [piece][row][272 bytes], one copy per piece and
+                // block touched -- far fewer and larger requests than per-thread loads.  (The pieces
+                // were written with ordinary stores and the copies read through the async proxy: the
+                // writers issued the proxy fence, before they published their piece.)
+                // Thread (row i, 16-byte chunk c, piece group g) then folds pieces g, g + G, ... of its
+                // row into a running (max, sum, weighted output); the groups' results meet in shared
+                // memory (the Q blocks, idle by now).  Everything that does not depend on the pieces'
+                // contents is computed in front of the wait for the call's arrivals.
+                constexpr int kRowBytes = kPartRowHalves * 2;               // 272
+                float* red = reinterpret_cast<float*>(q_sm);                // [256][10]: 8 outputs, sum, max
+                const int unit_rows = NB * kRowsPerBlock;                   // rows of a full row group
+                const int seq_rows = plan.n_kv_heads * qg * T;              // list entries per sequence
+                int phase = 0;
+                bool fin_ok = true, first_pass = true;
+                #pragma unroll 1
+                for (int row = my_begin; row < my_end && fin_ok;) {
+                    // sequence, KV head, row group and row of list entry `row`
+                    int b = 0, rest = row;
+                    while (plan.seq[b].n_splits == 1 || rest >= seq_rows) {
+                        if (plan.seq[b].n_splits > 1) rest -= seq_rows;
+                        ++b;
+                    }
+                    const int ns = plan.seq[b].n_splits;
+                    const int kvh = rest / (qg * T);
+                    rest -= kvh * qg * T;
+                    const int grp = rest / unit_rows, r0 = rest - grp * unit_rows;
+                    const int tok0 = grp * NB * tpb;                        // first token of this row group
+                    const int unit_left = qg * min(NB * tpb, T - tok0) - r0;
+                    // rows per pass: a power of two, no more than this finisher has, than fit the ring
+                    // with all their pieces, or than 16
+                    int R = 1;
+                    while (R < 16 && R < chunk) R <<= 1;
+                    while (R > 1 && R * ns * kRowBytes > NS * kStageBytes) R >>= 1;
+                    const int G = 16 / R;                                   // piece groups
+                    const int c16 = tid & 15, grp_p = (tid >> 4) % G, row_i = tid / (16 * G);
+                    const int n_here = min(R, min(unit_left, my_end - row));
+                    // the rows may straddle the unit's two blocks: rows [r0, split) and [split, r0 + n_here)
+                    const int bk0 = r0 / kRowsPerBlock;
+                    const int split = (r0 < kRowsPerBlock && r0 + n_here > kRowsPerBlock) ? kRowsPerBlock : r0 + n_here;
+                    const size_t item0 = (size_t)plan.seq[b].item_begin + (size_t)(kvh * plan.n_groups + grp) * ns;
+                    const size_t piece_pitch = (size_t)plan.part_rows * kPartRowHalves;      // halves between pieces
+                    const __half* first = args.o_part + (item0 * plan.part_rows + (size_t)(bk0 * kBlockRows + r0 - bk0 * kRowsPerBlock)) * kPartRowHalves;
+                    const __half* second = args.o_part + (item0 * plan.part_rows + (size_t)kBlockRows) * kPartRowHalves;
+                    const int idx = r0 + row_i;                            // row of the unit's list: token idx / g, head idx % g
+                    const int t = tok0 + idx / qg, h = kvh * qg + idx % qg;
+                    uint4* out_row = reinterpret_cast<uint4*>(args.out + (((size_t)b * T + t) * args.n_q_heads + h) * kD + c16 * 8);
+                    float* lse_row = args.lse + ((size_t)b * args.n_q_heads + h) * T + t;
+                    const uint32_t pstride = (uint32_t)n_here * kRowBytes;     // bytes between pieces in the ring
+                    const uint32_t row_sm = smem_u32(kv_sm) + (uint32_t)row_i * kRowBytes;
+                    if (tid == 0) {
+                        if (first_pass) {
+                            // every partial of the call in place, and the previous call's final results written
+                            // (both words are polled in one loop: the second is usually there already)
+                            bool have_all = false, prev_done = false;
                             #pragma unroll 1
-                            for (int r0 = row_begin; r0 < row_end; r0 += R, phase ^= 1) {
-                                const int n_here = min(R, row_end - r0);
-                                // the rows may straddle the unit's two blocks: rows [r0, split) and [split, r0 + n_here)
-                                const int split = (r0 < kRowsPerBlock && r0 + n_here > kRowsPerBlock) ? kRowsPerBlock : r0 + n_here;
-                                if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n_here * ns * kRowBytes));
-                                softmax_bar_sync();                                // the ring's previous contents have been read, the byte count is posted
-                                {
-                                    const int bk0 = r0 / kRowsPerBlock;
-                                    const __half* first = args.o_part + (item0 * plan.part_rows + (size_t)(bk0 * kBlockRows + r0 - bk0 * kRowsPerBlock)) * kPartRowHalves;
-                                    const __half* second = args.o_part + (item0 * plan.part_rows + (size_t)kBlockRows) * kPartRowHalves;
-                                    for (int sp = tid; sp < ns; sp += 256) {           // thread sp brings piece sp
-                                        const uint32_t dst = smem_u32(kv_sm) + (uint32_t)(sp * n_here * kRowBytes);
-                                        bulk_load(dst, first + (size_t)sp * piece_pitch, (uint32_t)(split - r0) * kRowBytes, B.fin());
-                                        if (split < r0 + n_here)
-                                            bulk_load(dst + (uint32_t)(split - r0) * kRowBytes, second + (size_t)sp * piece_pitch,
-                                                      (uint32_t)(r0 + n_here - split) * kRowBytes, B.fin());
-                                    }
-                                }
-                                if (tid == 0) SPARROW_STAMP(12);        // bulk copies issued
-                                fin_ok = fin_ok && mbar_wait_warp(B.fin(), phase);
-                                if (tid == 0) SPARROW_STAMP(15);        // bulk copies landed
-                                const int idx = r0 + row_i;                            // row of the unit's list: token idx / 7, head idx % 7
-                                const bool active = fin_ok && row_i < n_here;
-                                const uint32_t pstride = (uint32_t)n_here * kRowBytes;     // bytes between pieces in the ring
-                                const uint32_t row_sm = smem_u32(kv_sm) + (uint32_t)row_i * kRowBytes;
-                                float m_run = -INFINITY, s_run = 0.f;                  // natural-log units
-                                float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                                if (active) {
-                                    #pragma unroll 2
-                                    for (uint32_t sp = grp_p, a_o = row_sm + grp_p * pstride; sp < (uint32_t)ns; sp += G, a_o += G * pstride) {
-                                        const float l = lds_f32(a_o + 2 * kD);
-                                        uint32_t raw[4];
-                                        lds_v4(a_o + c16 * 16, raw);
-                                        if (l == -INFINITY) continue;                  // a piece that saw no visible key
-                                        const float m_new = fmaxf(m_run, l);
-                                        const float a = ex2((m_run - m_new) * 1.4426950408889634f);   // 0 for the first piece
-                                        const float w = ex2((l - m_new) * 1.4426950408889634f);
-                                        s_run = fmaf(s_run, a, w);
-                                        #pragma unroll
-                                        for (int q = 0; q < 4; ++q) {
-                                            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
-                                            acc[2 * q] = fmaf(acc[2 * q], a, w * f.x); acc[2 * q + 1] = fmaf(acc[2 * q + 1], a, w * f.y);
-                                        }
-                                        m_run = m_new;
-                                    }
-                                }
-                                if (tid == 0) SPARROW_STAMP(13);        // pieces folded
-                                if (G > 1) {                                           // (G is the same in every thread)
-                                    softmax_bar_sync();                                // the pass before has been read
-                                    #pragma unroll
-                                    for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
-                                    red[tid * 10 + 8] = s_run;
-                                    red[tid * 10 + 9] = m_run;
-                                    softmax_bar_sync();
-                                    if (grp_p == 0) {
-                                        const float* mine = red + tid * 10;
-                                        float m_all = m_run;
-                                        for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
-                                        const float a0 = m_run == -INFINITY ? 0.f : ex2((m_run - m_all) * 1.4426950408889634f);
-                                        s_run *= a0;
-                                        #pragma unroll
-                                        for (int q = 0; q < 8; ++q) acc[q] *= a0;
-                                        for (int g2 = 1; g2 < G; ++g2) {
-                                            const float* o = mine + g2 * 160;
-                                            if (o[9] == -INFINITY) continue;
-                                            const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
-                                            s_run = fmaf(o[8], ag, s_run);
-                                            #pragma unroll
-                                            for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
-                                        }
-                                        m_run = m_all;
-                                    }
-                                }
-                                if (tid == 0) SPARROW_STAMP(14);        // groups reduced
-                                if (active && grp_p == 0) {
-                                    const int t = tok0 + idx / qg;
-                                    const int h = kvh * qg + idx % qg;
-                                    const float inv = s_run > 0.f ? __fdividef(1.f, s_run) : 0.f;
-                                    uint4 pk;
-                                    pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-                                    pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
-                                    *reinterpret_cast<uint4*>(args.out + (((size_t)b * T + t) * args.n_q_heads + h) * kD + c16 * 8) = pk;
-                                    if (c16 == 0) args.lse[((size_t)b * args.n_q_heads + h) * T + t] = s_run > 0.f ? m_run + __logf(s_run) : -INFINITY;
-                                }
+                            for (uint32_t i = 0; i < kCounterPolls && !(have_all && prev_done); ++i) {
+                                if (!have_all) have_all = ld_acquire(arrive_word) == (unsigned)sync.n_arrive;
+                                if (!prev_done) prev_done = (int32_t)(ld_acquire(sync.fin_done + (sync.parity ^ 1)) - sync.fin_wait_other) >= 0;
+                                if (!(have_all && prev_done)) __nanosleep(i < 256 ? 20 : 200);
                             }
+                            SPARROW_STAMP(8);                               // all arrivals seen
+                            if (!have_all) atomicOr(args.status, timeout_bits(kSiteArrivals));
+                            else if (!prev_done) atomicOr(args.status, timeout_bits(kSiteFinOther));
+                            SPARROW_STAMP(9);                               // previous call's finishers seen
+                            *fin_go = (have_all && prev_done) ? 1 : 0;
+                        }
+                        if (*fin_go) mbar_expect_tx(B.fin(), (uint32_t)(n_here * ns * kRowBytes));
+                    }
+                    softmax_bar_sync();                                    // the ring's previous contents have been read, the byte count is posted
+                    fin_ok = *fin_go != 0;
+                    if (!fin_ok) break;
+                    for (int sp = tid; sp < ns; sp += 256) {               // thread sp brings piece sp
+                        const uint32_t dst = smem_u32(kv_sm) + (uint32_t)sp * pstride;
+                        bulk_load(dst, first + (size_t)sp * piece_pitch, (uint32_t)(split - r0) * kRowBytes, B.fin());
+                        if (split < r0 + n_here)
+                            bulk_load(dst + (uint32_t)(split - r0) * kRowBytes, second + (size_t)sp * piece_pitch,
+                                      (uint32_t)(r0 + n_here - split) * kRowBytes, B.fin());
+                    }
+                    if (tid == 0) SPARROW_STAMP(12);                       // bulk copies issued
+                    const bool landed = mbar_wait_warp(B.fin(), phase);
+                    phase ^= 1;
+                    first_pass = false;
+                    if (tid == 0) SPARROW_STAMP(15);                       // bulk copies landed
+                    if (!landed) { if (lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies)); }
+                    const bool active = landed && row_i < n_here;
+                    float m_run = -INFINITY, s_run = 0.f;                  // natural-log units
+                    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                    if (active) {
+                        #pragma unroll 2
+                        for (uint32_t sp = grp_p, a_o = row_sm + grp_p * pstride; sp < (uint32_t)ns; sp += G, a_o += G * pstride) {
+                            const float l = lds_f32(a_o + 2 * kD);
+                            uint32_t raw[4];
+                            lds_v4(a_o + c16 * 16, raw);
+                            if (l == -INFINITY) continue;                  // a piece that saw no visible key
+                            const float m_new = fmaxf(m_run, l);
+                            const float a = ex2((m_run - m_new) * 1.4426950408889634f);   // 0 for the first piece
+                            const float w = ex2((l - m_new) * 1.4426950408889634f);
+                            s_run = fmaf(s_run, a, w);
+                            #pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
+                                acc[2 * q] = fmaf(acc[2 * q], a, w * f.x); acc[2 * q + 1] = fmaf(acc[2 * q + 1], a, w * f.y);
+                            }
+                            m_run = m_new;
                         }
                     }
-                    if (!fin_ok) atomicOr(args.status, timeout_bits(kSiteFinCopies));
+                    if (tid == 0) SPARROW_STAMP(13);                       // pieces folded
+                    if (G > 1) {                                           // (G is the same in every thread)
+                        softmax_bar_sync();                                // the pass before has been read
+                        #pragma unroll
+                        for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
+                        red[tid * 10 + 8] = s_run;
+                        red[tid * 10 + 9] = m_run;
+                        softmax_bar_sync();
+                        if (grp_p == 0) {
+                            const float* mine = red + tid * 10;
+                            float m_all = m_run;
+                            for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
+                            const float a0 = m_run == -INFINITY ? 0.f : ex2((m_run - m_all) * 1.4426950408889634f);
+                            s_run *= a0;
+                            #pragma unroll
+                            for (int q = 0; q < 8; ++q) acc[q] *= a0;
+                            for (int g2 = 1; g2 < G; ++g2) {
+                                const float* o = mine + g2 * 160;
+                                if (o[9] == -INFINITY) continue;
+                                const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
+                                s_run = fmaf(o[8], ag, s_run);
+                                #pragma unroll
+                                for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
+                            }
+                            m_run = m_all;
+                        }
+                    }
+                    if (tid == 0) SPARROW_STAMP(14);                       // groups reduced
+                    if (active && grp_p == 0) {
+                        const float inv = s_run > 0.f ? __fdividef(1.f, s_run) : 0.f;
+                        uint4 pk;
+                        pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+                        pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+                        *out_row = pk;
+                        if (c16 == 0) *lse_row = s_run > 0.f ? m_run + __logf(s_run) : -INFINITY;
+                    }
+                    row += n_here;
                 }
                 if (tid == 0) SPARROW_STAMP(10);                        // merged rows written
                 softmax_bar_sync();
