@@ -91,8 +91,7 @@ constexpr float kRescaleLog2 = 8.0f;             // lazy-max threshold in log2 u
 
 __host__ __device__ constexpr int smem_bytes(int n_blocks, int n_stages)
 {
-    // two row blocks: 1 KB more for the per-row results the two warpgroups hand each other
-    return 1024 /*alignment slack*/ + n_blocks * kQBlockBytes + n_stages * kStageBytes + kMiscBytes + (n_blocks == 2 ? 1024 : 0);
+    return 1024 /*alignment slack*/ + n_blocks * kQBlockBytes + n_stages * kStageBytes + kMiscBytes;
 }
 // S blocks (score tiles in flight) for a given number of row blocks; TMEM: S blocks first, then
 // one 128-column O accumulator per row block, 512 columns in all.
@@ -158,10 +157,19 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
+// 1-D bulk copy shared -> global, and the wait until this thread's copies are complete (written, not only read)
+__device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_store_wait()
+{
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// Orders generic-proxy accesses to global memory that this thread has observed before its later
-// async-proxy (bulk copy) accesses to it.
+// Orders this thread's accesses to global memory across the generic and the async proxy (bulk copies).
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -890,83 +898,72 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             if (w == 1u && sync.enabled && blockIdx.x == 0) sync.arrivals[(sync.slot + 2) & 3] = 0u;   // the call after next: unused by now
             *write_ok = w == 1u ? 1u : 2u;
         }
-        float* xch2 = reinterpret_cast<float*>(misc + kMiscBytes);         // [2][128], two row blocks only
-        if constexpr (NB == 2) {
-            // each warpgroup hands over its block's per-row results: both warpgroups store both blocks
-            xch[wg * 128 + row_local] = my_l > 0.f ? 1.f / my_l : 0.f;
-            xch2[wg * 128 + row_local] = my_l > 0.f ? (my_m * c2 + log2f(my_l)) * 0.6931471805599453f : -INFINITY;
-            softmax_bar_sync();
+        // A thread finishes one row: its 64 output dims [64 wg, 64 wg + 64) of the one block, or all 128 of its
+        // warpgroup's own block.
+        const int blk = NB == 1 ? 0 : wg;
+        const int dim0 = NB == 1 ? 64 * wg : 0;
+        if constexpr (NB == 1) xch[wg * 128 + row_local] = l_run[0];       // the two halves' sums meet (the maxima are already the same)
+        softmax_bar_sync();
+        const float l_all = NB == 1 ? l_run[0] + xch[(wg ^ 1) * 128 + row_local] : my_l;
+        const float m_fin = NB == 1 ? m_ref[0] : my_m;
+        const bool my_row = NB == 1 ? row_ok[0] : (wg ? row_ok[NB - 1] : row_ok[0]);
+        const int my_t = (block0 + blk) * tpb + row_local / qg;
+        const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+        const float lse_val = l_all > 0.f ? (m_fin * c2 + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+        if (ok) ok = mbar_wait_warp(B.o_done(blk, n_tiles - 1), ((n_tiles - 1) >> 2) & 1);    // the last product is in
+        tc_fence_after();
+        if (tid == 0) SPARROW_STAMP(6);                                // last product complete
+        ok = ok && *write_ok == 1u;                                    // (thread 0 settled it before the barrier above)
+        const int h_row = it.kvh * qg + g_row;
+        // Partial rows are staged as they lie in the workspace ([row][272 bytes]: an odd number of 16-byte
+        // chunks, so a warp's rows do not share banks) and leave as one bulk copy per block: the copy's own
+        // completion orders them ahead of the publication, where ordinary stores needed a second pass
+        // and a proxy fence.  The staging area is the Q blocks and the start of the K ring: every Q K^T
+        // completed ahead of the product waited for above.
+        constexpr int kPartRowBytes = kPartRowHalves * 2;
+        unsigned char* stage = q_sm + blk * (kBlockRows * kPartRowBytes);
+        if (ok && my_row) {
+            if (wg == 0 || NB == 2) {
+                if (direct) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + my_t] = lse_val;
+                else *reinterpret_cast<float*>(stage + row_local * kPartRowBytes + kD * 2) = lse_val;
+            }
         }
-        #pragma unroll
-        for (int blk = 0; blk < NB; ++blk) {
-            const int last_product = n_tiles - 1;
-            if (ok) ok = mbar_wait_warp(B.o_done(blk, last_product), (last_product >> 2) & 1);    // the last product is in
-            tc_fence_after();
-            if (tid == 0 && blk == 0) SPARROW_STAMP(6);                // last product complete
-            float inv, lse_val;
-            if constexpr (NB == 2) {
-                inv = xch[blk * 128 + row_local];
-                lse_val = xch2[blk * 128 + row_local];
-            } else {
-                // the two halves' sums meet (the maxima are already the same)
-                xch[wg * 128 + row_local] = l_run[blk];
-                softmax_bar_sync();
-                const float l_all = l_run[blk] + xch[(wg ^ 1) * 128 + row_local];
-                softmax_bar_sync();                                    // xch is reused by the next block
-                inv = l_all > 0.f ? 1.f / l_all : 0.f;
-                lse_val = l_all > 0.f ? (m_ref[blk] * c2 + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
-            }
-            ok = ok && *write_ok == 1u;                                // (thread 0 settled it before the barriers above)
-            const int h_row = it.kvh * qg + g_row;
-            // Staging area for coalesced stores: the Q block (every MMA has completed by now).  Row r
-            // holds 16 chunks of 16 bytes (128 halves), chunk c stored at position c ^ (r & 15).
-            unsigned char* stage = q_sm + blk * kQBlockBytes;
-            const size_t prow0 = (size_t)blockIdx.x * plan.part_rows + blk * kBlockRows;   // first partial row of this block
-            if (ok) {
-                #pragma unroll 1
-                for (int hf = 0; hf < 2; ++hf) {                       // this thread's output dims [64 wg, 64 wg + 64)
-                    const int col = wg * 64 + hf * 32;
-                    float o[32];
-                    tmem_ld32(lane_addr + kOCol + blk * 128 + col, o);
-                    tmem_wait_ld();
-                    uint4 pk[4];
-                    uint32_t* w = reinterpret_cast<uint32_t*>(pk);
-                    if (direct) {
-                        if (row_ok[blk]) {
-                            #pragma unroll
-                            for (int c = 0; c < 16; ++c) w[c] = pack_bf16x2(o[2 * c] * inv, o[2 * c + 1] * inv);
-                            uint4* dst = reinterpret_cast<uint4*>(
-                                args.out + (((size_t)it.b * T + t_row[blk]) * args.n_q_heads + h_row) * kD + col);
-                            #pragma unroll
-                            for (int c = 0; c < 4; ++c) dst[c] = pk[c];
-                        }
-                    } else {
-                        #pragma unroll
-                        for (int c = 0; c < 16; ++c) w[c] = pack_half2(o[2 * c] * inv, o[2 * c + 1] * inv);
-                        #pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            *reinterpret_cast<uint4*>(stage + row_local * 256 + ((((col >> 3) + c) ^ (row_local & 15)) << 4)) = pk[c];
-                    }
+        if (ok) {
+            #pragma unroll 1
+            for (int col = dim0; col < dim0 + (NB == 1 ? 64 : 128); col += 32) {
+                float o[32];
+                tmem_ld32(lane_addr + kOCol + blk * 128 + col, o);
+                tmem_wait_ld();
+                uint4 pk[4];
+                uint32_t* w = reinterpret_cast<uint32_t*>(pk);
+                uint4* dst;
+                if (direct) {
+                    #pragma unroll
+                    for (int c = 0; c < 16; ++c) w[c] = pack_bf16x2(o[2 * c] * inv, o[2 * c + 1] * inv);
+                    dst = reinterpret_cast<uint4*>(args.out + (((size_t)it.b * T + my_t) * args.n_q_heads + h_row) * kD + col);
+                } else {
+                    #pragma unroll
+                    for (int c = 0; c < 16; ++c) w[c] = pack_half2(o[2 * c] * inv, o[2 * c + 1] * inv);
+                    dst = reinterpret_cast<uint4*>(stage + row_local * kPartRowBytes + col * 2);
                 }
-                if (row_ok[blk] && wg == 0) {
-                    if (direct) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + t_row[blk]] = lse_val;
-                    else *reinterpret_cast<float*>(args.o_part + (prow0 + row_local) * kPartRowHalves + kD) = lse_val;
+                if (my_row) {
+                    #pragma unroll
+                    for (int c = 0; c < 4; ++c) dst[c] = pk[c];
                 }
             }
-            softmax_bar_sync();                                        // both halves of every staged row are in place
-            if (ok && !direct) {
-                // warp w copies rows [16 w, 16 w + 16), two rows (512 contiguous bytes) per instruction
-                const int tok_here = min(tpb, max(0, T - (block0 + blk) * tpb));
-                const int rows_here = tok_here * qg;
-                #pragma unroll 4
-                for (int i = 0; i < 8; ++i) {
-                    const int r = warp * 16 + 2 * i + (lane >> 4), c = lane & 15;
-                    if (r < rows_here) {
-                        const uint4 val = *reinterpret_cast<const uint4*>(stage + r * 256 + ((c ^ (r & 15)) << 4));
-                        *reinterpret_cast<uint4*>(args.o_part + (prow0 + r) * kPartRowHalves + c * 8) = val;
-                    }
-                }
+        }
+        if (!direct) fence_proxy_async();                              // the staged rows, ahead of the bulk copies
+        softmax_bar_sync();                                            // every row is staged (or written)
+        if (tid == 0 && ok && !direct) {
+            #pragma unroll
+            for (int bk = 0; bk < NB; ++bk) {
+                const int rows_here = min(tpb, max(0, T - (block0 + bk) * tpb)) * qg;
+                if (rows_here > 0)
+                    bulk_store(args.o_part + ((size_t)blockIdx.x * plan.part_rows + bk * kBlockRows) * kPartRowHalves,
+                               smem_u32(q_sm + bk * (kBlockRows * kPartRowBytes)), (uint32_t)(rows_here * kPartRowBytes));
             }
+            bulk_store_wait();
+            fence_proxy_async_global();
         }
 
         // ---- publish this item; the call's finisher CTAs merge its partials ---------------------------
@@ -985,17 +982,12 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const int my_end = fin_idx >= 0 ? min(total, my_begin + chunk) : 0;
             const bool merges = my_begin < my_end;
             unsigned* arrive_word = sync.arrivals + sync.slot;
-            // the pieces are read by the finishers' bulk copies (async proxy): order this thread's stores ahead of them
-            if (!direct) fence_proxy_async_global();
-            softmax_bar_sync();                                        // every global store of this CTA has been issued
             if (tid == 0) SPARROW_STAMP(7);                            // partial rows stored
             if (tid == 0 && !direct) publish_counter(arrive_word);
             if (merges) {
                 // 16 R G threads merge R rows at a time.  The rows' pieces are first brought into the
                 // (idle) K/V ring by bulk copies, [piece][row][272 bytes], one copy per piece and
-                // block touched -- far fewer and larger requests than per-thread loads.  (The pieces
-                // were written with ordinary stores and the copies read through the async proxy: the
-                // writers issued the proxy fence, before they published their piece.)
+                // block touched -- far fewer and larger requests than per-thread loads.
                 // Thread (row i, 16-byte chunk c, piece group g) then folds pieces g, g + G, ... of its
                 // row into a running (max, sum, weighted output); the groups' results meet in shared
                 // memory (the Q blocks, idle by now).  Everything that does not depend on the pieces'
