@@ -382,6 +382,20 @@ struct Bars {
     __device__ __forceinline__ uint32_t o_done(int blk, int j) const { return base + 160u + 32u * (uint32_t)blk + 8u * (uint32_t)(j & 3); }
 };
 
+// What one pass of the merge takes: runs of rows of one unit (sequence, KV head, row group).
+struct MergeSegment {
+    int b, ns, n, split;             // sequence, pieces, rows, rows of them in the run's first block
+    int src, src2;                   // workspace row of the first piece's first row; of the unit's second block
+    int offset;                      // byte offset in the ring
+    int r0, tok0, head0;             // first row inside the unit, the unit's first token and query head
+};
+constexpr int kMaxSegments = 8;
+struct MergeList {
+    MergeSegment seg[kMaxSegments];
+    int n_seg, bytes, next_row;
+};
+static_assert(sizeof(MergeList) <= kMaxT * 8, "the list lies over the ancestor words");
+
 template <int NB>
 __global__ void __launch_bounds__(kBoundThreads, 1)
 verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ SyncArgs sync,
@@ -498,6 +512,20 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // the whole warp walks the jobs, converged; one elected lane issues (see elect_one)
         {
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
+            // V rows past the end of the sequence may hold anything: they are zeroed in shared memory, so that
+            // 0 * x stays 0, ahead of the last tile's first product and beside its softmax.
+            auto zero_v_tail = [&](int j) {
+                const int valid = n_keys_seq - (it.key_begin + j * kTile);
+                if (valid >= kTile) return;
+                unsigned char* v_tile = kv_sm + (j % NS) * kStageBytes + 2 * kSubTileBytes;
+                #pragma unroll 1
+                for (int i = valid * 8 + lane; i < kTile * 8; i += 32) {
+                    *reinterpret_cast<uint4*>(v_tile + i * 16) = make_uint4(0, 0, 0, 0);
+                    *reinterpret_cast<uint4*>(v_tile + kSubTileBytes + i * 16) = make_uint4(0, 0, 0, 0);
+                }
+                fence_proxy_async();
+                __syncwarp();
+            };
             // descriptors differ from job to job only in their 14-bit address field
             const uint64_t q_desc0 = smem_desc(smem_u32(q_sm), 16, 1024);
             const uint64_t k_desc0 = smem_desc(smem_u32(kv_sm), 16, 1024);
@@ -538,7 +566,10 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 #pragma unroll 1
                 for (int n = 0; n < n_jobs && ok; ++n) {
                     const int j = n >> 1, b = n & 1, st = j % NS;
-                    if (b == 0 && !mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
+                    if (b == 0) {
+                        if (!mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
+                        if (j == n_tiles - 1) zero_v_tail(j);
+                    }
                     if (!mbar_wait_warp(B.p_full(b), j & 1)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
@@ -592,7 +623,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             #pragma unroll 1
             for (int n = 0; n < n_jobs && ok; ++n) {
                 const int j = n / NB, blk = n % NB, sb = n % NSB, st = j % NS;
-                if (blk == 0 && !mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
+                if (!mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
+                if (j == n_tiles - 1) zero_v_tail(j);
                 if (!mbar_wait_warp(B.p_full(sb), (n / NSB) & 1)) { ok = false; break; }
                 tc_fence_after();
                 const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
@@ -711,20 +743,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 const int tile0 = it.key_begin + j * kTile;
                 if (!mbar_wait_warp(B.s_full(blk), j & 1)) { ok = false; break; }
                 tc_fence_after();
-                // V rows past the end of the sequence may hold anything: zero them so 0 * x stays 0
-                // (once per tile, by the threads of the first block, thread r taking key row r)
-                if (blk == 0 && tile0 + kTile > n_keys_seq && tile0 + row_local >= n_keys_seq) {
-                    const int st = j % NS;
-                    mbar_wait(B.v_full(st), (j / NS) & 1);
-                    unsigned char* vrow = kv_sm + st * kStageBytes + 2 * kSubTileBytes + row_local * 128;
-                    #pragma unroll 1
-                    for (int c = 0; c < 8; ++c) {
-                        *reinterpret_cast<uint4*>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
-                        *reinterpret_cast<uint4*>(vrow + kSubTileBytes + c * 16) = make_uint4(0, 0, 0, 0);
-                    }
-                    fence_proxy_async();
-                }
-                __syncwarp();
                 if (__any_sync(0xffffffffu, j >= j_tail || j < j_head)) {  // the tile crosses a visibility boundary of some row
                     const unsigned long long lo = vis_word(tile0, my_anc, my_lo), hi = vis_word(tile0 + 64, my_anc, my_lo);
                     #pragma unroll 1
@@ -817,19 +835,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             tmem_wait_ld();
             if (j >= j_tail || j < j_head) {
                 const int tile0 = it.key_begin + j * kTile;          // first key of the tile
-                // V rows past the end of the sequence may hold anything: zero them so 0 * x stays 0
-                // (once per tile, by the first warpgroup, thread r taking key row r)
-                if (wg == 0 && tile0 + row_local >= n_keys_seq) {
-                    const int st = j % NS;
-                    mbar_wait(B.v_full(st), (j / NS) & 1);
-                    unsigned char* vrow = kv_sm + st * kStageBytes + 2 * kSubTileBytes + row_local * 128;
-                    #pragma unroll 1
-                    for (int c = 0; c < 8; ++c) {
-                        *reinterpret_cast<uint4*>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
-                        *reinterpret_cast<uint4*>(vrow + kSubTileBytes + c * 16) = make_uint4(0, 0, 0, 0);
-                    }
-                    fence_proxy_async();
-                }
                 const unsigned long long vis = vis_word(tile0 + sb_wg, anc[0], lo_row[0]);
                 mask_chunk(x0, (uint32_t)vis);
                 mask_chunk(x1, (uint32_t)(vis >> 32));
@@ -962,171 +967,204 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     bulk_store(args.o_part + ((size_t)blockIdx.x * plan.part_rows + bk * kBlockRows) * kPartRowHalves,
                                smem_u32(q_sm + bk * (kBlockRows * kPartRowBytes)), (uint32_t)(rows_here * kPartRowBytes));
             }
-            bulk_store_wait();
-            fence_proxy_async_global();
         }
 
         // ---- publish this item; the call's finisher CTAs merge its partials ---------------------------
         // (overlapped mode: arrival words and finisher counters as described at SyncArgs; a
         // stream-ordered call only stores its partials, and a combine kernel follows)
-        if (sync.enabled) {
-            const int fin_idx = (int)blockIdx.x - (plan.n_items - sync.n_fin);     // >= 0: this CTA is a finisher
-            const int kRowsPerBlock = tpb * qg;                        // 126 for 7 heads x 18 tokens
-            // The call's row list: for every unit (sequence, KV head, row group) with several pieces,
-            // its valid query rows (7 per draft token).  Finisher f takes rows [f chunk, (f + 1) chunk).
+        constexpr int kRowBytes = kPartRowHalves * 2;                   // 272
+        const int fin_idx = (int)blockIdx.x - (plan.n_items - sync.n_fin);     // >= 0: this CTA is a finisher
+        const int rows_per_block = tpb * qg;                            // 126 for 7 heads x 18 tokens
+        const int seq_rows = plan.n_kv_heads * qg * T;                  // query rows of a sequence
+        // The call's row list: the query rows of every sequence with several pieces, (KV head, row group,
+        // row) in order.  Finisher f takes rows [f chunk, (f + 1) chunk).
+        int my_begin = 0, my_end = 0;
+        if (sync.enabled && fin_idx >= 0) {
             int total = 0;
             for (int b = 0; b < plan.batch; ++b)
-                if (plan.seq[b].n_splits > 1) total += plan.n_kv_heads * qg * T;
-            const int chunk = sync.n_fin > 0 ? (total + sync.n_fin - 1) / sync.n_fin : 0;
-            const int my_begin = fin_idx >= 0 ? min(total, fin_idx * chunk) : 0;
-            const int my_end = fin_idx >= 0 ? min(total, my_begin + chunk) : 0;
-            const bool merges = my_begin < my_end;
+                if (plan.seq[b].n_splits > 1) total += seq_rows;
+            const int chunk = (total + sync.n_fin - 1) / sync.n_fin;
+            my_begin = min(total, fin_idx * chunk);
+            my_end = min(total, my_begin + chunk);
+        }
+        const bool merges = my_begin < my_end;
+        MergeList* list = reinterpret_cast<MergeList*>(anc_s);          // (the tables are no longer needed)
+        // Fills the list with what one pass merges, from row `row` on: runs of rows of one unit, as many as
+        // fit the K/V ring with all their pieces.
+        auto list_rows = [&](int row) {
+            int n_seg = 0, bytes = 0;
+            #pragma unroll 1
+            while (row < my_end && n_seg < kMaxSegments) {
+                MergeSegment sg;
+                int rest = row;
+                sg.b = 0;
+                while (plan.seq[sg.b].n_splits == 1 || rest >= seq_rows) {
+                    if (plan.seq[sg.b].n_splits > 1) rest -= seq_rows;
+                    ++sg.b;
+                }
+                sg.ns = plan.seq[sg.b].n_splits;
+                const int kvh = rest / (qg * T);
+                rest -= kvh * qg * T;
+                const int grp = rest / (NB * rows_per_block);
+                sg.r0 = rest - grp * NB * rows_per_block;
+                sg.tok0 = grp * NB * tpb;
+                sg.head0 = kvh * qg;
+                const int unit_left = qg * min(NB * tpb, T - sg.tok0) - sg.r0;
+                sg.n = min(min(unit_left, my_end - row), (NS * kStageBytes - bytes) / (sg.ns * kRowBytes));
+                if (sg.n == 0) break;
+                // the run may straddle the unit's two blocks: `split` rows in the first of them
+                const int bk0 = sg.r0 / rows_per_block;
+                sg.split = (bk0 == 0 && sg.r0 + sg.n > rows_per_block) ? rows_per_block - sg.r0 : sg.n;
+                const int part_row0 = (plan.seq[sg.b].item_begin + (kvh * plan.n_groups + grp) * sg.ns) * plan.part_rows;
+                sg.src = part_row0 + bk0 * kBlockRows + sg.r0 - bk0 * rows_per_block;
+                sg.src2 = part_row0 + kBlockRows;
+                sg.offset = bytes;
+                list->seg[n_seg++] = sg;
+                bytes += sg.n * sg.ns * kRowBytes;
+                row += sg.n;
+            }
+            list->n_seg = n_seg;
+            list->bytes = bytes;
+            list->next_row = row;
+        };
+        // (thread 0, while its bulk copies are on their way)
+        if (tid == 0 && merges) list_rows(my_begin);
+        if (tid == 0 && ok && !direct) {
+            bulk_store_wait();
+            fence_proxy_async_global();
+        }
+        if (sync.enabled) {
             unsigned* arrive_word = sync.arrivals + sync.slot;
             if (tid == 0) SPARROW_STAMP(7);                            // partial rows stored
             if (tid == 0 && !direct) publish_counter(arrive_word);
             if (merges) {
-                // 16 R G threads merge R rows at a time.  The rows' pieces are first brought into the
-                // (idle) K/V ring by bulk copies, [piece][row][272 bytes], one copy per piece and
-                // block touched -- far fewer and larger requests than per-thread loads.
-                // Thread (row i, 16-byte chunk c, piece group g) then folds pieces g, g + G, ... of its
-                // row into a running (max, sum, weighted output); the groups' results meet in shared
-                // memory (the Q blocks, idle by now).  Everything that does not depend on the pieces'
-                // contents is computed in front of the wait for the call's arrivals.
-                constexpr int kRowBytes = kPartRowHalves * 2;               // 272
+                if (tid == 0) {
+                    // every partial of the call in place, and the previous call's final results written
+                    // (both words are polled in one loop: the second is usually there already)
+                    bool have_all = false, prev_done = false;
+                    #pragma unroll 1
+                    for (uint32_t i = 0; i < kCounterPolls && !(have_all && prev_done); ++i) {
+                        if (!have_all) have_all = ld_acquire(arrive_word) == (unsigned)sync.n_arrive;
+                        if (!prev_done) prev_done = (int32_t)(ld_acquire(sync.fin_done + (sync.parity ^ 1)) - sync.fin_wait_other) >= 0;
+                        if (!(have_all && prev_done)) __nanosleep(i < 256 ? 20 : 200);
+                    }
+                    SPARROW_STAMP(8);                                   // all arrivals seen
+                    if (!have_all) atomicOr(args.status, timeout_bits(kSiteArrivals));
+                    else if (!prev_done) atomicOr(args.status, timeout_bits(kSiteFinOther));
+                    SPARROW_STAMP(9);                                   // previous call's finishers seen
+                    *fin_go = (have_all && prev_done) ? 1 : 0;
+                }
+                // The rows' pieces are first brought into the (idle) K/V ring by bulk copies, [piece][row]
+                // [272 bytes], one copy per piece and block touched -- far fewer and larger requests than
+                // per-thread loads.  Then 16 R G threads merge R rows at a time: thread (row i, 16-byte chunk
+                // c, piece group g) folds pieces g, g + G, ... of its row into a running (max, sum, weighted
+                // output); the groups' results meet in shared memory (the Q blocks, idle by now).
                 float* red = reinterpret_cast<float*>(q_sm);                // [256][10]: 8 outputs, sum, max
-                const int unit_rows = NB * kRowsPerBlock;                   // rows of a full row group
-                const int seq_rows = plan.n_kv_heads * qg * T;              // list entries per sequence
-                int phase = 0;
-                bool fin_ok = true, first_pass = true;
+                const int inv_qg = (65536 + qg - 1) / qg;                   // x / qg = x * inv_qg >> 16 for x <= 512
+                const int c16 = tid & 15;
                 #pragma unroll 1
-                for (int row = my_begin; row < my_end && fin_ok;) {
-                    // sequence, KV head, row group and row of list entry `row`
-                    int b = 0, rest = row;
-                    while (plan.seq[b].n_splits == 1 || rest >= seq_rows) {
-                        if (plan.seq[b].n_splits > 1) rest -= seq_rows;
-                        ++b;
-                    }
-                    const int ns = plan.seq[b].n_splits;
-                    const int kvh = rest / (qg * T);
-                    rest -= kvh * qg * T;
-                    const int grp = rest / unit_rows, r0 = rest - grp * unit_rows;
-                    const int tok0 = grp * NB * tpb;                        // first token of this row group
-                    const int unit_left = qg * min(NB * tpb, T - tok0) - r0;
-                    // rows per pass: a power of two, no more than this finisher has, than fit the ring
-                    // with all their pieces, or than 16
-                    int R = 1;
-                    while (R < 16 && R < chunk) R <<= 1;
-                    while (R > 1 && R * ns * kRowBytes > NS * kStageBytes) R >>= 1;
-                    const int G = 16 / R;                                   // piece groups
-                    const int c16 = tid & 15, grp_p = (tid >> 4) % G, row_i = tid / (16 * G);
-                    const int n_here = min(R, min(unit_left, my_end - row));
-                    // the rows may straddle the unit's two blocks: rows [r0, split) and [split, r0 + n_here)
-                    const int bk0 = r0 / kRowsPerBlock;
-                    const int split = (r0 < kRowsPerBlock && r0 + n_here > kRowsPerBlock) ? kRowsPerBlock : r0 + n_here;
-                    const size_t item0 = (size_t)plan.seq[b].item_begin + (size_t)(kvh * plan.n_groups + grp) * ns;
-                    const size_t piece_pitch = (size_t)plan.part_rows * kPartRowHalves;      // halves between pieces
-                    const __half* first = args.o_part + (item0 * plan.part_rows + (size_t)(bk0 * kBlockRows + r0 - bk0 * kRowsPerBlock)) * kPartRowHalves;
-                    const __half* second = args.o_part + (item0 * plan.part_rows + (size_t)kBlockRows) * kPartRowHalves;
-                    const int idx = r0 + row_i;                            // row of the unit's list: token idx / g, head idx % g
-                    const int t = tok0 + idx / qg, h = kvh * qg + idx % qg;
-                    uint4* out_row = reinterpret_cast<uint4*>(args.out + (((size_t)b * T + t) * args.n_q_heads + h) * kD + c16 * 8);
-                    float* lse_row = args.lse + ((size_t)b * args.n_q_heads + h) * T + t;
-                    const uint32_t pstride = (uint32_t)n_here * kRowBytes;     // bytes between pieces in the ring
-                    const uint32_t row_sm = smem_u32(kv_sm) + (uint32_t)row_i * kRowBytes;
-                    if (tid == 0) {
-                        if (first_pass) {
-                            // every partial of the call in place, and the previous call's final results written
-                            // (both words are polled in one loop: the second is usually there already)
-                            bool have_all = false, prev_done = false;
-                            #pragma unroll 1
-                            for (uint32_t i = 0; i < kCounterPolls && !(have_all && prev_done); ++i) {
-                                if (!have_all) have_all = ld_acquire(arrive_word) == (unsigned)sync.n_arrive;
-                                if (!prev_done) prev_done = (int32_t)(ld_acquire(sync.fin_done + (sync.parity ^ 1)) - sync.fin_wait_other) >= 0;
-                                if (!(have_all && prev_done)) __nanosleep(i < 256 ? 20 : 200);
-                            }
-                            SPARROW_STAMP(8);                               // all arrivals seen
-                            if (!have_all) atomicOr(args.status, timeout_bits(kSiteArrivals));
-                            else if (!prev_done) atomicOr(args.status, timeout_bits(kSiteFinOther));
-                            SPARROW_STAMP(9);                               // previous call's finishers seen
-                            *fin_go = (have_all && prev_done) ? 1 : 0;
+                for (int phase = 0;; phase ^= 1) {
+                    if (tid == 0 && *fin_go) mbar_expect_tx(B.fin(), (uint32_t)list->bytes);
+                    softmax_bar_sync();                                    // the list and the byte count are posted
+                    if (!*fin_go) break;
+                    const int n_seg = list->n_seg;
+                    #pragma unroll 1
+                    for (int k = 0; k < n_seg; ++k) {
+                        const MergeSegment& sg = list->seg[k];
+                        const int ns = sg.ns, n = sg.n, split = sg.split;
+                        const __half* src = args.o_part + (size_t)sg.src * kPartRowHalves;
+                        const uint32_t dst = smem_u32(kv_sm) + (uint32_t)sg.offset;
+                        const size_t pitch = (size_t)plan.part_rows * kPartRowHalves;      // halves between pieces
+                        for (int sp = tid; sp < ns; sp += 256) {           // thread sp brings piece sp
+                            bulk_load(dst + (uint32_t)(sp * n * kRowBytes), src + sp * pitch, (uint32_t)split * kRowBytes, B.fin());
+                            if (split < n)
+                                bulk_load(dst + (uint32_t)((sp * n + split) * kRowBytes),
+                                          args.o_part + (size_t)sg.src2 * kPartRowHalves + sp * pitch, (uint32_t)(n - split) * kRowBytes, B.fin());
                         }
-                        if (*fin_go) mbar_expect_tx(B.fin(), (uint32_t)(n_here * ns * kRowBytes));
-                    }
-                    softmax_bar_sync();                                    // the ring's previous contents have been read, the byte count is posted
-                    fin_ok = *fin_go != 0;
-                    if (!fin_ok) break;
-                    for (int sp = tid; sp < ns; sp += 256) {               // thread sp brings piece sp
-                        const uint32_t dst = smem_u32(kv_sm) + (uint32_t)sp * pstride;
-                        bulk_load(dst, first + (size_t)sp * piece_pitch, (uint32_t)(split - r0) * kRowBytes, B.fin());
-                        if (split < r0 + n_here)
-                            bulk_load(dst + (uint32_t)(split - r0) * kRowBytes, second + (size_t)sp * piece_pitch,
-                                      (uint32_t)(r0 + n_here - split) * kRowBytes, B.fin());
                     }
                     if (tid == 0) SPARROW_STAMP(12);                       // bulk copies issued
                     const bool landed = mbar_wait_warp(B.fin(), phase);
-                    phase ^= 1;
-                    first_pass = false;
                     if (tid == 0) SPARROW_STAMP(15);                       // bulk copies landed
-                    if (!landed) { if (lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies)); }
-                    const bool active = landed && row_i < n_here;
-                    float m_run = -INFINITY, s_run = 0.f;                  // natural-log units
-                    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                    if (active) {
-                        #pragma unroll 2
-                        for (uint32_t sp = grp_p, a_o = row_sm + grp_p * pstride; sp < (uint32_t)ns; sp += G, a_o += G * pstride) {
-                            const float l = lds_f32(a_o + 2 * kD);
-                            uint32_t raw[4];
-                            lds_v4(a_o + c16 * 16, raw);
-                            if (l == -INFINITY) continue;                  // a piece that saw no visible key
-                            const float m_new = fmaxf(m_run, l);
-                            const float a = ex2((m_run - m_new) * 1.4426950408889634f);   // 0 for the first piece
-                            const float w = ex2((l - m_new) * 1.4426950408889634f);
-                            s_run = fmaf(s_run, a, w);
-                            #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
-                                acc[2 * q] = fmaf(acc[2 * q], a, w * f.x); acc[2 * q + 1] = fmaf(acc[2 * q + 1], a, w * f.y);
+                    if (!landed && lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies));
+                    #pragma unroll 1
+                    for (int k = 0; k < n_seg; ++k) {
+                        const MergeSegment& sg = list->seg[k];
+                        const int ns = sg.ns, n = sg.n;
+                        int lg_g = 4;                                       // G = 16 / R piece groups, R rows at a time
+                        while (lg_g > 0 && (16 >> lg_g) < n) --lg_g;
+                        const int G = 1 << lg_g, R = 16 >> lg_g;
+                        const int grp_p = (tid >> 4) & (G - 1);
+                        const uint32_t pstride = (uint32_t)n * kRowBytes;   // bytes between pieces in the ring
+                        #pragma unroll 1
+                        for (int r = 0; r < n; r += R) {
+                            const int i = r + (tid >> (4 + lg_g));
+                            const bool active = landed && i < n;
+                            float m_run = -INFINITY, s_run = 0.f;          // natural-log units
+                            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                            if (active) {
+                                uint32_t a_o = smem_u32(kv_sm) + (uint32_t)sg.offset + (uint32_t)i * kRowBytes + grp_p * pstride;
+                                #pragma unroll 2
+                                for (int sp = grp_p; sp < ns; sp += G, a_o += G * pstride) {
+                                    const float l = lds_f32(a_o + 2 * kD);
+                                    uint32_t raw[4];
+                                    lds_v4(a_o + c16 * 16, raw);
+                                    if (l == -INFINITY) continue;          // a piece that saw no visible key
+                                    const float m_new = fmaxf(m_run, l);
+                                    const float a = ex2((m_run - m_new) * 1.4426950408889634f);   // 0 for the first piece
+                                    const float w = ex2((l - m_new) * 1.4426950408889634f);
+                                    s_run = fmaf(s_run, a, w);
+                                    #pragma unroll
+                                    for (int q = 0; q < 4; ++q) {
+                                        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
+                                        acc[2 * q] = fmaf(acc[2 * q], a, w * f.x); acc[2 * q + 1] = fmaf(acc[2 * q + 1], a, w * f.y);
+                                    }
+                                    m_run = m_new;
+                                }
                             }
-                            m_run = m_new;
-                        }
-                    }
-                    if (tid == 0) SPARROW_STAMP(13);                       // pieces folded
-                    if (G > 1) {                                           // (G is the same in every thread)
-                        softmax_bar_sync();                                // the pass before has been read
-                        #pragma unroll
-                        for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
-                        red[tid * 10 + 8] = s_run;
-                        red[tid * 10 + 9] = m_run;
-                        softmax_bar_sync();
-                        if (grp_p == 0) {
-                            const float* mine = red + tid * 10;
-                            float m_all = m_run;
-                            for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
-                            const float a0 = m_run == -INFINITY ? 0.f : ex2((m_run - m_all) * 1.4426950408889634f);
-                            s_run *= a0;
-                            #pragma unroll
-                            for (int q = 0; q < 8; ++q) acc[q] *= a0;
-                            for (int g2 = 1; g2 < G; ++g2) {
-                                const float* o = mine + g2 * 160;
-                                if (o[9] == -INFINITY) continue;
-                                const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
-                                s_run = fmaf(o[8], ag, s_run);
+                            if (tid == 0) SPARROW_STAMP(13);               // pieces folded
+                            if (G > 1) {                                   // (G is the same in every thread; then one round does the run)
+                                softmax_bar_sync();                        // the run before has been read
                                 #pragma unroll
-                                for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
+                                for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
+                                red[tid * 10 + 8] = s_run;
+                                red[tid * 10 + 9] = m_run;
+                                softmax_bar_sync();
+                                if (grp_p == 0) {
+                                    const float* mine = red + tid * 10;
+                                    float m_all = m_run;
+                                    for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
+                                    const float a0 = m_run == -INFINITY ? 0.f : ex2((m_run - m_all) * 1.4426950408889634f);
+                                    s_run *= a0;
+                                    #pragma unroll
+                                    for (int q = 0; q < 8; ++q) acc[q] *= a0;
+                                    for (int g2 = 1; g2 < G; ++g2) {
+                                        const float* o = mine + g2 * 160;
+                                        if (o[9] == -INFINITY) continue;
+                                        const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
+                                        s_run = fmaf(o[8], ag, s_run);
+                                        #pragma unroll
+                                        for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
+                                    }
+                                    m_run = m_all;
+                                }
                             }
-                            m_run = m_all;
+                            if (tid == 0) SPARROW_STAMP(14);               // groups reduced
+                            if (active && grp_p == 0) {
+                                const int idx = sg.r0 + i, tok = (idx * inv_qg) >> 16;       // row of the unit: token idx / g, head idx % g
+                                const int t = sg.tok0 + tok, h = sg.head0 + idx - tok * qg;
+                                const float inv = s_run > 0.f ? __fdividef(1.f, s_run) : 0.f;
+                                uint4 pk;
+                                pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+                                pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+                                *reinterpret_cast<uint4*>(args.out + (((size_t)sg.b * T + t) * args.n_q_heads + h) * kD + c16 * 8) = pk;
+                                if (c16 == 0) args.lse[((size_t)sg.b * args.n_q_heads + h) * T + t] = s_run > 0.f ? m_run + __logf(s_run) : -INFINITY;
+                            }
                         }
                     }
-                    if (tid == 0) SPARROW_STAMP(14);                       // groups reduced
-                    if (active && grp_p == 0) {
-                        const float inv = s_run > 0.f ? __fdividef(1.f, s_run) : 0.f;
-                        uint4 pk;
-                        pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-                        pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
-                        *out_row = pk;
-                        if (c16 == 0) *lse_row = s_run > 0.f ? m_run + __logf(s_run) : -INFINITY;
-                    }
-                    row += n_here;
+                    const int next = list->next_row;
+                    if (!landed || next >= my_end) break;
+                    softmax_bar_sync();                                    // everybody is through with the ring and the list
+                    if (tid == 0) list_rows(next);
                 }
                 if (tid == 0) SPARROW_STAMP(10);                        // merged rows written
                 softmax_bar_sync();
