@@ -65,6 +65,7 @@ struct sparrow_ctx {
     bool log_plans;                          // SPARROW_LOG=1 when the context was created: one line per call on stderr
     bool overlap_single_calls;               // sparrow_set_call_overlap()
     bool in_batch;                           // the call being enqueued belongs to a sparrow_verify_attn_batch()
+    bool prev_lone;                          // the previous fused call published its end relaxed (SyncArgs::lone)
     bool chain_next;                         // the call being enqueued directly follows this context's previous fused call
     // Host mirror of the ordering counters in the workspace (see SyncArgs): call sequence number
     // of the fused calls and, per call parity, the cumulative number of finishers launched so far.
@@ -342,6 +343,7 @@ SyncArgs next_sync(const sparrow_ctx* c, const SplitPlan& p, bool overlaps, bool
     sy.fin_wait_same = c->fin_total[parity];
     sy.fin_wait_other = after_previous ? c->fin_total[parity ^ 1] : c->fin_before_last[parity ^ 1];
     sy.wait_first = 0;
+    sy.lone = overlaps && !may_share;
     sy.call = c->seq;
     return sy;
 }
@@ -640,7 +642,7 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     const CallRanges cr = call_ranges(c, q, k, v, parents, T_tree, T, first_visible, out, lse);
     const bool protocol = call_overlaps(c, st, true);                // not capturing, programmatic launch on
     const bool same_ctx_before = g_last_fused_ctx.exchange(c) == c;
-    const bool early = protocol && same_ctx_before && (c->chain_next || c->overlap_single_calls) &&
+    const bool early = protocol && same_ctx_before && !c->prev_lone && (c->chain_next || c->overlap_single_calls) &&
                        !inputs_touch_recent_outputs(c, cr);
     // Can another call of this context run beside this one?  Only inside a batch, or with the opt-in for
     // single calls.  A call that has the GPU to itself is cut into one wave whatever the policy: measured
@@ -671,6 +673,7 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
         advance_sync(c, plan, sy);
         std::memcpy(c->prev_ranges, cr.r, sizeof(cr.r));
         c->prev_valid = true;
+        c->prev_lone = sy.lone != 0;
         note_fused_launch(c, cr, early);
         return SPARROW_OK;                                   // the kernel merges its own partials
     }

@@ -128,6 +128,7 @@ struct SyncArgs {
     uint32_t fin_wait_same;
     uint32_t fin_wait_other;
     int32_t wait_first;      // launched with programmatic stream serialisation but ordered behind its predecessor: wait before the first global access
+    int32_t lone;            // no later call can start before this grid has ended
     uint32_t call;           // running number of the context's fused calls (the timeline build files its stamps under it)
 };
 
@@ -163,9 +164,9 @@ __device__ __forceinline__ bool wait_equal(const unsigned* addr, uint32_t value)
 }
 // Release-increment of a counter: orders every write this thread has observed (its own and, after
 // a CTA barrier, its CTA's) before the increment.
-__device__ __forceinline__ void publish_counter(unsigned* addr)
+__device__ __forceinline__ void publish_counter(unsigned* addr, unsigned n = 1u)
 {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(addr) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(addr), "r"(n) : "memory");
 }
 
 // Launch overlap between kernels in stream order.  A kernel launched with programmatic stream

@@ -1102,23 +1102,25 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                             float m_run = -INFINITY, s_run = 0.f;          // natural-log units
                             float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                             if (active) {
-                                uint32_t a_o = smem_u32(kv_sm) + (uint32_t)sg.offset + (uint32_t)i * kRowBytes + grp_p * pstride;
+                                // the largest LSE first, so that the pieces' weights do not depend on one another
+                                const uint32_t a0 = smem_u32(kv_sm) + (uint32_t)sg.offset + (uint32_t)i * kRowBytes + grp_p * pstride;
+                                const uint32_t step = (uint32_t)G * pstride;
+                                uint32_t a_o = a0 + 2 * kD;
+                                #pragma unroll 4
+                                for (int sp = grp_p; sp < ns; sp += G, a_o += step) m_run = fmaxf(m_run, lds_f32(a_o));
+                                const float m_log2 = m_run == -INFINITY ? 0.f : m_run * 1.4426950408889634f;   // (all pieces empty: weights 0)
+                                a_o = a0;
                                 #pragma unroll 2
-                                for (int sp = grp_p; sp < ns; sp += G, a_o += G * pstride) {
-                                    const float l = lds_f32(a_o + 2 * kD);
+                                for (int sp = grp_p; sp < ns; sp += G, a_o += step) {
+                                    const float w = ex2(fmaf(lds_f32(a_o + 2 * kD), 1.4426950408889634f, -m_log2));
                                     uint32_t raw[4];
                                     lds_v4(a_o + c16 * 16, raw);
-                                    if (l == -INFINITY) continue;          // a piece that saw no visible key
-                                    const float m_new = fmaxf(m_run, l);
-                                    const float a = ex2((m_run - m_new) * 1.4426950408889634f);   // 0 for the first piece
-                                    const float w = ex2((l - m_new) * 1.4426950408889634f);
-                                    s_run = fmaf(s_run, a, w);
+                                    s_run += w;
                                     #pragma unroll
                                     for (int q = 0; q < 4; ++q) {
                                         const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
-                                        acc[2 * q] = fmaf(acc[2 * q], a, w * f.x); acc[2 * q + 1] = fmaf(acc[2 * q + 1], a, w * f.y);
+                                        acc[2 * q] = fmaf(w, f.x, acc[2 * q]); acc[2 * q + 1] = fmaf(w, f.y, acc[2 * q + 1]);
                                     }
-                                    m_run = m_new;
                                 }
                             }
                             if (tid == 0) SPARROW_STAMP(13);               // pieces folded
@@ -1170,8 +1172,11 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 softmax_bar_sync();
             }
             if (tid == 0) {
-                if (direct) publish_counter(sync.fin_done + sync.parity);
-                if (fin_idx >= 0) publish_counter(sync.fin_done + sync.parity);
+                const unsigned done = (direct ? 1u : 0u) + (fin_idx >= 0 ? 1u : 0u);
+                if (done) {
+                    if (sync.lone) atomicAdd(sync.fin_done + sync.parity, done);       // (relaxed: nobody reads this call's results before the grid has ended)
+                    else publish_counter(sync.fin_done + sync.parity, done);
+                }
             }
         }
         if (!ok) { atomicOr(args.status, timeout_bits(kSiteSoftmax)); *abort_flag = 1; }
