@@ -92,8 +92,8 @@ __device__ __forceinline__ uint32_t cluster_rank()
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+using tc::cluster_arrive;
+using tc::cluster_wait;
 // 16 bytes into the same place of CTA `rank`'s shared memory, counted on its mbarrier.
 __device__ __forceinline__ void push_2x64(const void* local, const uint64_t* local_bar, uint32_t rank, long long a, long long b)
 {

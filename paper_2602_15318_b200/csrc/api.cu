@@ -60,6 +60,7 @@ struct sparrow_ctx {
     size_t part_offset;                      // first byte of the split-KV partials in the workspace
     int part_buffers;                        // 2: alternate by call parity (fused mode); 1: stream-ordered calls only
     std::atomic<long long> launches;
+    const int* max_clusters[2];              // by row blocks - 1: verification clusters of 1 .. 16 CTAs that can run at once
     int max_sample_cluster;                  // CTAs per cluster of the temperature-1 acceptance kernel the device takes
     bool use_pdl;
     bool log_plans;                          // SPARROW_LOG=1 when the context was created: one line per call on stderr
@@ -334,7 +335,7 @@ SyncArgs next_sync(const sparrow_ctx* c, const SplitPlan& p, bool overlaps, bool
     sy.slot = (int)(c->seq & 3u);
     int n_arrive = 0;
     for (int b = 0; b < p.batch; ++b)
-        if (p.seq[b].n_splits > 1) n_arrive += p.n_kv_heads * p.n_groups * p.seq[b].n_splits;
+        if (p.seq[b].n_splits > 1 && p.cluster <= 1) n_arrive += p.n_kv_heads * p.n_groups * p.seq[b].n_splits;
     sy.n_arrive = n_arrive;
     // Finishers wait, holding their SM, until the call's last piece is in: few of them where later
     // calls should move in beside this one, all CTAs where none can or under the latency policy.
@@ -513,14 +514,18 @@ sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const Syn
     cfg.blockDim = dim3(tc::kThreads);
     cfg.dynamicSmemBytes = tc::smem_bytes(nb, nb == 1 ? 3 : 2);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)(plan.cluster > 1 ? plan.cluster : 1);
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     // Programmatic: an early start (only where verify_call() has made sure that the kernel directly
     // before is this context's previous call), or, with wait_first, stream order with the launch and
     // the set-up overlapping the predecessor's end.
-    cfg.numAttrs = sy.enabled ? 1 : 0;
+    cfg.numAttrs = !sy.enabled ? 0 : plan.cluster > 1 ? 2 : 1;       // (clusters only occur among these)
     const cudaError_t e = nb == 1 ? cudaLaunchKernelEx(&cfg, tc::verify_tc_kernel<1>, a, sy, plan, mq, mk, mv)
                                   : cudaLaunchKernelEx(&cfg, tc::verify_tc_kernel<2>, a, sy, plan, mq, mk, mv);
     if (e != cudaSuccess) return SPARROW_ERR_CUDA;
@@ -588,6 +593,50 @@ int sample_cluster_limit(int device)
     return n;
 }
 
+// Clusters of n = 1 .. 16 CTAs of the verification kernel (one CTA per SM) that can run at once on the
+// current device, by row blocks - 1; asked once per device and process.
+using tc::kMaxMergeCluster;
+struct ClusterTable {
+    std::atomic<int> state;                   // 0 unknown, 1 being filled, 2 known
+    int n[2][kMaxMergeCluster + 1];
+};
+template <int NB>
+void query_max_clusters(int* n)
+{
+    n[0] = n[1] = 0;
+    const bool wide = cudaFuncSetAttribute(tc::verify_tc_kernel<NB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (int c = 2; c <= kMaxMergeCluster; ++c) {
+        n[c] = 0;
+        if (c > 8 && !wide) continue;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)c);
+        cfg.blockDim = dim3(tc::kThreads);
+        cfg.dynamicSmemBytes = tc::smem_bytes(NB, NB == 1 ? 3 : 2);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)c;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n[c], tc::verify_tc_kernel<NB>, &cfg) != cudaSuccess) n[c] = 0;
+    }
+    cudaGetLastError();
+}
+const ClusterTable* cluster_table(int device)
+{
+    static ClusterTable tables[kMaxStaticDevices];
+    if (device < 0 || device >= kMaxStaticDevices) return nullptr;
+    ClusterTable& t = tables[device];
+    int expected = 0;
+    if (t.state.compare_exchange_strong(expected, 1)) {
+        query_max_clusters<1>(t.n[0]);
+        query_max_clusters<2>(t.n[1]);
+        t.state.store(2);
+    }
+    return t.state.load() == 2 ? &t : nullptr;      // (a thread that comes while another one asks does without)
+}
+
 struct DeviceGuard {
     int prev = -1;
     bool ok = true;
@@ -606,6 +655,47 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
     for (int i = 0; i < T; ++i)
         if (parents[i] < -1 || parents[i] >= i) return SPARROW_ERR_TREE;
     return SPARROW_OK;
+}
+
+constexpr float kTileUs[2] = {1.2f, 2.0f};            // a tile of 128 keys, one / two row blocks
+constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f;
+// A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
+// be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
+// at most 16 pieces per unit, pieces short enough to leave a stage of the K/V ring free for the rows that are
+// sent around (2 tiles with one row block, 1 with two), and whole clusters per GPC.  Rewrites the plan where
+// that is estimated to pay.  Estimates in us, from single calls: PLACEHOLDER
+void plan_lone_call(const sparrow_ctx* c, SplitPlan* p)
+{
+    const int nb = p->blocks_per_group, units = p->batch * p->n_kv_heads * p->n_groups;
+    const float per_tile = nb == 1 ? kTileUs[0] : kTileUs[1];
+    const int free_stage_tiles = nb == 1 ? 2 : 1;
+    int most = 0, least = 1 << 30;                     // tiles of the longest and the shortest sequence
+    float best = 0.f;
+    for (int b = 0; b < p->batch; ++b) {
+        const int tiles = (p->seq[b].n_keys - p->seq[b].key0 + kKeyTile - 1) / kKeyTile;
+        const int piece = (tiles + p->seq[b].n_splits - 1) / p->seq[b].n_splits;
+        if (tiles > most) most = tiles;
+        if (tiles < least) least = tiles;
+        const float t = per_tile * piece + (p->seq[b].n_splits > 1 ? kMergeWorkspaceUs : 0.f);
+        if (t > best) best = t;
+    }
+    int pieces = 0;
+    for (int n = 1; n <= kMaxMergeCluster && n <= least; ++n) {
+        const int piece = (most + n - 1) / n;
+        if (n == 1 && units > c->n_sm) continue;
+        if (n > 1 && (piece > free_stage_tiles || !c->max_clusters[nb - 1] || units > c->max_clusters[nb - 1][n])) continue;
+        const float t = per_tile * piece + (n > 1 ? kMergeClusterUs : 0.f);
+        if (t < best) { best = t; pieces = n; }
+    }
+    if (pieces == 0) return;
+    int total = 0;
+    for (int b = 0; b < p->batch; ++b) {
+        p->seq[b].n_splits = pieces;
+        p->seq[b].item_begin = total;
+        total += p->n_kv_heads * p->n_groups * pieces;
+    }
+    p->n_items = total;
+    p->cluster = pieces;
 }
 
 // One verification call: T query tokens, the last T of the T_tree nodes whose K/V rows sit at
@@ -655,6 +745,7 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     sparrow_status s = make_plan(plan_target(c, may_share), c->layout.batch, c->layout.n_kv_heads, group, n_keys, T,
                                  blocks_per_group_tc(T, group), &plan, kMinPieceKeys, key0);
     if (s != SPARROW_OK) return s;
+    if (protocol && !may_share) plan_lone_call(c, &plan);
     plan.T_tree = T_tree;
     for (int b = 0; b < c->layout.batch; ++b) plan.seq[b].kv_len = kv_len[b];
     if ((s = check_ws(c, plan)) != SPARROW_OK) return s;
@@ -666,7 +757,8 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
                      protocol ? "counter protocol" : "stream-ordered", early ? "starts early" : "stream order");
         for (int b = 0; b < plan.batch; ++b)
             std::fprintf(stderr, " seq %d: keys [%d, %d) in %d piece(s)", b, plan.seq[b].key0, plan.seq[b].n_keys, plan.seq[b].n_splits);
-        std::fprintf(stderr, "; %d finisher(s)\n", sy.n_fin);
+        if (plan.cluster > 1) std::fprintf(stderr, "; merged in clusters of %d\n", plan.cluster);
+        else std::fprintf(stderr, "; %d finisher(s)\n", sy.n_fin);
     }
     if ((s = launch_verify_tc(c, plan, sy, q, k, v, parents, first_visible, out, lse, st)) != SPARROW_OK) return s;
     if (protocol) {
@@ -752,6 +844,10 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
     c->part_buffers = 2;
     c->launches.store(0);
     c->max_sample_cluster = sample_cluster_limit(device);
+    if (const ClusterTable* ct = cluster_table(device)) {
+        c->max_clusters[0] = ct->n[0];
+        c->max_clusters[1] = ct->n[1];
+    }
     const char* e = std::getenv("SPARROW_NO_PDL");
     // more SMs than the list of possibly-resident calls can hold: calls never start early
     c->use_pdl = !(e && e[0] == '1') && c->n_sm < kRecentCalls;

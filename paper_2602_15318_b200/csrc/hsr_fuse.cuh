@@ -63,14 +63,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8])
                  : "r"(taddr) : "memory");
 }
 
-__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
 __device__ __forceinline__ void st_cluster_v4(uint32_t addr, float a, float b, float c, float d)
 {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
@@ -233,8 +225,8 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
     if (args.n_slices > 1) {
         // one cluster barrier: every slice's pushes have landed; after it nobody touches a peer
         if (tid == 0) SPARROW_STAMP(5);                                 // partial sums pushed
-        cluster_arrive_release();
-        cluster_wait_acquire();
+        cluster_arrive();
+        cluster_wait();
         if (tid == 0) SPARROW_STAMP(6);                                 // cluster barrier passed
         if (warp < 4) {
             // part 2: the slices in fixed order (results do not depend on timing), bias, bf16 z

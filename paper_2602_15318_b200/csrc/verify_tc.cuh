@@ -85,13 +85,21 @@ constexpr int kTile = 128;                       // keys per stage and per job
 constexpr int kSubTileBytes = 128 * 64 * 2;      // one 128 x 64 bf16 box: 16 KB
 constexpr int kQBlockBytes = 2 * kSubTileBytes;  // 128 rows x 128 dims: 32 KB
 constexpr int kStageBytes = 4 * kSubTileBytes;   // K (32 KB) + V (32 KB)
+constexpr int kRowBytes = kPartRowHalves * 2;    // a partial row: 272 bytes
 constexpr int kMiscBytes = 2048;                 // barriers, flags, ancestor words, maxima exchange
 constexpr uint32_t kSpinLimit = 1u << 22;        // polls before a wait gives up
 constexpr float kRescaleLog2 = 8.0f;             // lazy-max threshold in log2 units
 
+// Rows received from the CTAs of a cluster lie in the ring's last stage; with two row blocks (up to 256 rows and
+// rounded-up shares) they need a little more behind it.
+constexpr int kMaxMergeCluster = 16;
+__host__ __device__ constexpr int recv_extra(int n_blocks)
+{
+    return n_blocks == 1 ? 0 : ((2 * kBlockRows + kMaxMergeCluster) * kRowBytes - kStageBytes + 1023) / 1024 * 1024;
+}
 __host__ __device__ constexpr int smem_bytes(int n_blocks, int n_stages)
 {
-    return 1024 /*alignment slack*/ + n_blocks * kQBlockBytes + n_stages * kStageBytes + kMiscBytes;
+    return 1024 /*alignment slack*/ + n_blocks * kQBlockBytes + n_stages * kStageBytes + recv_extra(n_blocks) + kMiscBytes;
 }
 // S blocks (score tiles in flight) for a given number of row blocks; TMEM: S blocks first, then
 // one 128-column O accumulator per row block, 512 columns in all.
@@ -182,6 +190,24 @@ __device__ __forceinline__ void softmax_bar_sync() { asm volatile("bar.sync 1, 2
 // The gatekeeper warp has filled the tables that the 256 softmax threads read (id 3).
 __device__ __forceinline__ void tables_ready_arrive() { asm volatile("bar.arrive 3, 288;" ::: "memory"); }
 __device__ __forceinline__ void tables_ready_sync() { asm volatile("bar.sync 3, 288;" ::: "memory"); }
+// ---- thread-block clusters
+// (relaxed: nothing but the barrier's own phase is ordered; a releasing arrive took 0.7 us of every set-up)
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// address of the same place in the shared memory of CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// 1-D bulk copy from this CTA's shared memory to a CTA of the cluster, counted on an mbarrier there
+__device__ __forceinline__ void bulk_push(uint32_t dst_cluster, uint32_t src, uint32_t bytes, uint32_t bar_cluster)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst_cluster), "r"(src), "r"(bytes), "r"(bar_cluster) : "memory");
+}
 // One lane of a converged warp.  The tensor-core instructions take their descriptors from uniform
 // registers, which the compiler only uses behind elect.sync in a warp whose control flow stays
 // converged.  Behind `if (lane == 0)` every tcgen05.mma first moves its operands over: 93 to 104
@@ -410,7 +436,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     constexpr int NS = NB == 1 ? 3 : 2;               // K/V ring depth
     unsigned char* q_sm = sm;
     unsigned char* kv_sm = sm + NB * kQBlockBytes;
-    unsigned char* misc = kv_sm + NS * kStageBytes;
+    unsigned char* misc = kv_sm + NS * kStageBytes + recv_extra(NB);
     uint64_t* bar_mem = reinterpret_cast<uint64_t*>(misc);                  // 28 barrier slots in 224 bytes
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 224);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(misc + 228);
@@ -487,6 +513,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (plan.cluster > 1) cluster_arrive_relaxed();      // (waited for ahead of the first access to a peer)
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 0) SPARROW_STAMP(1);                             // set-up done
     // (behind the wait above: a dependent that starts early may rely on everything before this call)
@@ -674,7 +701,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             // epilogue's critical path.  1 = go, 2 = a wait gave up.
             bool go = wait_counter(sync.fin_done + sync.parity, sync.fin_wait_same);
             if (!go) atomicOr(args.status, timeout_bits(kSiteWriteSame));
-            if (go && plan.seq[it.b].n_splits == 1) {
+            if (go && (plan.seq[it.b].n_splits == 1 || plan.cluster > 1)) {
                 go = wait_counter(sync.fin_done + (sync.parity ^ 1), sync.fin_wait_other);
                 if (!go) atomicOr(args.status, timeout_bits(kSiteWriteOther));
             }
@@ -894,6 +921,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // ---- epilogue: normalised partial output + natural-log LSE -------------------------------
         if (tid == 0) SPARROW_STAMP(5);                                 // softmax loop left
         const bool direct = plan.seq[it.b].n_splits == 1;                  // the only piece: write the final result
+        const bool clustered = plan.cluster > 1;                           // the unit's pieces meet in the cluster's shared memory
         if (tid == 0) {
             // Global writes start below.  In overlapped mode a lane of the MMA warp has been waiting,
             // since the kernel started, for the counters that allow them (see there).
@@ -925,12 +953,11 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // completion orders them ahead of the publication, where ordinary stores needed a second pass
         // and a proxy fence.  The staging area is the Q blocks and the start of the K ring: every Q K^T
         // completed ahead of the product waited for above.
-        constexpr int kPartRowBytes = kPartRowHalves * 2;
-        unsigned char* stage = q_sm + blk * (kBlockRows * kPartRowBytes);
+        unsigned char* stage = q_sm + blk * (kBlockRows * kRowBytes);
         if (ok && my_row) {
             if (wg == 0 || NB == 2) {
                 if (direct) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + my_t] = lse_val;
-                else *reinterpret_cast<float*>(stage + row_local * kPartRowBytes + kD * 2) = lse_val;
+                else *reinterpret_cast<float*>(stage + row_local * kRowBytes + kD * 2) = lse_val;
             }
         }
         if (ok) {
@@ -949,7 +976,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 } else {
                     #pragma unroll
                     for (int c = 0; c < 16; ++c) w[c] = pack_half2(o[2 * c] * inv, o[2 * c + 1] * inv);
-                    dst = reinterpret_cast<uint4*>(stage + row_local * kPartRowBytes + col * 2);
+                    dst = reinterpret_cast<uint4*>(stage + row_local * kRowBytes + col * 2);
                 }
                 if (my_row) {
                     #pragma unroll
@@ -959,20 +986,19 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
         if (!direct) fence_proxy_async();                              // the staged rows, ahead of the bulk copies
         softmax_bar_sync();                                            // every row is staged (or written)
-        if (tid == 0 && ok && !direct) {
+        if (tid == 0 && ok && !direct && !clustered) {
             #pragma unroll
             for (int bk = 0; bk < NB; ++bk) {
                 const int rows_here = min(tpb, max(0, T - (block0 + bk) * tpb)) * qg;
                 if (rows_here > 0)
                     bulk_store(args.o_part + ((size_t)blockIdx.x * plan.part_rows + bk * kBlockRows) * kPartRowHalves,
-                               smem_u32(q_sm + bk * (kBlockRows * kPartRowBytes)), (uint32_t)(rows_here * kPartRowBytes));
+                               smem_u32(q_sm + bk * (kBlockRows * kRowBytes)), (uint32_t)(rows_here * kRowBytes));
             }
         }
 
         // ---- publish this item; the call's finisher CTAs merge its partials ---------------------------
         // (overlapped mode: arrival words and finisher counters as described at SyncArgs; a
         // stream-ordered call only stores its partials, and a combine kernel follows)
-        constexpr int kRowBytes = kPartRowHalves * 2;                   // 272
         const int fin_idx = (int)blockIdx.x - (plan.n_items - sync.n_fin);     // >= 0: this CTA is a finisher
         const int rows_per_block = tpb * qg;                            // 126 for 7 heads x 18 tokens
         const int seq_rows = plan.n_kv_heads * qg * T;                  // query rows of a sequence
@@ -1027,16 +1053,129 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             list->bytes = bytes;
             list->next_row = row;
         };
+        // Merging is done by 16 R G threads, R rows at a time: thread (row i, 16-byte chunk c16, piece group
+        // g) folds pieces g, g + G, ... of its row; the groups' results meet in shared memory here, and the
+        // row is written.
+        // [256][10]: 8 outputs, sum, max; over the Q blocks, or where rows on their way to peers lie there, over a V tile
+        float* red = reinterpret_cast<float*>(clustered ? kv_sm + 2 * kSubTileBytes : q_sm);
+        const int inv_qg = (65536 + qg - 1) / qg;                       // x / qg = x * inv_qg >> 16 for x <= 512
+        const int c16 = tid & 15;
+        auto finish_row = [&](float (&acc)[8], float s_run, float m_run, bool active, int G, int grp_p, int b, int t, int h) {
+            if (G > 1) {                                               // (G is the same in every thread)
+                softmax_bar_sync();                                    // the run before has been read
+                #pragma unroll
+                for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
+                red[tid * 10 + 8] = s_run;
+                red[tid * 10 + 9] = m_run;
+                softmax_bar_sync();
+                if (grp_p == 0) {
+                    const float* mine = red + tid * 10;
+                    float m_all = m_run;
+                    for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
+                    const float a0 = m_run == -INFINITY ? 0.f : ex2((m_run - m_all) * 1.4426950408889634f);
+                    s_run *= a0;
+                    #pragma unroll
+                    for (int q = 0; q < 8; ++q) acc[q] *= a0;
+                    for (int g2 = 1; g2 < G; ++g2) {
+                        const float* o = mine + g2 * 160;
+                        if (o[9] == -INFINITY) continue;
+                        const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
+                        s_run = fmaf(o[8], ag, s_run);
+                        #pragma unroll
+                        for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
+                    }
+                    m_run = m_all;
+                }
+            }
+            if (tid == 0) SPARROW_STAMP(14);                           // groups reduced
+            if (active && grp_p == 0) {
+                const float inv = s_run > 0.f ? __fdividef(1.f, s_run) : 0.f;
+                uint4 pk;
+                pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+                pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+                *reinterpret_cast<uint4*>(args.out + (((size_t)b * T + t) * args.n_q_heads + h) * kD + c16 * 8) = pk;
+                if (c16 == 0) args.lse[((size_t)b * args.n_q_heads + h) * T + t] = s_run > 0.f ? m_run + __logf(s_run) : -INFINITY;
+            }
+        };
+        // Merges rows [0, n) of a run whose pieces lie at `base` as [piece][row][272 bytes]; row i is row r0 + i of
+        // its unit.
+        auto merge_run = [&](uint32_t base, int ns, int n, int r0, int b, int tok0, int head0, bool landed) {
+            int lg_g = 4;                                              // G = 16 / R piece groups, R rows at a time
+            while (lg_g > 0 && (16 >> lg_g) < n) --lg_g;
+            const int G = 1 << lg_g, R = 16 >> lg_g;
+            const int grp_p = (tid >> 4) & (G - 1);
+            const uint32_t pstride = (uint32_t)n * kRowBytes;          // bytes between pieces
+            #pragma unroll 1
+            for (int r = 0; r < n; r += R) {
+                const int i = r + (tid >> (4 + lg_g));
+                const bool active = landed && i < n;
+                float m_run = -INFINITY, s_run = 0.f;                  // natural-log units
+                float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                if (active) {
+                    // the largest LSE first, so that the pieces' weights do not depend on one another
+                    const uint32_t a0 = base + (uint32_t)i * kRowBytes + grp_p * pstride, step = (uint32_t)G * pstride;
+                    uint32_t a_o = a0 + 2 * kD;
+                    #pragma unroll 4
+                    for (int sp = grp_p; sp < ns; sp += G, a_o += step) m_run = fmaxf(m_run, lds_f32(a_o));
+                    const float m_log2 = m_run == -INFINITY ? 0.f : m_run * 1.4426950408889634f;   // (all pieces empty: weights 0)
+                    a_o = a0;
+                    #pragma unroll 2
+                    for (int sp = grp_p; sp < ns; sp += G, a_o += step) {
+                        const float w = ex2(fmaf(lds_f32(a_o + 2 * kD), 1.4426950408889634f, -m_log2));
+                        uint32_t raw[4];
+                        lds_v4(a_o + c16 * 16, raw);
+                        s_run += w;
+                        #pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
+                            acc[2 * q] = fmaf(w, f.x, acc[2 * q]); acc[2 * q + 1] = fmaf(w, f.y, acc[2 * q + 1]);
+                        }
+                    }
+                }
+                if (tid == 0) SPARROW_STAMP(13);                       // pieces folded
+                const int idx = r0 + i, tok = (idx * inv_qg) >> 16;    // token idx / g, head idx % g
+                finish_row(acc, s_run, m_run, active, G, grp_p, b, tok0 + tok, head0 + idx - tok * qg);
+            }
+        };
+        if (clustered) {
+            // Every CTA of the cluster merges a share of the unit's rows: it is sent its rows of every piece, one
+            // bulk copy from each peer, into the last stage of the K/V ring, which pieces this short never use.
+            const int cl = plan.cluster;
+            const int unit_rows = qg * min(NB * tpb, T - block0 * tpb);
+            const uint32_t recv = smem_u32(kv_sm) + (NS - 1) * kStageBytes;
+            const int r_begin = unit_rows * it.split / cl, n = unit_rows * (it.split + 1) / cl - r_begin;
+            cluster_wait();                                            // every peer runs, its barriers are initialised
+            if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n * cl * kRowBytes));
+            if (tid < cl) {
+                const int r0 = unit_rows * tid / cl, r1 = unit_rows * (tid + 1) / cl;      // peer tid's share
+                const uint32_t dst = map_to_rank(recv + (uint32_t)(it.split * (r1 - r0) * kRowBytes), (uint32_t)tid);
+                const uint32_t bar = map_to_rank(B.fin(), (uint32_t)tid);
+                // (staged block by block: the share may straddle the two)
+                const int mid = min(max(rows_per_block, r0), r1);
+                if (mid > r0) bulk_push(dst, smem_u32(q_sm) + (uint32_t)(r0 * kRowBytes), (uint32_t)((mid - r0) * kRowBytes), bar);
+                if (r1 > mid)
+                    bulk_push(dst + (uint32_t)((mid - r0) * kRowBytes),
+                              smem_u32(q_sm) + (uint32_t)((kBlockRows + mid - rows_per_block) * kRowBytes), (uint32_t)((r1 - mid) * kRowBytes), bar);
+            }
+            if (tid == 0) SPARROW_STAMP(12);                           // pushes issued
+            const bool landed = mbar_wait_warp(B.fin(), 0);
+            cluster_arrive_relaxed();                                  // (all pushes to this CTA are through: its peers may leave)
+            if (!landed && lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies));
+            if (tid == 0) SPARROW_STAMP(15);                           // every piece is here
+            merge_run(recv, cl, n, r_begin, it.b, block0 * tpb, it.kvh * qg, landed && ok);
+            if (tid == 0) SPARROW_STAMP(10);                           // merged rows written
+            softmax_bar_sync();
+        }
         // (thread 0, while its bulk copies are on their way)
         if (tid == 0 && merges) list_rows(my_begin);
-        if (tid == 0 && ok && !direct) {
+        if (tid == 0 && ok && !direct && !clustered) {
             bulk_store_wait();
             fence_proxy_async_global();
         }
         if (sync.enabled) {
             unsigned* arrive_word = sync.arrivals + sync.slot;
             if (tid == 0) SPARROW_STAMP(7);                            // partial rows stored
-            if (tid == 0 && !direct) publish_counter(arrive_word);
+            if (tid == 0 && !direct && !clustered) publish_counter(arrive_word);
             if (merges) {
                 if (tid == 0) {
                     // every partial of the call in place, and the previous call's final results written
@@ -1059,9 +1198,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 // per-thread loads.  Then 16 R G threads merge R rows at a time: thread (row i, 16-byte chunk
                 // c, piece group g) folds pieces g, g + G, ... of its row into a running (max, sum, weighted
                 // output); the groups' results meet in shared memory (the Q blocks, idle by now).
-                float* red = reinterpret_cast<float*>(q_sm);                // [256][10]: 8 outputs, sum, max
-                const int inv_qg = (65536 + qg - 1) / qg;                   // x / qg = x * inv_qg >> 16 for x <= 512
-                const int c16 = tid & 15;
                 #pragma unroll 1
                 for (int phase = 0;; phase ^= 1) {
                     if (tid == 0 && *fin_go) mbar_expect_tx(B.fin(), (uint32_t)list->bytes);
@@ -1089,79 +1225,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     #pragma unroll 1
                     for (int k = 0; k < n_seg; ++k) {
                         const MergeSegment& sg = list->seg[k];
-                        const int ns = sg.ns, n = sg.n;
-                        int lg_g = 4;                                       // G = 16 / R piece groups, R rows at a time
-                        while (lg_g > 0 && (16 >> lg_g) < n) --lg_g;
-                        const int G = 1 << lg_g, R = 16 >> lg_g;
-                        const int grp_p = (tid >> 4) & (G - 1);
-                        const uint32_t pstride = (uint32_t)n * kRowBytes;   // bytes between pieces in the ring
-                        #pragma unroll 1
-                        for (int r = 0; r < n; r += R) {
-                            const int i = r + (tid >> (4 + lg_g));
-                            const bool active = landed && i < n;
-                            float m_run = -INFINITY, s_run = 0.f;          // natural-log units
-                            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                            if (active) {
-                                // the largest LSE first, so that the pieces' weights do not depend on one another
-                                const uint32_t a0 = smem_u32(kv_sm) + (uint32_t)sg.offset + (uint32_t)i * kRowBytes + grp_p * pstride;
-                                const uint32_t step = (uint32_t)G * pstride;
-                                uint32_t a_o = a0 + 2 * kD;
-                                #pragma unroll 4
-                                for (int sp = grp_p; sp < ns; sp += G, a_o += step) m_run = fmaxf(m_run, lds_f32(a_o));
-                                const float m_log2 = m_run == -INFINITY ? 0.f : m_run * 1.4426950408889634f;   // (all pieces empty: weights 0)
-                                a_o = a0;
-                                #pragma unroll 2
-                                for (int sp = grp_p; sp < ns; sp += G, a_o += step) {
-                                    const float w = ex2(fmaf(lds_f32(a_o + 2 * kD), 1.4426950408889634f, -m_log2));
-                                    uint32_t raw[4];
-                                    lds_v4(a_o + c16 * 16, raw);
-                                    s_run += w;
-                                    #pragma unroll
-                                    for (int q = 0; q < 4; ++q) {
-                                        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
-                                        acc[2 * q] = fmaf(w, f.x, acc[2 * q]); acc[2 * q + 1] = fmaf(w, f.y, acc[2 * q + 1]);
-                                    }
-                                }
-                            }
-                            if (tid == 0) SPARROW_STAMP(13);               // pieces folded
-                            if (G > 1) {                                   // (G is the same in every thread; then one round does the run)
-                                softmax_bar_sync();                        // the run before has been read
-                                #pragma unroll
-                                for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
-                                red[tid * 10 + 8] = s_run;
-                                red[tid * 10 + 9] = m_run;
-                                softmax_bar_sync();
-                                if (grp_p == 0) {
-                                    const float* mine = red + tid * 10;
-                                    float m_all = m_run;
-                                    for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
-                                    const float a0 = m_run == -INFINITY ? 0.f : ex2((m_run - m_all) * 1.4426950408889634f);
-                                    s_run *= a0;
-                                    #pragma unroll
-                                    for (int q = 0; q < 8; ++q) acc[q] *= a0;
-                                    for (int g2 = 1; g2 < G; ++g2) {
-                                        const float* o = mine + g2 * 160;
-                                        if (o[9] == -INFINITY) continue;
-                                        const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
-                                        s_run = fmaf(o[8], ag, s_run);
-                                        #pragma unroll
-                                        for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
-                                    }
-                                    m_run = m_all;
-                                }
-                            }
-                            if (tid == 0) SPARROW_STAMP(14);               // groups reduced
-                            if (active && grp_p == 0) {
-                                const int idx = sg.r0 + i, tok = (idx * inv_qg) >> 16;       // row of the unit: token idx / g, head idx % g
-                                const int t = sg.tok0 + tok, h = sg.head0 + idx - tok * qg;
-                                const float inv = s_run > 0.f ? __fdividef(1.f, s_run) : 0.f;
-                                uint4 pk;
-                                pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-                                pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
-                                *reinterpret_cast<uint4*>(args.out + (((size_t)sg.b * T + t) * args.n_q_heads + h) * kD + c16 * 8) = pk;
-                                if (c16 == 0) args.lse[((size_t)sg.b * args.n_q_heads + h) * T + t] = s_run > 0.f ? m_run + __logf(s_run) : -INFINITY;
-                            }
-                        }
+                        merge_run(smem_u32(kv_sm) + (uint32_t)sg.offset, sg.ns, sg.n, sg.r0, sg.b, sg.tok0, sg.head0, landed);
                     }
                     const int next = list->next_row;
                     if (!landed || next >= my_end) break;
@@ -1172,7 +1236,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 softmax_bar_sync();
             }
             if (tid == 0) {
-                const unsigned done = (direct ? 1u : 0u) + (fin_idx >= 0 ? 1u : 0u);
+                const unsigned done = (direct || clustered ? 1u : 0u) + (fin_idx >= 0 ? 1u : 0u);
                 if (done) {
                     if (sync.lone) atomicAdd(sync.fin_done + sync.parity, done);       // (relaxed: nobody reads this call's results before the grid has ended)
                     else publish_counter(sync.fin_done + sync.parity, done);
@@ -1183,6 +1247,11 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     }
 
     // ---- teardown -------------------------------------------------------------------------------
+    if (plan.cluster > 1) {
+        // Nobody leaves before its peers have received what it sends them.
+        if (warp >= 8) { cluster_wait(); cluster_arrive_relaxed(); }    // (the softmax warps have done both)
+        cluster_wait();
+    }
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) {
