@@ -15,9 +15,9 @@ namespace sparrow {
 // from the root down, path[n .. T) = -1; bonus = target_next[last + 1] (target_next[0] if none).
 // A parent outside [-1, i) sets the tree status bit and counts as "root".
 __global__ void __launch_bounds__(kMaxBatch)
-accept_greedy_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __restrict__ parents,
-                     const int32_t* __restrict__ target_next, int batch, int T, int32_t* __restrict__ path,
-                     int32_t* __restrict__ n_accept, int32_t* __restrict__ bonus, unsigned* status)
+accept_greedy_kernel(const int32_t* draft_tokens, const int32_t* parents,
+                     const int32_t* target_next, int batch, int T, int32_t* path,
+                     int32_t* n_accept, int32_t* bonus, unsigned* status)
 {
     let_dependents_launch();
     wait_for_predecessors();

@@ -103,14 +103,6 @@ __device__ __forceinline__ void push_2x64(const void* local, const uint64_t* loc
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];"
                  ::"r"(addr), "l"(a), "l"(b), "r"(bar) : "memory");
 }
-// A load that stays where it is written: ahead of the wait it is meant to overlap.
-__device__ __forceinline__ float ld_now(const float* p)
-{
-    float v;
-    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
 struct Shared {
     Level lv;
     uint64_t bar[2];                                    // the cluster's pushes of even / odd steps have landed
@@ -164,10 +156,10 @@ __device__ __forceinline__ bool cluster_sum(Shared& sh, long long& a, long long&
 }
 
 __global__ void __launch_bounds__(kThreads)
-accept_sample_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __restrict__ parents,
-                     const float* __restrict__ p_target, const float* __restrict__ p_draft,
-                     const uint32_t* __restrict__ u_node, const uint32_t* __restrict__ u_bonus, int T, int V, int n_cta, int resident,
-                     int32_t* __restrict__ path, int32_t* __restrict__ n_accept, int32_t* __restrict__ bonus, unsigned* status)
+accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
+                     const float* p_target, const float* p_draft,
+                     const uint32_t* u_node, const uint32_t* u_bonus, int T, int V, int n_cta, int resident,
+                     int32_t* path, int32_t* n_accept, int32_t* bonus, unsigned* status)
 {
     let_dependents_launch();
     wait_for_predecessors();
@@ -189,8 +181,8 @@ accept_sample_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __
         #pragma unroll
         for (int k = 0; k < kAhead; ++k) {
             const int i = k * kThreads + tid;
-            fp[k] = i < n_mine ? ld_now(pt + i) : 0.f;
-            fq[k] = i < n_mine ? ld_now(pq + i) : 0.f;
+            fp[k] = i < n_mine ? ld_behind(pt + i) : 0.f;
+            fq[k] = i < n_mine ? ld_behind(pq + i) : 0.f;
         }
     };
     fetch_row(0);
@@ -212,8 +204,8 @@ accept_sample_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __
         sh.tok[tid] = x;
         atomicOr(&sh.kids[p + 1], 1ull << tid);
         if (x >= 0 && x < V) {
-            node_p = ld_now(p_seq + (size_t)(p + 1) * V + x);
-            node_q = ld_now(q_seq + (size_t)(p + 1) * V + x);
+            node_p = ld_behind(p_seq + (size_t)(p + 1) * V + x);
+            node_q = ld_behind(q_seq + (size_t)(p + 1) * V + x);
         }
     }
     cluster_arrive();
@@ -235,7 +227,7 @@ accept_sample_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __
         bool in_place = false;                         // row_s holds the current residual weights, not the original ones
         // entry i of this CTA's slice
         auto entry = [&](int i) -> uint2 {
-            return i < n_res && !reread ? row_s[i] : make_uint2(fixed_prob(__ldg(pt + i)), fixed_prob(__ldg(pq + i)));
+            return i < n_res && !reread ? row_s[i] : make_uint2(fixed_prob(ld_behind(pt + i)), fixed_prob(ld_behind(pq + i)));
         };
         // weights of entry i now
         auto weights = [&](int i, long long* P, long long* Q) {
@@ -260,7 +252,7 @@ accept_sample_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __
         }
         #pragma unroll 8
         for (int i = kAhead * kThreads + tid; i < n_mine; i += kThreads) {
-            const uint2 e = make_uint2(fixed_prob(__ldg(pt + i)), fixed_prob(__ldg(pq + i)));
+            const uint2 e = make_uint2(fixed_prob(ld_behind(pt + i)), fixed_prob(ld_behind(pq + i)));
             if (i < n_res) row_s[i] = e;
             A += e.x;
             Bq += e.y;

@@ -535,11 +535,9 @@ sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const Syn
 
 __global__ void ancestor_masks_kernel(const int32_t* parents, int T, unsigned long long* masks, unsigned* status)
 {
-    __shared__ int32_t par_s[kMaxT];
     __shared__ unsigned long long anc_s[kMaxT];
-    for (int i = threadIdx.x; i < T; i += 32) par_s[i] = parents[i];
-    __syncwarp();
-    build_ancestor_words(par_s, anc_s, T, status);
+    const int lane = threadIdx.x;
+    build_ancestor_words(lane < T ? parents[lane] : -1, lane + 32 < T ? parents[lane + 32] : -1, anc_s, T, status);
     for (int i = threadIdx.x; i < T; i += 32) masks[i] = anc_s[i];
 }
 

@@ -178,6 +178,27 @@ __device__ __forceinline__ void publish_counter(unsigned* addr, unsigned n = 1u)
 __device__ __forceinline__ void wait_for_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Loads that stay behind that wait and see what the predecessor wrote: ordinary loads, neither through the
+// non-coherent path nor open to reordering (which const __restrict__ parameters and __ldg would be).
+__device__ __forceinline__ int32_t ld_behind(const int32_t* p)
+{
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ld_behind(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_behind(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+
 struct Item {
     int b, kvh, group, split, key_begin, key_end;
 };
@@ -213,41 +234,37 @@ __device__ __forceinline__ Item decode_item(const SplitPlan& p, int item)
     return it;
 }
 
-// Ancestor words of a draft tree, built by one warp: anc[i] has bit a set iff a == i or a is an
-// ancestor of i.  On entry jump[i] (shared memory, T <= 64 entries) is the parent of node i; it is used
-// up.  A parent outside [-1, node) is treated as "root" and reported.  Pointer doubling: after round
-// r a word covers 2^r generations, so six rounds do for any tree (a walk from every node to its root is
-// a chain of up to 64 dependent reads: 4.5 us on the critical path of a 40-node chain, 0.3 us like this).
-__device__ __forceinline__ void build_ancestor_words(int32_t* jump, unsigned long long* anc, int T, unsigned* status)
+// Ancestor words of a draft tree of T <= 64 nodes, built by one warp: anc[i] (shared memory) gets bit a set iff
+// a == i or a is an ancestor of i.  Lane l brings the parents of nodes l and l + 32.  A parent outside
+// [-1, node) is treated as "root" and reported.  Pointer doubling in registers: after round r a word covers
+// 2^r generations, so six rounds do for any tree.  The CTA that holds the draft block is the one a short
+// call waits for: a walk from every node to its root, a chain of up to 64 dependent reads, made a 40-node
+// chain 4.5 us late; doubling in shared memory took 0.13 us a round, shuffles take 0.03.
+__device__ __forceinline__ void build_ancestor_words(int p0, int p1, unsigned long long* anc, int T, unsigned* status)
 {
     const int lane = threadIdx.x & 31;
-    for (int i = lane; i < T; i += 32) {
-        const int p = jump[i];
-        if (p < -1 || p >= i) {
-            if (status) atomicOr(status, kStatTree);
-            jump[i] = -1;
-        }
-        anc[i] = 1ull << i;
+    int j0 = lane < T ? p0 : -1, j1 = lane + 32 < T ? p1 : -1;
+    if (j0 < -1 || j0 >= lane || j1 < -1 || j1 >= lane + 32) {
+        if (status) atomicOr(status, kStatTree);
+        if (j0 < -1 || j0 >= lane) j0 = -1;
+        if (j1 < -1 || j1 >= lane + 32) j1 = -1;
     }
+    uint32_t lo0 = 1u << lane, lo1 = 0u, hi1 = 1u << lane;       // (a node below 32 has no ancestor above)
+    while (__any_sync(0xffffffffu, j0 >= 0 || j1 >= 0)) {
+        const uint32_t a0 = __shfl_sync(0xffffffffu, lo0, j0 & 31);
+        const int n0 = __shfl_sync(0xffffffffu, j0, j0 & 31);
+        if (T > 32) {
+            const uint32_t l0 = __shfl_sync(0xffffffffu, lo0, j1 & 31), l1 = __shfl_sync(0xffffffffu, lo1, j1 & 31);
+            const uint32_t h1 = __shfl_sync(0xffffffffu, hi1, j1 & 31);
+            const int m0 = __shfl_sync(0xffffffffu, j0, j1 & 31), m1 = __shfl_sync(0xffffffffu, j1, j1 & 31);
+            if (j1 >= 32) { lo1 |= l1; hi1 |= h1; j1 = m1; }
+            else if (j1 >= 0) { lo1 |= l0; j1 = m0; }
+        }
+        if (j0 >= 0) { lo0 |= a0; j0 = n0; }
+    }
+    if (lane < T) anc[lane] = lo0;
+    if (lane + 32 < T) anc[lane + 32] = (unsigned long long)hi1 << 32 | lo1;
     __syncwarp();
-    #pragma unroll 1
-    for (int reach = 1; reach < T; reach <<= 1) {
-        unsigned long long more[2];
-        int next[2];
-        #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int i = lane + 32 * k, p = i < T ? jump[i] : -1;
-            more[k] = p >= 0 ? anc[p] : 0ull;
-            next[k] = p >= 0 ? jump[p] : -1;
-        }
-        __syncwarp();
-        #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int i = lane + 32 * k;
-            if (i < T) { anc[i] |= more[k]; jump[i] = next[k]; }
-        }
-        __syncwarp();
-    }
 }
 
 }  // namespace sparrow

@@ -35,7 +35,7 @@ __device__ __forceinline__ void move_row_chunk(const RowMoveArgs& a, long long i
     const int r = (int)(rest % a.n_rows); rest /= a.n_rows;
     const int h = (int)(rest % a.n_kv_heads);
     const int b = (int)(rest / a.n_kv_heads);
-    int src = a.src_rows ? __ldg(a.src_rows + (size_t)b * a.n_rows + r) : r;
+    int src = a.src_rows ? ld_behind(a.src_rows + (size_t)b * a.n_rows + r) : r;
     const bool bad = src < 0 || src >= a.src_capacity;       // never read: the row is written as zeros
     if (bad && c == 0 && h == 0) atomicOr(a.status, kStatAnchor);
     const size_t s_off = (size_t)b * a.src_stride_batch + (size_t)h * a.src_stride_head + (size_t)(bad ? 0 : src) * kD + c * 8;

@@ -120,8 +120,8 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
         for (int i = 0; i < kPerThread; ++i) {
             const int r = (tid + i * kThreads) >> 4;
             const int j = it.key_begin + tile * kTile + r;
-            rows[i] = j < it.key_end ? (anchored ? __ldg(aidx + j) : j) : kAbsent;
-            before[i] = (checks_order && j > 0 && j < it.key_end) ? __ldg(aidx + j - 1) : kAbsent;
+            rows[i] = j < it.key_end ? (anchored ? ld_behind(aidx + j) : j) : kAbsent;
+            before[i] = (checks_order && j > 0 && j < it.key_end) ? ld_behind(aidx + j - 1) : kAbsent;
         }
     };
     auto issue_tile = [&](int stage, const int (&rows)[kPerThread], const int (&before)[kPerThread]) {
@@ -157,16 +157,20 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
 
     // ---- prologue: masks / query positions, packed Q block -> registers --------------------
     const int tree_nodes = anchored ? args.tree_nodes : 0;
-    __shared__ int32_t par_s[kMaxT];
     const int n_par = anchored ? tree_nodes : T;
-    if (tid < n_par) par_s[tid] = __ldg(args.parents + (size_t)it.b * n_par + tid);
+    int par[2] = {-1, -1};
+    if (warp == 0) {
+        #pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (lane + 32 * k < n_par) par[k] = ld_behind(args.parents + (size_t)it.b * n_par + lane + 32 * k);
+    }
     if (anchored && tid < T) {
         int p = aidx[args.n_anchor - T + tid];
         if (p < 0 || p >= args.kv_capacity) { atomicOr(args.status, kStatAnchor); p = -1; }
         qpos_s[tid] = p;
     }
     __syncthreads();
-    if (warp == 0) build_ancestor_words(par_s, anc_s, n_par, args.status);
+    if (warp == 0) build_ancestor_words(par[0], par[1], anc_s, n_par, args.status);
     {
         constexpr int kChunksPerThread = kRows * 16 / kThreads;      // 8: all loads first, then the stores
         uint4 val[kChunksPerThread];
@@ -177,7 +181,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
             const int t = it.group * plan.tok_per_block + r / plan.group, g = r % plan.group;
             val[u] = make_uint4(0, 0, 0, 0);
             if (r < plan.tok_per_block * plan.group && t < T) {
-                val[u] = __ldg(reinterpret_cast<const uint4*>(
+                val[u] = ld_behind(reinterpret_cast<const uint4*>(
                     args.q + (((size_t)it.b * T + t) * args.n_q_heads + it.kvh * plan.group + g) * kD + c * 8));
             }
         }

@@ -674,23 +674,30 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // The tree and the window bounds, beside the first loads; the softmax warps wait for them at a barrier.
         {
             const int Tt = plan.T_tree;
+            const bool needs_tree = it.key_end > kv_len;       // this piece reaches the draft block
             if (sync.wait_first) wait_for_predecessors();
-            if (it.key_end > kv_len) {                   // this piece reaches the draft block: it needs the tree
-                const int32_t* par_g = args.parents + (size_t)it.b * Tt;
-                for (int i = lane; i < Tt; i += 32) par_s[i] = __ldg(par_g + i);
-                __syncwarp();
-                build_ancestor_words(par_s, anc_s, Tt, args.status);
+            int par[2] = {-1, -1}, lo[2] = {0, 0};
+            #pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int i = lane + 32 * k;
+                if (needs_tree && i < Tt) par[k] = ld_behind(args.parents + (size_t)it.b * Tt + i);
+                if (args.first_visible && i < T) lo[k] = ld_behind(args.first_visible + (size_t)it.b * T + i);
             }
+            if (needs_tree) build_ancestor_words(par[0], par[1], anc_s, Tt, args.status);
             // Lower window bound of every query token, clamped to what this call streams: a bound
             // left of the first streamed key cannot be honoured (the keys in between were not planned)
             // and is reported.
-            for (int t = lane; t < T; t += 32) {
-                int lo = args.first_visible ? __ldg(args.first_visible + (size_t)it.b * T + t) : 0;
-                if (lo < plan.seq[it.b].key0) {
-                    if (args.first_visible) atomicOr(args.status, kStatAnchor);
-                    lo = plan.seq[it.b].key0;
+            const int key0 = plan.seq[it.b].key0;
+            #pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int t = lane + 32 * k;
+                if (t < T) {
+                    if (lo[k] < key0) {
+                        if (args.first_visible) atomicOr(args.status, kStatAnchor);
+                        lo[k] = key0;
+                    }
+                    par_s[t] = lo[k] < kv_len ? lo[k] : kv_len;
                 }
-                par_s[t] = lo < kv_len ? lo : kv_len;
             }
             tables_ready_arrive();
         }

@@ -20,8 +20,8 @@ __host__ __device__ __forceinline__ int first_anchor_above(const int32_t* anchor
 
 // One thread per (sequence, query token).  anchor_idx [B][n_anchor]: text anchors first, then the
 // T_tree rows of the draft tree; the queries are its last T_new nodes.
-__global__ void window_bounds_kernel(const int32_t* __restrict__ anchor_idx, int n_anchor, int window, int T_tree, int T_new,
-                                     int batch, int32_t* __restrict__ first_visible)
+__global__ void window_bounds_kernel(const int32_t* anchor_idx, int n_anchor, int window, int T_tree, int T_new,
+                                     int batch, int32_t* first_visible)
 {
     let_dependents_launch();
     wait_for_predecessors();
