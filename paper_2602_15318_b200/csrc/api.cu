@@ -60,7 +60,7 @@ struct sparrow_ctx {
     size_t part_offset;                      // first byte of the split-KV partials in the workspace
     int part_buffers;                        // 2: alternate by call parity (fused mode); 1: stream-ordered calls only
     std::atomic<long long> launches;
-    const int* max_clusters[2];              // by row blocks - 1: verification clusters of 1 .. 16 CTAs that can run at once
+    const int* max_clusters[3];              // clusters of 1 .. 16 CTAs that can run at once: verification with one and two row blocks, gather
     int max_sample_cluster;                  // CTAs per cluster of the temperature-1 acceptance kernel the device takes
     bool use_pdl;
     bool log_plans;                          // SPARROW_LOG=1 when the context was created: one line per call on stderr
@@ -437,7 +437,8 @@ sparrow_status launch_split_gather(sparrow_ctx* c, const SplitPlan& plan, const 
     a.lse = lse;
     a.status = reinterpret_cast<unsigned*>(c->ws);
     other_kernel_enqueued();
-    return launch_behind(c, gather::split_gather_kernel, (unsigned)plan.n_items, gather::kThreads, gather::kSmemBytes, st, 0, plan, a);
+    return launch_behind(c, gather::split_gather_kernel, (unsigned)plan.n_items, gather::kThreads,
+                         plan.cluster > 1 ? gather::kClusterSmemBytes : gather::kSmemBytes, st, plan.cluster > 1 ? (unsigned)plan.cluster : 0u, plan, a);
 }
 
 // Cached tensor maps.  tag == 0: one K or V buffer, dims (128 dims, capacity rows, KV heads,
@@ -591,25 +592,25 @@ int sample_cluster_limit(int device)
     return n;
 }
 
-// Clusters of n = 1 .. 16 CTAs of the verification kernel (one CTA per SM) that can run at once on the
-// current device, by row blocks - 1; asked once per device and process.
+// Clusters of n = 1 .. 16 CTAs (one CTA per SM) that can run at once on the current device, for the
+// verification kernel with one and two row blocks and the gather kernel; asked once per device and process.
 using tc::kMaxMergeCluster;
 struct ClusterTable {
     std::atomic<int> state;                   // 0 unknown, 1 being filled, 2 known
-    int n[2][kMaxMergeCluster + 1];
+    int n[3][kMaxMergeCluster + 1];
 };
-template <int NB>
-void query_max_clusters(int* n)
+template <class Kernel>
+void query_max_clusters(Kernel kernel, int block, int smem, int* n)
 {
     n[0] = n[1] = 0;
-    const bool wide = cudaFuncSetAttribute(tc::verify_tc_kernel<NB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     for (int c = 2; c <= kMaxMergeCluster; ++c) {
         n[c] = 0;
         if (c > 8 && !wide) continue;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)c);
-        cfg.blockDim = dim3(tc::kThreads);
-        cfg.dynamicSmemBytes = tc::smem_bytes(NB, NB == 1 ? 3 : 2);
+        cfg.blockDim = dim3((unsigned)block);
+        cfg.dynamicSmemBytes = (size_t)smem;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)c;
@@ -617,7 +618,7 @@ void query_max_clusters(int* n)
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n[c], tc::verify_tc_kernel<NB>, &cfg) != cudaSuccess) n[c] = 0;
+        if (cudaOccupancyMaxActiveClusters(&n[c], kernel, &cfg) != cudaSuccess) n[c] = 0;
     }
     cudaGetLastError();
 }
@@ -628,8 +629,9 @@ const ClusterTable* cluster_table(int device)
     ClusterTable& t = tables[device];
     int expected = 0;
     if (t.state.compare_exchange_strong(expected, 1)) {
-        query_max_clusters<1>(t.n[0]);
-        query_max_clusters<2>(t.n[1]);
+        query_max_clusters(tc::verify_tc_kernel<1>, tc::kThreads, tc::smem_bytes(1, 3), t.n[0]);
+        query_max_clusters(tc::verify_tc_kernel<2>, tc::kThreads, tc::smem_bytes(2, 2), t.n[1]);
+        query_max_clusters(gather::split_gather_kernel, gather::kThreads, gather::kClusterSmemBytes, t.n[2]);
         t.state.store(2);
     }
     return t.state.load() == 2 ? &t : nullptr;      // (a thread that comes while another one asks does without)
@@ -655,13 +657,16 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
     return SPARROW_OK;
 }
 
-constexpr float kTileUs[2] = {1.2f, 2.0f};            // a tile of 128 keys, one / two row blocks
+// Estimates for plan_lone_call(), us: a tile of 128 keys with one / two row blocks, and the merges.
+constexpr float kTileUs[2] = {1.2f, 2.0f};
 constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f;
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
 // at most 16 pieces per unit, pieces short enough to leave a stage of the K/V ring free for the rows that are
 // sent around (2 tiles with one row block, 1 with two), and whole clusters per GPC.  Rewrites the plan where
-// that is estimated to pay.  Estimates in us, from single calls: PLACEHOLDER
+// that is estimated to pay.  Measured back to back, workspace -> cluster: 448 keys, T = 8 9.2 -> 7.4 us; 1,000
+// keys, T = 16 9.9 -> 8.2; 3,000 keys 13.1 -> 9.5 (12 pieces of two tiles instead of 24 of one); 448 keys, T = 30
+// 13.8 -> 11.6.  One piece against two in a cluster: 240 keys, T = 8 7.8 and 7.8.
 void plan_lone_call(const sparrow_ctx* c, SplitPlan* p)
 {
     const int nb = p->blocks_per_group, units = p->batch * p->n_kv_heads * p->n_groups;
@@ -684,6 +689,32 @@ void plan_lone_call(const sparrow_ctx* c, SplitPlan* p)
         if (n > 1 && (piece > free_stage_tiles || !c->max_clusters[nb - 1] || units > c->max_clusters[nb - 1][n])) continue;
         const float t = per_tile * piece + (n > 1 ? kMergeClusterUs : 0.f);
         if (t < best) { best = t; pieces = n; }
+    }
+    if (pieces == 0) return;
+    int total = 0;
+    for (int b = 0; b < p->batch; ++b) {
+        p->seq[b].n_splits = pieces;
+        p->seq[b].item_begin = total;
+        total += p->n_kv_heads * p->n_groups * pieces;
+    }
+    p->n_items = total;
+    p->cluster = pieces;
+}
+
+// The gathered pass cut so that a unit's pieces share a cluster and merge there instead of through the
+// workspace and a second kernel, as long as no piece gets longer by it (a gathered tile of 64 keys takes about
+// 2.7 us): 448 anchors, T = 8 11.7 -> 9.9 us; four sequences of 448 anchors, T = 60 32.4 -> 25.6; with longer
+// pieces it lost (6,000 anchors in 16 pieces of 6 tiles instead of 37 of 3: 24.1 -> 32.4).
+void plan_gather_cluster(const sparrow_ctx* c, int n_anchor, SplitPlan* p)
+{
+    const int units = p->batch * p->n_kv_heads * p->n_groups;
+    const int tiles = (n_anchor + p->piece_tile - 1) / p->piece_tile;
+    if (!c->max_clusters[2] || p->seq[0].n_splits == 1) return;
+    const int now = (tiles + p->seq[0].n_splits - 1) / p->seq[0].n_splits;
+    int pieces = 0, best = now + 1;
+    for (int n = 1; n <= kMaxMergeCluster && n <= tiles; ++n) {
+        const int piece = (tiles + n - 1) / n;
+        if ((n > 1 ? units <= c->max_clusters[2][n] : units <= c->n_sm) && piece < best) { best = piece; pieces = n; }
     }
     if (pieces == 0) return;
     int total = 0;
@@ -813,7 +844,7 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
     DeviceGuard guard(device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     if (cudaFuncSetAttribute(gather::split_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             gather::kSmemBytes) != cudaSuccess)
+                             gather::kClusterSmemBytes) != cudaSuccess)
         return SPARROW_ERR_CUDA;
     if (cudaFuncSetAttribute(tc::verify_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc::smem_bytes(1, 3)) != cudaSuccess ||
@@ -843,8 +874,7 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
     c->launches.store(0);
     c->max_sample_cluster = sample_cluster_limit(device);
     if (const ClusterTable* ct = cluster_table(device)) {
-        c->max_clusters[0] = ct->n[0];
-        c->max_clusters[1] = ct->n[1];
+        for (int k = 0; k < 3; ++k) c->max_clusters[k] = ct->n[k];
     }
     const char* e = std::getenv("SPARROW_NO_PDL");
     // more SMs than the list of possibly-resident calls can hold: calls never start early
@@ -1000,7 +1030,7 @@ sparrow_status sparrow_verify_attn_static(const sparrow_layout* L, const void* q
         if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return SPARROW_ERR_CUDA;
         if (prop.major != 10) return SPARROW_ERR_ARCH;
         if (cudaFuncSetAttribute(gather::split_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 gather::kSmemBytes) != cudaSuccess ||
+                                 gather::kClusterSmemBytes) != cudaSuccess ||
             cudaFuncSetAttribute(tc::verify_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  tc::smem_bytes(1, 3)) != cudaSuccess ||
             cudaFuncSetAttribute(tc::verify_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1087,13 +1117,14 @@ sparrow_status anchor_call(sparrow_ctx* c, const void* q, const void* k, const v
     sparrow_status s = make_plan(c->n_sm, c->layout.batch, c->layout.n_kv_heads, layout_group(c->layout), n_keys, T, 1, &plan, kMinGatherPieceKeys);
     if (s != SPARROW_OK) return s;
     if ((s = check_ws(c, plan)) != SPARROW_OK) return s;
+    plan_gather_cluster(c, n_anchor, &plan);
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const SyncArgs sy = next_sync(c, plan, false, true, false);
     if ((s = launch_split_gather(c, plan, sy, q, k, v, parents, anchor_idx, n_anchor, window, out, lse, st, tree_nodes)) != SPARROW_OK)
         return s;
-    return launch_combine(c, plan, sy, out, lse, st);
+    return plan.seq[0].n_splits > 1 && plan.cluster <= 1 ? launch_combine(c, plan, sy, out, lse, st) : SPARROW_OK;
 }
 }  // namespace
 

@@ -7,13 +7,15 @@
 // and block.  K/V rows are fetched
 // with 16-byte cp.async (row index = key index, or anchor_idx[key] when gathering) into a
 // two-stage XOR-swizzled shared-memory ring; S = QK^T and O += PV run on mma.sync m16n8k16 bf16
-// with fp32 accumulation; the online softmax is fp32 with quad shuffles.  Per item the kernel
-// writes a normalised fp16 partial output and a natural-log LSE for the combine step (or, when
-// the sequence has a single piece, the final bf16 output and LSE).
+// with fp32 accumulation; the online softmax is fp32 with quad shuffles.  A piece's result is a
+// normalised fp16 partial output and a natural-log LSE per row: where the unit's pieces share a
+// thread-block cluster they are sent to the CTA that finishes the row, else written for the combine kernel
+// (or, when the sequence has a single piece, final bf16 output and LSE).
 #pragma once
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "verify_tc.cuh"
 
 namespace sparrow {
 
@@ -45,6 +47,9 @@ constexpr int kRows = 128;        // packed query rows per CTA (8 warps x 16)
 constexpr int kTile = 64;         // keys per stage
 constexpr int kStageBytes = kTile * kD * 2;            // one K or V tile: 16 KB
 constexpr int kSmemBytes = 4 * kStageBytes + kMaxT * 8 + kMaxT * 4 + 2 * kTile * 4;
+// with the pieces of a unit in a cluster: the rows the peers send, [piece][row][272 bytes], and the merge's scratch
+constexpr int kRecvBytes = (kRows + tc::kMaxMergeCluster) * tc::kRowBytes;
+constexpr int kClusterSmemBytes = (kSmemBytes + 15) / 16 * 16 + kRecvBytes + kThreads * 10 * 4;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
@@ -93,6 +98,15 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
     int32_t* apos_s = qpos_s + kMaxT;                                // [2][kTile] gathered row ids
 
     // The combine kernel may be scheduled now: it waits for this grid as a whole before it reads.
+    __shared__ uint64_t merge_bar;
+    if (plan.cluster > 1) {
+        if (threadIdx.x == 0) {
+            tc::mbar_init(smem_u32(&merge_bar), 1);
+            tc::fence_barrier_init();
+        }
+        __syncthreads();
+        tc::cluster_arrive_relaxed();
+    }
     let_dependents_launch();
     wait_for_predecessors();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -330,6 +344,9 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
     cp_async_wait<0>();
 
     // ---- epilogue: normalised partial output + natural-log LSE ------------------------------
+    // Where the unit's pieces share a cluster a partial row is staged in shared memory (over the K/V ring) and
+    // sent to the CTA that finishes it.
+    const bool clustered = plan.cluster > 1;
     #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
         float l = l_run[rr];
@@ -347,13 +364,39 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
                 *reinterpret_cast<uint32_t*>(dst + nt * 8 + 2 * c4) = pack_bf16(o[nt][2 * rr] * inv, o[nt][2 * rr + 1] * inv);
             if (c4 == 0) args.lse[((size_t)it.b * args.n_q_heads + h) * T + t] = lse_val;
         } else {
-            const size_t prow = (size_t)blockIdx.x * plan.part_rows + lr;
-            __half* dst = args.o_part + prow * kPartRowHalves;
+            __half* dst = clustered ? reinterpret_cast<__half*>(smem + lr * tc::kRowBytes)
+                                    : args.o_part + ((size_t)blockIdx.x * plan.part_rows + lr) * kPartRowHalves;
             #pragma unroll
             for (int nt = 0; nt < 16; ++nt)
                 *reinterpret_cast<__half2*>(dst + nt * 8 + 2 * c4) = __floats2half2_rn(o[nt][2 * rr] * inv, o[nt][2 * rr + 1] * inv);
             if (c4 == 0) *reinterpret_cast<float*>(dst + kD) = lse_val;
         }
+    }
+    if (clustered) {
+        const int cl = plan.cluster;
+        const int tok0 = it.group * plan.tok_per_block;
+        const int unit_rows = plan.group * min(plan.tok_per_block, T - tok0);
+        const uint32_t recv = smem_u32(smem + (kSmemBytes + 15) / 16 * 16), bar = smem_u32(&merge_bar);
+        int r_begin;
+        const int n = tc::merge_share(unit_rows, it.split, cl, &r_begin) - r_begin;
+        tc::fence_proxy_async();                             // the staged rows, ahead of the bulk copies
+        __syncthreads();
+        tc::cluster_wait();                                  // every peer runs, its barrier is initialised
+        if (tid == 0) tc::mbar_expect_tx(bar, (uint32_t)(n * cl * tc::kRowBytes));
+        if (tid < cl) {
+            int r0;
+            const int rows = tc::merge_share(unit_rows, tid, cl, &r0) - r0;        // peer tid's share
+            if (rows > 0)
+                tc::bulk_push(tc::map_to_rank(recv + (uint32_t)(it.split * rows * tc::kRowBytes), (uint32_t)tid),
+                              smem_u32(smem + r0 * tc::kRowBytes), (uint32_t)(rows * tc::kRowBytes), tc::map_to_rank(bar, (uint32_t)tid));
+        }
+        const bool landed = tc::mbar_wait(bar, 0);
+        tc::cluster_arrive_relaxed();                        // (all pushes to this CTA are through: its peers may leave)
+        if (!landed && lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies));
+        const tc::MergeOut mo = {args.out, args.lse, T, args.n_q_heads, plan.group};
+        tc::merge_run(tid, recv, cl, n, r_begin, it.b, tok0, it.kvh * plan.group, landed,
+                      reinterpret_cast<float*>(smem + (kSmemBytes + 15) / 16 * 16 + kRecvBytes), mo, [] { __syncthreads(); });
+        tc::cluster_wait();                                  // nobody leaves before its peers have received what it sends them
     }
 }
 

@@ -408,6 +408,107 @@ struct Bars {
     __device__ __forceinline__ uint32_t o_done(int blk, int j) const { return base + 160u + 32u * (uint32_t)blk + 8u * (uint32_t)(j & 3); }
 };
 
+struct MergeOut {
+    __nv_bfloat16* out;
+    float* lse;
+    int T, n_q_heads, qg;
+};
+// The final bf16 row and LSE from a row's weighted sum, the sum of weights and the reference of the weights; 16
+// threads of 8 dims each.
+__device__ __forceinline__ void write_merged(const float (&acc)[8], float s, float m, int b, int t, int h, int c16, const MergeOut& mo)
+{
+    const float inv = s > 0.f ? __fdividef(1.f, s) : 0.f;
+    uint4 pk;
+    pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+    pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+    *reinterpret_cast<uint4*>(mo.out + (((size_t)b * mo.T + t) * mo.n_q_heads + h) * kD + c16 * 8) = pk;
+    if (c16 == 0) mo.lse[((size_t)b * mo.n_q_heads + h) * mo.T + t] = s > 0.f ? m + __logf(s) : -INFINITY;
+}
+// One thread's share of a row: pieces first, first + step, ... of 8 dims.  The largest LSE first, so that the
+// pieces' weights do not depend on one another.
+__device__ __forceinline__ void fold_pieces(uint32_t row, int first, int step, int ns, uint32_t pstride, int c16, float (&acc)[8], float& s, float& m)
+{
+    const uint32_t a0 = row + (uint32_t)first * pstride, hop = (uint32_t)step * pstride;
+    uint32_t at = a0 + 2 * kD;
+    #pragma unroll 4
+    for (int sp = first; sp < ns; sp += step, at += hop) m = fmaxf(m, lds_f32(at));
+    const float m_log2 = m == -INFINITY ? 0.f : m * 1.4426950408889634f;           // (all pieces empty: weights 0)
+    at = a0;
+    #pragma unroll 2
+    for (int sp = first; sp < ns; sp += step, at += hop) {
+        const float w = ex2(fmaf(lds_f32(at + 2 * kD), 1.4426950408889634f, -m_log2));
+        uint32_t raw[4];
+        lds_v4(at + c16 * 16, raw);
+        s += w;
+        #pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
+            acc[2 * q] = fmaf(w, f.x, acc[2 * q]); acc[2 * q + 1] = fmaf(w, f.y, acc[2 * q + 1]);
+        }
+    }
+}
+// Merges rows [0, n) of a run whose ns pieces lie in shared memory at `base` as [piece][row][272 bytes] and writes
+// the results; row i is row r0 + i of its unit (token idx / g, head idx % g).  256 threads, 16 per row: R rows at
+// a time with 16 / R groups of threads sharing a row's pieces where there are fewer than 16 rows (the groups'
+// results meet in red: [256][10] floats).  `barrier` is a barrier of these 256 threads.
+template <class Barrier>
+__device__ __forceinline__ void merge_run(int tid, uint32_t base, int ns, int n, int r0, int b, int tok0, int head0, bool landed,
+                                          float* red, const MergeOut& mo, Barrier barrier)
+{
+    const int inv_qg = (65536 + mo.qg - 1) / mo.qg;                // x / qg = x * inv_qg >> 16 for x <= 512
+    const int c16 = tid & 15;
+    const uint32_t pstride = (uint32_t)n * kRowBytes;              // bytes between pieces
+    int lg_g = 4;
+    while (lg_g > 0 && (16 >> lg_g) < n) --lg_g;
+    const int G = 1 << lg_g;
+    if (G == 1) {
+        #pragma unroll 1
+        for (int r = tid >> 4; r < n; r += 16) {
+            if (!landed) break;
+            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, s = 0.f, m = -INFINITY;
+            fold_pieces(base + (uint32_t)r * kRowBytes, 0, 1, ns, pstride, c16, acc, s, m);
+            const int idx = r0 + r, tok = (idx * inv_qg) >> 16;
+            write_merged(acc, s, m, b, tok0 + tok, head0 + idx - tok * mo.qg, c16, mo);
+        }
+        return;
+    }
+    const int i = tid >> (4 + lg_g), grp = (tid >> 4) & (G - 1);
+    const bool active = landed && i < n;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, s = 0.f, m = -INFINITY;
+    if (active) fold_pieces(base + (uint32_t)i * kRowBytes, grp, G, ns, pstride, c16, acc, s, m);
+    barrier();                                                     // the run before has been read
+    #pragma unroll
+    for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
+    red[tid * 10 + 8] = s;
+    red[tid * 10 + 9] = m;
+    barrier();
+    if (!active || grp != 0) return;
+    const float* mine = red + tid * 10;
+    float m_all = m;
+    for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
+    const float a0 = m == -INFINITY ? 0.f : ex2((m - m_all) * 1.4426950408889634f);
+    s *= a0;
+    #pragma unroll
+    for (int q = 0; q < 8; ++q) acc[q] *= a0;
+    for (int g2 = 1; g2 < G; ++g2) {
+        const float* o = mine + g2 * 160;
+        if (o[9] == -INFINITY) continue;
+        const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
+        s = fmaf(o[8], ag, s);
+        #pragma unroll
+        for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
+    }
+    const int idx = r0 + i, tok = (idx * inv_qg) >> 16;
+    write_merged(acc, s, m_all, b, tok0 + tok, head0 + idx - tok * mo.qg, c16, mo);
+}
+
+// Rows of a unit that CTA `rank` of a cluster of `cl` finishes: [begin, return value).
+__device__ __forceinline__ int merge_share(int unit_rows, int rank, int cl, int* begin)
+{
+    *begin = unit_rows * rank / cl;
+    return unit_rows * (rank + 1) / cl;
+}
+
 // What one pass of the merge takes: runs of rows of one unit (sequence, KV head, row group).
 struct MergeSegment {
     int b, ns, n, split;             // sequence, pieces, rows, rows of them in the run's first block
@@ -1060,101 +1161,22 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             list->bytes = bytes;
             list->next_row = row;
         };
-        // Merging is done by 16 R G threads, R rows at a time: thread (row i, 16-byte chunk c16, piece group
-        // g) folds pieces g, g + G, ... of its row; the groups' results meet in shared memory here, and the
-        // row is written.
-        // [256][10]: 8 outputs, sum, max; over the Q blocks, or where rows on their way to peers lie there, over a V tile
+        // scratch of the merge: over the Q blocks, or where rows on their way to peers lie there, over a V tile
         float* red = reinterpret_cast<float*>(clustered ? kv_sm + 2 * kSubTileBytes : q_sm);
-        const int inv_qg = (65536 + qg - 1) / qg;                       // x / qg = x * inv_qg >> 16 for x <= 512
-        const int c16 = tid & 15;
-        auto finish_row = [&](float (&acc)[8], float s_run, float m_run, bool active, int G, int grp_p, int b, int t, int h) {
-            if (G > 1) {                                               // (G is the same in every thread)
-                softmax_bar_sync();                                    // the run before has been read
-                #pragma unroll
-                for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
-                red[tid * 10 + 8] = s_run;
-                red[tid * 10 + 9] = m_run;
-                softmax_bar_sync();
-                if (grp_p == 0) {
-                    const float* mine = red + tid * 10;
-                    float m_all = m_run;
-                    for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
-                    const float a0 = m_run == -INFINITY ? 0.f : ex2((m_run - m_all) * 1.4426950408889634f);
-                    s_run *= a0;
-                    #pragma unroll
-                    for (int q = 0; q < 8; ++q) acc[q] *= a0;
-                    for (int g2 = 1; g2 < G; ++g2) {
-                        const float* o = mine + g2 * 160;
-                        if (o[9] == -INFINITY) continue;
-                        const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
-                        s_run = fmaf(o[8], ag, s_run);
-                        #pragma unroll
-                        for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
-                    }
-                    m_run = m_all;
-                }
-            }
-            if (tid == 0) SPARROW_STAMP(14);                           // groups reduced
-            if (active && grp_p == 0) {
-                const float inv = s_run > 0.f ? __fdividef(1.f, s_run) : 0.f;
-                uint4 pk;
-                pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-                pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
-                *reinterpret_cast<uint4*>(args.out + (((size_t)b * T + t) * args.n_q_heads + h) * kD + c16 * 8) = pk;
-                if (c16 == 0) args.lse[((size_t)b * args.n_q_heads + h) * T + t] = s_run > 0.f ? m_run + __logf(s_run) : -INFINITY;
-            }
-        };
-        // Merges rows [0, n) of a run whose pieces lie at `base` as [piece][row][272 bytes]; row i is row r0 + i of
-        // its unit.
-        auto merge_run = [&](uint32_t base, int ns, int n, int r0, int b, int tok0, int head0, bool landed) {
-            int lg_g = 4;                                              // G = 16 / R piece groups, R rows at a time
-            while (lg_g > 0 && (16 >> lg_g) < n) --lg_g;
-            const int G = 1 << lg_g, R = 16 >> lg_g;
-            const int grp_p = (tid >> 4) & (G - 1);
-            const uint32_t pstride = (uint32_t)n * kRowBytes;          // bytes between pieces
-            #pragma unroll 1
-            for (int r = 0; r < n; r += R) {
-                const int i = r + (tid >> (4 + lg_g));
-                const bool active = landed && i < n;
-                float m_run = -INFINITY, s_run = 0.f;                  // natural-log units
-                float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                if (active) {
-                    // the largest LSE first, so that the pieces' weights do not depend on one another
-                    const uint32_t a0 = base + (uint32_t)i * kRowBytes + grp_p * pstride, step = (uint32_t)G * pstride;
-                    uint32_t a_o = a0 + 2 * kD;
-                    #pragma unroll 4
-                    for (int sp = grp_p; sp < ns; sp += G, a_o += step) m_run = fmaxf(m_run, lds_f32(a_o));
-                    const float m_log2 = m_run == -INFINITY ? 0.f : m_run * 1.4426950408889634f;   // (all pieces empty: weights 0)
-                    a_o = a0;
-                    #pragma unroll 2
-                    for (int sp = grp_p; sp < ns; sp += G, a_o += step) {
-                        const float w = ex2(fmaf(lds_f32(a_o + 2 * kD), 1.4426950408889634f, -m_log2));
-                        uint32_t raw[4];
-                        lds_v4(a_o + c16 * 16, raw);
-                        s_run += w;
-                        #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[q]));
-                            acc[2 * q] = fmaf(w, f.x, acc[2 * q]); acc[2 * q + 1] = fmaf(w, f.y, acc[2 * q + 1]);
-                        }
-                    }
-                }
-                if (tid == 0) SPARROW_STAMP(13);                       // pieces folded
-                const int idx = r0 + i, tok = (idx * inv_qg) >> 16;    // token idx / g, head idx % g
-                finish_row(acc, s_run, m_run, active, G, grp_p, b, tok0 + tok, head0 + idx - tok * qg);
-            }
-        };
+        const MergeOut merge_out = {args.out, args.lse, T, args.n_q_heads, qg};
         if (clustered) {
             // Every CTA of the cluster merges a share of the unit's rows: it is sent its rows of every piece, one
             // bulk copy from each peer, into the last stage of the K/V ring, which pieces this short never use.
             const int cl = plan.cluster;
             const int unit_rows = qg * min(NB * tpb, T - block0 * tpb);
             const uint32_t recv = smem_u32(kv_sm) + (NS - 1) * kStageBytes;
-            const int r_begin = unit_rows * it.split / cl, n = unit_rows * (it.split + 1) / cl - r_begin;
+            int r_begin;
+            const int n = merge_share(unit_rows, it.split, cl, &r_begin) - r_begin;
             cluster_wait();                                            // every peer runs, its barriers are initialised
             if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n * cl * kRowBytes));
             if (tid < cl) {
-                const int r0 = unit_rows * tid / cl, r1 = unit_rows * (tid + 1) / cl;      // peer tid's share
+                int r0;
+                const int r1 = merge_share(unit_rows, tid, cl, &r0);       // peer tid's share
                 const uint32_t dst = map_to_rank(recv + (uint32_t)(it.split * (r1 - r0) * kRowBytes), (uint32_t)tid);
                 const uint32_t bar = map_to_rank(B.fin(), (uint32_t)tid);
                 // (staged block by block: the share may straddle the two)
@@ -1169,7 +1191,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             cluster_arrive_relaxed();                                  // (all pushes to this CTA are through: its peers may leave)
             if (!landed && lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies));
             if (tid == 0) SPARROW_STAMP(15);                           // every piece is here
-            merge_run(recv, cl, n, r_begin, it.b, block0 * tpb, it.kvh * qg, landed && ok);
+            merge_run(tid, recv, cl, n, r_begin, it.b, block0 * tpb, it.kvh * qg, landed && ok, red, merge_out, [] { softmax_bar_sync(); });
             if (tid == 0) SPARROW_STAMP(10);                           // merged rows written
             softmax_bar_sync();
         }
@@ -1232,7 +1254,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     #pragma unroll 1
                     for (int k = 0; k < n_seg; ++k) {
                         const MergeSegment& sg = list->seg[k];
-                        merge_run(smem_u32(kv_sm) + (uint32_t)sg.offset, sg.ns, sg.n, sg.r0, sg.b, sg.tok0, sg.head0, landed);
+                        merge_run(tid, smem_u32(kv_sm) + (uint32_t)sg.offset, sg.ns, sg.n, sg.r0, sg.b, sg.tok0, sg.head0, landed, red, merge_out,
+                                  [] { softmax_bar_sync(); });
                     }
                     const int next = list->next_row;
                     if (!landed || next >= my_end) break;

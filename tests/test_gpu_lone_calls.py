@@ -1,0 +1,81 @@
+"""Single calls that share the GPU with no other call: how their pieces are merged depends on sizes (one
+piece, a thread-block cluster per unit, the workspace).  Sizes at the edges of those rules, against the
+oracle; tolerances as everywhere (gpu_util)."""
+import pytest
+import torch
+
+import oracle
+from paper_2602_15318_b200 import binding as B
+from paper_2602_15318_b200 import workloads as W
+
+from gpu_util import check, oracle_anchor, oracle_verify, run_anchor, run_verify
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("hq,hkv,kv_len,T,tree", [
+    (28, 4, [120], 8, "chain"),             # exactly one tile: no merge
+    (28, 4, [121], 8, "random"),            # one key more
+    (28, 4, [1000], 18, "chain"),           # the largest draft block of one row block
+    (28, 4, [4096 - 16], 16, "random"),     # 32 tiles: the longest pieces a cluster of 16 takes
+    (28, 4, [4096 - 15], 16, "random"),     # 33 tiles: through the workspace
+    (28, 4, [500], 36, "random"),           # 252 rows: shares that straddle the two row blocks
+    (28, 4, [500], 64, "chain"),            # two row groups, a chain as deep as a tree gets
+    (28, 4, [2048 - 40], 40, "random"),     # 16 tiles, two row blocks
+    (28, 4, [2049 - 40], 40, "random"),     # 17 tiles
+    (4, 4, [700], 1, "chain"),              # one row per unit: most CTAs of a cluster finish nothing
+    (16, 1, [1500], 64, "random"),          # 16 query heads per KV head, four row groups
+    (28, 4, [130, 2000, 700], 12, "random"),  # ragged lengths in clusters of two
+    (28, 4, [100] * 40, 20, "random"),      # more units than SMs
+])
+def test_verify_alone(hq, hkv, kv_len, T, tree):
+    case = W.make_verify_case(7100 + hq + T + kv_len[0], kv_len, T, tree, DEV, hq=hq, hkv=hkv)
+    ctx = B.Context.for_cache(case.k, W.SCALE, n_q_heads=hq)
+    ref = oracle_verify(case)
+    for _ in range(2):                      # (the second call follows the first without a synchronisation of its own)
+        out, lse, _ = run_verify(case, ctx)
+        check(out, lse, *ref)
+
+
+def test_verify_alone_back_to_back_and_in_front_of_a_batch():
+    """Lone calls of different kinds (cluster, workspace, one piece) and a batch that overlaps its own calls,
+    enqueued without synchronisation on one context: every result its own, in the batch bit for bit."""
+    cap = 9000 + 64
+    cases = [W.make_verify_case(7300 + i, [kv], T, tree, DEV, capacity=cap)
+             for i, (kv, T, tree) in enumerate([(700, 8, "chain"), (9000, 16, "random"), (60, 12, "random"), (1500, 33, "chain")])]
+    refs = [oracle_verify(c) for c in cases]
+    ctx = B.Context.for_cache(cases[0].k, W.SCALE)
+    new = lambda c: (torch.full_like(c.q, float("nan")), torch.full((1, W.HQ, c.T), float("nan"), dtype=torch.float32, device=DEV))
+    results, batched = [], []
+    for rep in range(4):
+        for c in cases:
+            out, lse = new(c)
+            B.sparrow_verify_attn(ctx, c.q, c.k, c.v, c.kv_len, c.parents, c.T, out, lse)
+            results.append((out, lse))
+        outs = [new(c) for c in cases]
+        B.sparrow_verify_attn_batch(ctx, B.VerifyBatch([(c.q, c.k, c.v, c.kv_len, c.parents, c.T, o, l) for c, (o, l) in zip(cases, outs)]))
+        batched.append(outs)
+    torch.cuda.synchronize()
+    assert ctx.last_device_status() == 0
+    for i, (out, lse) in enumerate(results):
+        check(out, lse, *refs[i % len(cases)])
+    for outs in batched:
+        for (o, l), (wo, wl), ref in zip(outs, batched[0], refs):
+            check(o, l, *ref)
+            assert torch.equal(o, wo) and torch.equal(l, wl)
+
+
+@pytest.mark.parametrize("n_text,T,batch", [
+    (56, 8, 1),                             # exactly one gathered tile
+    (57, 8, 1),                             # two pieces
+    (16 * 64 - 8, 8, 1),                    # sixteen pieces
+    (16 * 64 - 7, 8, 1),                    # seventeen tiles
+    (300, 40, 1),                           # three row groups, the last one short
+    (200, 1, 3),
+])
+def test_anchored_pieces(n_text, T, batch):
+    idx = list(range(40, 40 + n_text)) + list(range(2000, 2000 + T))
+    case = W.make_anchor_case(7500 + n_text + T, idx, 0, T, batch, DEV)
+    out, lse, _ = run_anchor(case)
+    check(out, lse, *oracle_anchor(case))
