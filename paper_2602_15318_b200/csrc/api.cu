@@ -66,6 +66,8 @@ struct sparrow_ctx {
     bool log_plans;                          // SPARROW_LOG=1 when the context was created: one line per call on stderr
     bool overlap_single_calls;               // sparrow_set_call_overlap()
     bool in_batch;                           // the call being enqueued belongs to a sparrow_verify_attn_batch()
+    bool prefix_ready;                       // the kernel directly before the call being enqueued writes only what the call finds behind
+                                             // the prefix, and was launched behind everything earlier (sparrow_verify_step_host)
     bool prev_lone;                          // the previous fused call published its end relaxed (SyncArgs::lone)
     bool chain_next;                         // the call being enqueued directly follows this context's previous fused call
     // Host mirror of the ordering counters in the workspace (see SyncArgs): call sequence number
@@ -779,7 +781,7 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     for (int b = 0; b < c->layout.batch; ++b) plan.seq[b].kv_len = kv_len[b];
     if ((s = check_ws(c, plan)) != SPARROW_OK) return s;
     SyncArgs sy = next_sync(c, plan, protocol, outputs_touch_previous(c, cr), may_share);
-    sy.wait_first = protocol && !early;
+    sy.wait_first = protocol && !early ? (c->prefix_ready ? 2 : 1) : 0;
     if (c->log_plans) {
         std::fprintf(stderr, "[sparrow] verify call %u: T %d of %d nodes, %d row block(s) x %d group(s), %d items (target %d), %s, %s;",
                      c->seq, T, T_tree, plan.blocks_per_group, plan.n_groups, plan.n_items, plan_target(c, may_share),
@@ -1437,8 +1439,10 @@ sparrow_status sparrow_verify_step_host(sparrow_ctx* c, const void* q_host, cons
         other_kernel_enqueued();
         const sparrow_status is = launch_behind(c, ingest_step_kernel, (unsigned)((work + 255) / 256), 256, 0, st, 0, ia);
         if (is != SPARROW_OK) return is;
+        c->prefix_ready = true;
         const sparrow_status s = sparrow_verify_attn(c, q_dev, k_cache, v_cache, kv_len, par_dev, T, out_view,
                                                      static_cast<float*>(lse_view), stream);
+        c->prefix_ready = false;
         if (s != SPARROW_OK) return s;
         return cudaStreamSynchronize(st) == cudaSuccess ? SPARROW_OK : SPARROW_ERR_CUDA;
     }

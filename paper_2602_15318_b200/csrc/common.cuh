@@ -128,7 +128,7 @@ struct SyncArgs {
     int32_t n_fin;           // finisher CTAs of this call (0 when no unit has several pieces)
     uint32_t fin_wait_same;
     uint32_t fin_wait_other;
-    int32_t wait_first;      // launched with programmatic stream serialisation but ordered behind its predecessor: wait before the first global access
+    int32_t wait_first;      // launched with programmatic stream serialisation but ordered behind its predecessor: wait before the first global access (2: but for key tiles that lie in the prefix)
     int32_t lone;            // no later call can start before this grid has ended
     uint32_t call;           // running number of the context's fused calls (the timeline build files its stamps under it)
 };

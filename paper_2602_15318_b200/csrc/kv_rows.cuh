@@ -76,8 +76,10 @@ struct IngestArgs {
 __global__ void __launch_bounds__(256)
 ingest_step_kernel(const __grid_constant__ IngestArgs a)
 {
-    let_dependents_launch();
+    // in this order: the attention call behind this kernel starts streaming the cache's prefix, which this
+    // kernel does not write, as soon as it is launched, and relies on everything earlier being complete
     wait_for_predecessors();
+    let_dependents_launch();
     const long long row_chunks = (long long)a.rows.batch * a.rows.n_kv_heads * a.rows.n_rows * 16;
     const long long total = row_chunks + a.q_chunks + a.n_parents;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {

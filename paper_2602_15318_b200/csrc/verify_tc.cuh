@@ -594,7 +594,12 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         *abort_flag = 0;
         *write_ok = sync.enabled ? 0u : 1u;
         fence_barrier_init();
-        if (sync.wait_first) wait_for_predecessors();
+        int j_first = 0;                                 // tiles requested ahead of the wait
+        if (sync.wait_first) {
+            if (sync.wait_first == 2)
+                for (; j_first < n_tiles && j_first < NS && it.key_begin + (j_first + 1) * kTile <= kv_len; ++j_first) { issue_k(j_first); issue_v(j_first); }
+            wait_for_predecessors();
+        }
         // Q first (the first S = Q K^T needs it and it is small), then K and V tiles in the order
         // they are consumed.
         mbar_expect_tx(B.q_full(), (uint32_t)(NB * 2 * 64 * qg * tpb * 2));   // two boxes of 64 dims x g heads x p tokens per block
@@ -605,7 +610,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             tma_load_4d(dst, &tmap_q, 0, 0, it.kvh, tok, B.q_full());
             tma_load_4d(dst + kSubTileBytes, &tmap_q, 64, 0, it.kvh, tok, B.q_full());
         }
-        for (int j = 0; j < n_tiles && j < NS; ++j) { issue_k(j); issue_v(j); }
+        for (int j = j_first; j < n_tiles && j < NS; ++j) { issue_k(j); issue_v(j); }
     }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
