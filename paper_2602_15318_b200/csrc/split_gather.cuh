@@ -383,12 +383,13 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
         __syncthreads();
         tc::cluster_wait();                                  // every peer runs, its barrier is initialised
         if (tid == 0) tc::mbar_expect_tx(bar, (uint32_t)(n * cl * tc::kRowBytes));
-        if (tid < cl) {
+        const int peer = warp + 8 * lane;                    // (spread over the warps: a warp's lanes issue one after the other)
+        if (peer < cl) {
             int r0;
-            const int rows = tc::merge_share(unit_rows, tid, cl, &r0) - r0;        // peer tid's share
+            const int rows = tc::merge_share(unit_rows, peer, cl, &r0) - r0;        // the peer's share
             if (rows > 0)
-                tc::bulk_push(tc::map_to_rank(recv + (uint32_t)(it.split * rows * tc::kRowBytes), (uint32_t)tid),
-                              smem_u32(smem + r0 * tc::kRowBytes), (uint32_t)(rows * tc::kRowBytes), tc::map_to_rank(bar, (uint32_t)tid));
+                tc::bulk_push(tc::map_to_rank(recv + (uint32_t)(it.split * rows * tc::kRowBytes), (uint32_t)peer),
+                              smem_u32(smem + r0 * tc::kRowBytes), (uint32_t)(rows * tc::kRowBytes), tc::map_to_rank(bar, (uint32_t)peer));
         }
         const bool landed = tc::mbar_wait(bar, 0);
         tc::cluster_arrive_relaxed();                        // (all pushes to this CTA are through: its peers may leave)

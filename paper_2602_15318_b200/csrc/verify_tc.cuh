@@ -1179,11 +1179,12 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const int n = merge_share(unit_rows, it.split, cl, &r_begin) - r_begin;
             cluster_wait();                                            // every peer runs, its barriers are initialised
             if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n * cl * kRowBytes));
-            if (tid < cl) {
+            const int peer = warp + 8 * lane;                          // (spread over the warps: a warp's lanes issue one after the other)
+            if (peer < cl) {
                 int r0;
-                const int r1 = merge_share(unit_rows, tid, cl, &r0);       // peer tid's share
-                const uint32_t dst = map_to_rank(recv + (uint32_t)(it.split * (r1 - r0) * kRowBytes), (uint32_t)tid);
-                const uint32_t bar = map_to_rank(B.fin(), (uint32_t)tid);
+                const int r1 = merge_share(unit_rows, peer, cl, &r0);      // the peer's share
+                const uint32_t dst = map_to_rank(recv + (uint32_t)(it.split * (r1 - r0) * kRowBytes), (uint32_t)peer);
+                const uint32_t bar = map_to_rank(B.fin(), (uint32_t)peer);
                 // (staged block by block: the share may straddle the two)
                 const int mid = min(max(rows_per_block, r0), r1);
                 if (mid > r0) bulk_push(dst, smem_u32(q_sm) + (uint32_t)(r0 * kRowBytes), (uint32_t)((mid - r0) * kRowBytes), bar);
@@ -1245,7 +1246,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                         const __half* src = args.o_part + (size_t)sg.src * kPartRowHalves;
                         const uint32_t dst = smem_u32(kv_sm) + (uint32_t)sg.offset;
                         const size_t pitch = (size_t)plan.part_rows * kPartRowHalves;      // halves between pieces
-                        for (int sp = tid; sp < ns; sp += 256) {           // thread sp brings piece sp
+                        // one copy per thread, spread over the warps (a warp's lanes issue theirs one after the other)
+                        for (int sp = warp + 8 * lane; sp < ns; sp += 256) {
                             bulk_load(dst + (uint32_t)(sp * n * kRowBytes), src + sp * pitch, (uint32_t)split * kRowBytes, B.fin());
                             if (split < n)
                                 bulk_load(dst + (uint32_t)((sp * n + split) * kRowBytes),
