@@ -877,36 +877,34 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             // tiles whose every key is visible to this row: [j_head, j_tail)
             const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
             const int j_head = my_lo > it.key_begin ? (my_lo - it.key_begin + kTile - 1) / kTile : 0;
-            // (visibility masks are applied in TMEM, by a pass of their own over the few tiles that need one)
             #pragma unroll 1
             for (int j = 0; j < n_tiles && ok; ++j) {
                 const int tile0 = it.key_begin + j * kTile;
                 if (!mbar_wait_warp(B.s_full(blk), j & 1)) { ok = false; break; }
                 tc_fence_after();
-                if (__any_sync(0xffffffffu, j >= j_tail || j < j_head)) {  // the tile crosses a visibility boundary of some row
-                    const unsigned long long lo = vis_word(tile0, my_anc, my_lo), hi = vis_word(tile0 + 64, my_anc, my_lo);
-                    #pragma unroll 1
-                    for (int ch = 0; ch < 4; ++ch) {                       // 32 keys at a time, where any row has one to hide
-                        const uint32_t vis = (uint32_t)((ch & 2 ? hi : lo) >> (32 * (ch & 1)));
-                        if (!__any_sync(0xffffffffu, vis != ~0u)) continue;
-                        float x[32];
-                        tmem_ld32(s_addr + 32 * ch, x);
-                        tmem_wait_ld();
-                        mask_chunk(x, vis);
-                        tmem_st32(s_addr + 32 * ch, reinterpret_cast<uint32_t*>(x));
-                    }
-                    tmem_wait_st();
-                }
-                // first pass over the row's 128 scores, 64 at a time: the maximum
+                // First pass over the row's 128 scores, 64 at a time: the maximum.  In a tile that crosses a
+                // visibility boundary of some row the scores are masked on the way; the lower 64, which are
+                // fetched again for the second pass, go back to TMEM masked.
+                const bool edge = __any_sync(0xffffffffu, j >= j_tail || j < j_head);
                 float x0[32], x1[32];
-                tmem_ld32(s_addr, x0);
-                tmem_ld32(s_addr + 32, x1);
-                tmem_wait_ld();
-                float mx = fmaxf(chunk_max(x0), chunk_max(x1));
-                tmem_ld32(s_addr + 64, x0);
-                tmem_ld32(s_addr + 96, x1);
-                tmem_wait_ld();
-                mx = fmaxf(mx, fmaxf(chunk_max(x0), chunk_max(x1)));
+                float mx = -INFINITY;
+                #pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+                    tmem_ld32(s_addr + 64 * half, x0);
+                    tmem_ld32(s_addr + 64 * half + 32, x1);
+                    tmem_wait_ld();
+                    if (edge) {
+                        const unsigned long long vis = vis_word(tile0 + 64 * half, my_anc, my_lo);
+                        mask_chunk(x0, (uint32_t)vis);
+                        mask_chunk(x1, (uint32_t)(vis >> 32));
+                        if (half == 0) {
+                            tmem_st32(s_addr, reinterpret_cast<uint32_t*>(x0));
+                            tmem_st32(s_addr + 32, reinterpret_cast<uint32_t*>(x1));
+                            tmem_wait_st();
+                        }
+                    }
+                    mx = fmaxf(mx, fmaxf(chunk_max(x0), chunk_max(x1)));
+                }
                 // lazy reference maximum, per row; the accumulator is rescaled by the whole warp (the
                 // TMEM accesses are warp-wide) whenever one of its rows moved
                 const bool need = my_ok && (mx > my_m + thr || (my_m == -INFINITY && mx > -INFINITY));
@@ -1081,25 +1079,37 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 tmem_wait_ld();
                 uint4 pk[4];
                 uint32_t* w = reinterpret_cast<uint32_t*>(pk);
-                uint4* dst;
                 if (direct) {
                     #pragma unroll
                     for (int c = 0; c < 16; ++c) w[c] = pack_bf16x2(o[2 * c] * inv, o[2 * c + 1] * inv);
-                    dst = reinterpret_cast<uint4*>(args.out + (((size_t)it.b * T + my_t) * args.n_q_heads + h_row) * kD + col);
                 } else {
                     #pragma unroll
                     for (int c = 0; c < 16; ++c) w[c] = pack_half2(o[2 * c] * inv, o[2 * c + 1] * inv);
-                    dst = reinterpret_cast<uint4*>(stage + row_local * kRowBytes + col * 2);
                 }
                 if (my_row) {
+                    uint4* dst = reinterpret_cast<uint4*>(stage + row_local * kRowBytes + col * 2);
                     #pragma unroll
                     for (int c = 0; c < 4; ++c) dst[c] = pk[c];
                 }
             }
         }
         if (!direct) fence_proxy_async();                              // the staged rows, ahead of the bulk copies
-        softmax_bar_sync();                                            // every row is staged (or written)
-        if (tid == 0 && ok && !direct && !clustered) {
+        softmax_bar_sync();                                            // every row is staged
+        if (direct) {
+            // final rows: 16 threads write a row's 256 bytes (a row per thread took 2 us longer)
+            const int inv_qg = (65536 + qg - 1) / qg;                  // x / qg = x * inv_qg >> 16 for x <= 512
+            #pragma unroll
+            for (int bk = 0; bk < NB; ++bk) {
+                const int t0 = (block0 + bk) * tpb, rows_here = ok ? min(tpb, max(0, T - t0)) * qg : 0;
+                #pragma unroll 4
+                for (int r = tid >> 4; r < rows_here; r += 16) {
+                    const int tok = (r * inv_qg) >> 16, h = it.kvh * qg + r - tok * qg;
+                    *reinterpret_cast<uint4*>(args.out + (((size_t)it.b * T + t0 + tok) * args.n_q_heads + h) * kD + (tid & 15) * 8) =
+                        *reinterpret_cast<const uint4*>(q_sm + bk * (kBlockRows * kRowBytes) + r * kRowBytes + (tid & 15) * 16);
+                }
+            }
+            softmax_bar_sync();                                        // every row is written
+        } else if (tid == 0 && ok && !clustered) {
             #pragma unroll
             for (int bk = 0; bk < NB; ++bk) {
                 const int rows_here = min(tpb, max(0, T - (block0 + bk) * tpb)) * qg;
