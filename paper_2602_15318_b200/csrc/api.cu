@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -117,7 +118,7 @@ Staging staging_layout(const sparrow_layout& L)
     return s;
 }
 
-// 128-row blocks (18 draft tokens each) one work item of the tensor-core pass handles
+// Most 128-row blocks (18 draft tokens each at a group of 7) that one work item of the tensor-core pass takes
 int blocks_per_group_tc(int T, int group) { return T <= tokens_per_block(group) ? 1 : 2; }
 
 int max_items(int n_sm, int batch, int n_kv_heads, int n_groups)
@@ -659,17 +660,19 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
     return SPARROW_OK;
 }
 
-// Estimates for plan_lone_call(), us: a tile of 128 keys with one / two row blocks, and the merges.
+// Estimates for the choice of a plan, us: a tile of 128 keys with one / two row blocks, the merges of a lone
+// call, and what an item of a call in a batch costs besides its tiles.
 constexpr float kTileUs[2] = {1.2f, 2.0f};
-constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f;
+constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 2.5f;
+constexpr float kItemUs[2] = {5.f, 11.f};
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
 // at most 16 pieces per unit, pieces short enough to leave a stage of the K/V ring free for the rows that are
 // sent around (2 tiles with one row block, 1 with two), and whole clusters per GPC.  Rewrites the plan where
 // that is estimated to pay.  Measured back to back, workspace -> cluster: 448 keys, T = 8 9.2 -> 7.4 us; 1,000
 // keys, T = 16 9.9 -> 8.2; 3,000 keys 13.1 -> 9.5 (12 pieces of two tiles instead of 24 of one); 448 keys, T = 30
-// 13.8 -> 11.6.  One piece against two in a cluster: 240 keys, T = 8 7.8 and 7.8.
-void plan_lone_call(const sparrow_ctx* c, SplitPlan* p)
+// 13.8 -> 11.6.  One piece against two in a cluster: 240 keys, T = 8 7.8 and 7.8.  Returns the estimate.
+float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
 {
     const int nb = p->blocks_per_group, units = p->batch * p->n_kv_heads * p->n_groups;
     const float per_tile = nb == 1 ? kTileUs[0] : kTileUs[1];
@@ -685,14 +688,14 @@ void plan_lone_call(const sparrow_ctx* c, SplitPlan* p)
         if (t > best) best = t;
     }
     int pieces = 0;
-    for (int n = 1; n <= kMaxMergeCluster && n <= least; ++n) {
+    for (int n = 1; may_rewrite && n <= kMaxMergeCluster && n <= least; ++n) {
         const int piece = (most + n - 1) / n;
         if (n == 1 && units > c->n_sm) continue;
         if (n > 1 && (piece > free_stage_tiles || !c->max_clusters[nb - 1] || units > c->max_clusters[nb - 1][n])) continue;
         const float t = per_tile * piece + (n > 1 ? kMergeClusterUs : 0.f);
         if (t < best) { best = t; pieces = n; }
     }
-    if (pieces == 0) return;
+    if (pieces == 0) return best;
     int total = 0;
     for (int b = 0; b < p->batch; ++b) {
         p->seq[b].n_splits = pieces;
@@ -701,6 +704,63 @@ void plan_lone_call(const sparrow_ctx* c, SplitPlan* p)
     }
     p->n_items = total;
     p->cluster = pieces;
+    return best;
+}
+
+// What a call in a batch takes of the GPU, in SM microseconds.
+float batch_cost(const SplitPlan& p)
+{
+    long long tiles = 0;
+    for (int b = 0; b < p.batch; ++b) tiles += (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile;
+    return kItemUs[p.blocks_per_group - 1] * p.n_items + kTileUs[p.blocks_per_group - 1] * (float)(tiles * p.n_kv_heads * p.n_groups);
+}
+
+// The split of a verification call, and whether its items take one row block or two.
+//
+// Calls that may share the GPU get the policy's item count; where that leaves pieces of more than
+// kMaxPieceTiles they are cut further, up to one item for every second SM: a piece that long is the last
+// thing running while other SMs have nothing left.  Calls of one batch, throughput policy, longest piece as
+// the item count gave it -> cut: four sequences of 30,000 keys, T = 36, 10 layers 838 -> 517 us; four of 20,000,
+// T = 10, 20 layers 525 -> 459; 20,000 keys, 8 KV heads, T = 50, 12 layers 338 -> 276; two of 8,000, 8 KV heads,
+// T = 20 157 -> 139; eight of 32,768, T = 32, 28 layers 3,025 -> 2,860, where one item per SM gave 3,055.  At 28
+// tiles the merges cost: 26,112 keys, T = 16, 28 layers 275 -> 287.  Neither rule looks at the other calls of a
+// batch: a call's bits do not depend on them.
+//
+// A draft block of more than one row block: an item with two of them reads its keys once for both and keeps the
+// tensor pipe fuller on long pieces (2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
+// and merge, no empty half where the blocks are odd in number, and twice as many of them fill the chip.
+// Lone calls, two blocks -> one: 448 keys, T = 40 11.1 -> 7.9 us; 2,048 keys, T = 24 12.6 -> 9.1; 16,384 keys, T = 64
+// 28.1 -> 26.7; 26,112 keys, T = 24 25.9 -> 24.5 but T = 60 34.6 -> 35.3 (stays with two).  In a batch: 5,000 keys x 4,
+// T = 50, 12 layers 240 -> 181; 2,000 keys, T = 20, 28 layers 152 -> 128; 10,000 keys, T = 40, latency policy 343 ->
+// 288; 30,000 keys, T = 30, throughput policy, 20 layers 335 -> 411 and eight of 32,768, T = 32 2,860 -> 3,240 (two).
+constexpr int kMaxPieceTiles = 48;
+sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluster, int group, const int32_t* n_keys, int T,
+                           const int32_t* key0, SplitPlan* plan)
+{
+    const sparrow_layout& L = c->layout;
+    float best = 0.f;
+    for (int nb = 1; nb <= blocks_per_group_tc(T, group); ++nb) {
+        SplitPlan p;
+        sparrow_status s = make_plan(plan_target(c, may_share), L.batch, L.n_kv_heads, group, n_keys, T, nb, &p, kMinPieceKeys, key0);
+        if (s != SPARROW_OK) return s;
+        float cost;
+        if (may_share) {
+            int longest = 0;
+            for (int b = 0; b < p.batch; ++b) {
+                const int tiles = (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile;
+                longest = std::max(longest, (tiles + p.seq[b].n_splits - 1) / p.seq[b].n_splits);
+            }
+            if (longest > kMaxPieceTiles)
+                s = make_plan(std::max(c->n_sm / 2, plan_target(c, true)), L.batch, L.n_kv_heads, group, n_keys, T, nb, &p,
+                              kMaxPieceTiles * kKeyTile, key0);
+            if (s != SPARROW_OK) return s;
+            cost = batch_cost(p);
+        } else {
+            cost = plan_lone_call(c, may_cluster, &p) + (nb - 1) * kTwoBlocksUs;
+        }
+        if (nb == 1 || cost < best) { *plan = p; best = cost; }
+    }
+    return SPARROW_OK;
 }
 
 // The gathered pass cut so that a unit's pieces share a cluster and merge there instead of through the
@@ -773,18 +833,16 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     const bool may_share = protocol && (c->in_batch || c->overlap_single_calls);
     SplitPlan plan;
     const int group = layout_group(c->layout);
-    sparrow_status s = make_plan(plan_target(c, may_share), c->layout.batch, c->layout.n_kv_heads, group, n_keys, T,
-                                 blocks_per_group_tc(T, group), &plan, kMinPieceKeys, key0);
+    sparrow_status s = plan_verify(c, may_share, protocol, group, n_keys, T, key0, &plan);
     if (s != SPARROW_OK) return s;
-    if (protocol && !may_share) plan_lone_call(c, &plan);
     plan.T_tree = T_tree;
     for (int b = 0; b < c->layout.batch; ++b) plan.seq[b].kv_len = kv_len[b];
     if ((s = check_ws(c, plan)) != SPARROW_OK) return s;
     SyncArgs sy = next_sync(c, plan, protocol, outputs_touch_previous(c, cr), may_share);
     sy.wait_first = protocol && !early ? (c->prefix_ready ? 2 : 1) : 0;
     if (c->log_plans) {
-        std::fprintf(stderr, "[sparrow] verify call %u: T %d of %d nodes, %d row block(s) x %d group(s), %d items (target %d), %s, %s;",
-                     c->seq, T, T_tree, plan.blocks_per_group, plan.n_groups, plan.n_items, plan_target(c, may_share),
+        std::fprintf(stderr, "[sparrow] verify call %u: T %d of %d nodes, %d row block(s), %d per item, %d items (target %d), %s, %s;",
+                     c->seq, T, T_tree, (T + plan.tok_per_block - 1) / plan.tok_per_block, plan.blocks_per_group, plan.n_items, plan_target(c, may_share),
                      protocol ? "counter protocol" : "stream-ordered", early ? "starts early" : "stream order");
         for (int b = 0; b < plan.batch; ++b)
             std::fprintf(stderr, " seq %d: keys [%d, %d) in %d piece(s)", b, plan.seq[b].key0, plan.seq[b].n_keys, plan.seq[b].n_splits);

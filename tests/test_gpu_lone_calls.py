@@ -79,3 +79,25 @@ def test_anchored_pieces(n_text, T, batch):
     case = W.make_anchor_case(7500 + n_text + T, idx, 0, T, batch, DEV)
     out, lse, _ = run_anchor(case)
     check(out, lse, *oracle_anchor(case))
+
+
+@pytest.mark.parametrize("hq,hkv,kv_len,T", [
+    (32, 8, [48 * 128 - 12] * 3, 12),       # pieces of 48 tiles: as long as a call in a batch leaves them
+    (32, 8, [48 * 128 - 11, 300, 6000], 12),  # one key more: two pieces, the second of one tile
+    (28, 4, [2000], 19),                    # two row blocks in items of one
+    (28, 4, [30000], 36),                   # two row blocks in items of two
+    (28, 4, [10000], 37),                   # three
+    (16, 1, [900], 64),                     # eight
+])
+def test_split_of_calls_in_a_batch(hq, hkv, kv_len, T):
+    """Two calls that overlap in a batch, where their pieces and row blocks are chosen differently from a lone call's."""
+    cases = [W.make_verify_case(7700 + T + i, kv_len, T, "random", DEV, hq=hq, hkv=hkv) for i in range(2)]
+    ctx = B.Context.for_cache(cases[0].k, W.SCALE, n_q_heads=hq)
+    ctx.set_plan_policy(B.PLAN_THROUGHPUT)
+    outs = [(torch.full_like(c.q, float("nan")), torch.full((len(kv_len), hq, T), float("nan"), dtype=torch.float32, device=DEV))
+            for c in cases]
+    B.sparrow_verify_attn_batch(ctx, B.VerifyBatch([(c.q, c.k, c.v, c.kv_len, c.parents, c.T, o, l) for c, (o, l) in zip(cases, outs)]))
+    torch.cuda.synchronize()
+    assert ctx.last_device_status() == 0
+    for c, (o, l) in zip(cases, outs):
+        check(o, l, *oracle_verify(c))
