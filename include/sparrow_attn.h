@@ -435,7 +435,8 @@ sparrow_status sparrow_debug_ancestor_masks_device(sparrow_ctx* ctx, const int32
  * splits_out[b] = key-range pieces per (sequence, KV head, row group) and the total number of
  * work items.  Pieces are whole 128-key tiles, as even as whole tiles allow (the last one takes
  * the ragged end): sparrow_plan_piece_range() gives the keys [begin, end) of piece `piece` of
- * `n_splits`; SPARROW_ERR_SHAPE unless 0 <= piece < n_splits <= ceil(n_keys / 128). */
+ * `n_splits`; SPARROW_ERR_SHAPE unless 0 <= piece < n_splits <= ceil(n_keys / 128).  (The kernels
+ * cut into pieces of the same sizes and take the longer ones first.) */
 sparrow_status sparrow_plan_splits(int32_t n_sm, int32_t batch, int32_t n_kv_heads, int32_t gqa_group,
                                    const int32_t* n_keys, int32_t T, int32_t* splits_out,
                                    int32_t* n_items_out);
