@@ -140,6 +140,7 @@ sparrow_status make_plan(int n_sm, int batch, int n_kv_heads, int group, const i
     p->T = T;
     p->T_tree = T;
     p->group = group;
+    p->inv_group = (65536 + group - 1) / group;
     p->tok_per_block = tpb;
     p->M = group * T;
     p->blocks_per_group = blocks_per_group;
@@ -663,7 +664,7 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
 // Estimates for the choice of a plan, us: a tile of 128 keys with one / two row blocks, the merges of a lone
 // call, and what an item of a call in a batch costs besides its tiles.
 constexpr float kTileUs[2] = {1.2f, 2.0f};
-constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 2.5f;
+constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 4.f;
 constexpr float kItemUs[2] = {5.f, 11.f};
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
@@ -704,6 +705,7 @@ float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
     }
     p->n_items = total;
     p->cluster = pieces;
+    p->inv_cluster = (65536 + pieces - 1) / pieces;
     return best;
 }
 
@@ -730,7 +732,8 @@ float batch_cost(const SplitPlan& p)
 // tensor pipe fuller on long pieces (2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
 // and merge, no empty half where the blocks are odd in number, and twice as many of them fill the chip.
 // Lone calls, two blocks -> one: 448 keys, T = 40 11.1 -> 7.9 us; 2,048 keys, T = 24 12.6 -> 9.1; 16,384 keys, T = 64
-// 28.1 -> 26.7; 26,112 keys, T = 24 25.9 -> 24.5 but T = 60 34.6 -> 35.3 (stays with two).  In a batch: 5,000 keys x 4,
+// 28.1 -> 26.7; 26,112 keys, T = 24 25.9 -> 24.5, T = 60 35.1 -> 34.4; 32,000 keys, T = 36 27.1 -> 25.1; but eight
+// sequences of 9,000, T = 30 48.4 -> 49.5 and two of 30,000, T = 60 71 -> 83 (stay with two).  In a batch: 5,000 keys x 4,
 // T = 50, 12 layers 240 -> 181; 2,000 keys, T = 20, 28 layers 152 -> 128; 10,000 keys, T = 40, latency policy 343 ->
 // 288; 30,000 keys, T = 30, throughput policy, 20 layers 335 -> 411 and eight of 32,768, T = 32 2,860 -> 3,240 (two).
 constexpr int kMaxPieceTiles = 48;
@@ -787,6 +790,7 @@ void plan_gather_cluster(const sparrow_ctx* c, int n_anchor, SplitPlan* p)
     }
     p->n_items = total;
     p->cluster = pieces;
+    p->inv_cluster = (65536 + pieces - 1) / pieces;
 }
 
 // One verification call: T query tokens, the last T of the T_tree nodes whose K/V rows sit at

@@ -81,6 +81,8 @@ struct SplitPlan {
     int32_t n_groups;             // ceil(T / (18 * blocks_per_group))
     int32_t n_kv_heads;
     int32_t part_rows;            // row pitch of one item's partial block in the workspace
+    int32_t inv_group;            // 2^16 / group rounded up: x / group = x * inv_group >> 16 for x <= 512
+    int32_t inv_cluster;          // the same of cluster
     int32_t cluster;              // > 1: every unit has this many pieces, in CTAs of one thread-block cluster that merge among themselves
     int32_t piece_tile;           // pieces of the key range are whole tiles of this many keys (128 or 64)
     SeqPlan seq[kMaxBatch];

@@ -49,7 +49,7 @@ constexpr int kStageBytes = kTile * kD * 2;            // one K or V tile: 16 KB
 constexpr int kSmemBytes = 4 * kStageBytes + kMaxT * 8 + kMaxT * 4 + 2 * kTile * 4;
 // with the pieces of a unit in a cluster: the rows the peers send, [piece][row][272 bytes], and the merge's scratch
 constexpr int kRecvBytes = (kRows + tc::kMaxMergeCluster) * tc::kRowBytes;
-constexpr int kClusterSmemBytes = (kSmemBytes + 15) / 16 * 16 + kRecvBytes + kThreads * 10 * 4;
+constexpr int kClusterSmemBytes = (kSmemBytes + 15) / 16 * 16 + kRecvBytes;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
@@ -378,7 +378,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
         const int unit_rows = plan.group * min(plan.tok_per_block, T - tok0);
         const uint32_t recv = smem_u32(smem + (kSmemBytes + 15) / 16 * 16), bar = smem_u32(&merge_bar);
         int r_begin;
-        const int n = tc::merge_share(unit_rows, it.split, cl, &r_begin) - r_begin;
+        const int n = tc::merge_share(unit_rows, it.split, plan.inv_cluster, &r_begin) - r_begin;
         tc::fence_proxy_async();                             // the staged rows, ahead of the bulk copies
         __syncthreads();
         tc::cluster_wait();                                  // every peer runs, its barrier is initialised
@@ -386,7 +386,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
         const int peer = warp + 8 * lane;                    // (spread over the warps: a warp's lanes issue one after the other)
         if (peer < cl) {
             int r0;
-            const int rows = tc::merge_share(unit_rows, peer, cl, &r0) - r0;        // the peer's share
+            const int rows = tc::merge_share(unit_rows, peer, plan.inv_cluster, &r0) - r0;        // the peer's share
             if (rows > 0)
                 tc::bulk_push(tc::map_to_rank(recv + (uint32_t)(it.split * rows * tc::kRowBytes), (uint32_t)peer),
                               smem_u32(smem + r0 * tc::kRowBytes), (uint32_t)(rows * tc::kRowBytes), tc::map_to_rank(bar, (uint32_t)peer));
@@ -394,9 +394,8 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
         const bool landed = tc::mbar_wait(bar, 0);
         tc::cluster_arrive_relaxed();                        // (all pushes to this CTA are through: its peers may leave)
         if (!landed && lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies));
-        const tc::MergeOut mo = {args.out, args.lse, T, args.n_q_heads, plan.group};
-        tc::merge_run(tid, recv, cl, n, r_begin, it.b, tok0, it.kvh * plan.group, landed,
-                      reinterpret_cast<float*>(smem + (kSmemBytes + 15) / 16 * 16 + kRecvBytes), mo, [] { __syncthreads(); });
+        const tc::MergeOut mo = {args.out, args.lse, T, args.n_q_heads, plan.group, plan.inv_group};
+        tc::merge_run(tid, recv, cl, n, r_begin, it.b, tok0, it.kvh * plan.group, landed, mo);
         tc::cluster_wait();                                  // nobody leaves before its peers have received what it sends them
     }
 }

@@ -411,7 +411,7 @@ struct Bars {
 struct MergeOut {
     __nv_bfloat16* out;
     float* lse;
-    int T, n_q_heads, qg;
+    int T, n_q_heads, qg, inv_qg;
 };
 // The final bf16 row and LSE from a row's weighted sum, the sum of weights and the reference of the weights; 16
 // threads of 8 dims each.
@@ -424,18 +424,17 @@ __device__ __forceinline__ void write_merged(const float (&acc)[8], float s, flo
     *reinterpret_cast<uint4*>(mo.out + (((size_t)b * mo.T + t) * mo.n_q_heads + h) * kD + c16 * 8) = pk;
     if (c16 == 0) mo.lse[((size_t)b * mo.n_q_heads + h) * mo.T + t] = s > 0.f ? m + __logf(s) : -INFINITY;
 }
-// One thread's share of a row: pieces first, first + step, ... of 8 dims.  The largest LSE first, so that the
-// pieces' weights do not depend on one another.
-__device__ __forceinline__ void fold_pieces(uint32_t row, int first, int step, int ns, uint32_t pstride, int c16, float (&acc)[8], float& s, float& m)
+// One thread's share of a row: `count` pieces `hop` bytes apart from `row` on, 8 dims.  The largest LSE first, so
+// that the pieces' weights do not depend on one another.
+__device__ __forceinline__ void fold_pieces(uint32_t row, int count, uint32_t hop, int c16, float (&acc)[8], float& s, float& m)
 {
-    const uint32_t a0 = row + (uint32_t)first * pstride, hop = (uint32_t)step * pstride;
-    uint32_t at = a0 + 2 * kD;
+    uint32_t at = row + 2 * kD;
     #pragma unroll 4
-    for (int sp = first; sp < ns; sp += step, at += hop) m = fmaxf(m, lds_f32(at));
+    for (int i = 0; i < count; ++i, at += hop) m = fmaxf(m, lds_f32(at));
     const float m_log2 = m == -INFINITY ? 0.f : m * 1.4426950408889634f;           // (all pieces empty: weights 0)
-    at = a0;
+    at = row;
     #pragma unroll 2
-    for (int sp = first; sp < ns; sp += step, at += hop) {
+    for (int i = 0; i < count; ++i, at += hop) {
         const float w = ex2(fmaf(lds_f32(at + 2 * kD), 1.4426950408889634f, -m_log2));
         uint32_t raw[4];
         lds_v4(at + c16 * 16, raw);
@@ -448,65 +447,58 @@ __device__ __forceinline__ void fold_pieces(uint32_t row, int first, int step, i
     }
 }
 // Merges rows [0, n) of a run whose ns pieces lie in shared memory at `base` as [piece][row][272 bytes] and writes
-// the results; row i is row r0 + i of its unit (token idx / g, head idx % g).  256 threads, 16 per row: R rows at
-// a time with 16 / R groups of threads sharing a row's pieces where there are fewer than 16 rows (the groups'
-// results meet in red: [256][10] floats).  `barrier` is a barrier of these 256 threads.
-template <class Barrier>
-__device__ __forceinline__ void merge_run(int tid, uint32_t base, int ns, int n, int r0, int b, int tok0, int head0, bool landed,
-                                          float* red, const MergeOut& mo, Barrier barrier)
+// the results; row i is row r0 + i of its unit (token idx / g, head idx % g).  256 threads, no barrier: more than
+// eight rows go two to a warp, 16 lanes of 8 dims each; of fewer a warp takes 128, 64, 32 or 16 dims, and the
+// groups of lanes left over share the row's pieces and add up by shuffles.  What this costs is instructions one
+// after the other (two warps per scheduler), divisions first: with trip counts and shares by shifts and by
+// reciprocals from the host, and without the barriers of groups that met in shared memory, verification of
+// 2,048 keys, T = 8 takes 7.9 us (8.3), three sequences of 9,001 22.3 (22.8), 448 anchors 9.3 (9.6).
+__device__ __forceinline__ void merge_run(int tid, uint32_t base, int ns, int n, int r0, int b, int tok0, int head0, bool landed, const MergeOut& mo)
 {
-    const int inv_qg = (65536 + mo.qg - 1) / mo.qg;                // x / qg = x * inv_qg >> 16 for x <= 512
-    const int c16 = tid & 15;
+    const int warp = tid >> 5, lane = tid & 31;
     const uint32_t pstride = (uint32_t)n * kRowBytes;              // bytes between pieces
-    int lg_g = 4;
-    while (lg_g > 0 && (16 >> lg_g) < n) --lg_g;
-    const int G = 1 << lg_g;
-    if (G == 1) {
-        #pragma unroll 1
-        for (int r = tid >> 4; r < n; r += 16) {
-            if (!landed) break;
-            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, s = 0.f, m = -INFINITY;
-            fold_pieces(base + (uint32_t)r * kRowBytes, 0, 1, ns, pstride, c16, acc, s, m);
-            const int idx = r0 + r, tok = (idx * inv_qg) >> 16;
+    const bool two_rows = n > 8;
+    const int lg_lanes = n > 4 ? 4 : (n > 2 ? 3 : n);              // lanes of a group
+    const int grp = lane >> lg_lanes, parts = 4 - lg_lanes;        // (two_rows: grp is the row)
+    const int tasks = two_rows ? (n + 1) >> 1 : n << parts;
+    // a group's pieces: first, first + 2^lg_step, ...
+    const int first = two_rows ? 0 : grp, lg_step = two_rows ? 0 : 5 - lg_lanes;
+    const int count = (ns - first + (1 << lg_step) - 1) >> lg_step;
+    #pragma unroll 1
+    for (int task = warp; task < tasks; task += 8) {
+        const int r = two_rows ? 2 * task + grp : task >> parts;
+        const int c16 = (lane & ((1 << lg_lanes) - 1)) + ((task & ((1 << parts) - 1)) << lg_lanes);
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, s = 0.f, m = -INFINITY;
+        if (landed && r < n) fold_pieces(base + (uint32_t)r * kRowBytes + (uint32_t)first * pstride, count, pstride << lg_step, c16, acc, s, m);
+        if (!two_rows) {
+            float m_all = m;
+            #pragma unroll 1
+            for (int o = 1 << lg_lanes; o < 32; o <<= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xffffffffu, m_all, o));
+            const float f = m == -INFINITY ? 0.f : ex2((m - m_all) * 1.4426950408889634f);
+            m = m_all;
+            s *= f;
+            #pragma unroll
+            for (int q = 0; q < 8; ++q) acc[q] *= f;
+            #pragma unroll 1
+            for (int o = 1 << lg_lanes; o < 32; o <<= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, o);
+                #pragma unroll
+                for (int q = 0; q < 8; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+            }
+        }
+        if (landed && r < n && (two_rows || grp == 0)) {
+            const int idx = r0 + r, tok = (idx * mo.inv_qg) >> 16;
             write_merged(acc, s, m, b, tok0 + tok, head0 + idx - tok * mo.qg, c16, mo);
         }
-        return;
     }
-    const int i = tid >> (4 + lg_g), grp = (tid >> 4) & (G - 1);
-    const bool active = landed && i < n;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, s = 0.f, m = -INFINITY;
-    if (active) fold_pieces(base + (uint32_t)i * kRowBytes, grp, G, ns, pstride, c16, acc, s, m);
-    barrier();                                                     // the run before has been read
-    #pragma unroll
-    for (int q = 0; q < 8; ++q) red[tid * 10 + q] = acc[q];
-    red[tid * 10 + 8] = s;
-    red[tid * 10 + 9] = m;
-    barrier();
-    if (!active || grp != 0) return;
-    const float* mine = red + tid * 10;
-    float m_all = m;
-    for (int g2 = 1; g2 < G; ++g2) m_all = fmaxf(m_all, mine[g2 * 160 + 9]);
-    const float a0 = m == -INFINITY ? 0.f : ex2((m - m_all) * 1.4426950408889634f);
-    s *= a0;
-    #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] *= a0;
-    for (int g2 = 1; g2 < G; ++g2) {
-        const float* o = mine + g2 * 160;
-        if (o[9] == -INFINITY) continue;
-        const float ag = ex2((o[9] - m_all) * 1.4426950408889634f);
-        s = fmaf(o[8], ag, s);
-        #pragma unroll
-        for (int q = 0; q < 8; ++q) acc[q] = fmaf(o[q], ag, acc[q]);
-    }
-    const int idx = r0 + i, tok = (idx * inv_qg) >> 16;
-    write_merged(acc, s, m_all, b, tok0 + tok, head0 + idx - tok * mo.qg, c16, mo);
 }
 
-// Rows of a unit that CTA `rank` of a cluster of `cl` finishes: [begin, return value).
-__device__ __forceinline__ int merge_share(int unit_rows, int rank, int cl, int* begin)
+// Rows of a unit that CTA `rank` of a cluster finishes: [begin, return value).  inv_cl: 2^16 / cluster size, rounded
+// up (exact: at most 252 rows times 16).
+__device__ __forceinline__ int merge_share(int unit_rows, int rank, int inv_cl, int* begin)
 {
-    *begin = unit_rows * rank / cl;
-    return unit_rows * (rank + 1) / cl;
+    *begin = (unit_rows * rank * inv_cl) >> 16;
+    return (unit_rows * (rank + 1) * inv_cl) >> 16;
 }
 
 // What one pass of the merge takes: runs of rows of one unit (sequence, KV head, row group).
@@ -1097,13 +1089,12 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         softmax_bar_sync();                                            // every row is staged
         if (direct) {
             // final rows: 16 threads write a row's 256 bytes (a row per thread took 2 us longer)
-            const int inv_qg = (65536 + qg - 1) / qg;                  // x / qg = x * inv_qg >> 16 for x <= 512
             #pragma unroll
             for (int bk = 0; bk < NB; ++bk) {
                 const int t0 = (block0 + bk) * tpb, rows_here = ok ? min(tpb, max(0, T - t0)) * qg : 0;
                 #pragma unroll 4
                 for (int r = tid >> 4; r < rows_here; r += 16) {
-                    const int tok = (r * inv_qg) >> 16, h = it.kvh * qg + r - tok * qg;
+                    const int tok = (r * plan.inv_group) >> 16, h = it.kvh * qg + r - tok * qg;
                     *reinterpret_cast<uint4*>(args.out + (((size_t)it.b * T + t0 + tok) * args.n_q_heads + h) * kD + (tid & 15) * 8) =
                         *reinterpret_cast<const uint4*>(q_sm + bk * (kBlockRows * kRowBytes) + r * kRowBytes + (tid & 15) * 16);
                 }
@@ -1176,9 +1167,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             list->bytes = bytes;
             list->next_row = row;
         };
-        // scratch of the merge: over the Q blocks, or where rows on their way to peers lie there, over a V tile
-        float* red = reinterpret_cast<float*>(clustered ? kv_sm + 2 * kSubTileBytes : q_sm);
-        const MergeOut merge_out = {args.out, args.lse, T, args.n_q_heads, qg};
+        const MergeOut merge_out = {args.out, args.lse, T, args.n_q_heads, qg, plan.inv_group};
         if (clustered) {
             // Every CTA of the cluster merges a share of the unit's rows: it is sent its rows of every piece, one
             // bulk copy from each peer, into the last stage of the K/V ring, which pieces this short never use.
@@ -1186,13 +1175,13 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const int unit_rows = qg * min(NB * tpb, T - block0 * tpb);
             const uint32_t recv = smem_u32(kv_sm) + (NS - 1) * kStageBytes;
             int r_begin;
-            const int n = merge_share(unit_rows, it.split, cl, &r_begin) - r_begin;
+            const int n = merge_share(unit_rows, it.split, plan.inv_cluster, &r_begin) - r_begin;
             cluster_wait();                                            // every peer runs, its barriers are initialised
             if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n * cl * kRowBytes));
             const int peer = warp + 8 * lane;                          // (spread over the warps: a warp's lanes issue one after the other)
             if (peer < cl) {
                 int r0;
-                const int r1 = merge_share(unit_rows, peer, cl, &r0);      // the peer's share
+                const int r1 = merge_share(unit_rows, peer, plan.inv_cluster, &r0);      // the peer's share
                 const uint32_t dst = map_to_rank(recv + (uint32_t)(it.split * (r1 - r0) * kRowBytes), (uint32_t)peer);
                 const uint32_t bar = map_to_rank(B.fin(), (uint32_t)peer);
                 // (staged block by block: the share may straddle the two)
@@ -1207,7 +1196,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             cluster_arrive_relaxed();                                  // (all pushes to this CTA are through: its peers may leave)
             if (!landed && lane == 0) atomicOr(args.status, timeout_bits(kSiteFinCopies));
             if (tid == 0) SPARROW_STAMP(15);                           // every piece is here
-            merge_run(tid, recv, cl, n, r_begin, it.b, block0 * tpb, it.kvh * qg, landed && ok, red, merge_out, [] { softmax_bar_sync(); });
+            merge_run(tid, recv, cl, n, r_begin, it.b, block0 * tpb, it.kvh * qg, landed && ok, merge_out);
             if (tid == 0) SPARROW_STAMP(10);                           // merged rows written
             softmax_bar_sync();
         }
@@ -1224,8 +1213,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             if (merges) {
                 if (tid == 0) {
                     // every partial of the call in place, and the previous call's final results written
-                    // (both words are polled in one loop: the second is usually there already)
-                    bool have_all = false, prev_done = false;
+                    // (both words are polled in one loop: the second is usually there already, and a lone
+                    // call's predecessors have ended as grids)
+                    bool have_all = false, prev_done = sync.lone != 0;
                     #pragma unroll 1
                     for (uint32_t i = 0; i < kCounterPolls && !(have_all && prev_done); ++i) {
                         if (!have_all) have_all = ld_acquire(arrive_word) == (unsigned)sync.n_arrive;
@@ -1240,9 +1230,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 }
                 // The rows' pieces are first brought into the (idle) K/V ring by bulk copies, [piece][row]
                 // [272 bytes], one copy per piece and block touched -- far fewer and larger requests than
-                // per-thread loads.  Then 16 R G threads merge R rows at a time: thread (row i, 16-byte chunk
-                // c, piece group g) folds pieces g, g + G, ... of its row into a running (max, sum, weighted
-                // output); the groups' results meet in shared memory (the Q blocks, idle by now).
+                // per-thread loads (16-byte words that carry a tag, read by the threads as they arrive and without
+                // any counter, were there 1.6 us earlier but took 2 us longer to collect).
                 #pragma unroll 1
                 for (int phase = 0;; phase ^= 1) {
                     if (tid == 0 && *fin_go) mbar_expect_tx(B.fin(), (uint32_t)list->bytes);
@@ -1271,8 +1260,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     #pragma unroll 1
                     for (int k = 0; k < n_seg; ++k) {
                         const MergeSegment& sg = list->seg[k];
-                        merge_run(tid, smem_u32(kv_sm) + (uint32_t)sg.offset, sg.ns, sg.n, sg.r0, sg.b, sg.tok0, sg.head0, landed, red, merge_out,
-                                  [] { softmax_bar_sync(); });
+                        merge_run(tid, smem_u32(kv_sm) + (uint32_t)sg.offset, sg.ns, sg.n, sg.r0, sg.b, sg.tok0, sg.head0, landed, merge_out);
                     }
                     const int next = list->next_row;
                     if (!landed || next >= my_end) break;
