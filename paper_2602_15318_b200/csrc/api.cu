@@ -497,6 +497,9 @@ void clear_tensor_maps(sparrow_ctx* c)
     c->evict_tick = 0;
 }
 
+// K and V of a call that are not worth keeping in L2 (126 MB): with those of a second layer they do not fit.
+constexpr long long kStreamOutBytes = 64ll << 20;
+
 sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const SyncArgs& sy, const void* q, const void* k, const void* v,
                                 const int32_t* parents, const int32_t* first_visible, void* out, float* lse, cudaStream_t st)
 {
@@ -513,6 +516,9 @@ sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const Syn
     a.out = static_cast<__nv_bfloat16*>(out);
     a.lse = lse;
     a.status = reinterpret_cast<unsigned*>(c->ws);
+    long long keys = 0;
+    for (int b = 0; b < plan.batch; ++b) keys += plan.seq[b].n_keys - plan.seq[b].key0;
+    a.leave_l2 = !sy.lone ? 0 : keys * plan.n_kv_heads * 2 * kD * 2 > kStreamOutBytes ? 2 : 1;
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3(plan.n_items);

@@ -69,6 +69,7 @@ struct TcArgs {
     const int32_t* first_visible;   // DEV [B][T] or nullptr: query t sees prefix key j only if j >= first_visible[b][t]
     int32_t n_q_heads;
     float scale_log2e;           // softmax_scale * log2(e)
+    int32_t leave_l2;            // K and V tiles that are the first to leave L2: none, half (1), all (2)
     __half* o_part;              // [n_items][part_rows] partial rows: 128 fp16 outputs + fp32 LSE (kPartRowHalves)
     __nv_bfloat16* out;          // final output
     float* lse;
@@ -158,6 +159,13 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
         ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar) : "memory");
+}
+// the same with an L2 eviction policy
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, uint32_t bar, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
+        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar), "l"(policy) : "memory");
 }
 // 1-D bulk copy global -> shared (16-byte aligned, size a multiple of 16), completion on an mbarrier
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
@@ -555,21 +563,31 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     const int n_jobs = n_tiles * NB;
     const int block0 = it.group * NB;                       // first 128-row block of this item
 
+    // K and V tiles of a lone call leave L2 before anything else does: a cache is streamed once per call, and would
+    // otherwise push out the code, the queries and the partial rows, which then come back from DRAM behind the
+    // stream of tiles.  All tiles of a call that takes more than half of L2, half of them of a shorter one,
+    // whose next call on the same cache then finds as much as before (26,112 keys on one and the same cache: none
+    // 15.9 us, half 16.0, all 17.3).  Caches out of L2, none -> this: 26,112 keys, T = 16 18.6 -> 18.2 us (all: 17.9);
+    // three sequences of 9,001, 8 KV heads 26.5 -> 25.0; two of 20,000, T = 16 21.6 -> 21.4.  In batches it gave nothing.
+    uint64_t stream_policy;
+    if (args.leave_l2 == 0) asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(stream_policy));
+    else if (args.leave_l2 == 1) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 0.5;" : "=l"(stream_policy));
+    else asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_policy));
     auto issue_k = [&](int j) {                     // producer thread only
         const int st = j % NS;
         const uint32_t dst = smem_u32(kv_sm + st * kStageBytes);
         const int row = it.key_begin + j * kTile;
         mbar_expect_tx(B.k_full(st), 2 * kSubTileBytes);
-        tma_load_4d(dst, &tmap_k, 0, row, it.kvh, it.b, B.k_full(st));
-        tma_load_4d(dst + kSubTileBytes, &tmap_k, 64, row, it.kvh, it.b, B.k_full(st));
+        tma_load_4d(dst, &tmap_k, 0, row, it.kvh, it.b, B.k_full(st), stream_policy);
+        tma_load_4d(dst + kSubTileBytes, &tmap_k, 64, row, it.kvh, it.b, B.k_full(st), stream_policy);
     };
     auto issue_v = [&](int j) {
         const int st = j % NS;
         const uint32_t dst = smem_u32(kv_sm + st * kStageBytes + 2 * kSubTileBytes);
         const int row = it.key_begin + j * kTile;
         mbar_expect_tx(B.v_full(st), 2 * kSubTileBytes);
-        tma_load_4d(dst, &tmap_v, 0, row, it.kvh, it.b, B.v_full(st));
-        tma_load_4d(dst + kSubTileBytes, &tmap_v, 64, row, it.kvh, it.b, B.v_full(st));
+        tma_load_4d(dst, &tmap_v, 0, row, it.kvh, it.b, B.v_full(st), stream_policy);
+        tma_load_4d(dst + kSubTileBytes, &tmap_v, 64, row, it.kvh, it.b, B.v_full(st), stream_policy);
     };
 
     // ---- setup: barriers and the first ring-full of loads, TMEM, ancestor words ------------------
