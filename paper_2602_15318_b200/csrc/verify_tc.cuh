@@ -590,7 +590,11 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         tma_load_4d(dst + kSubTileBytes, &tmap_v, 64, row, it.kvh, it.b, B.v_full(st), stream_policy);
     };
 
-    // ---- setup: barriers and the first ring-full of loads, TMEM, ancestor words ------------------
+    // ---- setup: barriers, TMEM.  Nothing here waits for an earlier kernel: every warp runs on to its own first
+    // wait before the loads start.  With the wait and the first loads in front of the CTA barrier the MMA
+    // warp fetched its code behind the stream of tiles, up to 2 us late; now, before -> after: 2,048 keys, T = 8
+    // 7.8 -> 7.6 us, 26,112 keys, T = 16 18.3 -> 17.7, 16,384 keys, T = 64 25.8 -> 25.2, three sequences of 9,001, 8
+    // KV heads 21.6 -> 21.0, eight of 9,000, T = 30 48.1 -> 46.7.
     if (warp == kProducerWarp && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_q) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_k) : "memory");
@@ -604,23 +608,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         *abort_flag = 0;
         *write_ok = sync.enabled ? 0u : 1u;
         fence_barrier_init();
-        int j_first = 0;                                 // tiles requested ahead of the wait
-        if (sync.wait_first) {
-            if (sync.wait_first == 2)
-                for (; j_first < n_tiles && j_first < NS && it.key_begin + (j_first + 1) * kTile <= kv_len; ++j_first) { issue_k(j_first); issue_v(j_first); }
-            wait_for_predecessors();
-        }
-        // Q first (the first S = Q K^T needs it and it is small), then K and V tiles in the order
-        // they are consumed.
-        mbar_expect_tx(B.q_full(), (uint32_t)(NB * 2 * 64 * qg * tpb * 2));   // two boxes of 64 dims x g heads x p tokens per block
-        #pragma unroll
-        for (int blk = 0; blk < NB; ++blk) {
-            const uint32_t dst = smem_u32(q_sm + blk * kQBlockBytes);
-            const int tok = it.b * T + (block0 + blk) * tpb;
-            tma_load_4d(dst, &tmap_q, 0, 0, it.kvh, tok, B.q_full());
-            tma_load_4d(dst + kSubTileBytes, &tmap_q, 64, 0, it.kvh, tok, B.q_full());
-        }
-        for (int j = j_first; j < n_tiles && j < NS; ++j) { issue_k(j); issue_v(j); }
     }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
@@ -632,12 +619,27 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     if (plan.cluster > 1) cluster_arrive_relaxed();      // (waited for ahead of the first access to a peer)
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 0) SPARROW_STAMP(1);                             // set-up done
-    // (behind the wait above: a dependent that starts early may rely on everything before this call)
-    if (sync.enabled) let_dependents_launch();
 
     if (warp == kProducerWarp) {
         // ================= TMA producer =================
         if (lane == 0) {
+            int j_first = 0;                                 // tiles requested ahead of the wait
+            if (sync.wait_first) {
+                if (sync.wait_first == 2)
+                    for (; j_first < n_tiles && j_first < NS && it.key_begin + (j_first + 1) * kTile <= kv_len; ++j_first) { issue_k(j_first); issue_v(j_first); }
+                wait_for_predecessors();
+            }
+            // Q first (the first S = Q K^T needs it and it is small), then K and V tiles in the order
+            // they are consumed.
+            mbar_expect_tx(B.q_full(), (uint32_t)(NB * 2 * 64 * qg * tpb * 2));   // two boxes of 64 dims x g heads x p tokens per block
+            #pragma unroll
+            for (int blk = 0; blk < NB; ++blk) {
+                const uint32_t dst = smem_u32(q_sm + blk * kQBlockBytes);
+                const int tok = it.b * T + (block0 + blk) * tpb;
+                tma_load_4d(dst, &tmap_q, 0, 0, it.kvh, tok, B.q_full());
+                tma_load_4d(dst + kSubTileBytes, &tmap_q, 64, 0, it.kvh, tok, B.q_full());
+            }
+            for (int j = j_first; j < n_tiles && j < NS; ++j) { issue_k(j); issue_v(j); }
             // refill whichever ring has a free slot; K slots free up ahead of V slots
             int jk = NS < n_tiles ? NS : n_tiles, jv = jk;
             uint32_t idle = 0;
@@ -792,6 +794,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const int Tt = plan.T_tree;
             const bool needs_tree = it.key_end > kv_len;       // this piece reaches the draft block
             if (sync.wait_first) wait_for_predecessors();
+            // (behind the wait: a dependent that starts early may rely on everything before this call; not
+            // from the producer, whose refills it held up)
+            if (sync.enabled) let_dependents_launch();
             int par[2] = {-1, -1}, lo[2] = {0, 0};
             #pragma unroll
             for (int k = 0; k < 2; ++k) {
