@@ -1319,7 +1319,7 @@ sparrow_status sparrow_window_first_visible_device(sparrow_ctx* c, const int32_t
     if (!guard.ok) return SPARROW_ERR_CUDA;
     const int n = c->layout.batch * T_new;
     other_kernel_enqueued();
-    return launch_behind(c, window_bounds_kernel, (unsigned)((n + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream), 0, anchor_idx, n_anchor, window, T_tree,
+    return launch_behind(c, window_bounds_kernel, (unsigned)((n + 3) / 4), 128, 0, static_cast<cudaStream_t>(stream), 0, anchor_idx, n_anchor, window, T_tree,
                          T_new, c->layout.batch, first_visible);
 }
 

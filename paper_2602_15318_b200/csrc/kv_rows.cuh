@@ -27,37 +27,53 @@ struct RowMoveArgs {
     unsigned* status;
 };
 
-// Moves 16 bytes of K and of V: chunk i of the (sequence, KV head, row, 16-byte column) index space.
-__device__ __forceinline__ void move_row_chunk(const RowMoveArgs& a, long long i)
+// Where chunk i of the (sequence, KV head, row, 16-byte column) index space lies.  (Rows are counted in 32 bits: a
+// 64-bit division is a hundred dependent instructions.)
+struct RowChunk {
+    int b, h, r, c;
+    size_t src_head, dst;            // element offsets: the source's (sequence, KV head) with the column, the destination
+};
+__device__ __forceinline__ RowChunk find_row_chunk(const RowMoveArgs& a, long long i)
 {
-    const int c = (int)(i & 15);
-    long long rest = i >> 4;
-    const int r = (int)(rest % a.n_rows); rest /= a.n_rows;
-    const int h = (int)(rest % a.n_kv_heads);
-    const int b = (int)(rest / a.n_kv_heads);
-    int src = a.src_rows ? ld_behind(a.src_rows + (size_t)b * a.n_rows + r) : r;
+    RowChunk x;
+    x.c = (int)(i & 15);
+    const unsigned row = (unsigned)(i >> 4), unit = row / (unsigned)a.n_rows;
+    x.r = (int)(row - unit * (unsigned)a.n_rows);
+    x.b = (int)(unit / (unsigned)a.n_kv_heads);
+    x.h = (int)(unit - (unsigned)x.b * (unsigned)a.n_kv_heads);
+    x.src_head = (size_t)x.b * a.src_stride_batch + (size_t)x.h * a.src_stride_head + x.c * 8;
+    x.dst = (size_t)x.b * a.dst_stride_batch + (size_t)x.h * a.dst_stride_head + (size_t)(a.dst_row0[x.b] + x.r) * kD + x.c * 8;
+    return x;
+}
+// Moves 16 bytes of K and of V.
+__device__ __forceinline__ void move_row_chunk(const RowMoveArgs& a, const RowChunk& x)
+{
+    const int src = a.src_rows ? ld_behind(a.src_rows + (size_t)x.b * a.n_rows + x.r) : x.r;
     const bool bad = src < 0 || src >= a.src_capacity;       // never read: the row is written as zeros
-    if (bad && c == 0 && h == 0) atomicOr(a.status, kStatAnchor);
-    const size_t s_off = (size_t)b * a.src_stride_batch + (size_t)h * a.src_stride_head + (size_t)(bad ? 0 : src) * kD + c * 8;
-    const size_t d_off = (size_t)b * a.dst_stride_batch + (size_t)h * a.dst_stride_head +
-                         (size_t)(a.dst_row0[b] + r) * kD + c * 8;
+    if (bad && x.c == 0 && x.h == 0) atomicOr(a.status, kStatAnchor);
+    const size_t s_off = x.src_head + (size_t)(bad ? 0 : src) * kD;
     uint4 kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
     if (!bad) {
         kv = *reinterpret_cast<const uint4*>(a.k_src + s_off);
         vv = *reinterpret_cast<const uint4*>(a.v_src + s_off);
     }
-    *reinterpret_cast<uint4*>(a.k_dst + d_off) = kv;
-    *reinterpret_cast<uint4*>(a.v_dst + d_off) = vv;
+    *reinterpret_cast<uint4*>(a.k_dst + x.dst) = kv;
+    *reinterpret_cast<uint4*>(a.v_dst + x.dst) = vv;
 }
 
 __global__ void __launch_bounds__(256)
 move_rows_kernel(const __grid_constant__ RowMoveArgs a)
 {
     let_dependents_launch();
-    wait_for_predecessors();
     const long long total = (long long)a.batch * a.n_kv_heads * a.n_rows * 16;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
-        move_row_chunk(a, i);
+    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    RowChunk x = find_row_chunk(a, i < total ? i : 0);       // (before the wait: the addresses need nothing of it)
+    wait_for_predecessors();
+    while (i < total) {
+        move_row_chunk(a, x);
+        i += (long long)gridDim.x * blockDim.x;
+        if (i < total) x = find_row_chunk(a, i);
+    }
 }
 
 // One step's inputs straight from host memory that the GPU can address (pinned or registered):
@@ -78,12 +94,17 @@ ingest_step_kernel(const __grid_constant__ IngestArgs a)
 {
     // in this order: the attention call behind this kernel starts streaming the cache's prefix, which this
     // kernel does not write, as soon as it is launched, and relies on everything earlier being complete
-    wait_for_predecessors();
-    let_dependents_launch();
     const long long row_chunks = (long long)a.rows.batch * a.rows.n_kv_heads * a.rows.n_rows * 16;
     const long long total = row_chunks + a.q_chunks + a.n_parents;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        if (i < row_chunks) move_row_chunk(a.rows, i);
+    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    RowChunk x = find_row_chunk(a.rows, i < row_chunks ? i : 0);
+    wait_for_predecessors();
+    let_dependents_launch();
+    for (; i < total; i += (long long)gridDim.x * blockDim.x) {
+        if (i < row_chunks) {
+            if (i >= (long long)gridDim.x * blockDim.x) x = find_row_chunk(a.rows, i);
+            move_row_chunk(a.rows, x);
+        }
         else if (i < row_chunks + a.q_chunks) a.q_dst[i - row_chunks] = a.q_src[i - row_chunks];
         else a.parents_dst[i - row_chunks - a.q_chunks] = a.parents_src[i - row_chunks - a.q_chunks];
     }
