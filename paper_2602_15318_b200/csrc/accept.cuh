@@ -50,6 +50,7 @@ accept_greedy_kernel(const int32_t* draft_tokens, const int32_t* parents,
     bonus[b] = nxt[best + 1];
 }
 
+template <int N>                     // room for the sequences (see RowMoveArgs)
 struct KeepArgs {
     __nv_bfloat16* k;
     __nv_bfloat16* v;
@@ -57,14 +58,15 @@ struct KeepArgs {
     const int32_t* n_accept;         // DEV [batch]
     int32_t T, n_kv_heads;
     int64_t stride_batch, stride_head;
-    int32_t kv_len[kMaxBatch];
+    int32_t kv_len[N];
 };
 
 // One CTA per (sequence, KV head): rows kv_len + path[i] -> rows kv_len + i, i < n_accept.  The
 // move is in place and sources and destinations overlap, so every row is read into shared
 // memory before any is written.  256 threads, 16 per row and pass.
+template <int N>
 __global__ void __launch_bounds__(256)
-keep_accepted_rows_kernel(const __grid_constant__ KeepArgs a)
+keep_accepted_rows_kernel(const __grid_constant__ KeepArgs<N> a)
 {
     let_dependents_launch();
     wait_for_predecessors();

@@ -14,6 +14,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 
 #include "combine.cuh"
 #include "common.cuh"
@@ -403,6 +404,15 @@ sparrow_status launch_behind(sparrow_ctx* c, void (*kernel)(KArgs...), unsigned 
     if (cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...) != cudaSuccess) { cudaGetLastError(); return SPARROW_ERR_CUDA; }
     c->launches.fetch_add(1);
     return SPARROW_OK;
+}
+
+// Calls f with the number of sequences its kernel's arguments have room for (see RowMoveArgs).
+constexpr int kFewSequences = 4;
+template <class F>
+sparrow_status with_room(int batch, F f)
+{
+    if (batch <= kFewSequences) return f(std::integral_constant<int, kFewSequences>{});
+    return f(std::integral_constant<int, kMaxBatch>{});
 }
 
 sparrow_status launch_combine(sparrow_ctx* c, const SplitPlan& plan, const SyncArgs& sy, void* out, float* lse, cudaStream_t st)
@@ -1226,31 +1236,31 @@ sparrow_status sparrow_kv_append(sparrow_ctx* c, const void* k_new, const void* 
     if (!aligned16(k_new) || !aligned16(v_new) || !aligned16(k_cache) || !aligned16(v_cache)) return SPARROW_ERR_SHAPE;
     if (!c->ws) return SPARROW_ERR_WORKSPACE;
     const sparrow_layout& L = c->layout;
-    RowMoveArgs a;
-    std::memset(&a, 0, sizeof a);
-    for (int b = 0; b < L.batch; ++b) {
+    for (int b = 0; b < L.batch; ++b)
         if (kv_len[b] < 0 || (int64_t)kv_len[b] + T > L.kv_capacity) return SPARROW_ERR_SHAPE;
-        a.dst_row0[b] = kv_len[b];
-    }
-    a.k_src = static_cast<const __nv_bfloat16*>(k_new);
-    a.v_src = static_cast<const __nv_bfloat16*>(v_new);
-    a.k_dst = static_cast<__nv_bfloat16*>(k_cache);
-    a.v_dst = static_cast<__nv_bfloat16*>(v_cache);
-    a.src_rows = nullptr;
-    a.n_rows = T;
-    a.batch = L.batch;
-    a.n_kv_heads = L.n_kv_heads;
-    a.src_capacity = T;
-    a.src_stride_head = (int64_t)T * kD;
-    a.src_stride_batch = a.src_stride_head * L.n_kv_heads;
-    a.dst_stride_batch = L.kv_stride_batch;
-    a.dst_stride_head = L.kv_stride_head;
-    a.status = reinterpret_cast<unsigned*>(c->ws);
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
-    const long long threads = (long long)L.batch * L.n_kv_heads * T * 16;
     other_kernel_enqueued();
-    return launch_behind(c, move_rows_kernel, (unsigned)((threads + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream), 0, a);
+    return with_room(L.batch, [&](auto room) {
+        RowMoveArgs<room()> a = {};
+        for (int b = 0; b < L.batch; ++b) a.dst_row0[b] = kv_len[b];
+        a.k_src = static_cast<const __nv_bfloat16*>(k_new);
+        a.v_src = static_cast<const __nv_bfloat16*>(v_new);
+        a.k_dst = static_cast<__nv_bfloat16*>(k_cache);
+        a.v_dst = static_cast<__nv_bfloat16*>(v_cache);
+        a.src_rows = nullptr;
+        a.n_rows = T;
+        a.batch = L.batch;
+        a.n_kv_heads = L.n_kv_heads;
+        a.src_capacity = T;
+        a.src_stride_head = (int64_t)T * kD;
+        a.src_stride_batch = a.src_stride_head * L.n_kv_heads;
+        a.dst_stride_batch = L.kv_stride_batch;
+        a.dst_stride_head = L.kv_stride_head;
+        a.status = reinterpret_cast<unsigned*>(c->ws);
+        const long long threads = (long long)L.batch * L.n_kv_heads * T * 16;
+        return launch_behind(c, move_rows_kernel<room()>, (unsigned)((threads + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream), 0, a);
+    });
 }
 
 sparrow_status sparrow_compact_anchors(sparrow_ctx* c, const void* k, const void* v, const int32_t* anchor_idx,
@@ -1263,30 +1273,31 @@ sparrow_status sparrow_compact_anchors(sparrow_ctx* c, const void* k, const void
     if (compact_capacity < 1 || dst_row < 0 || (int64_t)dst_row + n_anchor > compact_capacity) return SPARROW_ERR_SHAPE;
     if (!c->ws) return SPARROW_ERR_WORKSPACE;
     const sparrow_layout& L = c->layout;
-    RowMoveArgs a;
-    std::memset(&a, 0, sizeof a);
-    for (int b = 0; b < L.batch; ++b) a.dst_row0[b] = dst_row;
-    a.k_src = static_cast<const __nv_bfloat16*>(k);
-    a.v_src = static_cast<const __nv_bfloat16*>(v);
-    a.k_dst = static_cast<__nv_bfloat16*>(k_compact);
-    a.v_dst = static_cast<__nv_bfloat16*>(v_compact);
-    a.src_rows = anchor_idx;
-    a.n_rows = n_anchor;
-    a.batch = L.batch;
-    a.n_kv_heads = L.n_kv_heads;
-    a.src_capacity = L.kv_capacity;
-    a.src_stride_batch = L.kv_stride_batch;
-    a.src_stride_head = L.kv_stride_head;
-    a.dst_stride_head = (int64_t)compact_capacity * kD;
-    a.dst_stride_batch = a.dst_stride_head * L.n_kv_heads;
-    a.status = reinterpret_cast<unsigned*>(c->ws);
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     const long long threads = (long long)L.batch * L.n_kv_heads * n_anchor * 16;
     long long blocks = (threads + 255) / 256;
     if (blocks > 8LL * c->n_sm) blocks = 8LL * c->n_sm;
     other_kernel_enqueued();
-    return launch_behind(c, move_rows_kernel, (unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream), 0, a);
+    return with_room(L.batch, [&](auto room) {
+        RowMoveArgs<room()> a = {};
+        for (int b = 0; b < L.batch; ++b) a.dst_row0[b] = dst_row;
+        a.k_src = static_cast<const __nv_bfloat16*>(k);
+        a.v_src = static_cast<const __nv_bfloat16*>(v);
+        a.k_dst = static_cast<__nv_bfloat16*>(k_compact);
+        a.v_dst = static_cast<__nv_bfloat16*>(v_compact);
+        a.src_rows = anchor_idx;
+        a.n_rows = n_anchor;
+        a.batch = L.batch;
+        a.n_kv_heads = L.n_kv_heads;
+        a.src_capacity = L.kv_capacity;
+        a.src_stride_batch = L.kv_stride_batch;
+        a.src_stride_head = L.kv_stride_head;
+        a.dst_stride_head = (int64_t)compact_capacity * kD;
+        a.dst_stride_batch = a.dst_stride_head * L.n_kv_heads;
+        a.status = reinterpret_cast<unsigned*>(c->ws);
+        return launch_behind(c, move_rows_kernel<room()>, (unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream), 0, a);
+    });
 }
 
 sparrow_status sparrow_window_first_visible(const int32_t* anchor_idx, int32_t n_anchor, int32_t window, int32_t T_tree,
@@ -1423,24 +1434,25 @@ sparrow_status sparrow_kv_keep_accepted(sparrow_ctx* c, void* k_cache, void* v_c
     if (T < 1 || T > kMaxT) return SPARROW_ERR_SHAPE;
     if (!aligned16(k_cache) || !aligned16(v_cache)) return SPARROW_ERR_SHAPE;
     const sparrow_layout& L = c->layout;
-    KeepArgs a;
-    std::memset(&a, 0, sizeof a);
-    for (int b = 0; b < L.batch; ++b) {
+    for (int b = 0; b < L.batch; ++b)
         if (kv_len[b] < 0 || (int64_t)kv_len[b] + T > L.kv_capacity) return SPARROW_ERR_SHAPE;
-        a.kv_len[b] = kv_len[b];
-    }
-    a.k = static_cast<__nv_bfloat16*>(k_cache);
-    a.v = static_cast<__nv_bfloat16*>(v_cache);
-    a.path = path;
-    a.n_accept = n_accept;
-    a.T = T;
-    a.n_kv_heads = L.n_kv_heads;
-    a.stride_batch = L.kv_stride_batch;
-    a.stride_head = L.kv_stride_head;
     DeviceGuard guard(c->device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
     other_kernel_enqueued();
-    return launch_behind(c, keep_accepted_rows_kernel, (unsigned)(L.batch * L.n_kv_heads), 256, (size_t)2 * T * 256, static_cast<cudaStream_t>(stream), 0, a);
+    return with_room(L.batch, [&](auto room) {
+        KeepArgs<room()> a = {};
+        for (int b = 0; b < L.batch; ++b) a.kv_len[b] = kv_len[b];
+        a.k = static_cast<__nv_bfloat16*>(k_cache);
+        a.v = static_cast<__nv_bfloat16*>(v_cache);
+        a.path = path;
+        a.n_accept = n_accept;
+        a.T = T;
+        a.n_kv_heads = L.n_kv_heads;
+        a.stride_batch = L.kv_stride_batch;
+        a.stride_head = L.kv_stride_head;
+        return launch_behind(c, keep_accepted_rows_kernel<room()>, (unsigned)(L.batch * L.n_kv_heads), 256, (size_t)2 * T * 256,
+                             static_cast<cudaStream_t>(stream), 0, a);
+    });
 }
 
 sparrow_status sparrow_verify_step_host(sparrow_ctx* c, const void* q_host, const void* k_new_host,
