@@ -142,7 +142,7 @@ class _Calls:
         except ImportError as e:
             raise RuntimeError("the _pycall extension is not built: run `python -m paper_2602_15318_b200.build`") from e
         torch.cuda.current_stream()                       # brings torch's CUDA state up
-        _pycall.set_stream_functions(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        _pycall.set_stream_functions(None, None)          # torch's
         for fn, sig in _SIGNATURES.items():
             setattr(self, fn, _pycall.bind(ctypes.cast(getattr(L, fn), ctypes.c_void_p).value, sig, fn, _chk))
         return self.__dict__[name]

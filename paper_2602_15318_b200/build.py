@@ -1,5 +1,6 @@
 """Builds libsparrow_attn.so (C ABI, sm_100a only; nvcc) and _pycall.so (the Python binding's argument
-marshalling; gcc) in-tree."""
+marshalling; g++) in-tree."""
+import importlib.util
 import os
 import subprocess
 import sys
@@ -10,7 +11,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsparrow_attn.so")
 PYCALL = os.path.join(HERE, "_pycall.so")
-PYCALL_SOURCE = os.path.join(CSRC, "pycall.c")
+PYCALL_SOURCES = [os.path.join(CSRC, "pycall.c"), os.path.join(CSRC, "pycall_torch.cpp")]
 SOURCES = [os.path.join(CSRC, "api.cu")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC"]
@@ -32,9 +33,15 @@ def nvcc() -> str:
 
 
 def build_pycall(force: bool = False) -> str:
-    if force or not os.path.exists(PYCALL) or os.path.getmtime(PYCALL) < os.path.getmtime(PYCALL_SOURCE):
-        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], "-o", PYCALL,
-                        PYCALL_SOURCE], check=True)
+    if force or not os.path.exists(PYCALL) or os.path.getmtime(PYCALL) < max(os.path.getmtime(s) for s in PYCALL_SOURCES):
+        torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
+        torch_lib = os.path.join(torch_dir, "lib")
+        include = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+                   os.path.join(os.path.dirname(os.path.dirname(nvcc())), "include"), sysconfig.get_paths()["include"]]
+        subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-shared", "-fPIC", *["-I" + i for i in include], "-o", PYCALL,
+                        "-x", "c", PYCALL_SOURCES[0], "-x", "c++", PYCALL_SOURCES[1], "-x", "none",
+                        "-L" + torch_lib, "-Wl,-rpath," + torch_lib, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"],
+                       check=True)
     return PYCALL
 
 

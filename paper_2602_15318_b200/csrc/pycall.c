@@ -10,7 +10,7 @@
  *   s  a stream: None (the current one), an object with `cuda_stream`, or an int handle
  * Every argument is an integer or a pointer, i.e. one 64-bit slot of the calling convention.  A non-zero
  * status calls on_error(status, name), which raises.  The interpreter lock is released during the
- * call.  set_stream_functions(get_device, get_raw_stream) says how to ask for the current stream. */
+ * call.  set_stream_functions(get_device, get_raw_stream) says how to ask for the current stream, if not torch. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -26,6 +26,10 @@ typedef struct {
     PyObject* name;
     PyObject* on_error;
 } Bound;
+
+/* pycall_torch.cpp */
+int sparrow_tensor_address(PyObject* o, int64_t* out);
+int sparrow_current_stream(int64_t* out);
 
 static PyObject *s_address, *s_data_ptr, *s_cuda_stream, *g_get_device, *g_get_raw_stream;
 
@@ -61,7 +65,8 @@ static int stolen_slot(PyObject* o, int64_t* out)      /* the same, dropping the
 static int stream_slot(PyObject* o, int64_t* out)
 {
     if (o == Py_None) {
-        if (!g_get_device || !g_get_raw_stream) { PyErr_SetString(PyExc_RuntimeError, "no stream functions set"); return -1; }
+        if (!g_get_device && sparrow_current_stream(out)) return 0;
+        if (!g_get_device || !g_get_raw_stream) { PyErr_SetString(PyExc_RuntimeError, "no current stream"); return -1; }
         PyObject* dev = PyObject_CallNoArgs(g_get_device);
         if (!dev) return -1;
         PyObject* st = PyObject_CallOneArg(g_get_raw_stream, dev);
@@ -107,7 +112,9 @@ static PyObject* bound_call(PyObject* self, PyObject* const* args, Py_ssize_t na
         PyObject* o = args[k];
         switch (b->sig[k]) {
             case 'c': bad = stolen_slot(PyObject_GetAttr(o, s_address), &a[k]); break;
-            case 't': if (o != Py_None) bad = stolen_slot(PyObject_CallMethodNoArgs(o, s_data_ptr), &a[k]); break;
+            case 't':
+                if (o != Py_None && !sparrow_tensor_address(o, &a[k])) bad = stolen_slot(PyObject_CallMethodNoArgs(o, s_data_ptr), &a[k]);
+                break;
             case 'i': bad = as_slot(o, &a[k]); a[k] = (int64_t)(int32_t)a[k]; break;
             case 'L': if (o == Py_None) break; /* fall through */
             case 'l': bad = int_array(o, ints[n_arrays], &heap[n_arrays], &a[k]); ++n_arrays; break;
@@ -161,8 +168,8 @@ static PyObject* py_set_stream_functions(PyObject* self, PyObject* args)
     PyObject *dev, *raw;
     (void)self;
     if (!PyArg_ParseTuple(args, "OO", &dev, &raw)) return NULL;
-    Py_XSETREF(g_get_device, Py_NewRef(dev));
-    Py_XSETREF(g_get_raw_stream, Py_NewRef(raw));
+    Py_XSETREF(g_get_device, dev == Py_None ? NULL : Py_NewRef(dev));
+    Py_XSETREF(g_get_raw_stream, raw == Py_None ? NULL : Py_NewRef(raw));
     Py_RETURN_NONE;
 }
 
