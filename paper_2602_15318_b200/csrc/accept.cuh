@@ -69,12 +69,12 @@ __global__ void __launch_bounds__(256)
 keep_accepted_rows_kernel(const __grid_constant__ KeepArgs<N> a)
 {
     let_dependents_launch();
-    wait_for_predecessors();
     extern __shared__ uint4 rows_sm[];                       // [2][T][16] chunks of 16 bytes
-    const int b = blockIdx.x / a.n_kv_heads, h = blockIdx.x % a.n_kv_heads;
+    const int b = blockIdx.x / a.n_kv_heads, h = blockIdx.x - b * a.n_kv_heads;
+    const size_t base = (size_t)b * a.stride_batch + (size_t)h * a.stride_head + (size_t)a.kv_len[b] * kD;
+    wait_for_predecessors();
     int n = a.n_accept[b];
     n = n < 0 ? 0 : (n > a.T ? a.T : n);
-    const size_t base = (size_t)b * a.stride_batch + (size_t)h * a.stride_head + (size_t)a.kv_len[b] * kD;
     for (int e = threadIdx.x; e < n * 16; e += blockDim.x) {
         const int i = e >> 4, c = e & 15;
         int src = a.path[(size_t)b * a.T + i];

@@ -162,7 +162,6 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
                      int32_t* path, int32_t* n_accept, int32_t* bonus, unsigned* status)
 {
     let_dependents_launch();
-    wait_for_predecessors();
     extern __shared__ uint2 row_s[];                   // the first `resident` entries of this CTA's slice: (P, Q) fixed point
     __shared__ Shared sh;
     const int b = blockIdx.x / n_cta, tid = threadIdx.x;
@@ -185,7 +184,6 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
             fq[k] = i < n_mine ? ld_behind(pq + i) : 0.f;
         }
     };
-    fetch_row(0);
     if (tid == 0) {
         tc::mbar_init(tc::smem_u32(&sh.bar[0]), 1);
         tc::mbar_init(tc::smem_u32(&sh.bar[1]), 1);
@@ -194,6 +192,8 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
     if (tid < 2 * kMaxCluster) sh.part[tid & 1][tid >> 1][0] = sh.part[tid & 1][tid >> 1][1] = 0;
     if (tid <= kMaxT) sh.kids[tid] = 0ull;
     __syncthreads();
+    wait_for_predecessors();                           // (everything above needs nothing of them)
+    fetch_row(0);
     if (tid <= T) sh.u_bonus[tid] = u_bonus[(size_t)b * (T + 1) + tid];
     float node_p = 0.f, node_q = 0.f;                  // the node's token in its parent's rows
     if (tid < T) {

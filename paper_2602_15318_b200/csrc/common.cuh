@@ -201,6 +201,13 @@ __device__ __forceinline__ float ld_behind(const float* p)
     return v;
 }
 
+__device__ __forceinline__ __nv_bfloat16 ld_behind(const __nv_bfloat16* p)
+{
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return __ushort_as_bfloat16(v);
+}
+
 struct Item {
     int b, kvh, group, split, key_begin, key_end;
 };

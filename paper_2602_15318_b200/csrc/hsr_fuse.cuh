@@ -99,10 +99,11 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     SPARROW_TIMELINE_CALL(0);
     if (tid == 0) SPARROW_STAMP(0);                                     // entry
-    const int f_tile = blockIdx.x / args.n_slices, slice = blockIdx.x - f_tile * args.n_slices;
+    const int lg_slices = 31 - __clz(args.n_slices);                    // (a power of two)
+    const int f_tile = (int)blockIdx.x >> lg_slices, slice = blockIdx.x - (f_tile << lg_slices);
     // K tiles of this slice: as even as whole tiles allow
-    const int kt_begin = (int)((long long)args.k_tiles * slice / args.n_slices);
-    const int kt_end = (int)((long long)args.k_tiles * (slice + 1) / args.n_slices);
+    const int kt_begin = (int)(((long long)args.k_tiles * slice) >> lg_slices);
+    const int kt_end = (int)(((long long)args.k_tiles * (slice + 1)) >> lg_slices);
     const int n_kt = kt_end - kt_begin;
     const int n_st = (n_kt + kBoxes - 1) / kBoxes;                      // ring fills of this item (the last may be short)
     const int d_tiles = args.d / kKTile;                                // K tiles that belong to e
@@ -129,8 +130,6 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
         mbar_init(done, 1);
         *abort_flag = 0;
         fence_barrier_init();
-        wait_for_predecessors();
-        for (int i = 0; i < n_st && i < kStages; ++i) issue(i);
     }
     if (warp == 5) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(64u) : "memory");
@@ -145,9 +144,12 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
 
     const int feat_local = (warp & 3) * 32 + lane;
     // n_slices is a power of two: each CTA of the cluster finishes `share` of the 64 token columns
-    const int share = kTok / args.n_slices, lg_share = 31 - __clz(share), row_floats = share + 4;
+    const int share = kTok >> lg_slices, lg_share = 31 - __clz(share), row_floats = share + 4;
+    float b = 0.f;                                                      // epilogue: the feature's bias
     if (warp == 4) {
-        if (lane == 0) {                                                // ---- TMA producer: refill freed stages
+        if (lane == 0) {                                                // ---- TMA producer: fill the ring, refill freed stages
+            wait_for_predecessors();
+            for (int i = 0; i < n_st && i < kStages; ++i) issue(i);
             #pragma unroll 1
             for (int i = kStages; i < n_st; ++i) {
                 if (!mbar_wait(empty(i % kStages), (i / kStages - 1) & 1)) {
@@ -191,13 +193,14 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
         // ---- epilogue warps, part 1: thread = one output feature (TMEM lane), 64 token columns.
         // Everything from here on runs once per CTA, i.e. from a cold instruction cache: the loops
         // are kept rolled (8 token columns per trip) so that few distinct instructions are fetched.
+        wait_for_predecessors();
+        if (args.bias) b = __bfloat162float(ld_behind(args.bias + f_tile * kFeat + feat_local));      // beside the products
         bool ok = n_kt == 0 || mbar_wait_warp(done, 0);
         tc_fence_after();
         if (!ok) { atomicOr(args.status, timeout_bits(kSiteSoftmax)); *abort_flag = 1; }
         const bool have = ok && n_kt > 0;
         if (tid == 0) SPARROW_STAMP(4);                                 // accumulator complete
         if (args.n_slices == 1) {                                       // a single slice writes z itself
-            const float b = args.bias ? __bfloat162float(args.bias[f_tile * kFeat + feat_local]) : 0.f;
             #pragma unroll 1
             for (int c = 0; c < args.M; c += 8) {
                 float v[8];
@@ -230,7 +233,6 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
         if (tid == 0) SPARROW_STAMP(6);                                 // cluster barrier passed
         if (warp < 4) {
             // part 2: the slices in fixed order (results do not depend on timing), bias, bf16 z
-            const float b = args.bias ? __bfloat162float(args.bias[f_tile * kFeat + feat_local]) : 0.f;
             const float* mine = reinterpret_cast<const float*>(recv) + feat_local * row_floats;
             const int t0 = slice * share;
             const int n_mine = min(share, args.M - t0);                 // may be <= 0: nothing to finish
