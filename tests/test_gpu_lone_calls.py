@@ -26,6 +26,9 @@ DEV = "cuda:0"
     (28, 4, [2049 - 40], 40, "random"),     # 17 tiles
     (4, 4, [700], 1, "chain"),              # one row per unit: most CTAs of a cluster finish nothing
     (16, 1, [1500], 64, "random"),          # 16 query heads per KV head, four row groups
+    (8, 8, [1100], 9, "chain"),             # 9 rows in a cluster: one or two for each CTA to merge
+    (28, 4, [26000], 3, "chain"),           # 84 rows through the workspace, one for each finisher
+    (28, 4, [9000], 30, "random"),          # 840 rows, six or fewer for each
     (28, 4, [130, 2000, 700], 12, "random"),  # ragged lengths in clusters of two
     (28, 4, [100] * 40, 20, "random"),      # more units than SMs
 ])
