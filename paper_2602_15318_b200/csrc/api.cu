@@ -1158,7 +1158,6 @@ sparrow_status sparrow_verify_attn_static(const sparrow_layout* L, const void* q
         return SPARROW_ERR_SHAPE;
     if (check_ws(c, plan) != SPARROW_OK) return SPARROW_ERR_WORKSPACE;
     // the status word is the one thing that must start clean
-    // the status word is the one thing that must start clean
     if (cudaMemsetAsync(c->ws, 0, sizeof(unsigned), static_cast<cudaStream_t>(stream)) != cudaSuccess) return SPARROW_ERR_CUDA;
     return sparrow_verify_attn(c, q, k, v, kv_len, parents, T, out, lse, stream);
 }

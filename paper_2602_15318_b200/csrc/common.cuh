@@ -59,7 +59,7 @@ enum WaitSite { kSiteProducer = 0, kSiteMma = 1, kSiteSoftmax = 2, kSiteWriteSam
 //
 // One work item = (sequence b, KV head, row group, key-range piece).  Items of sequence b occupy
 // [seq[b].item_begin, seq[b+1].item_begin); inside, the index runs (kv head, row group, piece) with the
-// piece fastest.  Piece s of n covers keys [n_keys*s/n, n_keys*(s+1)/n).
+// piece fastest.  Pieces are whole tiles, the longer ones first (decode_item).
 struct SeqPlan {                  // per sequence
     int32_t item_begin;           // first work item of the sequence
     int32_t n_splits;             // key-range pieces per unit
@@ -89,7 +89,6 @@ struct SplitPlan {
 };
 
 constexpr int kFinisherCtas = 32;  // CTAs of a call that share its combine step
-constexpr int kMaxGroups = 4;      // row groups per (sequence, KV head): at most 8 blocks (g = 16), 2 per group
 constexpr int kArrivalSlots = 4;   // arrival words rotate over the call number modulo 4
 // A partial row in the workspace: 128 fp16 outputs, then the row's fp32 LSE, padded to 16 bytes,
 // so that one bulk copy brings a run of rows with everything needed to merge them.

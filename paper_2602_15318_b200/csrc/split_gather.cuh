@@ -47,7 +47,7 @@ constexpr int kRows = 128;        // packed query rows per CTA (8 warps x 16)
 constexpr int kTile = 64;         // keys per stage
 constexpr int kStageBytes = kTile * kD * 2;            // one K or V tile: 16 KB
 constexpr int kSmemBytes = 4 * kStageBytes + kMaxT * 8 + kMaxT * 4 + 2 * kTile * 4;
-// with the pieces of a unit in a cluster: the rows the peers send, [piece][row][272 bytes], and the merge's scratch
+// with the pieces of a unit in a cluster: the rows the peers send, [piece][row][272 bytes]
 constexpr int kRecvBytes = (kRows + tc::kMaxMergeCluster) * tc::kRowBytes;
 constexpr int kClusterSmemBytes = (kSmemBytes + 15) / 16 * 16 + kRecvBytes;
 
