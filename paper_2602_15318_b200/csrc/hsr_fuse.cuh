@@ -176,6 +176,7 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             constexpr uint32_t idesc = idesc_bf16(false, kTok);
             bool ok = true;
+            wait_for_predecessors();                                    // (its remaining time is not part of the bounded waits)
             #pragma unroll 1
             for (int i = 0; i < n_st && ok; ++i) {
                 const int st = i % kStages;

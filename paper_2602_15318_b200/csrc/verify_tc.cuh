@@ -675,6 +675,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const uint64_t q_desc0 = smem_desc(smem_u32(q_sm), 16, 1024);
             const uint64_t k_desc0 = smem_desc(smem_u32(kv_sm), 16, 1024);
             const uint64_t v_desc0 = smem_desc(smem_u32(kv_sm) + 2 * kSubTileBytes, kSubTileBytes, 1024);
+            // (a bounded wait must not include what is left of the predecessor's time: kernels that let their
+            // dependents start early may run on for longer than its polls)
+            if (sync.wait_first) wait_for_predecessors();
             bool ok = mbar_wait_warp(B.q_full(), 0);
             if (lane == 0) SPARROW_STAMP(2);                                           // Q landed
             if constexpr (NB == 2) {

@@ -1,0 +1,39 @@
+"""Rules of the kernels' source that no run shows: breaking one costs a result only behind a predecessor that runs
+for seconds, or only where a thread block starts late."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_15318_b200", "csrc")
+
+
+def _code(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def _between(text, start, end):
+    i = text.index(start)
+    return text[i:text.index(end, i)]
+
+
+@pytest.mark.parametrize("name,start,end", [
+    ("verify_tc.cuh", "if (warp == kProducerWarp) {", "else if (warp == kMmaWarp)"),
+    ("verify_tc.cuh", "else if (warp == kMmaWarp) {", "else if (warp == kGateWarp)"),
+    ("verify_tc.cuh", "else if (warp == kGateWarp) {", "else if (warp < 8)"),
+    ("hsr_fuse.cuh", "if (warp == 4) {\n        if (lane == 0) {", "else if (warp == 5)"),
+    ("hsr_fuse.cuh", "else if (warp == 5) {", "} else {"),
+    ("hsr_fuse.cuh", "bool ok = n_kt == 0", None),
+])
+def test_no_bounded_wait_in_front_of_the_wait_for_the_predecessor(name, start, end):
+    """A wait that gives up after a number of polls must not start while the predecessor may still run: a kernel
+    that lets its dependents start early may take longer than those polls."""
+    code = _code(name)
+    if end is None:                                     # the projection's epilogue warps: the wait stands just before
+        i = code.index(start)
+        assert "wait_for_predecessors()" in code[i - 300:i]
+        return
+    part = _between(code, start, end)
+    first = re.search(r"\b(mbar_wait|mbar_wait_warp|mbar_try_wait|wait_counter|ld_acquire)\(", part)
+    assert first and 0 <= part.find("wait_for_predecessors()") < first.start()
