@@ -94,7 +94,10 @@ sparrow_status sparrow_destroy(sparrow_ctx* ctx);
  * Results differ between policies only by the rounding order of the split-KV merge.  Calls that
  * share the GPU with no other call of the context (single calls without sparrow_set_call_overlap(), graph
  * capture, SPARROW_NO_PDL, sparrow_anchor_attn, sparrow_verify_attn_static) always use one wave
- * over all SMs. */
+ * over all SMs.  They do not need that wave to be resident as a whole: kernels of other streams and
+ * contexts may hold SMs at the same time.  Calls that may overlap (batches, the opt-in) do need SMs for
+ * the CTAs that merge them -- the last 32, under LATENCY all of them -- at one time: keep calls
+ * of several contexts that overlap under LATENCY from running concurrently. */
 typedef enum {
     SPARROW_PLAN_LATENCY    = 0,
     SPARROW_PLAN_BALANCED   = 1,

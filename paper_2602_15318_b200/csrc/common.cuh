@@ -89,7 +89,12 @@ struct SplitPlan {
 };
 
 constexpr int kFinisherCtas = 32;  // CTAs of a call that share its combine step
-constexpr int kArrivalSlots = 4;   // arrival words rotate over the call number modulo 4
+// An arrival word counts arrivals in its lower half and, in a lone call, finishers that have left above; the top bit is
+// taken by the CTA that merges for them.
+constexpr uint32_t kArrivedMask = 0xFFFFu, kOneLeft = 0x10000u, kAdopted = 0x80000000u;
+// Polls after which a finisher of a lone call leaves its rows to the last CTA to arrive, some 200 us: the CTAs of one
+// wave end within a few microseconds of one another, unless kernels of other streams hold SMs that some have yet to start on.
+constexpr uint32_t kPatiencePolls = 256;
 // A partial row in the workspace: 128 fp16 outputs, then the row's fp32 LSE, padded to 16 bytes,
 // so that one bulk copy brings a run of rows with everything needed to merge them.
 constexpr int kPartRowHalves = 136;
@@ -117,6 +122,12 @@ constexpr int kPartRowHalves = 136;
 // results land in call order.  CTA 0 then clears the arrival word of slot (n + 2) % 4: its last
 // user was call n-2, and the items of call n+2 cannot arrive before the finishers of call n are
 // done, which in turn have seen CTA 0's arrival (or, if it had none, follow it in the stream).
+// In a lone call every CTA is a finisher, and the grid may fill the GPU: waiting for all of it would need all of
+// it resident at once, and two such calls of different contexts, each holding the SMs that the other's last CTAs
+// need, would wait for each other.  There nobody waits without end: a finisher that has polled kPatiencePolls
+// times adds kOneLeft to the arrival word and leaves.  The first CTA that finds all arrivals counted and somebody gone
+// merges the rows of every finisher; there always is one, the last CTA to arrive, if no other.  It goes share by share, so
+// that the results are the same bits (a finisher that has not left writes the same values into its own share).
 // With enabled == 0 the kernels are ordered by the stream alone: they touch no counter, and a
 // separate combine kernel follows the split-KV kernel.
 struct SyncArgs {
@@ -163,6 +174,13 @@ __device__ __forceinline__ bool wait_equal(const unsigned* addr, uint32_t value)
         __nanosleep(i < 64 ? 40 : 200);
     }
     return false;
+}
+// Increment of a counter that also returns what it was; orders as publish_counter() and ld_acquire() do.
+__device__ __forceinline__ unsigned add_acquire_release(unsigned* addr, unsigned n)
+{
+    unsigned v;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(v) : "l"(addr), "r"(n) : "memory");
+    return v;
 }
 // Release-increment of a counter: orders every write this thread has observed (its own and, after
 // a CTA barrier, its CTA's) before the increment.

@@ -1144,23 +1144,22 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const int seq_rows = plan.n_kv_heads * qg * T;                  // query rows of a sequence
         // The call's row list: the query rows of every sequence with several pieces, (KV head, row group,
         // row) in order.  Finisher f takes rows [f chunk, (f + 1) chunk).
-        int my_begin = 0, my_end = 0;
-        if (sync.enabled && fin_idx >= 0) {
-            int total = 0;
+        int total = 0, chunk = 0;
+        if (sync.enabled && fin_idx >= 0) {                             // (in a lone call every CTA is one)
             for (int b = 0; b < plan.batch; ++b)
                 if (plan.seq[b].n_splits > 1) total += seq_rows;
-            const int chunk = (total + sync.n_fin - 1) / sync.n_fin;
-            my_begin = min(total, fin_idx * chunk);
-            my_end = min(total, my_begin + chunk);
+            chunk = (total + sync.n_fin - 1) / sync.n_fin;
         }
-        const bool merges = my_begin < my_end;
+        const int my_begin = fin_idx >= 0 ? min(total, fin_idx * chunk) : 0;
+        int share_end = fin_idx >= 0 ? min(total, my_begin + chunk) : 0;       // end of the share being merged
+        const bool merges = my_begin < share_end;
         MergeList* list = reinterpret_cast<MergeList*>(anc_s);          // (the tables are no longer needed)
         // Fills the list with what one pass merges, from row `row` on: runs of rows of one unit, as many as
         // fit the K/V ring with all their pieces.
         auto list_rows = [&](int row) {
             int n_seg = 0, bytes = 0;
             #pragma unroll 1
-            while (row < my_end && n_seg < kMaxSegments) {
+            while (row < share_end && n_seg < kMaxSegments) {
                 MergeSegment sg;
                 int rest = row;
                 sg.b = 0;
@@ -1176,7 +1175,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 sg.tok0 = grp * NB * tpb;
                 sg.head0 = kvh * qg;
                 const int unit_left = qg * min(NB * tpb, T - sg.tok0) - sg.r0;
-                sg.n = min(min(unit_left, my_end - row), (NS * kStageBytes - bytes) / (sg.ns * kRowBytes));
+                sg.n = min(min(unit_left, share_end - row), (NS * kStageBytes - bytes) / (sg.ns * kRowBytes));
                 if (sg.n == 0) break;
                 // the run may straddle the unit's two blocks: `split` rows in the first of them
                 const int bk0 = sg.r0 / rows_per_block;
@@ -1235,34 +1234,51 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         if (sync.enabled) {
             unsigned* arrive_word = sync.arrivals + sync.slot;
             if (tid == 0) SPARROW_STAMP(7);                            // partial rows stored
-            if (tid == 0 && !direct && !clustered) publish_counter(arrive_word);
-            if (merges) {
+            const bool arrives = !direct && !clustered;
+            if (tid == 0 && arrives) publish_counter(arrive_word);
+            if (merges || (sync.lone && arrives)) {
                 if (tid == 0) {
                     // every partial of the call in place, and the previous call's final results written
                     // (both words are polled in one loop: the second is usually there already, and a lone
                     // call's predecessors have ended as grids)
                     bool have_all = false, prev_done = sync.lone != 0;
+                    uint32_t word = 0;
+                    const uint32_t polls = !merges ? 1u : sync.lone ? kPatiencePolls : kCounterPolls;
                     #pragma unroll 1
-                    for (uint32_t i = 0; i < kCounterPolls && !(have_all && prev_done); ++i) {
-                        if (!have_all) have_all = ld_acquire(arrive_word) == (unsigned)sync.n_arrive;
+                    for (uint32_t i = 0; i < polls && !(have_all && prev_done); ++i) {
+                        if (!have_all) {
+                            word = ld_acquire(arrive_word);
+                            have_all = (word & kArrivedMask) == (unsigned)sync.n_arrive;
+                        }
                         if (!prev_done) prev_done = (int32_t)(ld_acquire(sync.fin_done + (sync.parity ^ 1)) - sync.fin_wait_other) >= 0;
                         if (!(have_all && prev_done)) __nanosleep(i < 256 ? 20 : 200);
                     }
                     SPARROW_STAMP(8);                                   // all arrivals seen
-                    if (!have_all) atomicOr(args.status, timeout_bits(kSiteArrivals));
-                    else if (!prev_done) atomicOr(args.status, timeout_bits(kSiteFinOther));
+                    bool adopts = false;
+                    if (sync.lone) {
+                        // (one that would leave but finds all arrivals counted stays: nobody needs to have noticed it)
+                        if (merges && !have_all) have_all = (add_acquire_release(arrive_word, kOneLeft) & kArrivedMask) == (unsigned)sync.n_arrive;
+                        else if (have_all && word >= kOneLeft) adopts = (atomicOr(arrive_word, kAdopted) & kAdopted) == 0u;
+                    } else if (!have_all) {
+                        atomicOr(args.status, timeout_bits(kSiteArrivals));
+                    } else if (!prev_done) {
+                        atomicOr(args.status, timeout_bits(kSiteFinOther));
+                    }
                     SPARROW_STAMP(9);                                   // previous call's finishers seen
-                    *fin_go = (have_all && prev_done) ? 1 : 0;
+                    *fin_go = !(have_all && prev_done) ? 0 : adopts ? 2 : merges ? 1 : 0;
                 }
                 // The rows' pieces are first brought into the (idle) K/V ring by bulk copies, [piece][row]
                 // [272 bytes], one copy per piece and block touched -- far fewer and larger requests than
                 // per-thread loads (16-byte words that carry a tag, read by the threads as they arrive and without
                 // any counter, were there 1.6 us earlier but took 2 us longer to collect).
+                int adopted = 0;                                           // (thread 0) next finisher whose share is taken over
+                if (tid == 0 && !merges) list->n_seg = list->bytes = list->next_row = 0;
                 #pragma unroll 1
                 for (int phase = 0;; phase ^= 1) {
                     if (tid == 0 && *fin_go) mbar_expect_tx(B.fin(), (uint32_t)list->bytes);
                     softmax_bar_sync();                                    // the list and the byte count are posted
-                    if (!*fin_go) break;
+                    const int go = *fin_go;
+                    if (!go) break;
                     const int n_seg = list->n_seg;
                     #pragma unroll 1
                     for (int k = 0; k < n_seg; ++k) {
@@ -1289,9 +1305,18 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                         merge_run(tid, smem_u32(kv_sm) + (uint32_t)sg.offset, sg.ns, sg.n, sg.r0, sg.b, sg.tok0, sg.head0, landed, merge_out);
                     }
                     const int next = list->next_row;
-                    if (!landed || next >= my_end) break;
+                    if (!landed || (next >= share_end && go == 1)) break;
                     softmax_bar_sync();                                    // everybody is through with the ring and the list
-                    if (tid == 0) list_rows(next);
+                    if (tid == 0) {
+                        int row = next;
+                        while (row >= share_end && adopted < sync.n_fin) { // (only where go is 2)
+                            row = adopted == fin_idx ? total : min(total, adopted * chunk);
+                            share_end = min(total, row + chunk);
+                            ++adopted;
+                        }
+                        if (row < share_end) list_rows(row);
+                        else *fin_go = 0;
+                    }
                 }
                 if (tid == 0) SPARROW_STAMP(10);                        // merged rows written
                 softmax_bar_sync();
