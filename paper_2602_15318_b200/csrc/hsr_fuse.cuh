@@ -13,7 +13,7 @@
 // operands staged by TMA through a 6-stage mbarrier ring (16 KB of weights + 8 KB of activations per
 // stage), accumulator in TMEM.  The slices of one feature tile form a thread-block cluster (2, 4 or
 // 8 CTAs).  The CTA of rank r finishes tokens [r 64/n, (r + 1) 64/n): every CTA pushes its fp32
-// partial sums for those tokens into that CTA's shared memory, and after one cluster barrier each
+// partial sums for those tokens into that CTA's shared memory, and after a cluster barrier each
 // CTA adds the slices in fixed order (deterministic), adds the bias and writes z (bf16).  Nothing
 // goes through global scratch and no counter is needed.  Every mbarrier wait is bounded; a CTA
 // whose wait ran out still takes part in the cluster barrier.
@@ -152,6 +152,7 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (args.n_slices > 1) cluster_arrive_relaxed();                    // (waited for ahead of the first push: the peer must run)
     let_dependents_launch();
     if (tid == 0) SPARROW_STAMP(1);                                     // set-up done
 
@@ -228,6 +229,7 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
             // for them are pushed into that CTA's receive buffer, laid out [slice][feature][token in
             // share] with padded rows.  Remote stores are not waited for.  Columns past M hold
             // zeros (TMA fills the token rows past M with zeros), so whole chunks are pushed.
+            cluster_wait();
             const uint32_t row0 = smem_u32(recv) + (uint32_t)((slice * kFeat + feat_local) * row_floats) * 4u;
             #pragma unroll 1
             for (int c = 0; c < args.M; c += 8) {
@@ -240,7 +242,8 @@ hsr_fuse_kernel(const __grid_constant__ HsrArgs args, const __grid_constant__ CU
         }
     }
     if (args.n_slices > 1) {
-        // one cluster barrier: every slice's pushes have landed; after it nobody touches a peer
+        // second cluster barrier: every slice's pushes have landed; after it nobody touches a peer
+        if (warp >= 4) cluster_wait();                                  // (the first one)
         if (tid == 0) SPARROW_STAMP(5);                                 // partial sums pushed
         cluster_arrive();
         cluster_wait();

@@ -37,3 +37,17 @@ def test_no_bounded_wait_in_front_of_the_wait_for_the_predecessor(name, start, e
     part = _between(code, start, end)
     first = re.search(r"\b(mbar_wait|mbar_wait_warp|mbar_try_wait|wait_counter|ld_acquire)\(", part)
     assert first and 0 <= part.find("wait_for_predecessors()") < first.start()
+
+
+@pytest.mark.parametrize("name,start", [
+    ("verify_tc.cuh", "if (clustered) {\n"),
+    ("split_gather.cuh", "if (clustered) {\n"),
+    ("hsr_fuse.cuh", "if (args.n_slices == 1) {"),
+    ("accept_sample.cuh", "accept_sample_kernel(const int32_t*"),
+])
+def test_a_cluster_meets_before_its_first_push(name, start):
+    """Shared memory of another CTA of the cluster may only be written once that CTA is known to run."""
+    code = _code(name)
+    body = code[code.index(start):]
+    push = re.search(r"\b(bulk_push|st_cluster_v4|cluster_sum)\(", body).start()
+    assert 0 <= body.find("cluster_wait()") < push
