@@ -14,6 +14,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <thread>
 #include <type_traits>
 
 #include "combine.cuh"
@@ -654,7 +655,8 @@ const ClusterTable* cluster_table(int device)
         query_max_clusters(gather::split_gather_kernel, gather::kThreads, gather::kClusterSmemBytes, t.n[2]);
         t.state.store(2);
     }
-    return t.state.load() == 2 ? &t : nullptr;      // (a thread that comes while another one asks does without)
+    while (t.state.load() != 2) std::this_thread::yield();      // another thread is asking
+    return &t;
 }
 
 struct DeviceGuard {

@@ -1,5 +1,8 @@
 """Lone verification calls whose one wave over all SMs cannot be resident at once, because calls of other contexts on
 other streams hold SMs: the results are the bits of undisturbed calls and no wait gives up."""
+import os
+import subprocess
+import sys
 import time
 
 import pytest
@@ -12,6 +15,7 @@ from gpu_util import check, oracle_verify, sample_rows
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _new(case):
@@ -64,3 +68,48 @@ def test_two_contexts_with_one_wave_each_beside_a_long_call(kv_a, T_a, kv_b, T_b
     for c in (ctx, ctx_a, ctx_b):
         assert c.last_device_status() == 0
     assert worst < 0.2, f"{worst:.3f} s"
+
+
+def test_contexts_created_at_once_by_several_threads_are_alike():
+    """The first contexts of a process, created by sixteen threads at the same time: none may do without what another
+    one is still asking the device for.  All of them plan a call alike, with merges in clusters."""
+    code = """
+import ctypes, sys, threading
+import torch
+from paper_2602_15318_b200 import binding as B
+from paper_2602_15318_b200 import workloads as W
+case = W.make_verify_case(8300, [1500], 16, "random", "cuda:0")
+torch.cuda.synchronize()
+L, n = B.lib(), 16
+create, gate, made = L.sparrow_create, threading.Barrier(n), []
+layout = B.Layout(1, W.HQ, W.HKV, W.D, case.k.shape[2], W.SCALE, W.HKV * case.k.shape[2] * W.D, case.k.shape[2] * W.D)
+handles = [ctypes.c_void_p() for _ in range(n)]
+def make(i):
+    h, l = ctypes.byref(handles[i]), ctypes.byref(layout)
+    gate.wait()
+    made.append(create(h, l, 0))
+sys.setswitchinterval(1e-6)
+threads = [threading.Thread(target=make, args=(i,)) for i in range(n)]
+[t.start() for t in threads]
+[t.join() for t in threads]
+assert made == [0] * n
+ctx = []
+for h in handles:
+    c = B.Context(1, case.k.shape[2], layout.kv_stride_batch, layout.kv_stride_head, W.SCALE, allocate_workspace=False)
+    L.sparrow_destroy(c.handle)
+    c.handle, c.address = h, h.value
+    size = c.workspace_bytes(16)
+    c.workspace = torch.empty(size + 256, dtype=torch.uint8, device="cuda:0")
+    c.set_workspace((c.workspace.data_ptr() + 255) // 256 * 256, size)
+    ctx.append(c)
+for c in ctx:
+    out = torch.empty_like(case.q)
+    lse = torch.empty((1, W.HQ, 16), dtype=torch.float32, device="cuda:0")
+    B.sparrow_verify_attn(c, case.q, case.k, case.v, case.kv_len, case.parents, 16, out, lse)
+torch.cuda.synchronize()
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env={**os.environ, "SPARROW_LOG": "1", "PYTHONPATH": ROOT},
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    plans = [line.split(";", 1)[1] for line in r.stderr.splitlines() if line.startswith("[sparrow] verify call")]
+    assert len(plans) == 16 and len(set(plans)) == 1 and "merged in clusters of" in plans[0], plans
