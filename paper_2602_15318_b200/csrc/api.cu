@@ -844,7 +844,7 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     // launches: the split-KV pass and the combine kernel.
     const CallRanges cr = call_ranges(c, q, k, v, parents, T_tree, T, first_visible, out, lse);
     const bool protocol = call_overlaps(c, st, true);                // not capturing, programmatic launch on
-    const bool same_ctx_before = g_last_fused_ctx.exchange(c) == c;
+    const bool same_ctx_before = g_last_fused_ctx.exchange(nullptr) == c;      // (nobody's, until this call is in the stream)
     const bool early = protocol && same_ctx_before && !c->prev_lone && (c->chain_next || c->overlap_single_calls) &&
                        !inputs_touch_recent_outputs(c, cr);
     // Can another call of this context run beside this one?  Only inside a batch, or with the opt-in for
@@ -878,6 +878,7 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
         c->prev_valid = true;
         c->prev_lone = sy.lone != 0;
         note_fused_launch(c, cr, early);
+        g_last_fused_ctx.store(c);
         return SPARROW_OK;                                   // the kernel merges its own partials
     }
     bool needs_combine = false;
