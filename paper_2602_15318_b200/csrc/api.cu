@@ -682,8 +682,10 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
 // Estimates for the choice of a plan, us: a tile of 128 keys with one / two row blocks, the merges of a lone
 // call, and what an item of a call in a batch costs besides its tiles.
 constexpr float kTileUs[2] = {1.2f, 2.0f};
-constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 4.f;
-constexpr float kItemUs[2] = {5.f, 11.f};
+constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 4.f, kTwoBlocksWholeUs = 1.f;
+constexpr float kItemUs[2] = {5.f, 11.f}, kWholeItemUs[2] = {7.f, 8.5f};      // its rows are merged; it is its unit's only piece
+constexpr float kBatchTileUs[2] = {1.1f, 2.0f};
+constexpr float kWaveUs[2] = {6.f, 8.f};                                       // a further wave of a call with more units than SMs
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
 // at most 16 pieces per unit, pieces short enough to leave a stage of the K/V ring free for the rows that are
@@ -730,9 +732,27 @@ float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
 // What a call in a batch takes of the GPU, in SM microseconds.
 float batch_cost(const SplitPlan& p)
 {
+    const int nb = p.blocks_per_group - 1, units = p.n_kv_heads * p.n_groups;      // (of one sequence)
+    float cost = 0.f;
+    for (int b = 0; b < p.batch; ++b) {
+        const int tiles = (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile, ns = p.seq[b].n_splits;
+        cost += (float)units * ((float)ns * (ns > 1 ? kItemUs[nb] : kWholeItemUs[nb]) + kBatchTileUs[nb] * (float)tiles);
+    }
+    return cost;
+}
+
+// What a lone call pays for its item form: the heavier prologue and merge of two row blocks, and the waves after
+// the first where the units alone are more than the SMs.
+float lone_cost_of_items(const sparrow_ctx* c, const SplitPlan& p)
+{
+    const int nb = p.blocks_per_group - 1;
+    const bool whole = p.n_items == p.batch * p.n_kv_heads * p.n_groups;
+    const float own = nb == 0 ? 0.f : whole ? kTwoBlocksWholeUs : kTwoBlocksUs;
+    if (p.n_items <= c->n_sm) return own;
     long long tiles = 0;
     for (int b = 0; b < p.batch; ++b) tiles += (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile;
-    return kItemUs[p.blocks_per_group - 1] * p.n_items + kTileUs[p.blocks_per_group - 1] * (float)(tiles * p.n_kv_heads * p.n_groups);
+    const int more_waves = (p.n_items + c->n_sm - 1) / c->n_sm - 1;
+    return own + (float)more_waves * (kWaveUs[nb] + kTileUs[nb] * (float)tiles / (float)p.batch);
 }
 
 // The split of a verification call, and whether its items take one row block or two.
@@ -749,11 +769,11 @@ float batch_cost(const SplitPlan& p)
 // A draft block of more than one row block: an item with two of them reads its keys once for both and keeps the
 // tensor pipe fuller on long pieces (2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
 // and merge, no empty half where the blocks are odd in number, and twice as many of them fill the chip.
-// Lone calls, two blocks -> one: 448 keys, T = 40 11.1 -> 7.9 us; 2,048 keys, T = 24 12.6 -> 9.1; 16,384 keys, T = 64
-// 28.1 -> 26.7; 26,112 keys, T = 24 25.9 -> 24.5, T = 60 35.1 -> 34.4; 32,000 keys, T = 36 27.1 -> 25.1; but eight
-// sequences of 9,000, T = 30 48.4 -> 49.5 and two of 30,000, T = 60 71 -> 83 (stay with two).  In a batch: 5,000 keys x 4,
-// T = 50, 12 layers 240 -> 181; 2,000 keys, T = 20, 28 layers 152 -> 128; 10,000 keys, T = 40, latency policy 343 ->
-// 288; 30,000 keys, T = 30, throughput policy, 20 layers 335 -> 411 and eight of 32,768, T = 32 2,860 -> 3,240 (two).
+// Where units are whole an item of two blocks costs less than two items of one, the more so the shorter the
+// sequences (24 sequences of 100 keys, T = 20: 96 items 6.1 us a call in a batch, 192 items 9.8), unless the blocks are odd in
+// number and the sequences longer (16 of 1,600, T = 40: 30.7 and 26.1); a lone call takes one block as long as that
+// gives no further wave (16 of 100, T = 20: 6.8 and 7.8; 24 of 100: 13.1 and 8.3).  Where pieces are merged: 2,048 keys, T = 24
+// alone 12.6 us with two blocks, 9.1 with one; 30,000 keys, T = 30, throughput policy, 20 layers 335 and 411.
 constexpr int kMaxPieceTiles = 48;
 sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluster, int group, const int32_t* n_keys, int T,
                            const int32_t* key0, SplitPlan* plan)
@@ -777,7 +797,8 @@ sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluste
             if (s != SPARROW_OK) return s;
             cost = batch_cost(p);
         } else {
-            cost = plan_lone_call(c, may_cluster, &p) + (nb - 1) * kTwoBlocksUs;
+            cost = plan_lone_call(c, may_cluster, &p);
+            cost += lone_cost_of_items(c, p);
         }
         if (nb == 1 || cost < best) { *plan = p; best = cost; }
     }
