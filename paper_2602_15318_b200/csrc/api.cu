@@ -757,14 +757,14 @@ float lone_cost_of_items(const sparrow_ctx* c, const SplitPlan& p)
 
 // The split of a verification call, and whether its items take one row block or two.
 //
-// Calls that may share the GPU get the policy's item count; where that leaves pieces of more than
-// kMaxPieceTiles they are cut further, up to one item for every second SM: a piece that long is the last
-// thing running while other SMs have nothing left.  Calls of one batch, throughput policy, longest piece as
-// the item count gave it -> cut: four sequences of 30,000 keys, T = 36, 10 layers 838 -> 517 us; four of 20,000,
-// T = 10, 20 layers 525 -> 459; 20,000 keys, 8 KV heads, T = 50, 12 layers 338 -> 276; two of 8,000, 8 KV heads,
-// T = 20 157 -> 139; eight of 32,768, T = 32, 28 layers 3,025 -> 2,860, where one item per SM gave 3,055.  At 28
-// tiles the merges cost: 26,112 keys, T = 16, 28 layers 275 -> 287.  Neither rule looks at the other calls of a
-// batch: a call's bits do not depend on them.
+// Calls that may share the GPU get the policy's item count; pieces of more than kMaxPieceTiles are cut further, up to
+// one item for every second SM, where the policy cuts units anyway or the sequences are uneven: such a piece is
+// the last thing running while other SMs have nothing left.  Sequences of about one length that are whole pieces stay whole:
+// the merge that a cut brings costs a stream of calls more than the tail it shortens.  Calls of a batch, throughput policy:
+// 8 of the 28-layer calls of eight ragged sequences up to 32,768 keys, T = 32 166 -> 115 us a call; 28 calls of eight
+// sequences of 8,000, T = 16 whole 22, cut 28; of four of 9,000, 8 KV heads, T = 20 24, cut 34 (balanced).  64: pieces
+// of 52 tiles that the policy has already made cost 9 % cut again (four of 21,000, T = 16, balanced), of 85 nothing.
+// Neither rule looks at the other calls of a batch: a call's bits do not depend on them.
 //
 // A draft block of more than one row block: an item with two of them reads its keys once for both and keeps the
 // tensor pipe fuller on long pieces (2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
@@ -774,7 +774,7 @@ float lone_cost_of_items(const sparrow_ctx* c, const SplitPlan& p)
 // number and the sequences longer (16 of 1,600, T = 40: 30.7 and 26.1); a lone call takes one block as long as that
 // gives no further wave (16 of 100, T = 20: 6.8 and 7.8; 24 of 100: 13.1 and 8.3).  Where pieces are merged: 2,048 keys, T = 24
 // alone 12.6 us with two blocks, 9.1 with one; 30,000 keys, T = 30, throughput policy, 20 layers 335 and 411.
-constexpr int kMaxPieceTiles = 48;
+constexpr int kMaxPieceTiles = 64;
 sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluster, int group, const int32_t* n_keys, int T,
                            const int32_t* key0, SplitPlan* plan)
 {
@@ -786,12 +786,16 @@ sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluste
         if (s != SPARROW_OK) return s;
         float cost;
         if (may_share) {
-            int longest = 0;
+            int longest = 0, most = 0, units = p.batch * p.n_kv_heads * p.n_groups;
+            long long all = 0;
             for (int b = 0; b < p.batch; ++b) {
                 const int tiles = (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile;
                 longest = std::max(longest, (tiles + p.seq[b].n_splits - 1) / p.seq[b].n_splits);
+                most = std::max(most, tiles);
+                all += tiles;
             }
-            if (longest > kMaxPieceTiles)
+            const bool even = 4 * all > 3ll * most * p.batch;
+            if (longest > kMaxPieceTiles && !(p.n_items == units && even))
                 s = make_plan(std::max(c->n_sm / 2, plan_target(c, true)), L.batch, L.n_kv_heads, group, n_keys, T, nb, &p,
                               kMaxPieceTiles * kKeyTile, key0);
             if (s != SPARROW_OK) return s;

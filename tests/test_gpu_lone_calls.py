@@ -85,8 +85,8 @@ def test_anchored_pieces(n_text, T, batch):
 
 
 @pytest.mark.parametrize("hq,hkv,kv_len,T", [
-    (32, 8, [48 * 128 - 12] * 3, 12),       # pieces of 48 tiles: as long as a call in a batch leaves them
-    (32, 8, [48 * 128 - 11, 300, 6000], 12),  # one key more: two pieces, the second of one tile
+    (32, 8, [48 * 128 - 12] * 3, 12),       # one piece of 48 tiles a unit
+    (32, 8, [48 * 128 - 11, 300, 6000], 12),  # ragged lengths, 49 tiles the longest
     (28, 4, [2000], 19),                    # two row blocks in items of one
     (28, 4, [30000], 36),                   # two row blocks in items of two
     (28, 4, [10000], 37),                   # three

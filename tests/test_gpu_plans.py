@@ -46,3 +46,16 @@ def _plan(capfd, monkeypatch, hq, hkv, kv_len, T, route, policy):
 def test_row_blocks_per_item(hq, hkv, kv_len, T, route, per_item, items, capfd, monkeypatch):
     got = _plan(capfd, monkeypatch, hq, hkv, kv_len, T, route, B.PLAN_BALANCED)
     assert got[:2] == (per_item, items)
+
+
+@pytest.mark.parametrize("hq,hkv,kv_len,T,policy,pieces", [
+    (28, 4, [9000] * 8, 16, B.PLAN_THROUGHPUT, [1] * 8),                  # whole, of one length: stay whole
+    (32, 8, [9000, 8000, 8500], 20, B.PLAN_THROUGHPUT, [1] * 3),          # nearly of one length
+    (32, 8, [64 * 128 - 20, 900, 800], 20, B.PLAN_THROUGHPUT, [1] * 3),   # uneven, pieces of 64 tiles
+    (32, 8, [64 * 128 - 19, 900, 800], 20, B.PLAN_THROUGHPUT, [2, 1, 1]),  # one key more
+    (28, 4, [30000], 16, B.PLAN_THROUGHPUT, [5]),                         # 47 tiles a piece as the policy makes them
+    (28, 4, [41000], 16, B.PLAN_THROUGHPUT, [6]),                         # 65 tiles: cut again
+])
+def test_long_pieces_of_a_batch(hq, hkv, kv_len, T, policy, pieces, capfd, monkeypatch):
+    got = _plan(capfd, monkeypatch, hq, hkv, kv_len, T, "batch", policy)
+    assert got[2] == pieces
