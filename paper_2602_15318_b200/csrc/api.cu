@@ -683,8 +683,7 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
 // call, and what an item of a call in a batch costs besides its tiles.
 constexpr float kTileUs[2] = {1.2f, 2.0f};
 constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 4.f, kTwoBlocksWholeUs = 1.f;
-constexpr float kItemUs[2] = {5.f, 11.f}, kWholeItemUs[2] = {7.f, 8.5f};      // its rows are merged; it is its unit's only piece
-constexpr float kBatchTileUs[2] = {1.1f, 2.0f};
+constexpr float kItemUs[2] = {5.f, 11.f}, kWholeItemUs[2] = {6.5f, 8.5f};      // its rows are merged; it is its unit's only piece
 constexpr float kWaveUs[2] = {6.f, 8.f};                                       // a further wave of a call with more units than SMs
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
@@ -736,7 +735,7 @@ float batch_cost(const SplitPlan& p)
     float cost = 0.f;
     for (int b = 0; b < p.batch; ++b) {
         const int tiles = (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile, ns = p.seq[b].n_splits;
-        cost += (float)units * ((float)ns * (ns > 1 ? kItemUs[nb] : kWholeItemUs[nb]) + kBatchTileUs[nb] * (float)tiles);
+        cost += (float)units * ((float)ns * (ns > 1 ? kItemUs[nb] : kWholeItemUs[nb]) + kTileUs[nb] * (float)tiles);
     }
     return cost;
 }
@@ -757,14 +756,14 @@ float lone_cost_of_items(const sparrow_ctx* c, const SplitPlan& p)
 
 // The split of a verification call, and whether its items take one row block or two.
 //
-// Calls that may share the GPU get the policy's item count; pieces of more than kMaxPieceTiles are cut further, up to
-// one item for every second SM, where the policy cuts units anyway or the sequences are uneven: such a piece is
-// the last thing running while other SMs have nothing left.  Sequences of about one length that are whole pieces stay whole:
-// the merge that a cut brings costs a stream of calls more than the tail it shortens.  Calls of a batch, throughput policy:
-// 8 of the 28-layer calls of eight ragged sequences up to 32,768 keys, T = 32 166 -> 115 us a call; 28 calls of eight
-// sequences of 8,000, T = 16 whole 22, cut 28; of four of 9,000, 8 KV heads, T = 20 24, cut 34 (balanced).  64: pieces
-// of 52 tiles that the policy has already made cost 9 % cut again (four of 21,000, T = 16, balanced), of 85 nothing.
-// Neither rule looks at the other calls of a batch: a call's bits do not depend on them.
+// Calls that may share the GPU get the policy's item count; pieces of more than kMaxPieceTiles are cut further: such a
+// piece is the last thing running while other SMs have nothing left.  Up to one item for every fifth SM, for uneven sequences
+// with two row blocks up to one for every second: the merge that a cut brings costs a stream of calls more than the
+// tail it shortens once many units are whole pieces, and with one row block the stream is bound by memory besides.
+// 28 calls, throughput policy: eight sequences of 8,000 keys, T = 16 whole 24.5 us a call, cut in two 28.4; of four of 9,000, 8 KV
+// heads, T = 20 (balanced) 24 and 34; 9,000 keys, T = 50 whole 12.1, 24 pieces 9.1; two of 13,000, T = 20 in 16 pieces 18.2,
+// in 24 15.2; 8 calls of eight ragged sequences up to 32,768, T = 32 whole 166, cut 115.  Neither rule looks at the other
+// calls of a batch: a call's bits do not depend on them.
 //
 // A draft block of more than one row block: an item with two of them reads its keys once for both and keeps the
 // tensor pipe fuller on long pieces (2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
@@ -774,7 +773,7 @@ float lone_cost_of_items(const sparrow_ctx* c, const SplitPlan& p)
 // number and the sequences longer (16 of 1,600, T = 40: 30.7 and 26.1); a lone call takes one block as long as that
 // gives no further wave (16 of 100, T = 20: 6.8 and 7.8; 24 of 100: 13.1 and 8.3).  Where pieces are merged: 2,048 keys, T = 24
 // alone 12.6 us with two blocks, 9.1 with one; 30,000 keys, T = 30, throughput policy, 20 layers 335 and 411.
-constexpr int kMaxPieceTiles = 64;
+constexpr int kMaxPieceTiles = 48;
 sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluster, int group, const int32_t* n_keys, int T,
                            const int32_t* key0, SplitPlan* plan)
 {
@@ -786,7 +785,7 @@ sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluste
         if (s != SPARROW_OK) return s;
         float cost;
         if (may_share) {
-            int longest = 0, most = 0, units = p.batch * p.n_kv_heads * p.n_groups;
+            int longest = 0, most = 0;
             long long all = 0;
             for (int b = 0; b < p.batch; ++b) {
                 const int tiles = (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile;
@@ -794,10 +793,10 @@ sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluste
                 most = std::max(most, tiles);
                 all += tiles;
             }
-            const bool even = 4 * all > 3ll * most * p.batch;
-            if (longest > kMaxPieceTiles && !(p.n_items == units && even))
-                s = make_plan(std::max(c->n_sm / 2, plan_target(c, true)), L.batch, L.n_kv_heads, group, n_keys, T, nb, &p,
-                              kMaxPieceTiles * kKeyTile, key0);
+            const bool even = 5 * all > 4ll * most * p.batch;
+            const int limit = std::max(nb == 2 && !even ? c->n_sm / 2 : c->n_sm / 5, plan_target(c, true));
+            if (longest > kMaxPieceTiles)
+                s = make_plan(limit, L.batch, L.n_kv_heads, group, n_keys, T, nb, &p, kMaxPieceTiles * kKeyTile, key0);
             if (s != SPARROW_OK) return s;
             cost = batch_cost(p);
         } else {

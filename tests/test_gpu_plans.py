@@ -49,12 +49,14 @@ def test_row_blocks_per_item(hq, hkv, kv_len, T, route, per_item, items, capfd, 
 
 
 @pytest.mark.parametrize("hq,hkv,kv_len,T,policy,pieces", [
-    (28, 4, [9000] * 8, 16, B.PLAN_THROUGHPUT, [1] * 8),                  # whole, of one length: stay whole
-    (32, 8, [9000, 8000, 8500], 20, B.PLAN_THROUGHPUT, [1] * 3),          # nearly of one length
-    (32, 8, [64 * 128 - 20, 900, 800], 20, B.PLAN_THROUGHPUT, [1] * 3),   # uneven, pieces of 64 tiles
-    (32, 8, [64 * 128 - 19, 900, 800], 20, B.PLAN_THROUGHPUT, [2, 1, 1]),  # one key more
+    (28, 4, [9000] * 8, 16, B.PLAN_THROUGHPUT, [1] * 8),                  # 32 whole units stay whole
+    (28, 4, [9000, 5000] * 4, 16, B.PLAN_THROUGHPUT, [1] * 8),            # uneven ones too, with one row block
+    (32, 8, [9000, 8000, 8500], 20, B.PLAN_THROUGHPUT, [1] * 3),
+    (28, 4, [48 * 128 - 32] + [1000] * 5, 32, B.PLAN_THROUGHPUT, [1] * 6),        # uneven, two row blocks, 48 tiles
+    (28, 4, [48 * 128 - 31] + [1000] * 5, 32, B.PLAN_THROUGHPUT, [2] + [1] * 5),  # one key more
+    (28, 4, [9000], 50, B.PLAN_THROUGHPUT, [2]),                          # 12 units: 24 pieces
     (28, 4, [30000], 16, B.PLAN_THROUGHPUT, [5]),                         # 47 tiles a piece as the policy makes them
-    (28, 4, [41000], 16, B.PLAN_THROUGHPUT, [6]),                         # 65 tiles: cut again
+    (28, 4, [41000], 16, B.PLAN_THROUGHPUT, [7]),                         # 65 tiles: cut again
 ])
 def test_long_pieces_of_a_batch(hq, hkv, kv_len, T, policy, pieces, capfd, monkeypatch):
     got = _plan(capfd, monkeypatch, hq, hkv, kv_len, T, "batch", policy)
