@@ -7,7 +7,7 @@
  *   t  a tensor (its data_ptr()) or None (NULL)
  *   i  an int, passed as int32
  *   l  a sequence of ints -> int32 array, valid during the call;  L  the same, or None -> NULL
- *   s  a stream: None (the current one), an object with `cuda_stream`, or an int handle
+ *   s  a stream: None (the current one), an object with `cuda_stream`, an int handle, or one in a ctypes.c_void_p
  * Every argument is an integer or a pointer, i.e. one 64-bit slot of the calling convention.  A non-zero
  * status calls on_error(status, name), which raises.  The interpreter lock is released during the
  * call.  set_stream_functions(get_device, get_raw_stream) says how to ask for the current stream, if not torch. */
@@ -31,7 +31,7 @@ typedef struct {
 int sparrow_tensor_address(PyObject* o, int64_t* out);
 int sparrow_current_stream(int64_t* out);
 
-static PyObject *s_address, *s_data_ptr, *s_cuda_stream, *g_get_device, *g_get_raw_stream;
+static PyObject *s_address, *s_data_ptr, *s_cuda_stream, *s_value, *g_void_p, *g_get_device, *g_get_raw_stream;
 
 static const char kCapsule[] = "sparrow.bound";
 
@@ -74,7 +74,13 @@ static int stream_slot(PyObject* o, int64_t* out)
         return stolen_slot(st, out);
     }
     if (PyLong_Check(o)) return as_slot(o, out);
-    return stolen_slot(PyObject_GetAttr(o, s_cuda_stream), out);
+    const int is_handle = PyObject_IsInstance(o, g_void_p);
+    if (is_handle < 0) return -1;
+    if (!is_handle) return stolen_slot(PyObject_GetAttr(o, s_cuda_stream), out);
+    PyObject* v = PyObject_GetAttr(o, s_value);
+    if (v != Py_None) return stolen_slot(v, out);
+    Py_DECREF(v);                                               /* (a null handle: the default stream) */
+    return 0;
 }
 
 /* Sequence of ints -> int32 array in *buf (STACK_INTS entries) or on the heap (*heap). */
@@ -183,6 +189,10 @@ PyMODINIT_FUNC PyInit__pycall(void)
     s_address = PyUnicode_InternFromString("address");
     s_data_ptr = PyUnicode_InternFromString("data_ptr");
     s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
-    if (!s_address || !s_data_ptr || !s_cuda_stream) return NULL;
+    s_value = PyUnicode_InternFromString("value");
+    PyObject* ctypes = PyImport_ImportModule("ctypes");
+    g_void_p = ctypes ? PyObject_GetAttrString(ctypes, "c_void_p") : NULL;
+    Py_XDECREF(ctypes);
+    if (!s_address || !s_data_ptr || !s_cuda_stream || !s_value || !g_void_p) return NULL;
     return PyModule_Create(&module);
 }

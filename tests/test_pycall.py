@@ -81,3 +81,15 @@ def test_signatures_match_the_library():
         want = getattr(L, name).argtypes
         assert len(want) == len(sig), name
         assert all((w is ctypes.c_int32) == (s == "i") for w, s in zip(want, sig)), name
+
+
+@pytest.mark.parametrize("handle,want", [(0, 0), (None, 0), (5, 5), (2 ** 47 - 16, 2 ** 47 - 16)])
+def test_a_stream_handle_in_a_void_pointer(handle, want):
+    """What ctypes takes for a pointer argument is taken here too."""
+    fn, seen = _bound("s")
+    fn(ctypes.c_void_p(handle))
+    assert seen == [[want]]
+    for wrong in (ctypes.c_int(5), 1.5, "5"):
+        with pytest.raises((TypeError, AttributeError)):
+            fn(wrong)
+    assert seen == [[want]]
