@@ -140,7 +140,8 @@ class _Calls:
         try:
             from . import _pycall
         except ImportError as e:
-            raise RuntimeError("the _pycall extension is not built: run `python -m paper_2602_15318_b200.build`") from e
+            raise RuntimeError("the _pycall extension is not built, or for another Python or torch: "
+                               "run `python -m paper_2602_15318_b200.build`") from e
         torch.cuda.current_stream()                       # brings torch's CUDA state up
         _pycall.set_stream_functions(None, None)          # torch's
         for fn, sig in _SIGNATURES.items():

@@ -93,3 +93,12 @@ def test_a_stream_handle_in_a_void_pointer(handle, want):
         with pytest.raises((TypeError, AttributeError)):
             fn(wrong)
     assert seen == [[want]]
+
+
+def test_the_extension_is_built_again_for_another_torch_or_python(monkeypatch, tmp_path):
+    assert build.pycall_is_current()
+    monkeypatch.setattr(build, "pycall_versions", lambda: "cpython-399 torch 9.9")
+    assert not build.pycall_is_current()
+    monkeypatch.undo()
+    monkeypatch.setattr(build, "PYCALL_VERSIONS", str(tmp_path / "none"))
+    assert not build.pycall_is_current()
