@@ -91,7 +91,9 @@ sparrow_status sparrow_destroy(sparrow_ctx* ctx);
  *   BALANCED    about 3/8 n_sm items (the default);
  *   THROUGHPUT  about n_sm / 7 items: longest pieces, several calls resident at once; best when
  *               many independent calls are queued back to back (one per layer or per request).
- * Results differ between policies only by the rounding order of the split-KV merge.  Calls that
+ * Pieces of more than 48 tiles of 128 keys are cut further, up to n_sm / 5 items (uneven sequences with draft blocks of
+ * more than 128 rows: n_sm / 2).  Results differ between policies by rounding only: weights are rounded to bf16 against the
+ * largest score of their piece, and pieces are merged in another order.  Calls that
  * share the GPU with no other call of the context (single calls without sparrow_set_call_overlap(), graph
  * capture, SPARROW_NO_PDL, sparrow_anchor_attn, sparrow_verify_attn_static) always use one wave
  * over all SMs.  They do not need that wave to be resident as a whole: kernels of other streams and
@@ -112,8 +114,8 @@ sparrow_status sparrow_set_plan_policy(sparrow_ctx* ctx, int32_t policy);
  * ordering rules at sparrow_verify_attn()).  Off by default.  Host state only. */
 sparrow_status sparrow_set_call_overlap(sparrow_ctx* ctx, int32_t enable);
 
-/* Work items the planner currently aims for in fused mode (pass it to sparrow_plan_splits() as
- * n_sm to see the schedule of a call).  0 when ctx is NULL. */
+/* Work items the policy currently aims for in calls that may overlap others (see sparrow_plan_policy; other
+ * calls aim for n_sm).  0 when ctx is NULL. */
 int32_t sparrow_plan_target_items(const sparrow_ctx* ctx);
 
 /* Bytes of device scratch the calls need for draft blocks of up to max_T tokens (split-KV partial
@@ -208,8 +210,9 @@ sparrow_status sparrow_window_first_visible_device(sparrow_ctx* ctx, const int32
 
 /* Several verification calls enqueued back to back on one stream -- e.g. the layers of one
  * decode step, each with its own KV cache (Section 4: the target verifies the draft tree in one
- * forward pass, i.e. one such call per decoder layer).  Same results as calling
- * sparrow_verify_attn() n_calls times; the calls after the first start early (nothing can sit
+ * forward pass, i.e. one such call per decoder layer).  The same as calling sparrow_verify_attn() n_calls
+ * times up to rounding: a call in a batch is cut as the policy says, a single one into one wave.  A call's bits do not
+ * depend on the other calls of its batch.  The calls after the first start early (nothing can sit
  * between them in the stream).  Stops at the first error.  `calls` is HOST memory. */
 typedef struct {
     const void*    q;
@@ -258,7 +261,7 @@ sparrow_status sparrow_anchor_attn_tree(sparrow_ctx* ctx, const void* q, const v
 
 /* Row movers (Section 3.1: the draft model keeps the text-anchored states and discards the visual
  * KV cache; the paper gives no procedure, these two calls are this library's).  Both are plain
- * copies, bit-exact, one ordinary kernel each, ordered by the stream like any other kernel.
+ * copies, bit-exact, one kernel each, ordered by the stream.
  *
  * sparrow_kv_append: writes the T new rows of every (sequence, KV head) into cache rows
  * [kv_len[b], kv_len[b] + T) -- what sparrow_verify_attn() expects to find there.
@@ -434,9 +437,11 @@ sparrow_status sparrow_debug_ancestor_masks_device(sparrow_ctx* ctx, const int32
 /* Host-side split schedule, exported for inspection (pure host code, needs no GPU): for `batch`
  * sequences of n_keys[b] keys, gqa_group query heads per KV head, draft blocks of T tokens and a
  * target of n_sm work items (the SM
- * count, or sparrow_plan_target_items() for calls in fused mode), writes
+ * count, or sparrow_plan_target_items() for calls that may overlap), writes
  * splits_out[b] = key-range pieces per (sequence, KV head, row group) and the total number of
- * work items.  Pieces are whole 128-key tiles, as even as whole tiles allow (the last one takes
+ * work items, for items of as many row blocks as T needs (1 or 2).  This is the rule a call starts from: it may take items of
+ * one row block instead of two, merge its pieces in thread-block clusters, which fixes their number, or cut long
+ * pieces again.  SPARROW_LOG=1 prints what each call takes.  Pieces are whole 128-key tiles, as even as whole tiles allow (the last one takes
  * the ragged end): sparrow_plan_piece_range() gives the keys [begin, end) of piece `piece` of
  * `n_splits`; SPARROW_ERR_SHAPE unless 0 <= piece < n_splits <= ceil(n_keys / 128).  (The kernels
  * cut into pieces of the same sizes and take the longer ones first.) */

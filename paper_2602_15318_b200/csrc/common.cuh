@@ -230,13 +230,29 @@ struct Item {
 };
 
 // Key range of piece `split` of `ns` over `n_keys` keys in whole tiles of `tile` keys, as even as whole tiles
-// allow; the last piece takes the ragged end.  Needs ns <= number of tiles.
+// allow; the last piece takes the ragged end.  Needs ns <= number of tiles.  (What sparrow_plan_piece_range() reports: the
+// sizes are the kernels', which take the longer pieces first, see piece_tiles.)
 inline void piece_range(int n_keys, int ns, int split, int tile, int* begin, int* end)
 {
     const long long n_tiles = (n_keys + tile - 1) / tile;
     const long long b = n_tiles * split / ns * tile, e = n_tiles * (split + 1) / ns * tile;
     *begin = (int)b;
     *end = (int)(e < n_keys ? e : n_keys);
+}
+
+// Tiles of piece `split` of `ns` over `tiles` tiles as the kernels take them: as even as whole tiles allow, the longer
+// pieces first.  The last one holds the draft block, whose masks and tables already make it the latest (26,112 keys,
+// T = 16: 0.7 us behind pieces of the same six tiles, one tile is 1.1 us).
+struct TileRun {
+    int first, count;
+};
+__host__ __device__ __forceinline__ TileRun piece_tiles(int tiles, int ns, int split)
+{
+    const int least = tiles / ns, longer = tiles - least * ns;
+    TileRun r;
+    r.first = split * least + (split < longer ? split : longer);
+    r.count = least + (split < longer ? 1 : 0);
+    return r;
 }
 
 __device__ __forceinline__ Item decode_item(const SplitPlan& p, int item)
@@ -251,13 +267,10 @@ __device__ __forceinline__ Item decode_item(const SplitPlan& p, int item)
     const int unit = local / ns;
     it.group = unit % p.n_groups;
     it.kvh = unit / p.n_groups;
-    // The longer pieces first: the last one holds the draft block, whose masks and tables already make it the
-    // latest (26,112 keys, T = 16: 0.7 us behind pieces of the same six tiles, one tile is 1.1 us).
     const int key0 = p.seq[b].key0, n_keys = p.seq[b].n_keys - key0;
-    const int tiles = (n_keys + p.piece_tile - 1) / p.piece_tile, least = tiles / ns, longer = tiles - least * ns;
-    const int first = it.split * least + min(it.split, longer);
-    it.key_begin = key0 + first * p.piece_tile;
-    it.key_end = key0 + min(n_keys, (first + least + (it.split < longer ? 1 : 0)) * p.piece_tile);
+    const TileRun run = piece_tiles((n_keys + p.piece_tile - 1) / p.piece_tile, ns, it.split);
+    it.key_begin = key0 + run.first * p.piece_tile;
+    it.key_end = key0 + min(n_keys, (run.first + run.count) * p.piece_tile);
     return it;
 }
 

@@ -2,8 +2,11 @@
 for seconds, or only where a thread block starts late."""
 import os
 import re
+import subprocess
 
 import pytest
+
+from paper_2602_15318_b200 import build
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_15318_b200", "csrc")
 
@@ -51,3 +54,50 @@ def test_a_cluster_meets_before_its_first_push(name, start):
     body = code[code.index(start):]
     push = re.search(r"\b(bulk_push|st_cluster_v4|cluster_sum)\(", body).start()
     assert 0 <= body.find("cluster_wait()") < push
+
+
+HARNESS = r"""
+#include <cstdio>
+#include <vector>
+#include <algorithm>
+#include "common.cuh"
+using namespace sparrow;
+int main()
+{
+    for (int tile : {64, 128})
+        for (int tiles = 1; tiles <= 300; tiles += tiles < 40 ? 1 : 37)
+            for (int ns = 1; ns <= tiles; ++ns) {
+                int at = 0;
+                std::vector<int> mine, reported;
+                for (int split = 0; split < ns; ++split) {
+                    const TileRun r = piece_tiles(tiles, ns, split);
+                    if (r.first != at || r.count < 1) { std::printf("gap: %d tiles, piece %d of %d\n", tiles, split, ns); return 1; }
+                    if (!mine.empty() && r.count > mine.back()) { std::printf("a longer piece behind a shorter one\n"); return 1; }
+                    at += r.count;
+                    mine.push_back(r.count);
+                    for (int rest : {1, tile / 2, tile}) {
+                        int b, e;
+                        const int n_keys = (tiles - 1) * tile + rest;
+                        piece_range(n_keys, ns, split, tile, &b, &e);
+                        if (b % tile || e <= b || (split == ns - 1) != (e == n_keys)) { std::printf("piece_range %d %d %d\n", n_keys, ns, split); return 1; }
+                        if (rest == tile) reported.push_back((e - b) / tile);
+                    }
+                }
+                if (at != tiles || mine.front() - mine.back() > 1) { std::printf("%d tiles in %d pieces end at %d\n", tiles, ns, at); return 1; }
+                std::sort(reported.rbegin(), reported.rend());
+                if (reported != mine) { std::printf("other sizes than reported: %d tiles, %d pieces\n", tiles, ns); return 1; }
+            }
+    std::puts("ok");
+    return 0;
+}
+"""
+
+
+def test_the_kernels_pieces_tile_the_key_range(tmp_path):
+    """The kernels' own rule on the host: no gap, no overlap, whole tiles within one of each other, the longer ones
+    first, and the sizes that sparrow_plan_piece_range() reports."""
+    src, exe = tmp_path / "pieces.cu", tmp_path / "pieces"
+    src.write_text(HARNESS)
+    subprocess.run([build.nvcc(), *build.NVCC_FLAGS[:2], "-std=c++17", "-I" + CSRC, "-o", str(exe), str(src)], check=True, timeout=600)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
