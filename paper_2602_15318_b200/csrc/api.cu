@@ -226,9 +226,6 @@ __half* o_part_ptr(const sparrow_ctx* c, int parity)
     return reinterpret_cast<__half*>(c->ws + c->part_offset + (c->part_buffers > 1 ? parity : 0) * part_half_bytes(c));
 }
 
-// Ordering arguments of the next call and, once it is enqueued, the advance of the host mirror.
-// Calls that are being captured into a graph, or made with programmatic launch switched off, or
-// served by the gathered kernel run in stream-ordered mode: their kernels touch no counter.
 // Will this call run in fused mode, i.e. may it overlap its neighbours in the stream?  Not while the
 // stream is being captured, not with programmatic launch switched off, not on the gathered kernel.
 bool call_overlaps(const sparrow_ctx* c, cudaStream_t st, bool fused_kernel)
@@ -328,6 +325,9 @@ void note_fused_launch(sparrow_ctx* c, const CallRanges& cr, bool launched_early
     if (c->n_recent < kRecentCalls) ++c->n_recent;
 }
 
+// Ordering arguments of the next call (advance_sync() moves the host mirror on once it is enqueued).  Calls that are being
+// captured into a graph, made with programmatic launch switched off or served by the gathered kernel run in
+// stream-ordered mode: their kernels touch no counter.
 // `after_previous`: the call's final results must wait for the previous fused call as a whole (its
 // outputs overlap that call's memory); otherwise they only wait for the calls before that one.
 SyncArgs next_sync(const sparrow_ctx* c, const SplitPlan& p, bool overlaps, bool after_previous, bool may_share)
@@ -689,9 +689,8 @@ constexpr float kWaveUs[2] = {6.f, 8.f};                                       /
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
 // at most 16 pieces per unit, pieces short enough to leave a stage of the K/V ring free for the rows that are
 // sent around (2 tiles with one row block, 1 with two), and whole clusters per GPC.  Rewrites the plan where
-// that is estimated to pay.  Measured back to back, workspace -> cluster: 448 keys, T = 8 9.2 -> 7.4 us; 1,000
-// keys, T = 16 9.9 -> 8.2; 3,000 keys 13.1 -> 9.5 (12 pieces of two tiles instead of 24 of one); 448 keys, T = 30
-// 13.8 -> 11.6.  One piece against two in a cluster: 240 keys, T = 8 7.8 and 7.8.  Returns the estimate.
+// that is estimated to pay (448 keys, T = 8 9.2 -> 7.4 us; 3,000 keys in 12 pieces of two tiles instead of 24 of one
+// 13.1 -> 9.5).  Returns the estimate.
 float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
 {
     const int nb = p->blocks_per_group, units = p->batch * p->n_kv_heads * p->n_groups;
@@ -872,10 +871,8 @@ sparrow_status verify_call(sparrow_ctx* c, const void* q, const void* k, const v
     const bool early = protocol && same_ctx_before && !c->prev_lone && (c->chain_next || c->overlap_single_calls) &&
                        !inputs_touch_recent_outputs(c, cr);
     // Can another call of this context run beside this one?  Only inside a batch, or with the opt-in for
-    // single calls.  A call that has the GPU to itself is cut into one wave whatever the policy: measured
-    // single calls, balanced policy's 55 items -> 148 items: 33.0 -> 24.8 us (26,112 keys, T = 16), 52.6 ->
-    // 32.2 (three sequences of 9,001 keys and fewer, T = 23, 8 KV heads), 105 -> 50 (six of 9,000, T = 30),
-    // 16.5 -> 14.8 (2,048 keys, T = 8), no size slower.
+    // single calls.  A call that has the GPU to itself is cut into one wave whatever the policy (26,112 keys, T = 16,
+    // balanced policy's 55 items -> 148: 33.0 -> 24.8 us; no size was slower).
     const bool may_share = protocol && (c->in_batch || c->overlap_single_calls);
     SplitPlan plan;
     const int group = layout_group(c->layout);

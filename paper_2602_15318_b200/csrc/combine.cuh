@@ -4,13 +4,13 @@
 // [B][T][Hq][128] and fp32 lse [B][Hq][T].  Pieces that saw no visible key carry lse_s = -inf and
 // weigh zero; a row with no visible key anywhere gets out = 0, lse = -inf.
 //
-// One warp per query row, registers and shuffles only, so the same routine serves the finisher
-// CTAs of the fused split-KV kernel (whose shared memory is taken) and the stand-alone combine
-// kernel of the stream-ordered mode.  Lane l keeps the LSEs of pieces
-// l, l+32, ...  The four quarter-warps take pieces q, q+4, q+8, ...; inside a quarter each of the 8
-// lanes owns 16 of the 128 output dims (two 16-byte loads per piece), and the quarters' sums meet
-// through two shuffle steps.  The code is kept small on purpose: every warp runs it exactly once,
-// so instruction fetch, not arithmetic, is what a long unrolled body would pay for.
+// The second kernel of calls that do not merge in their own: verification captured into a graph or without
+// programmatic launch, and the gathered pass of more pieces than a cluster takes.  One warp per query row,
+// registers and shuffles only.  Lane l keeps the LSEs of pieces l, l+32, ...  The four quarter-warps
+// take pieces q, q+4, q+8, ...; inside a quarter each of the 8 lanes owns 16 of the 128 output dims (two
+// 16-byte loads per piece), and the quarters' sums meet through two shuffle steps.  The code is kept small on
+// purpose: every warp runs it exactly once, so instruction fetch, not arithmetic, is what a long unrolled body would
+// pay for.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -140,8 +140,7 @@ __device__ __forceinline__ void combine_row(const SplitPlan& plan, const Combine
     }
 }
 
-// The stand-alone combine kernel of the stream-ordered mode: grid-stride over the rows, one warp
-// per row, launched behind the split-KV kernel (ordinarily, or programmatically in anchored mode).
+// Grid-stride over the rows, launched behind the split-KV kernel (ordinarily, or programmatically behind the gathered pass).
 __global__ void __launch_bounds__(kWarps * 32)
 combine_kernel(const __grid_constant__ SplitPlan plan, const __grid_constant__ CombineArgs args)
 {

@@ -165,16 +165,6 @@ __device__ __forceinline__ bool wait_counter(const unsigned* addr, uint32_t targ
     }
     return false;
 }
-// Bounded acquire-wait until a word equals `value`.
-__device__ __forceinline__ bool wait_equal(const unsigned* addr, uint32_t value)
-{
-    #pragma unroll 1
-    for (uint32_t i = 0; i < kCounterPolls; ++i) {
-        if (ld_acquire(addr) == value) return true;
-        __nanosleep(i < 64 ? 40 : 200);
-    }
-    return false;
-}
 // Increment of a counter that also returns what it was; orders as publish_counter() and ld_acquire() do.
 __device__ __forceinline__ unsigned add_acquire_release(unsigned* addr, unsigned n)
 {

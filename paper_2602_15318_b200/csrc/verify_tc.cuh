@@ -8,7 +8,7 @@
 //                        each, which land exactly in the K-major 128-byte-swizzled operand
 //                        layout), then K and V tiles of 128 keys x 128 dims (4 boxes of 128 x 64)
 //                        into a 2- or 3-stage shared-memory ring, mbarrier full / empty handshakes.
-//   warp 9, one thread   tcgen05.mma issuer.  A job is one key tile against one row block:
+//   warp 9               tcgen05.mma issuer: the warp stays converged, an elected lane issues.  A job is one key tile against one row block:
 //                        S = Q K^T (A, B from shared memory, K-major) into a 128 x 128 fp32 TMEM
 //                        block; O += P V with P read from TMEM (bf16, aliasing the S block) and V
 //                        from shared memory as an MN-major operand.  The scores of up to three
@@ -127,17 +127,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-// Non-blocking probe of a phase.
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
@@ -395,12 +384,12 @@ __device__ __forceinline__ bool softmax_bar_or(bool pred)
 // only after its last O += P V, so the K stream runs ahead of the V stream.
 struct Bars {
     uint32_t base;
-    // at most 3 stages and 3 S blocks: 28 slots in all
+    // slots of 8 bytes: 0-27 here and in o_done, 30 and 31 below (28 and 29 hold the TMEM address and flags)
     __device__ __forceinline__ uint32_t k_full(int i) const { return base + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t k_empty(int i) const { return base + 24u + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t v_full(int i) const { return base + 48u + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t v_empty(int i) const { return base + 72u + 8u * (uint32_t)i; }
-    // (a fourth score / P slot, used with two row blocks, sits behind the other barriers)
+    // (a fourth score / P slot, used with two row blocks)
     __device__ __forceinline__ uint32_t s_full(int i) const { return i < 3 ? base + 96u + 8u * (uint32_t)i : base + 240u; }
     __device__ __forceinline__ uint32_t p_full(int i) const { return i < 3 ? base + 120u + 8u * (uint32_t)i : base + 248u; }
     __device__ __forceinline__ uint32_t q_full() const { return base + 144u; }
@@ -415,6 +404,9 @@ struct Bars {
     // this warp's P of that tile.
     __device__ __forceinline__ uint32_t o_done(int blk, int j) const { return base + 160u + 32u * (uint32_t)blk + 8u * (uint32_t)(j & 3); }
 };
+
+constexpr uint32_t kBarrierBytes = 256;      // what the slots above and the words between them take of the barrier area
+static_assert(kMiscBytes >= 1024 + 2 * 128 * 4 && kBarrierBytes + kMaxT * 8 == 768, "barriers, ancestor words, bounds, exchange");
 
 struct MergeOut {
     __nv_bfloat16* out;
@@ -458,9 +450,8 @@ __device__ __forceinline__ void fold_pieces(uint32_t row, int count, uint32_t ho
 // the results; row i is row r0 + i of its unit (token idx / g, head idx % g).  256 threads, no barrier: more than
 // eight rows go two to a warp, 16 lanes of 8 dims each; of fewer a warp takes 128, 64, 32 or 16 dims, and the
 // groups of lanes left over share the row's pieces and add up by shuffles.  What this costs is instructions one
-// after the other (two warps per scheduler), divisions first: with trip counts and shares by shifts and by
-// reciprocals from the host, and without the barriers of groups that met in shared memory, verification of
-// 2,048 keys, T = 8 takes 7.9 us (8.3), three sequences of 9,001 22.3 (22.8), 448 anchors 9.3 (9.6).
+// after the other (two warps per scheduler), divisions first: trip counts and shares go by shifts and by
+// reciprocals from the host (verification of 2,048 keys, T = 8 8.3 -> 7.9 us).
 __device__ __forceinline__ void merge_run(int tid, uint32_t base, int ns, int n, int r0, int b, int tok0, int head0, bool landed, const MergeOut& mo)
 {
     const int warp = tid >> 5, lane = tid & 31;
@@ -502,7 +493,7 @@ __device__ __forceinline__ void merge_run(int tid, uint32_t base, int ns, int n,
 }
 
 // Rows of a unit that CTA `rank` of a cluster finishes: [begin, return value).  inv_cl: 2^16 / cluster size, rounded
-// up (exact: at most 252 rows times 16).
+// up (exact: for c CTAs and x = rows * rank <= 256 * 16, x (c inv_cl - 2^16) <= 4096 * 15 < 2^16).
 __device__ __forceinline__ int merge_share(int unit_rows, int rank, int inv_cl, int* begin)
 {
     *begin = (unit_rows * rank * inv_cl) >> 16;
@@ -538,12 +529,12 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     unsigned char* q_sm = sm;
     unsigned char* kv_sm = sm + NB * kQBlockBytes;
     unsigned char* misc = kv_sm + NS * kStageBytes + recv_extra(NB);
-    uint64_t* bar_mem = reinterpret_cast<uint64_t*>(misc);                  // 28 barrier slots in 224 bytes
+    uint64_t* bar_mem = reinterpret_cast<uint64_t*>(misc);                  // barriers in bytes 0-223 and 240-255 (see Bars)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 224);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(misc + 228);
     volatile uint32_t* write_ok = reinterpret_cast<volatile uint32_t*>(misc + 232);   // the counters allow global writes
     volatile int32_t* fin_go = reinterpret_cast<volatile int32_t*>(misc + 236);       // finishers: their waits succeeded
-    unsigned long long* anc_s = reinterpret_cast<unsigned long long*>(misc + 256);   // [64]
+    unsigned long long* anc_s = reinterpret_cast<unsigned long long*>(misc + kBarrierBytes);   // [64]
     int32_t* par_s = reinterpret_cast<int32_t*>(misc + 768);                          // [64]: parents in the prologue, then the rows' first visible keys
     float* xch = reinterpret_cast<float*>(misc + 1024);                               // [2][128] maxima / sums exchange
 
@@ -559,16 +550,14 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     const int kv_len = plan.seq[it.b].kv_len;
     const int n_keys_seq = plan.seq[it.b].n_keys;
     const int n_tiles = (it.key_end - it.key_begin + kTile - 1) / kTile;
-    // job n: key tile n / NB, row block (and O accumulator) n % NB, S block n % NSB
-    const int n_jobs = n_tiles * NB;
+    const int n_jobs = n_tiles * NB;                        // key tile x row block
     const int block0 = it.group * NB;                       // first 128-row block of this item
 
     // K and V tiles of a lone call leave L2 before anything else does: a cache is streamed once per call, and would
     // otherwise push out the code, the queries and the partial rows, which then come back from DRAM behind the
     // stream of tiles.  All tiles of a call that takes more than half of L2, half of them of a shorter one,
     // whose next call on the same cache then finds as much as before (26,112 keys on one and the same cache: none
-    // 15.9 us, half 16.0, all 17.3).  Caches out of L2, none -> this: 26,112 keys, T = 16 18.6 -> 18.2 us (all: 17.9);
-    // three sequences of 9,001, 8 KV heads 26.5 -> 25.0; two of 20,000, T = 16 21.6 -> 21.4.  In batches it gave nothing.
+    // 15.9 us, half 16.0, all 17.3; caches out of L2: 18.6, 18.2, 17.9).  In batches it gave nothing.
     uint64_t stream_policy;
     if (args.leave_l2 == 0) asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(stream_policy));
     else if (args.leave_l2 == 1) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 0.5;" : "=l"(stream_policy));
@@ -592,9 +581,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
 
     // ---- setup: barriers, TMEM.  Nothing here waits for an earlier kernel: every warp runs on to its own first
     // wait before the loads start.  With the wait and the first loads in front of the CTA barrier the MMA
-    // warp fetched its code behind the stream of tiles, up to 2 us late; now, before -> after: 2,048 keys, T = 8
-    // 7.8 -> 7.6 us, 26,112 keys, T = 16 18.3 -> 17.7, 16,384 keys, T = 64 25.8 -> 25.2, three sequences of 9,001, 8
-    // KV heads 21.6 -> 21.0, eight of 9,000, T = 30 48.1 -> 46.7.
+    // warp fetched its code behind the stream of tiles, up to 2 us late (26,112 keys, T = 16 18.3 -> 17.7 us).
     if (warp == kProducerWarp && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_q) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_k) : "memory");
@@ -743,50 +730,47 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     if (n + 2 < n_jobs) ok = issue_qk2(n + 2);                // this block's next scores
                 }
             } else {
-            constexpr uint32_t idesc_qk = idesc_bf16(false);
-            constexpr uint32_t idesc_pv = idesc_bf16(true);
-            // S = Q K^T of job m into S block m % NSB
-            auto issue_qk = [&](int m) -> bool {
-                const int j = m / NB, blk = m % NB, sb = m % NSB, st = j % NS;
-                if (blk == 0) {                                           // first use of this K tile
+                // One row block: a job is a key tile, the scores of tile j lie in S block j % NSB.
+                constexpr uint32_t idesc_qk = idesc_bf16(false);
+                constexpr uint32_t idesc_pv = idesc_bf16(true);
+                auto issue_qk = [&](int j) -> bool {                      // S = Q K^T
+                    const int sb = j % NSB, st = j % NS;
                     if (!mbar_wait_warp(B.k_full(st), (j / NS) & 1)) return false;
                     tc_fence_after();
                     if (j == 0 && lane == 0) SPARROW_STAMP(3);                       // first K tile landed
-                }
-                const uint64_t qd = q_desc0 + (uint64_t)((blk * kQBlockBytes) >> 4);
-                const uint64_t kd = k_desc0 + (uint64_t)((st * kStageBytes) >> 4);
-                if (elect_one()) {
-                    #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
-                        const uint32_t off = ((ks >> 2) * kSubTileBytes + (ks & 3) * 32) >> 4;
-                        mma_ss(tmem_u + sb * 128, qd + off, kd + off, idesc_qk, ks > 0);
+                    const uint64_t kd = k_desc0 + (uint64_t)((st * kStageBytes) >> 4);
+                    if (elect_one()) {
+                        #pragma unroll
+                        for (int ks = 0; ks < 8; ++ks) {
+                            const uint32_t off = ((ks >> 2) * kSubTileBytes + (ks & 3) * 32) >> 4;
+                            mma_ss(tmem_u + sb * 128, q_desc0 + off, kd + off, idesc_qk, ks > 0);
+                        }
+                        tc_commit(B.s_full(sb));
+                        tc_commit(B.k_empty(st));
                     }
-                    tc_commit(B.s_full(sb));
-                    if (blk == NB - 1) tc_commit(B.k_empty(st));          // last use of the tile
+                    __syncwarp();
+                    return true;
+                };
+                for (int j = 0; j < NSB && j < n_tiles && ok; ++j) ok = issue_qk(j);
+                #pragma unroll 1
+                for (int j = 0; j < n_tiles && ok; ++j) {
+                    const int sb = j % NSB, st = j % NS;
+                    if (!mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
+                    if (j == n_tiles - 1) zero_v_tail(j);
+                    if (!mbar_wait_warp(B.p_full(sb), (j / NSB) & 1)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
+                    if (elect_one()) {
+                        #pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            mma_ts(tmem_u + kOCol, tmem_u + sb * 128 + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)((kk * 2048) >> 4),
+                                   idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+                        tc_commit(B.o_done(0, j));
+                        tc_commit(B.v_empty(st));
+                    }
+                    __syncwarp();
+                    if (j + NSB < n_tiles) ok = issue_qk(j + NSB);        // its S block was tile j's
                 }
-                __syncwarp();
-                return true;
-            };
-            for (int m = 0; m < NSB && m < n_jobs && ok; ++m) ok = issue_qk(m);
-            #pragma unroll 1
-            for (int n = 0; n < n_jobs && ok; ++n) {
-                const int j = n / NB, blk = n % NB, sb = n % NSB, st = j % NS;
-                if (!mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
-                if (j == n_tiles - 1) zero_v_tail(j);
-                if (!mbar_wait_warp(B.p_full(sb), (n / NSB) & 1)) { ok = false; break; }
-                tc_fence_after();
-                const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
-                if (elect_one()) {
-                    #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_ts(tmem_u + kOCol + blk * 128, tmem_u + sb * 128 + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)((kk * 2048) >> 4),
-                               idesc_pv, (n >= NB || kk > 0) ? 1u : 0u);
-                    tc_commit(B.o_done(blk, j));
-                    if (blk == NB - 1) tc_commit(B.v_empty(st));
-                }
-                __syncwarp();
-                if (n + NSB < n_jobs) ok = issue_qk(n + NSB);             // its S block was job n's
-            }
             }
             if (lane == 0) SPARROW_STAMP(4);                            // last product issued
             if (!ok && lane == 0) { atomicOr(args.status, timeout_bits(kSiteMma)); *abort_flag = 1; }
@@ -1052,7 +1036,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const bool direct = plan.seq[it.b].n_splits == 1;                  // the only piece: write the final result
         const bool clustered = plan.cluster > 1;                           // the unit's pieces meet in the cluster's shared memory
         if (tid == 0) {
-            // Global writes start below.  In overlapped mode a lane of the MMA warp has been waiting,
+            // Global writes start below.  In overlapped mode a lane of the gate warp has been waiting,
             // since the kernel started, for the counters that allow them (see there).
             uint32_t w = *write_ok;
             for (uint32_t i = 0; w == 0u && i < (1u << 26); ++i) { __nanosleep(20); w = *write_ok; }
