@@ -7,7 +7,8 @@ position just before the call).
     python -m paper_2602_15318_b200.timeline --config C2 --policy throughput --burst 20
     python -m paper_2602_15318_b200.timeline --hsr
 
-With --burst N the N calls are enqueued back to back from C (one sparrow_verify_attn_batch, as the
+A call of its own takes one wave over all SMs (--policy latency); the other policies' pieces are those of a
+call in a batch, here a batch of one.  With --burst N the N calls are enqueued back to back from C (one sparrow_verify_attn_batch, as the
 bench's timed region does) and one line per call says when its CTAs started, left their main loop,
 stored their partial rows and when its merged rows were written.
 
@@ -32,8 +33,7 @@ CALLS, CTAS, SLOTS = 32, 256, 16
 VERIFY_SLOTS = ["kernel entered", "set-up done (barriers, TMEM)", "Q landed", "first K tile landed",
                 "last product issued", "softmax loop left", "last product complete", "partial rows stored",
                 "finisher: all arrivals seen", "finisher: previous call done", "finisher: merged rows written",
-                "leaving", "finisher: bulk copies issued", "finisher: pieces folded", "finisher: groups reduced",
-                "finisher: bulk copies landed"]
+                "leaving", "merge: copies issued", "", "", "merge: every piece here"]
 HSR_SLOTS = ["kernel entered", "set-up done (barriers, TMEM)", "first tile landed", "last MMA issued",
              "accumulator complete", "partial sums pushed", "cluster barrier passed", "z written, leaving"]
 
@@ -96,9 +96,14 @@ def main():
         outs = [torch.empty_like(c.q) for c in cases]
         lses = [torch.empty((c.B, W.HQ, c.T), dtype=torch.float32, device=dev) for c in cases]
 
+        ones = [B.VerifyBatch([(c.q, c.k, c.v, c.kv_len, c.parents, c.T, o, l)]) for c, o, l in zip(cases, outs, lses)]
+
         def call(i):
             c = cases[i % n_rot]
-            B.sparrow_verify_attn(ctx, c.q, c.k, c.v, c.kv_len, c.parents, c.T, outs[i % n_rot], lses[i % n_rot])
+            if args.policy == "latency":
+                B.sparrow_verify_attn(ctx, c.q, c.k, c.v, c.kv_len, c.parents, c.T, outs[i % n_rot], lses[i % n_rot])
+            else:
+                B.sparrow_verify_attn_batch(ctx, ones[i % n_rot])
         names, what = VERIFY_SLOTS, f"sparrow_verify_attn, {args.config}, {args.policy} policy"
 
     def read_table():
