@@ -159,7 +159,8 @@ sparrow_status sparrow_set_workspace(sparrow_ctx* ctx, void* dev_ptr, size_t byt
  * that follows a call of another context.  Writes of consecutive calls of one context are ordered
  * through counters in its workspace.  All calls of a context belong on one stream (or must be kept
  * from running concurrently by events): the counters assume that calls run in the order they were
- * enqueued.  While a stream is being captured into a graph, or with SPARROW_NO_PDL=1 in the
+ * enqueued.  (Calls of several contexts may run at once; what that asks of the SMs stands at
+ * sparrow_plan_policy.)  While a stream is being captured into a graph, or with SPARROW_NO_PDL=1 in the
  * environment when the context is created, a call is two ordinary launches (split-KV pass over
  * one wave of pieces, combine kernel) ordered by the stream alone and touches no counter.
  * Results are deterministic for fixed arguments. */
