@@ -17,25 +17,29 @@
 //                        masking, fp32 online softmax with a lazy maximum, P packed to bf16 and
 //                        stored back with tcgen05.st.
 //                        One row block (T <= 18): the two threads with the same lane (warps w and
-//                        w + 4) share a row, warpgroup g taking key columns [64 g, 64 g + 64) of every
-//                        tile, with its P over its own scores.  They keep the same reference maximum:
-//                        one barrier with an OR reduction per tile tells whether any row's maximum grew
-//                        by more than 2^8; only then the halves' maxima meet in shared memory and O is
-//                        rescaled in TMEM.  Each thread sums its own columns; the halves' sums meet
-//                        once, in the epilogue.
+//                        w + 4, one scheduler) share a row, warpgroup g taking key columns [64 g, 64 g + 64) of every
+//                        tile, with its P over its own scores.  They use the same reference maximum, taken from
+//                        the first tile, and run apart from one another: what one does besides its exponentials
+//                        is filled by the exponentials of the other.  A reference moves only where a score exceeds it by
+//                        more than 2^16 (P and its sums are floating point: nothing is lost before that); then
+//                        the pair meets at a barrier, the halves' maxima meet in shared memory, and O and the P that is
+//                        still waiting are rescaled in TMEM.  Each thread sums its own columns; the halves'
+//                        sums meet once, in the epilogue.
+//                        Cycles per tile (41 tiles a CTA, 20 CTAs): 1,985 with a barrier of all softmax warps in every tile, 1,880
+//                        with one between the two of a pair, 1,600 without; the exponentials alone are 1,024, the
+//                        products 1,030 (a wait at a barrier that is complete costs the issuing warp another 100,
+//                        three or four times a tile).  Two warps that issue products, one for S and one for O, take 1,450,
+//                        but start a lone call 0.2 us later and gain nothing there.
 //                        Two row blocks: warpgroup g owns block g, one thread per row and all 128
 //                        keys of a tile, and works through its block's tiles on its own (no
 //                        barrier between the warpgroups); per block the chain is scores -> softmax
 //                        -> O += P V -> next scores, and the two chains interleave on the tensor
 //                        pipe and the exponential unit.  P is handed over in two halves, the first
-//                        half's product running beside the exponentials of the second.
-//                        The loops are rolled around 64 scores: what a tile costs beyond its
-//                        exponentials (1,024 cycles a block) is mostly instruction supply and hand-over
-//                        latency.  Two blocks, 36 tokens, cycles per tile: 3,900 with both passes unrolled
-//                        over 128 scores, 3,480 like this; sixteen softmax warps (a warpgroup per half row)
-//                        3,500; 64-key steps with their own N = 64 products slower (the 64-column product
-//                        takes 48 cycles instead of 32).  Long streams of calls run at the power limit
-//                        (1,000 W, 1.5 GHz) whatever the loop looks like.
+//                        half's product running beside the exponentials of the second.  3,200 cycles per tile: 2,030 of
+//                        softmax and 1,100 until the next scores are there.
+//                        What a score costs: packed fp32 multiply-add and addition (half an instruction each), 2^x, half a
+//                        conversion to bf16, half a maximum; with single fp32 operations and bf16 packed by integer
+//                        ones 8.5 cycles a score and scheduler instead of 8.1 (the unit for 2^x alone: 8.0).
 //   warp 10              gatekeeper: fills the tables of ancestor words and window bounds, then one
 //                        thread waits (overlapped mode), beside the main loop, for the counters that
 //                        allow this CTA's first global write.
@@ -89,7 +93,7 @@ constexpr int kStageBytes = 4 * kSubTileBytes;   // K (32 KB) + V (32 KB)
 constexpr int kRowBytes = kPartRowHalves * 2;    // a partial row: 272 bytes
 constexpr int kMiscBytes = 2048;                 // barriers, flags, ancestor words, maxima exchange
 constexpr uint32_t kSpinLimit = 1u << 22;        // polls before a wait gives up
-constexpr float kRescaleLog2 = 8.0f;             // lazy-max threshold in log2 units
+constexpr float kRescaleLog2 = 16.0f;             // lazy-max threshold in log2 units
 
 // Rows received from the CTAs of a cluster lie in the ring's last stage; with two row blocks (up to 256 rows and
 // rounded-up shares) they need a little more behind it.
@@ -127,6 +131,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// The same without being held up where the phase is not complete.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
@@ -299,13 +314,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// Two non-negative finite floats -> packed bf16, rounded to nearest (ties up) with integer
-// instructions: the conversion instruction shares the quarter-rate pipe with ex2, which is the
-// softmax's bottleneck.
-__device__ __forceinline__ uint32_t pack_bf16x2_pos(float lo, float hi)
-{
-    return __byte_perm(__float_as_uint(lo) + 0x8000u, __float_as_uint(hi) + 0x8000u, 0x7632);
-}
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
 {
     const __half2 h2 = __floats2half2_rn(lo, hi);
@@ -352,30 +360,58 @@ __device__ __forceinline__ float chunk_max(const float (&x)[32])
     for (int c = 6; c < 30; c += 4) { a = max3(a, x[c], x[c + 1]); b = max3(b, x[c + 2], x[c + 3]); }
     return max3(a, b, fmaxf(x[30], x[31]));
 }
-// p = 2^(x c2 - mc) for 32 scores; adds the unrounded p to sum4 and stores the 16 packed bf16
+// Two fp32 operations per instruction (a pair of registers each).
+__device__ __forceinline__ uint64_t pair_of(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void pair_parts(uint64_t p, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p)); }
+__device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_pair(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// p = 2^(x c2 - mc) for 32 scores (c2 and -mc twice each); adds the unrounded p to sum and stores the 16 packed bf16
 // pairs to 16 TMEM columns at p_addr.
-__device__ __forceinline__ void exp_chunk(const float (&x)[32], float c2, float mc, float (&sum4)[4], uint32_t p_addr)
+__device__ __forceinline__ void exp_chunk(const float (&x)[32], uint64_t c2, uint64_t neg_mc, uint64_t (&sum)[2], uint32_t p_addr)
 {
     uint32_t p[16];
     #pragma unroll
     for (int c = 0; c < 16; ++c) {
-        const float p0 = ex2(fmaf(x[2 * c], c2, -mc));
-        const float p1 = ex2(fmaf(x[2 * c + 1], c2, -mc));
-        sum4[c & 3] += p0 + p1;
-        p[c] = pack_bf16x2_pos(p0, p1);
+        float p0, p1;
+        pair_parts(fma_pair(pair_of(x[2 * c], x[2 * c + 1]), c2, neg_mc), p0, p1);
+        p0 = ex2(p0);
+        p1 = ex2(p1);
+        sum[c & 1] = add_pair(sum[c & 1], pair_of(p0, p1));
+        p[c] = pack_bf16x2(p0, p1);
     }
     tmem_st16(p_addr, p);
 }
+__device__ __forceinline__ float sum_of(const uint64_t (&sum)[2])
+{
+    float a, b;
+    pair_parts(add_pair(sum[0], sum[1]), a, b);
+    return a + b;
+}
 
-// Barrier among the 256 softmax threads with an OR reduction of a predicate (id 2).
-__device__ __forceinline__ bool softmax_bar_or(bool pred)
+// Barriers between the two softmax warps that share a scheduler and 32 rows (ids 4 to 11), with an OR of a predicate.
+__device__ __forceinline__ bool pair_or(uint32_t id, bool pred)
 {
     uint32_t r;
     asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 2, 256, p;\n\t"
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %2, 0;\n\t"
+        "bar.red.or.pred q, %1, 64, p;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r) : "r"((uint32_t)pred) : "memory");
+        : "=r"(r) : "r"(id), "r"((uint32_t)pred) : "memory");
     return r != 0;
 }
 
@@ -396,12 +432,12 @@ struct Bars {
     __device__ __forceinline__ uint32_t fin() const { return base + 152u; }       // finishers' bulk copies
     // Completion of O += P V of key tile j on row block blk: a ring of four barriers per block,
     // tile j on barrier j % 4 with phase parity (j / 4) & 1.  The softmax only looks at it when a
-    // row maximum moves and in the epilogue, asking for tile j - 1 while it works on tile j.  A
-    // parity wait is only meaningful for the phase in progress or the one just completed; here the
-    // barrier is in exactly that state: its previous use (tile j - 5) completed before the scores
-    // of tile j, which the warp has seen (the tensor pipe completes in issue order and the scores
-    // of tile j were issued after the product of tile j - 3), and its next use (tile j + 3) needs
-    // this warp's P of that tile.
+    // row maximum moves and in the epilogue, asking for the last tile that both halves of the row have handed
+    // over.  A parity wait is only meaningful for the phase in progress or the one just completed; here the
+    // barrier is in exactly that state: with tile t asked for, its previous use (tile t - 4) completed before the
+    // scores of tile t, which the warp has seen (the tensor pipe completes in issue order and they
+    // were issued after the product of tile t - 3), and its next use (tile t + 4) needs P that this warp or its
+    // partner has yet to make.
     __device__ __forceinline__ uint32_t o_done(int blk, int j) const { return base + 160u + 32u * (uint32_t)blk + 8u * (uint32_t)(j & 3); }
 };
 
@@ -534,6 +570,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(misc + 228);
     volatile uint32_t* write_ok = reinterpret_cast<volatile uint32_t*>(misc + 232);   // the counters allow global writes
     volatile int32_t* fin_go = reinterpret_cast<volatile int32_t*>(misc + 236);       // finishers: their waits succeeded
+    // one row block, in slots of barriers that only two blocks use: [4] a warp of the pair waits for its partner; [8] where the warps stand
+    volatile int32_t* meet_s = reinterpret_cast<volatile int32_t*>(misc + 240);
+    volatile int32_t* tile_s = reinterpret_cast<volatile int32_t*>(misc + 192);
     unsigned long long* anc_s = reinterpret_cast<unsigned long long*>(misc + kBarrierBytes);   // [64]
     int32_t* par_s = reinterpret_cast<int32_t*>(misc + 768);                          // [64]: parents in the prologue, then the rows' first visible keys
     float* xch = reinterpret_cast<float*>(misc + 1024);                               // [2][128] maxima / sums exchange
@@ -586,10 +625,16 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_q) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_k) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_v) : "memory");
-        for (int i = 0; i < 3; ++i) { mbar_init(B.k_full(i), 1); mbar_init(B.k_empty(i), 1); mbar_init(B.v_full(i), 1); mbar_init(B.v_empty(i), 1); }
+        for (int i = 0; i < 3; ++i) { mbar_init(B.k_full(i), 1); mbar_init(B.k_empty(i), 1); mbar_init(B.v_full(i), 1); mbar_init(B.v_empty(i), 1); }      // (a tile is read by every block)
         // one row block: a P block comes from all eight softmax warps; two: from the block's own four
-        for (int i = 0; i < 4; ++i) { mbar_init(B.s_full(i), 1); mbar_init(B.p_full(i), NB == 1 ? 8 : 4); }
-        for (int i = 0; i < 4; ++i) { mbar_init(B.o_done(0, i), 1); mbar_init(B.o_done(1, i), 1); }
+        for (int i = 0; i < 3; ++i) { mbar_init(B.s_full(i), 1); mbar_init(B.p_full(i), NB == 1 ? 8 : 4); }
+        for (int i = 0; i < 4; ++i) mbar_init(B.o_done(0, i), 1);
+        if (NB == 2) {
+            mbar_init(B.p_full(3), 4);
+            for (int i = 0; i < 4; ++i) mbar_init(B.o_done(1, i), 1);
+        } else {
+            for (int i = 0; i < 4; ++i) meet_s[i] = 0;
+        }
         mbar_init(B.q_full(), 1);
         mbar_init(B.fin(), 1);
         *abort_flag = 0;
@@ -733,43 +778,56 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 // One row block: a job is a key tile, the scores of tile j lie in S block j % NSB.
                 constexpr uint32_t idesc_qk = idesc_bf16(false);
                 constexpr uint32_t idesc_pv = idesc_bf16(true);
-                auto issue_qk = [&](int j) -> bool {                      // S = Q K^T
-                    const int sb = j % NSB, st = j % NS;
-                    if (!mbar_wait_warp(B.k_full(st), (j / NS) & 1)) return false;
-                    tc_fence_after();
-                    if (j == 0 && lane == 0) SPARROW_STAMP(3);                       // first K tile landed
-                    const uint64_t kd = k_desc0 + (uint64_t)((st * kStageBytes) >> 4);
+                auto issue_qk = [&](int ring) {                           // S = Q K^T of the tile in stage and S block `ring`
+                    const uint64_t kd = k_desc0 + (uint64_t)((ring * kStageBytes) >> 4);
                     if (elect_one()) {
                         #pragma unroll
                         for (int ks = 0; ks < 8; ++ks) {
                             const uint32_t off = ((ks >> 2) * kSubTileBytes + (ks & 3) * 32) >> 4;
-                            mma_ss(tmem_u + sb * 128, q_desc0 + off, kd + off, idesc_qk, ks > 0);
+                            mma_ss(tmem_u + ring * 128, q_desc0 + off, kd + off, idesc_qk, ks > 0);
                         }
-                        tc_commit(B.s_full(sb));
-                        tc_commit(B.k_empty(st));
+                        tc_commit(B.s_full(ring));
+                        tc_commit(B.k_empty(ring));
                     }
                     __syncwarp();
-                    return true;
                 };
-                for (int j = 0; j < NSB && j < n_tiles && ok; ++j) ok = issue_qk(j);
+                static_assert(NB == 2 || NS == NSB, "one ring index for stages and S blocks");
+                #pragma unroll 1
+                for (int j = 0; j < NS && j < n_tiles && ok; ++j) {
+                    ok = mbar_wait_warp(B.k_full(j), 0);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (j == 0 && lane == 0) SPARROW_STAMP(3);                       // first K tile landed
+                    issue_qk(j);
+                }
+                int ring = 0;                                             // tile modulo 3
+                uint32_t parity = 0;
+                ok = ok && mbar_wait_warp(B.v_full(0), 0);
                 #pragma unroll 1
                 for (int j = 0; j < n_tiles && ok; ++j) {
-                    const int sb = j % NSB, st = j % NS;
-                    if (!mbar_wait_warp(B.v_full(st), (j / NS) & 1)) { ok = false; break; }
                     if (j == n_tiles - 1) zero_v_tail(j);
-                    if (!mbar_wait_warp(B.p_full(sb), (j / NSB) & 1)) { ok = false; break; }
+                    if (!mbar_wait_warp(B.p_full(ring), parity)) { ok = false; break; }
                     tc_fence_after();
-                    const uint64_t vd = v_desc0 + (uint64_t)((st * kStageBytes) >> 4);
+                    const uint64_t vd = v_desc0 + (uint64_t)((ring * kStageBytes) >> 4);
                     if (elect_one()) {
                         #pragma unroll
                         for (int kk = 0; kk < 8; ++kk)
-                            mma_ts(tmem_u + kOCol, tmem_u + sb * 128 + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)((kk * 2048) >> 4),
+                            mma_ts(tmem_u + kOCol, tmem_u + ring * 128 + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)((kk * 2048) >> 4),
                                    idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
                         tc_commit(B.o_done(0, j));
-                        tc_commit(B.v_empty(st));
+                        tc_commit(B.v_empty(ring));
                     }
                     __syncwarp();
-                    if (j + NSB < n_tiles) ok = issue_qk(j + NSB);        // its S block was tile j's
+                    const uint32_t parity_next = parity ^ 1u;
+                    const int this_ring = ring;
+                    if (++ring == NS) { ring = 0; parity = parity_next; }
+                    // (the next tile's V is waited for while the pipe has work)
+                    if (j + 1 < n_tiles && !mbar_wait_warp(B.v_full(ring), parity)) { ok = false; break; }
+                    if (j + NS < n_tiles) {                               // the S block and the stage that have become free
+                        if (!mbar_wait_warp(B.k_full(this_ring), this_ring == NS - 1 ? parity : parity_next)) { ok = false; break; }
+                        tc_fence_after();
+                        issue_qk(this_ring);
+                    }
                 }
             }
             if (lane == 0) SPARROW_STAMP(4);                            // last product issued
@@ -831,6 +889,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const float c2 = args.scale_log2e;
         const float thr = kRescaleLog2 / c2;             // threshold in raw score units
+        const uint64_t c22 = pair_of(c2, c2);
         const int g_row = row_local % qg;
         int t_row[NB], lo_row[NB];
         bool row_ok[NB];
@@ -878,35 +937,39 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const uint32_t s_addr = lane_addr + blk * 128;
             // tiles whose every key is visible to this row: [j_head, j_tail)
             const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
-            const int j_head = my_lo > it.key_begin ? (my_lo - it.key_begin + kTile - 1) / kTile : 0;
+            const int j_head = __reduce_max_sync(0xffffffffu, my_lo > it.key_begin ? (my_lo - it.key_begin + kTile - 1) / kTile : 0);
             #pragma unroll 1
-            for (int j = 0; j < n_tiles && ok; ++j) {
+            for (int j = 0; j < n_tiles; ++j) {
                 const int tile0 = it.key_begin + j * kTile;
                 if (!mbar_wait_warp(B.s_full(blk), j & 1)) { ok = false; break; }
                 tc_fence_after();
                 // First pass over the row's 128 scores, 64 at a time: the maximum.  In a tile that crosses a
                 // visibility boundary of some row the scores are masked on the way; the lower 64, which are
                 // fetched again for the second pass, go back to TMEM masked.
-                const bool edge = __any_sync(0xffffffffu, j >= j_tail || j < j_head);
+                const bool edge = j >= j_tail || j < j_head;
                 float x0[32], x1[32];
-                float mx = -INFINITY;
-                #pragma unroll 1
-                for (int half = 0; half < 2; ++half) {
-                    tmem_ld32(s_addr + 64 * half, x0);
-                    tmem_ld32(s_addr + 64 * half + 32, x1);
-                    tmem_wait_ld();
-                    if (edge) {
-                        const unsigned long long vis = vis_word(tile0 + 64 * half, my_anc, my_lo);
-                        mask_chunk(x0, (uint32_t)vis);
-                        mask_chunk(x1, (uint32_t)(vis >> 32));
-                        if (half == 0) {
-                            tmem_st32(s_addr, reinterpret_cast<uint32_t*>(x0));
-                            tmem_st32(s_addr + 32, reinterpret_cast<uint32_t*>(x1));
-                            tmem_wait_st();
-                        }
-                    }
-                    mx = fmaxf(mx, fmaxf(chunk_max(x0), chunk_max(x1)));
+                tmem_ld32(s_addr, x0);
+                tmem_ld32(s_addr + 32, x1);
+                tmem_wait_ld();
+                if (edge) {
+                    const unsigned long long vis = vis_word(tile0, my_anc, my_lo);
+                    mask_chunk(x0, (uint32_t)vis);
+                    mask_chunk(x1, (uint32_t)(vis >> 32));
+                    tmem_st32(s_addr, reinterpret_cast<uint32_t*>(x0));
+                    tmem_st32(s_addr + 32, reinterpret_cast<uint32_t*>(x1));
+                    tmem_wait_st();
                 }
+                float mx = chunk_max(x0);
+                tmem_ld32(s_addr + 64, x0);
+                mx = fmaxf(mx, chunk_max(x1));
+                tmem_ld32(s_addr + 96, x1);
+                tmem_wait_ld();
+                if (edge) {
+                    const unsigned long long vis = vis_word(tile0 + 64, my_anc, my_lo);
+                    mask_chunk(x0, (uint32_t)vis);
+                    mask_chunk(x1, (uint32_t)(vis >> 32));
+                }
+                mx = fmaxf(mx, fmaxf(chunk_max(x0), chunk_max(x1)));
                 // lazy reference maximum, per row; the accumulator is rescaled by the whole warp (the
                 // TMEM accesses are warp-wide) whenever one of its rows moved
                 const bool need = my_ok && (mx > my_m + thr || (my_m == -INFINITY && mx > -INFINITY));
@@ -937,98 +1000,143 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 // columns are the ones P overwrites), then the lower 64, fetched again.  The upper keys'
                 // half of O += P V runs beside the exponentials of the lower ones.
                 const float mc = (my_m == -INFINITY) ? 0.f : my_m * c2;
-                float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-                #pragma unroll 1
-                for (int half = 1; half >= 0; --half) {
-                    if (half == 0) {
-                        tmem_ld32(s_addr, x0);
-                        tmem_ld32(s_addr + 32, x1);
-                        tmem_wait_ld();
-                    }
-                    exp_chunk(x0, c2, mc, sum4, s_addr + 64 + 32 * half);
-                    exp_chunk(x1, c2, mc, sum4, s_addr + 80 + 32 * half);
-                    tmem_wait_st();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(B.p_full(2 * (1 - half) + blk));
-                }
-                my_l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
+                const uint64_t neg_mc2 = pair_of(-mc, -mc);
+                uint64_t sum[2] = {0ull, 0ull};
+                exp_chunk(x0, c22, neg_mc2, sum, s_addr + 96);
+                tmem_ld32(s_addr, x0);
+                exp_chunk(x1, c22, neg_mc2, sum, s_addr + 112);
+                tmem_ld32(s_addr + 32, x1);
+                tmem_wait_st();
+                tc_fence_before();
+                if (lane == 0) mbar_arrive(B.p_full(blk));
+                tmem_wait_ld();
+                exp_chunk(x0, c22, neg_mc2, sum, s_addr + 64);
+                exp_chunk(x1, c22, neg_mc2, sum, s_addr + 80);
+                tmem_wait_st();
+                tc_fence_before();
+                if (lane == 0) mbar_arrive(B.p_full(2 + blk));
+                my_l += sum_of(sum);
             }
         } else {
-        // One row block: the two warpgroups split a tile's 128 keys; thread = one row, 64 keys.  The scores
-        // of a tile are requested from TMEM at the end of the tile before it, ahead of the wait for that
-        // tile's P stores, so the two latencies overlap.
+        // One row block: the two warpgroups split a tile's 128 keys; thread = one row, 64 keys.  The two warps that share
+        // 32 rows run apart from one another and meet only where a reference has to move (see the head of this file).
         const int sb_wg = 64 * wg;
+        const uint32_t pair_id = 4u + (uint32_t)(warp & 3);
         float x0[32], x1[32];
-        if (n_tiles > 0) {
-            ok = mbar_wait_warp(B.s_full(0), 0);
-            tc_fence_after();
-            if (ok) { tmem_ld32(lane_addr + sb_wg, x0); tmem_ld32(lane_addr + sb_wg + 32, x1); }
-        }
-        // tiles whose every key is visible to the row: [j_head, j_tail)
+        // tiles whose every key is visible to the warp's rows: [j_head, j_tail)
         const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
-        const int j_head = lo_row[0] > it.key_begin ? (lo_row[0] - it.key_begin + kTile - 1) / kTile : 0;
+        const int j_head = __reduce_max_sync(0xffffffffu, lo_row[0] > it.key_begin ? (lo_row[0] - it.key_begin + kTile - 1) / kTile : 0);
+        // scores above this need a new reference.  (Rows of padding hold whatever the Q box left there: they never do.)
+        float limit = row_ok[0] ? -INFINITY : INFINITY;
+        float mc = 0.f;                                                     // reference in log2 units, 0 as long as there is none
+        int j = 0, sb = 0, sb_before = 0;                                   // tile, its S block, the S block of the tile before
+        uint32_t s_parity = 0;
+        bool have = false, owes = false;                                    // tile j's scores are requested; P of tile j - 1 is not handed over
         #pragma unroll 1
-        for (int j = 0; j < n_tiles && ok; ++j) {
-            const int sb = j % NSB;
-            const uint32_t x_addr = lane_addr + sb * 128 + sb_wg;           // this thread's scores, then its P
-            tmem_wait_ld();
-            if (j >= j_tail || j < j_head) {
-                const int tile0 = it.key_begin + j * kTile;          // first key of the tile
-                const unsigned long long vis = vis_word(tile0 + sb_wg, anc[0], lo_row[0]);
-                mask_chunk(x0, (uint32_t)vis);
-                mask_chunk(x1, (uint32_t)(vis >> 32));
+        for (;;) {
+            if (__builtin_expect(!have, 0)) {
+                // not there when the tile before looked for them, or no tile is left
+                if (owes) {
+                    tmem_wait_st();
+                    tc_fence_before();
+                    if (lane == 0) mbar_arrive(B.p_full(sb_before));
+                    owes = false;
+                }
+                #pragma unroll 1
+                for (uint32_t i = 0; j < n_tiles; ++i) {
+                    if (__all_sync(0xffffffffu, mbar_try_wait(B.s_full(sb), s_parity))) { have = true; break; }
+                    if (__any_sync(0xffffffffu, meet_s[warp & 3] != 0)) break;
+                    if (i >= kSpinLimit) { ok = false; j = n_tiles; }
+                }
+                tc_fence_after();
+                if (have) { tmem_ld32(lane_addr + sb * 128 + sb_wg, x0); tmem_ld32(lane_addr + sb * 128 + sb_wg + 32, x1); }
             }
-            const float mx = fmaxf(chunk_max(x0), chunk_max(x1));
-            // Rows of padding hold whatever the Q box left there: they never force a rescale.
-            const bool need = row_ok[0] && (mx > m_ref[0] + thr || (m_ref[0] == -INFINITY && mx > -INFINITY));
-            if (softmax_bar_or(need)) {
-                // some row's maximum moved: the two halves of every row agree on the new reference
-                xch[wg * 128 + row_local] = need ? mx : -INFINITY;
-                softmax_bar_sync();
-                const float cand = fmaxf(need ? mx : -INFINITY, xch[(wg ^ 1) * 128 + row_local]);
+            float mx = -INFINITY;
+            if (have) {
+                tmem_wait_ld();
+                if (owes) {                                                 // the previous tile's P is in TMEM
+                    tmem_wait_st();
+                    tc_fence_before();
+                    if (lane == 0) mbar_arrive(B.p_full(sb_before));
+                }
+                if (j >= j_tail || j < j_head) {
+                    const unsigned long long vis = vis_word(it.key_begin + j * kTile + sb_wg, anc[0], lo_row[0]);
+                    mask_chunk(x0, (uint32_t)vis);
+                    mask_chunk(x1, (uint32_t)(vis >> 32));
+                }
+                mx = fmaxf(chunk_max(x0), chunk_max(x1));
+            }
+            const bool moves = __any_sync(0xffffffffu, mx > limit) != 0;
+            if (__builtin_expect(moves || !have || j == 0, 0)) {
+                // The two warps of the pair meet: one whose row has outgrown its reference, and its partner, wherever that
+                // stands (it runs at most to the scores that wait for this warp's P), or both at their end.
+                const float mine = mx > limit ? mx : -INFINITY;
+                xch[wg * 128 + row_local] = mine;
+                if (lane == 0) {
+                    tile_s[warp] = j;
+                    if (moves) meet_s[warp & 3] = 1;
+                }
+                if (!pair_or(pair_id, moves || j == 0)) break;              // both are through
+                const float cand = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
+                const int j_other = tile_s[warp ^ 4], j_done = min(j, j_other);
+                const bool moved = cand > -INFINITY;
                 float alpha = 1.f;
-                if (cand > -INFINITY) {
+                if (moved) {
                     alpha = (m_ref[0] == -INFINITY) ? 0.f : ex2((m_ref[0] - cand) * c2);
                     m_ref[0] = cand;
                     l_run[0] *= alpha;
+                    limit = cand + thr;
+                    mc = cand * c2;
                 }
-                if (j > 0 && __any_sync(0xffffffffu, cand > -INFINITY)) {     // O holds earlier tiles: rescale this half of it
-                    // every earlier tile's product has been added (they complete in order)
-                    if (!mbar_wait_warp(B.o_done(0, j - 1), ((j - 1) >> 2) & 1)) { ok = false; break; }
+                if (j_done > 0 || j > j_other) {
+                    // the accumulator holds the tiles before j_done (this half of it), and P of this warp's further tiles waits
+                    // for the partner's
+                    if (j_done > 0 && ok) ok = mbar_wait_warp(B.o_done(0, j_done - 1), ((j_done - 1) >> 2) & 1);
                     tc_fence_after();
-                    const uint32_t o_addr = lane_addr + kOCol + sb_wg;
                     #pragma unroll 1
-                    for (int ch = 0; ch < 4; ++ch) {
+                    for (int ch = 0; j_done > 0 && ch < 4; ++ch) {
+                        const uint32_t o_addr = lane_addr + kOCol + sb_wg + ch * 16;
                         float o[16];
-                        tmem_ld16(o_addr + ch * 16, o);
+                        tmem_ld16(o_addr, o);
                         tmem_wait_ld();
                         #pragma unroll
                         for (int c = 0; c < 16; ++c) o[c] *= alpha;
-                        tmem_st16(o_addr + ch * 16, reinterpret_cast<uint32_t*>(o));
+                        tmem_st16(o_addr, reinterpret_cast<uint32_t*>(o));
                     }
+                    #pragma unroll 1
+                    for (int t = 2 * j_done; t < 2 * j; ++t) {
+                        const uint32_t p_addr = lane_addr + ((t >> 1) % NSB) * 128 + sb_wg + 16 * (t & 1);
+                        uint32_t p[16];
+                        tmem_ld16(p_addr, reinterpret_cast<float*>(p));
+                        tmem_wait_ld();
+                        #pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            p[c] = pack_bf16x2(__uint_as_float(p[c] << 16) * alpha, __uint_as_float(p[c] & 0xffff0000u) * alpha);
+                        tmem_st16(p_addr, p);
+                    }
+                    tmem_wait_st();
+                    tc_fence_before();
                 }
+                if (lane == 0) meet_s[warp & 3] = 0;
+                pair_or(pair_id + 4u, false);                               // everything is rescaled, everybody has read
+                if (!have) continue;
             }
             // p = 2^(s c2 - m c2), row sum from the unrounded p, P (bf16) over this thread's own scores
-            const float mc = (m_ref[0] == -INFINITY) ? 0.f : m_ref[0] * c2;
-            float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-            exp_chunk(x0, c2, mc, sum4, x_addr);
-            exp_chunk(x1, c2, mc, sum4, x_addr + 16);
-            l_run[0] += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-            if (j + 1 < n_tiles) {                                     // request the next tile's scores
-                if (!mbar_wait_warp(B.s_full((j + 1) % NSB), (uint32_t)((j + 1) / NSB) & 1u)) {
-                    ok = false;
-                } else {
-                    tc_fence_after();
-                    const uint32_t s_next = lane_addr + ((j + 1) % NSB) * 128 + sb_wg;
-                    tmem_ld32(s_next, x0);
-                    tmem_ld32(s_next + 32, x1);
-                }
-            }
-            tmem_wait_st();                                            // this tile's P is in TMEM
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(B.p_full(sb));
+            const uint64_t neg_mc2 = pair_of(-mc, -mc);
+            uint64_t sum[2] = {0ull, 0ull};
+            const uint32_t x_addr = lane_addr + sb * 128 + sb_wg;           // this thread's scores, then its P
+            exp_chunk(x0, c22, neg_mc2, sum, x_addr);
+            sb_before = sb;
+            ++j;
+            if (++sb == NSB) { sb = 0; s_parity ^= 1u; }
+            const uint32_t s_next = lane_addr + sb * 128 + sb_wg;
+            have = j < n_tiles && __all_sync(0xffffffffu, mbar_test_wait(B.s_full(sb), s_parity));
+            tc_fence_after();
+            if (have) tmem_ld32(s_next, x0);
+            exp_chunk(x1, c22, neg_mc2, sum, x_addr + 16);
+            if (have) tmem_ld32(s_next + 32, x1);
+            l_run[0] += sum_of(sum);
+            owes = true;
         }
         }
         // ---- epilogue: normalised partial output + natural-log LSE -------------------------------
@@ -1048,9 +1156,16 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // warpgroup's own block.
         const int blk = NB == 1 ? 0 : wg;
         const int dim0 = NB == 1 ? 64 * wg : 0;
-        if constexpr (NB == 1) xch[wg * 128 + row_local] = l_run[0];       // the two halves' sums meet (the maxima are already the same)
+        // Partial rows are staged as they lie in the workspace ([row][272 bytes]: an odd number of 16-byte
+        // chunks, so a warp's rows do not share banks) and leave as one bulk copy per block: the copy's own
+        // completion orders them ahead of the publication, where ordinary stores needed a second pass
+        // and a proxy fence.  The staging area is the Q blocks and the start of the K ring: every Q K^T
+        // completed ahead of the product waited for below (the Q blocks are free with the last scores).
+        unsigned char* stage = q_sm + blk * (kBlockRows * kRowBytes);
+        float* tail = reinterpret_cast<float*>(stage + row_local * kRowBytes + kD * 2);      // LSE and 12 bytes of padding
+        if constexpr (NB == 1) tail[1 + wg] = l_run[0];                    // the two halves' sums meet (the maxima are already the same)
         softmax_bar_sync();
-        const float l_all = NB == 1 ? l_run[0] + xch[(wg ^ 1) * 128 + row_local] : my_l;
+        const float l_all = NB == 1 ? tail[1] + tail[2] : my_l;
         const float m_fin = NB == 1 ? m_ref[0] : my_m;
         const bool my_row = NB == 1 ? row_ok[0] : (wg ? row_ok[NB - 1] : row_ok[0]);
         const int my_t = (block0 + blk) * tpb + row_local / qg;
@@ -1061,12 +1176,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         if (tid == 0) SPARROW_STAMP(6);                                // last product complete
         ok = ok && *write_ok == 1u;                                    // (thread 0 settled it before the barrier above)
         const int h_row = it.kvh * qg + g_row;
-        // Partial rows are staged as they lie in the workspace ([row][272 bytes]: an odd number of 16-byte
-        // chunks, so a warp's rows do not share banks) and leave as one bulk copy per block: the copy's own
-        // completion orders them ahead of the publication, where ordinary stores needed a second pass
-        // and a proxy fence.  The staging area is the Q blocks and the start of the K ring: every Q K^T
-        // completed ahead of the product waited for above.
-        unsigned char* stage = q_sm + blk * (kBlockRows * kRowBytes);
         if (ok && my_row) {
             if (wg == 0 || NB == 2) {
                 if (direct) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + my_t] = lse_val;

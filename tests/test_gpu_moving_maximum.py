@@ -1,0 +1,55 @@
+"""Rows whose largest score keeps growing along the keys: the softmax's reference has to move in the middle of a piece,
+in either half of a tile, with the halves of a row at different tiles, and by more than an fp32 exponent holds."""
+import pytest
+import torch
+
+from paper_2602_15318_b200 import binding as B
+from paper_2602_15318_b200 import workloads as W
+
+from gpu_util import TOL_LSE, compare, oracle_verify
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+KV = 1800
+
+# P and the output are rounded to bf16 (2^-9 relative each) and a partial row to fp16 (2^-12); where a few keys hold the whole
+# weight nothing averages out: |v| <= 4.3 times the sum of the three.
+TOL = 4.3 * (2 ** -9 + 2 ** -9 + 2 ** -12)
+
+
+def _profile(kind, n):
+    """Added to every key's first component; one unit is about 2^1 in the weight of a row with +8 there."""
+    j = torch.arange(n)
+    tile, low = j // 128, (j % 128) < 64
+    if kind == "stairs": return 20.0 * tile                                # every tile, both halves at once
+    if kind == "low": return torch.where(low, 24.0 * (tile // 2), 0.0)     # the lower halves only, every other tile
+    if kind == "high": return torch.where(low, 0.0, 24.0 * (tile // 3))    # the upper halves only
+    if kind == "turns": return torch.where(low, 18.0 * tile, 18.0 * tile + 9.0)
+    if kind == "cliff": return torch.where(j == n - 300, 250.0, 0.0)       # one key, by more than 2^126
+    if kind == "falls": return -20.0 * tile                                # (rows with the other sign climb)
+    if kind == "late": return torch.where(j >= n - 20, 60.0, 0.0)          # among the last keys
+    return torch.zeros(n)
+
+
+@pytest.mark.parametrize("alone", [False, True])
+@pytest.mark.parametrize("T,hq,hkv", [(16, 28, 4), (30, 28, 4), (3, 8, 8)])
+def test_growing_scores(T, hq, hkv, alone):
+    kinds = ["stairs", "low", "high", "turns", "cliff", "falls", "late", "none"]
+    case = W.make_verify_case(8300 + T, [KV] * len(kinds), T, "random", DEV, hq=hq, hkv=hkv)
+    for b, kind in enumerate(kinds):
+        case.k[b, :, :KV + T, 0] = _profile(kind, KV + T).to(DEV, torch.bfloat16)
+    sign = torch.tensor([8.0, 0.0, -8.0], device=DEV)
+    rows = torch.arange(hq, device=DEV)[None, :] + torch.arange(T, device=DEV)[:, None]       # neighbours differ
+    case.q[..., 0] = sign[rows % 3].to(torch.bfloat16)
+    ctx = B.Context.for_cache(case.k, W.SCALE, n_q_heads=hq)
+    ctx.set_plan_policy(B.PLAN_THROUGHPUT)
+    out = torch.full_like(case.q, float("nan"))
+    lse = torch.full((case.B, hq, T), float("nan"), dtype=torch.float32, device=DEV)
+    if alone:
+        B.sparrow_verify_attn(ctx, case.q, case.k, case.v, case.kv_len, case.parents, T, out, lse)
+    else:                                                                  # (pieces of up to 15 tiles)
+        B.sparrow_verify_attn_batch(ctx, B.VerifyBatch([(case.q, case.k, case.v, case.kv_len, case.parents, T, out, lse)]))
+    torch.cuda.synchronize()
+    assert ctx.last_device_status() == 0
+    d_out, d_lse = compare(out, lse, *oracle_verify(case))
+    assert d_out <= TOL and d_lse <= TOL_LSE, (d_out, d_lse)
