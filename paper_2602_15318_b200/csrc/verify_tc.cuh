@@ -93,6 +93,7 @@ constexpr int kStageBytes = 4 * kSubTileBytes;   // K (32 KB) + V (32 KB)
 constexpr int kRowBytes = kPartRowHalves * 2;    // a partial row: 272 bytes
 constexpr int kMiscBytes = 2048;                 // barriers, flags, ancestor words, maxima exchange
 constexpr uint32_t kSpinLimit = 1u << 22;        // polls before a wait gives up
+constexpr int kPrefetchTiles = 2;                // brought into L2 ahead of the wait for the predecessor
 constexpr float kRescaleLog2 = 16.0f;             // lazy-max threshold in log2 units
 
 // Rows received from the CTAs of a cluster lie in the ring's last stage; with two row blocks (up to 256 rows and
@@ -170,6 +171,12 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
         ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar), "l"(policy) : "memory");
+}
+// Brings a box into L2 only: a hint, which neither reads nor orders anything.
+__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int c0, int c1, int c2, int c3, uint64_t policy)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %3, %4}], %5;"
+                 ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(policy) : "memory");
 }
 // 1-D bulk copy global -> shared (16-byte aligned, size a multiple of 16), completion on an mbarrier
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
@@ -617,6 +624,21 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         tma_load_4d(dst, &tmap_v, 0, row, it.kvh, it.b, B.v_full(st), stream_policy);
         tma_load_4d(dst + kSubTileBytes, &tmap_v, 64, row, it.kvh, it.b, B.v_full(st), stream_policy);
     };
+
+    // The first tiles are on their way into L2 while the kernel waits to be released behind its predecessor (1.7 us), which may
+    // still write them: the loads behind the wait find what it wrote, in L2 like everything else.  Two tiles: 26,112 keys alone
+    // 17.4 -> 16.9 us, three sequences of 9,001 21.6 -> 20.2, caches that L2 holds as before; one tile 16.9 and 21.1, three
+    // 17.7 and 20.9, all of them 19.6 and 23.3 (the loads queue behind them).  Row groups share their tiles: the first one's items ask.
+    if (warp == kGateWarp && lane == 0 && sync.wait_first == 1 && it.group == 0) {
+        #pragma unroll 1
+        for (int j = 0; j < n_tiles && j < kPrefetchTiles; ++j) {
+            const int row = it.key_begin + j * kTile;
+            tma_prefetch_4d(&tmap_k, 0, row, it.kvh, it.b, stream_policy);
+            tma_prefetch_4d(&tmap_k, 64, row, it.kvh, it.b, stream_policy);
+            tma_prefetch_4d(&tmap_v, 0, row, it.kvh, it.b, stream_policy);
+            tma_prefetch_4d(&tmap_v, 64, row, it.kvh, it.b, stream_policy);
+        }
+    }
 
     // ---- setup: barriers, TMEM.  Nothing here waits for an earlier kernel: every warp runs on to its own first
     // wait before the loads start.  With the wait and the first loads in front of the CTA barrier the MMA
