@@ -26,10 +26,11 @@
 // of the receiver: 0.9 us less per step than a cluster barrier), after which all CTAs take the same
 // decision; while the sums travel, the rows of the child that is tested next are already on their way
 // into registers.  The partial sums also tell which CTA holds the bonus token.
-// Measured on a 32-node tree over 151,936 entries (kernel time; the walk's length depends on the
-// uniforms): 16 to 35 us with clusters of 16; one CTA per sequence, with the rows read again from L2 in
-// every pass and the serial scan of the draw, took 145 to 420 us.  Stamps of a level: 1.1 us to turn
-// two rows into fixed point, 0.5 us to request the next, 0.9 us for the cluster's sum.
+// Measured on a 32-node tree over 151,936 entries (back to back; the walk's length depends on the
+// uniforms): 14 to 22 us with clusters of 16; one CTA per sequence, with the rows read again from L2 in
+// every pass and the serial scan of the draw, took 145 to 420 us.  Stamps: a level 0.8 us to turn two rows into fixed point
+// (1.0 a value at a time), 0.3 us to request the next (0.4 with 4-byte loads), 0.95 us for the cluster's sum and 0.4 for the
+// decision; a rejection 0.15 to 0.5 us in front of the pass, 1.0 for it (1.25 with single entries), the sum, the decision; the draw 1.4.
 #pragma once
 #include "verify_tc.cuh"
 
@@ -57,6 +58,41 @@ __device__ __forceinline__ uint32_t fixed_prob(float p)
     return r;
 }
 
+// The same for N values at once, in place (the bits of f become the weights); returns their sum.  y = p 2^30 + 1/2 keeps everything
+// that matters of p: as unsigned words the y of ordinary small weights lie below 2^23's, and a negative p, a NaN or a
+// weight of 2^-7 or more anywhere among them shows as a larger one; only then is each of them looked at.  Half the instructions
+// a value of the function above.
+template <int N>
+__device__ __forceinline__ long long fixed_probs(float (&f)[N])
+{
+    static_assert(N <= 256, "N small weights fit 32 bits");
+    uint32_t most = 0;
+    #pragma unroll
+    for (int k = 0; k < N; ++k) {
+        f[k] = __fmaf_rd(f[k], 1073741824.0f, 0.5f);
+        most = max(most, __float_as_uint(f[k]));
+    }
+    if (most < 0x4B000000u) {
+        uint32_t sum = 0;
+        #pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const uint32_t r = __float_as_uint(__fadd_rd(f[k], 8388608.0f)) - 0x4B000000u;
+            f[k] = __uint_as_float(r);
+            sum += r;
+        }
+        return sum;
+    }
+    long long sum = 0;
+    #pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const float y = fminf(fmaxf(f[k], 0.f), 1073741824.0f);              // (NaN: 0)
+        const uint32_t r = y < 8388608.0f ? __float_as_uint(__fadd_rd(y, 8388608.0f)) - 0x4B000000u : (uint32_t)y;
+        f[k] = __uint_as_float(r);
+        sum += r;
+    }
+    return sum;
+}
+
 // Rows whose sums stay below this (1 + 2^-7 in fixed point) keep every residual weight below 2^31, through
 // up to 64 rejections: P' <= (B P) / 2^30 and A' <= (B A) / 2^30, and (1 + 2^-7)^64 < 1.7.
 constexpr long long kPlainSum = (1ll << kProbBits) + (1ll << (kProbBits - 7));
@@ -64,17 +100,16 @@ constexpr long long kPlainSum = (1ll << kProbBits) + (1ll << (kProbBits - 7));
 struct Level {                      // history of the rejections at the current node
     long long A[kMaxT], B[kMaxT];
     int x[kMaxT];
-    int n;
 };
 
 // Current residual target weight and current draft weight of an entry with original weights P0, Q0
-// at vocabulary index v.
-__device__ __forceinline__ void weights_at(uint32_t P0, uint32_t Q0, int v, const Level& lv, long long* P_out, long long* Q_out)
+// at vocabulary index v, after the level's first n rejections.
+__device__ __forceinline__ void weights_at(uint32_t P0, uint32_t Q0, int v, const Level& lv, int n, long long* P_out, long long* Q_out)
 {
     long long P = P0;
     const long long q0 = Q0;
     bool gone = false;               // v was a rejected candidate: the draft distribution has lost it
-    for (int s = 0; s < lv.n; ++s) {
+    for (int s = 0; s < n; ++s) {
         const long long Q = gone ? 0ll : q0;
         if (lv.B[s] > 0) {
             const long long d = lv.B[s] * P - lv.A[s] * Q;
@@ -85,6 +120,9 @@ __device__ __forceinline__ void weights_at(uint32_t P0, uint32_t Q0, int v, cons
     *P_out = P;
     *Q_out = gone ? 0ll : q0;
 }
+
+// Entries of the vocabulary that a CTA of the cluster owns (the last ones fewer, or none): whole quads.
+__host__ __device__ __forceinline__ int entries_per_cta(int V, int n_cta) { return ((V + n_cta - 1) / n_cta + 3) & ~3; }
 
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -126,19 +164,20 @@ __device__ __forceinline__ long long warp_sum(long long v)
     return (long long)(lo + (mid << 27) + (hi << 54));
 }
 
-// Sums (a, b) over the cluster; every thread gets the totals, sh.part[step & 1] the CTAs' shares.
+// Sums (a, b), or a alone (b is 0), over the cluster; every thread gets the totals, sh.part[step & 1] the CTAs' shares.
 // False when the peers' pushes did not arrive within the poll limit.
+template <bool BOTH>
 __device__ __forceinline__ bool cluster_sum(Shared& sh, long long& a, long long& b, int n_cta, uint32_t rank, uint32_t step)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     a = warp_sum(a);
-    b = warp_sum(b);
-    if (lane == 0) { sh.red[0][warp] = a; sh.red[1][warp] = b; }
+    if (BOTH) b = warp_sum(b);
+    if (lane == 0) { sh.red[0][warp] = a; if (BOTH) sh.red[1][warp] = b; }
     __syncthreads();
     if (warp == 0) {
         if (lane == 0) tc::mbar_expect_tx(tc::smem_u32(&sh.bar[step & 1]), 16u * (uint32_t)n_cta);
         a = warp_sum(lane < kWarps ? sh.red[0][lane] : 0ll);
-        b = warp_sum(lane < kWarps ? sh.red[1][lane] : 0ll);
+        if (BOTH) b = warp_sum(lane < kWarps ? sh.red[1][lane] : 0ll);
         if (lane < n_cta) push_2x64(&sh.part[step & 1][rank][0], &sh.bar[step & 1], (uint32_t)lane, a, b);
     }
     // A slot is written again two steps later, by a CTA that has by then received this CTA's push of the
@@ -155,6 +194,9 @@ __device__ __forceinline__ bool cluster_sum(Shared& sh, long long& a, long long&
     return ok;
 }
 
+// VEC: a thread takes four neighbouring entries at a time, with 16-byte loads (rows that start on 16-byte boundaries: the vocabulary is
+// a multiple of four); otherwise single ones, 512 apart.
+template <bool VEC>
 __global__ void __launch_bounds__(kThreads)
 accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
                      const float* p_target, const float* p_draft,
@@ -162,11 +204,19 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
                      int32_t* path, int32_t* n_accept, int32_t* bonus, unsigned* status)
 {
     let_dependents_launch();
-    extern __shared__ uint2 row_s[];                   // the first `resident` entries of this CTA's slice: (P, Q) fixed point
+    // the first `resident` entries of this CTA's slice, fixed point: all P, then all Q (VEC), or pairs
+    extern __shared__ uint4 row_mem[];
+    uint32_t* const P_s = reinterpret_cast<uint32_t*>(row_mem);
+    uint32_t* const Q_s = P_s + resident;
+    uint2* const PQ_s = reinterpret_cast<uint2*>(row_mem);
+    auto put = [&](int i, uint32_t P, uint32_t Q) {
+        if (VEC) { P_s[i] = P; Q_s[i] = Q; } else PQ_s[i] = make_uint2(P, Q);
+    };
+    auto held = [&](int i) -> uint2 { return VEC ? make_uint2(P_s[i], Q_s[i]) : PQ_s[i]; };
     __shared__ Shared sh;
     const int b = blockIdx.x / n_cta, tid = threadIdx.x;
     const uint32_t rank = n_cta > 1 ? cluster_rank() : 0u;
-    const int per_cta = (V + n_cta - 1) / n_cta;
+    const int per_cta = entries_per_cta(V, n_cta);
     const int v_begin = min(V, (int)rank * per_cta), n_mine = min(V, v_begin + per_cta) - v_begin;
     const int n_res = min(n_mine, resident);
     const float* p_seq = p_target + (size_t)b * (T + 1) * V;       // row r of this sequence: p_seq + r V
@@ -174,14 +224,27 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
 
     // the first kAhead entries per thread of a row pair, on their way
     float fp[kAhead], fq[kAhead];
+    // entry of register k of those
+    auto entry_of = [&](int k) -> int { return VEC ? ((k >> 2) * kThreads + tid) * 4 + (k & 3) : k * kThreads + tid; };
     auto fetch_row = [&](int r) {
         const float* pt = p_seq + (size_t)r * V + v_begin;
         const float* pq = q_seq + (size_t)r * V + v_begin;
-        #pragma unroll
-        for (int k = 0; k < kAhead; ++k) {
-            const int i = k * kThreads + tid;
-            fp[k] = i < n_mine ? ld_behind(pt + i) : 0.f;
-            fq[k] = i < n_mine ? ld_behind(pq + i) : 0.f;
+        if (VEC) {
+            #pragma unroll
+            for (int k = 0; k < kAhead; k += 4) {
+                const int i = entry_of(k);                          // (n_mine is a multiple of four)
+                uint4 p4 = make_uint4(0u, 0u, 0u, 0u), q4 = p4;
+                if (i < n_mine) { p4 = ld_behind(reinterpret_cast<const uint4*>(pt + i)); q4 = ld_behind(reinterpret_cast<const uint4*>(pq + i)); }
+                fp[k] = __uint_as_float(p4.x); fp[k + 1] = __uint_as_float(p4.y); fp[k + 2] = __uint_as_float(p4.z); fp[k + 3] = __uint_as_float(p4.w);
+                fq[k] = __uint_as_float(q4.x); fq[k + 1] = __uint_as_float(q4.y); fq[k + 2] = __uint_as_float(q4.z); fq[k + 3] = __uint_as_float(q4.w);
+            }
+        } else {
+            #pragma unroll
+            for (int k = 0; k < kAhead; ++k) {
+                const int i = entry_of(k);
+                fp[k] = i < n_mine ? ld_behind(pt + i) : 0.f;
+                fq[k] = i < n_mine ? ld_behind(pq + i) : 0.f;
+            }
         }
     };
     if (tid == 0) {
@@ -223,45 +286,58 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
         // (the row pair of node cur is in fp / fq, or on its way there)
         const float* pt = p_seq + (size_t)(cur + 1) * V + v_begin;
         const float* pq = q_seq + (size_t)(cur + 1) * V + v_begin;
-        bool reread = false;                           // row_s no longer holds what is asked for
-        bool in_place = false;                         // row_s holds the current residual weights, not the original ones
+        bool reread = false;                           // the row in shared memory is no longer what is asked for
+        bool in_place = false;                         // it holds the current residual weights, not the original ones
+        int n_rej = 0;                                 // rejections so far
         // entry i of this CTA's slice
         auto entry = [&](int i) -> uint2 {
-            return i < n_res && !reread ? row_s[i] : make_uint2(fixed_prob(ld_behind(pt + i)), fixed_prob(ld_behind(pq + i)));
+            return i < n_res && !reread ? held(i) : make_uint2(fixed_prob(ld_behind(pt + i)), fixed_prob(ld_behind(pq + i)));
         };
         // weights of entry i now
         auto weights = [&](int i, long long* P, long long* Q) {
             const uint2 e = entry(i);
             if (in_place) { *P = e.x; *Q = e.y; }
-            else weights_at(e.x, e.y, v_begin + i, sh.lv, P, Q);
+            else weights_at(e.x, e.y, v_begin + i, sh.lv, n_rej, P, Q);
         };
         long long A = 0, Bq = 0;
-        #pragma unroll
-        for (int k0 = 0; k0 < kAhead; k0 += 3) {                   // (three weights fit 32 bits)
-            uint32_t a3 = 0, b3 = 0;
+        if (VEC) {
+            A = fixed_probs(fp);
+            Bq = fixed_probs(fq);                                  // (entries past the slice are zeros)
             #pragma unroll
-            for (int k = k0; k < k0 + 3 && k < kAhead; ++k) {
-                const int i = k * kThreads + tid;
-                const uint2 e = make_uint2(fixed_prob(fp[k]), fixed_prob(fq[k]));
-                if (i < n_res) row_s[i] = e;
-                a3 += e.x;
-                b3 += e.y;
+            for (int k = 0; k < kAhead; k += 4) {
+                const int i = entry_of(k);
+                if (i < n_res) {                                   // (n_res is a multiple of four)
+                    *reinterpret_cast<float4*>(P_s + i) = make_float4(fp[k], fp[k + 1], fp[k + 2], fp[k + 3]);
+                    *reinterpret_cast<float4*>(Q_s + i) = make_float4(fq[k], fq[k + 1], fq[k + 2], fq[k + 3]);
+                }
             }
-            A += a3;
-            Bq += b3;
+        } else {
+            #pragma unroll
+            for (int k0 = 0; k0 < kAhead; k0 += 3) {               // (three weights fit 32 bits)
+                uint32_t a3 = 0, b3 = 0;
+                #pragma unroll
+                for (int k = k0; k < k0 + 3 && k < kAhead; ++k) {
+                    const int i = entry_of(k);
+                    const uint2 e = make_uint2(fixed_prob(fp[k]), fixed_prob(fq[k]));
+                    if (i < n_res) PQ_s[i] = e;
+                    a3 += e.x;
+                    b3 += e.y;
+                }
+                A += a3;
+                Bq += b3;
+            }
         }
         #pragma unroll 8
         for (int i = kAhead * kThreads + tid; i < n_mine; i += kThreads) {
             const uint2 e = make_uint2(fixed_prob(ld_behind(pt + i)), fixed_prob(ld_behind(pq + i)));
-            if (i < n_res) row_s[i] = e;
+            if (i < n_res) put(i, e.x, e.y);
             A += e.x;
             Bq += e.y;
         }
         if (level == 0 && tid < T) { sh.node_P[tid] = fixed_prob(node_p); sh.node_Q[tid] = fixed_prob(node_q); }
         int c = next_child(cur, cur + 1);
         if (c >= 0) fetch_row(c + 1);
-        if (tid == 0) sh.lv.n = 0;
-        ok = cluster_sum(sh, A, Bq, n_cta, rank, step++);
+        ok = cluster_sum<true>(sh, A, Bq, n_cta, rank, step++);
         if (tid < n_cta) sh.row_part[tid] = sh.part[(step - 1) & 1][tid][0];
         // The residual replaces the row where nothing can leave 32 bits.
         in_place = n_res == n_mine && A <= kPlainSum && Bq <= kPlainSum;
@@ -272,7 +348,7 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
             const int x = sh.tok[c];
             const bool in = x >= 0 && x < V;
             long long Px = 0, Qx = 0;
-            if (in) weights_at(sh.node_P[c], sh.node_Q[c], x, sh.lv, &Px, &Qx);
+            if (in) weights_at(sh.node_P[c], sh.node_Q[c], x, sh.lv, n_rej, &Px, &Qx);
             else if (tid == 0 && rank == 0) atomicOr(status, kStatTree);        // a token outside the vocabulary is never accepted
             const unsigned __int128 lhs = (unsigned __int128)sh.u_node[c] * (unsigned long long)Qx * (unsigned long long)A;
             const unsigned __int128 rhs = ((unsigned __int128)(unsigned long long)Px * (unsigned long long)Bq) << 32;
@@ -280,20 +356,38 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
             // rejected: the level's history grows by (A, B, x); the new A is the sum of the new residual
             const int sibling = next_child(cur, c + 1);
             if (sibling >= 0) fetch_row(sibling + 1);
-            __syncthreads();                                       // everybody has read the history as it was
-            if (tid == 0) { sh.lv.A[sh.lv.n] = A; sh.lv.B[sh.lv.n] = Bq; sh.lv.x[sh.lv.n] = in ? x : -1; sh.lv.n += 1; }
-            __syncthreads();
+            if (tid == 0) { sh.lv.A[n_rej] = A; sh.lv.B[n_rej] = Bq; sh.lv.x[n_rej] = in ? x : -1; }
+            ++n_rej;
+            // (read behind the barriers of the sum below, but where the pass itself reads it or there is none)
+            if (!in_place || Bq <= 0) __syncthreads();
             if (Bq > 0) {
                 long long s = 0, none = 0;
                 if (in_place) {
                     const uint32_t A0 = (uint32_t)A, B0 = (uint32_t)Bq;
-                    #pragma unroll 5
-                    for (int i = tid; i < n_mine; i += kThreads) {
-                        const uint2 e = row_s[i];
-                        const long long d = (long long)((unsigned long long)B0 * e.x) - (long long)((unsigned long long)A0 * e.y);
-                        const uint32_t P = d > 0 ? (uint32_t)(d >> kProbBits) : 0u;
-                        row_s[i] = make_uint2(P, v_begin + i == x ? 0u : e.y);
-                        s += P;
+                    auto residual = [&](uint32_t P, uint32_t Q) -> uint32_t {
+                        const long long d = (long long)((unsigned long long)B0 * P) - (long long)((unsigned long long)A0 * Q);
+                        return d > 0 ? (uint32_t)(d >> kProbBits) : 0u;
+                    };
+                    if (VEC) {
+                        #pragma unroll 5
+                        for (int i = 4 * tid; i < n_mine; i += 4 * kThreads) {
+                            uint4 P = *reinterpret_cast<const uint4*>(P_s + i);
+                            const uint4 Q = *reinterpret_cast<const uint4*>(Q_s + i);
+                            P = make_uint4(residual(P.x, Q.x), residual(P.y, Q.y), residual(P.z, Q.z), residual(P.w, Q.w));
+                            *reinterpret_cast<uint4*>(P_s + i) = P;
+                            s += (long long)((unsigned long long)P.x + P.y) + (long long)((unsigned long long)P.z + P.w);
+                        }
+                        // the draft distribution loses x, by the thread that has just read it
+                        const int at = x - v_begin;
+                        if (in && at >= 0 && at < n_mine && (at >> 2) % kThreads == tid) Q_s[at] = 0u;
+                    } else {
+                        #pragma unroll 5
+                        for (int i = tid; i < n_mine; i += kThreads) {
+                            const uint2 e = PQ_s[i];
+                            const uint32_t P = residual(e.x, e.y);
+                            PQ_s[i] = make_uint2(P, v_begin + i == x ? 0u : e.y);
+                            s += P;
+                        }
                     }
                 } else {
                     for (int i = tid; i < n_mine; i += kThreads) {
@@ -303,7 +397,7 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
                     }
                 }
                 a_step = step;
-                ok = cluster_sum(sh, s, none, n_cta, rank, step++);
+                ok = cluster_sum<false>(sh, s, none, n_cta, rank, step++);
                 A = s;
             }
             Bq -= Qx;
@@ -322,9 +416,8 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
         // nobody accepted: draw the next token from the residual (the original row if nothing is left of it)
         const bool original = A == 0;
         if (original) {
-            __syncthreads();
-            if (tid == 0) sh.lv.n = 0;
-            __syncthreads();
+            __syncthreads();                                       // (row_part is there)
+            n_rej = 0;
             reread = in_place;                                     // the residuals have replaced the row
             in_place = false;
             A = 0;

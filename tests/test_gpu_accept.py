@@ -211,3 +211,32 @@ def test_accept_sample_slices(batch, T, vocab, sharp, scale):
         ref_path, ref_bonus = oracle.sample_accept(tok[b], par[b], p[b], q[b], u_node[b], u_bonus[b])
         assert path[b].tolist() == ref_path + [-1] * (T - len(ref_path))
         assert int(n_acc[b]) == len(ref_path) and int(bonus[b]) == ref_bonus
+
+
+@pytest.mark.parametrize("vocab", [1024, 1023, 16384, 16382, 16381])        # whole quads (one CTA, two or more), and not
+def test_accept_sample_odd_probabilities(vocab):
+    """Values that are no probabilities (clamped) and the bounds between the ways of rounding, anywhere in a row; rows that are
+    not aligned to 16 bytes although the vocabulary is a multiple of four.  Bit-exact."""
+    T = 6
+    tok, par, p, q, u_node, u_bonus = _sampling_problem(9800 + vocab, 1, T, vocab, 0.3)
+    odd = np.array([np.nan, -0.5, -1e-12, 2.0, np.inf, -np.inf, 1.0, 2.0 ** -7, np.nextafter(np.float32(2.0 ** -7), np.float32(0)),
+                    2.0 ** -31, np.nextafter(np.float32(2.0 ** -31), np.float32(0)), 1e-40, -0.0], np.float32)
+    rng = np.random.default_rng(vocab)
+    for r in range(1, T + 1, 2):                                            # (every other row: the rest stays ordinary)
+        n = int(rng.integers(1, len(odd)))
+        p[0, r, rng.choice(vocab, n, replace=False)] = rng.choice(odd, n, replace=False)
+        q[0, r, rng.choice(vocab, n, replace=False)] = rng.choice(odd, n, replace=False)
+    clamped = [np.clip(np.nan_to_num(x, nan=0.0, posinf=1.0, neginf=0.0), 0.0, 1.0) for x in (p, q)]
+    ref_path, ref_bonus = oracle.sample_accept(tok[0], par[0], clamped[0][0], clamped[1][0], u_node[0], u_bonus[0])
+    ctx = B.Context(1, 128, W.HKV * 128 * W.D, 128 * W.D, W.SCALE)
+    d = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32, device=DEV)
+    for shift in (0, 1):
+        held = [torch.zeros(x.size + 1, dtype=torch.float32, device=DEV) for x in (p, q)]
+        pd, qd = (h[shift:shift + x.size].view(x.shape) for h, x in zip(held, (p, q)))
+        pd.copy_(torch.from_numpy(p)); qd.copy_(torch.from_numpy(q))
+        path, n_acc, bonus = d([[99] * T]), d([99]), d([99])
+        B.sparrow_accept_sample(ctx, d(tok), d(par), pd, qd, _u32(u_node), _u32(u_bonus), vocab, T, path, n_acc, bonus)
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == 0
+        assert path[0].tolist() == ref_path + [-1] * (T - len(ref_path))
+        assert int(n_acc[0]) == len(ref_path) and int(bonus[0]) == ref_bonus
