@@ -1094,6 +1094,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 // stands (it runs at most to the scores that wait for this warp's P), or both at their end.
                 const float mine = mx > limit ? mx : -INFINITY;
                 xch[wg * 128 + row_local] = mine;
+                // (at the end the sums meet, behind the row as it is staged below: every Q K^T is complete, Q's place is free)
+                if (j == n_tiles) reinterpret_cast<float*>(q_sm + row_local * kRowBytes + kD * 2)[1 + wg] = l_run[0];
                 if (lane == 0) {
                     tile_s[warp] = j;
                     if (moves) meet_s[warp & 3] = 1;
@@ -1181,12 +1183,12 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // Partial rows are staged as they lie in the workspace ([row][272 bytes]: an odd number of 16-byte
         // chunks, so a warp's rows do not share banks) and leave as one bulk copy per block: the copy's own
         // completion orders them ahead of the publication, where ordinary stores needed a second pass
-        // and a proxy fence.  The staging area is the Q blocks and the start of the K ring: every Q K^T
-        // completed ahead of the product waited for below (the Q blocks are free with the last scores).
+        // and a proxy fence.  The staging area is the Q blocks and the start of the K ring: every Q K^T of the one block has
+        // completed with its last scores; with two, the other block's may not have.
         unsigned char* stage = q_sm + blk * (kBlockRows * kRowBytes);
-        float* tail = reinterpret_cast<float*>(stage + row_local * kRowBytes + kD * 2);      // LSE and 12 bytes of padding
-        if constexpr (NB == 1) tail[1 + wg] = l_run[0];                    // the two halves' sums meet (the maxima are already the same)
-        softmax_bar_sync();
+        float* tail = reinterpret_cast<float*>(stage + row_local * kRowBytes + kD * 2);
+        if constexpr (NB == 2) softmax_bar_sync();
+        // (one row block: the halves' sums met with the pair's last barrier; the maxima are the same)
         const float l_all = NB == 1 ? tail[1] + tail[2] : my_l;
         const float m_fin = NB == 1 ? m_ref[0] : my_m;
         const bool my_row = NB == 1 ? row_ok[0] : (wg ? row_ok[NB - 1] : row_ok[0]);
@@ -1196,14 +1198,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         if (ok) ok = mbar_wait_warp(B.o_done(blk, n_tiles - 1), ((n_tiles - 1) >> 2) & 1);    // the last product is in
         tc_fence_after();
         if (tid == 0) SPARROW_STAMP(6);                                // last product complete
-        ok = ok && *write_ok == 1u;                                    // (thread 0 settled it before the barrier above)
         const int h_row = it.kvh * qg + g_row;
-        if (ok && my_row) {
-            if (wg == 0 || NB == 2) {
-                if (direct) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + my_t] = lse_val;
-                else *reinterpret_cast<float*>(stage + row_local * kRowBytes + kD * 2) = lse_val;
-            }
-        }
+        const bool has_lse = my_row && (wg == 0 || NB == 2);
+        if (ok && has_lse && !direct) *tail = lse_val;
         if (ok) {
             #pragma unroll 1
             for (int col = dim0; col < dim0 + (NB == 1 ? 64 : 128); col += 32) {
@@ -1228,7 +1225,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
         if (!direct) fence_proxy_async();                              // the staged rows, ahead of the bulk copies
         softmax_bar_sync();                                            // every row is staged
+        ok = ok && *write_ok == 1u;                                    // (thread 0 settled it ahead of the barrier)
         if (direct) {
+            if (ok && has_lse) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + my_t] = lse_val;
             // final rows: 16 threads write a row's 256 bytes (a row per thread took 2 us longer)
             #pragma unroll
             for (int bk = 0; bk < NB; ++bk) {
