@@ -167,7 +167,7 @@ __device__ __forceinline__ long long warp_sum(long long v)
 // Sums (a, b), or a alone (b is 0), over the cluster; every thread gets the totals, sh.part[step & 1] the CTAs' shares.
 // False when the peers' pushes did not arrive within the poll limit.
 template <bool BOTH>
-__device__ __forceinline__ bool cluster_sum(Shared& sh, long long& a, long long& b, int n_cta, uint32_t rank, uint32_t step)
+__device__ __forceinline__ bool sum_over_cluster(Shared& sh, long long& a, long long& b, int n_cta, uint32_t rank, uint32_t step)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     a = warp_sum(a);
@@ -192,6 +192,16 @@ __device__ __forceinline__ bool cluster_sum(Shared& sh, long long& a, long long&
         b += s.y;
     }
     return ok;
+}
+
+__device__ __forceinline__ bool cluster_sum(Shared& sh, long long& a, long long& b, int n_cta, uint32_t rank, uint32_t step)
+{
+    return sum_over_cluster<true>(sh, a, b, n_cta, rank, step);
+}
+__device__ __forceinline__ bool cluster_sum(Shared& sh, long long& a, int n_cta, uint32_t rank, uint32_t step)
+{
+    long long none = 0;
+    return sum_over_cluster<false>(sh, a, none, n_cta, rank, step);
 }
 
 // VEC: a thread takes four neighbouring entries at a time, with 16-byte loads (rows that start on 16-byte boundaries: the vocabulary is
@@ -337,7 +347,7 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
         if (level == 0 && tid < T) { sh.node_P[tid] = fixed_prob(node_p); sh.node_Q[tid] = fixed_prob(node_q); }
         int c = next_child(cur, cur + 1);
         if (c >= 0) fetch_row(c + 1);
-        ok = cluster_sum<true>(sh, A, Bq, n_cta, rank, step++);
+        ok = cluster_sum(sh, A, Bq, n_cta, rank, step++);
         if (tid < n_cta) sh.row_part[tid] = sh.part[(step - 1) & 1][tid][0];
         // The residual replaces the row where nothing can leave 32 bits.
         in_place = n_res == n_mine && A <= kPlainSum && Bq <= kPlainSum;
@@ -361,7 +371,7 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
             // (read behind the barriers of the sum below, but where the pass itself reads it or there is none)
             if (!in_place || Bq <= 0) __syncthreads();
             if (Bq > 0) {
-                long long s = 0, none = 0;
+                long long s = 0;
                 if (in_place) {
                     const uint32_t A0 = (uint32_t)A, B0 = (uint32_t)Bq;
                     auto residual = [&](uint32_t P, uint32_t Q) -> uint32_t {
@@ -397,7 +407,7 @@ accept_sample_kernel(const int32_t* draft_tokens, const int32_t* parents,
                     }
                 }
                 a_step = step;
-                ok = cluster_sum<false>(sh, s, none, n_cta, rank, step++);
+                ok = cluster_sum(sh, s, n_cta, rank, step++);
                 A = s;
             }
             Bq -= Qx;
