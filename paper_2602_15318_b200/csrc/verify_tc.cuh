@@ -18,18 +18,21 @@
 //                        stored back with tcgen05.st.
 //                        One row block (T <= 18): the two threads with the same lane (warps w and
 //                        w + 4, one scheduler) share a row, warpgroup g taking key columns [64 g, 64 g + 64) of every
-//                        tile, with its P over its own scores.  They use the same reference maximum, taken from
-//                        the first tile, and run apart from one another: what one does besides its exponentials
-//                        is filled by the exponentials of the other.  A reference moves only where a score exceeds it by
-//                        more than 2^16 (P and its sums are floating point: nothing is lost before that); then
-//                        the pair meets at a barrier, the halves' maxima meet in shared memory, and O and the P that is
-//                        still waiting are rescaled in TMEM.  Each thread sums its own columns; the halves'
-//                        sums meet once, in the epilogue.
+//                        tile, with its P over its own scores.  They use the same reference maximum and run apart from one
+//                        another, by a tile at most: what one does besides its exponentials is filled by the
+//                        exponentials of the other.  A reference only moves when a score exceeds it by more than
+//                        2^16; the warp that finds one says so and goes on, and its partner follows
+//                        before it hands over P of that tile (softmax_pair.cuh: no barrier but in the first tile and at the end).
+//                        Each thread sums its own columns; the halves' sums meet once, in the epilogue.
 //                        Cycles per tile (41 tiles a CTA, 20 CTAs): 1,985 with a barrier of all softmax warps in every tile, 1,880
 //                        with one between the two of a pair, 1,600 without; the exponentials alone are 1,024, the
 //                        products 1,030 (a wait at a barrier that is complete costs the issuing warp another 100,
 //                        three or four times a tile).  Two warps that issue products, one for S and one for O, take 1,450,
 //                        but start a lone call 0.2 us later and gain nothing there.
+//                        References that move, 16,384 keys, 64 nodes, us (a barrier of all in every tile in brackets): nothing
+//                        moves 22.8 (25.1), one key in 700 stands out 23.5 (25.6), one half outgrows the reference in every
+//                        second tile 24.2 (27.2), both halves of every row in every tile 31.8 (28.6: there P of a half is
+//                        rescaled as well, and each waits for what the other posts).
 //                        Two row blocks: warpgroup g owns block g, one thread per row and all 128
 //                        keys of a tile, and works through its block's tiles on its own (no
 //                        barrier between the warpgroups); per block the chain is scores -> softmax
@@ -65,6 +68,7 @@
 
 #include "combine.cuh"
 #include "common.cuh"
+#include "softmax_pair.cuh"
 
 namespace sparrow {
 
@@ -410,17 +414,10 @@ __device__ __forceinline__ float sum_of(const uint64_t (&sum)[2])
     return a + b;
 }
 
-// Barriers between the two softmax warps that share a scheduler and 32 rows (ids 4 to 11), with an OR of a predicate.
-__device__ __forceinline__ bool pair_or(uint32_t id, bool pred)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %2, 0;\n\t"
-        "bar.red.or.pred q, %1, 64, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r) : "r"(id), "r"((uint32_t)pred) : "memory");
-    return r != 0;
-}
+// Barriers between the two softmax warps that share a scheduler and 32 rows (ids 4 to 11).
+__device__ __forceinline__ void pair_sync(uint32_t id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+// What is on reference m, brought to reference m_new >= m (raw scores; none yet: -inf).
+__device__ __forceinline__ float rescale(float m, float m_new, float c2) { return m == m_new ? 1.f : m == -INFINITY ? 0.f : ex2((m - m_new) * c2); }
 
 // Shared-memory addresses of the mbarriers (8-byte slots).  K and V tiles have their own full /
 // empty pairs: a K tile is released as soon as its last S = Q K^T has been computed, a V tile
@@ -439,12 +436,12 @@ struct Bars {
     __device__ __forceinline__ uint32_t fin() const { return base + 152u; }       // finishers' bulk copies
     // Completion of O += P V of key tile j on row block blk: a ring of four barriers per block,
     // tile j on barrier j % 4 with phase parity (j / 4) & 1.  The softmax only looks at it when a
-    // row maximum moves and in the epilogue, asking for the last tile that both halves of the row have handed
-    // over.  A parity wait is only meaningful for the phase in progress or the one just completed; here the
+    // row maximum moves and in the epilogue, asking for the last tile that this warp has handed over and its partner has
+    // or will on its own.  A parity wait is only meaningful for the phase in progress or the one just completed; here the
     // barrier is in exactly that state: with tile t asked for, its previous use (tile t - 4) completed before the
     // scores of tile t, which the warp has seen (the tensor pipe completes in issue order and they
-    // were issued after the product of tile t - 3), and its next use (tile t + 4) needs P that this warp or its
-    // partner has yet to make.
+    // were issued after the product of tile t - 3), and its next use (tile t + 4) needs P that this warp
+    // has yet to hand over.
     __device__ __forceinline__ uint32_t o_done(int blk, int j) const { return base + 160u + 32u * (uint32_t)blk + 8u * (uint32_t)(j & 3); }
 };
 
@@ -577,9 +574,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(misc + 228);
     volatile uint32_t* write_ok = reinterpret_cast<volatile uint32_t*>(misc + 232);   // the counters allow global writes
     volatile int32_t* fin_go = reinterpret_cast<volatile int32_t*>(misc + 236);       // finishers: their waits succeeded
-    // one row block, in slots of barriers that only two blocks use: [4] a warp of the pair waits for its partner; [8] where the warps stand
-    volatile int32_t* meet_s = reinterpret_cast<volatile int32_t*>(misc + 240);
-    volatile int32_t* tile_s = reinterpret_cast<volatile int32_t*>(misc + 192);
+    // one row block, in slots of barriers that only two blocks use: [8] what the softmax warps have posted (see pair_word)
+    volatile int32_t* pair_s = reinterpret_cast<volatile int32_t*>(misc + 192);
     unsigned long long* anc_s = reinterpret_cast<unsigned long long*>(misc + kBarrierBytes);   // [64]
     int32_t* par_s = reinterpret_cast<int32_t*>(misc + 768);                          // [64]: parents in the prologue, then the rows' first visible keys
     float* xch = reinterpret_cast<float*>(misc + 1024);                               // [2][128] maxima / sums exchange
@@ -655,7 +651,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             mbar_init(B.p_full(3), 4);
             for (int i = 0; i < 4; ++i) mbar_init(B.o_done(1, i), 1);
         } else {
-            for (int i = 0; i < 4; ++i) meet_s[i] = 0;
+            for (int i = 0; i < 8; ++i) pair_s[i] = 0;
         }
         mbar_init(B.q_full(), 1);
         mbar_init(B.fin(), 1);
@@ -1041,7 +1037,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             }
         } else {
         // One row block: the two warpgroups split a tile's 128 keys; thread = one row, 64 keys.  The two warps that share
-        // 32 rows run apart from one another and meet only where a reference has to move (see the head of this file).
+        // 32 rows run apart from one another, by a tile at most (softmax_pair.cuh).
         const int sb_wg = 64 * wg;
         const uint32_t pair_id = 4u + (uint32_t)(warp & 3);
         float x0[32], x1[32];
@@ -1051,117 +1047,145 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // scores above this need a new reference.  (Rows of padding hold whatever the Q box left there: they never do.)
         float limit = row_ok[0] ? -INFINITY : INFINITY;
         float mc = 0.f;                                                     // reference in log2 units, 0 as long as there is none
-        int j = 0, sb = 0, sb_before = 0;                                   // tile, its S block, the S block of the tile before
-        uint32_t s_parity = 0;
-        bool have = false, owes = false;                                    // tile j's scores are requested; P of tile j - 1 is not handed over
+        float m_acc = -INFINITY;                                            // what the accumulator is on; m_ref: what this tile's P is on
+        int sb = 0;                                                         // the tile's S block
+        uint32_t s_parity = 0, moved = 0;                                   // moved: bit 0 in this tile, bit 1 in the one before
+        bool have = false, owes = false;                                    // the tile's scores are requested; P of the tile before is not handed over
+        uint32_t p_bar = 0;                                                 // (its barrier)
+        auto hand_over = [&]() {
+            tmem_wait_st();
+            tc_fence_before();
+            if (lane == 0) mbar_arrive(p_bar);
+        };
+        auto post = [&](float mine) {                                       // (the partner has read what was posted before)
+            xch[wg * 128 + row_local] = mine;
+            __threadfence_block();
+            __syncwarp();
+        };
         #pragma unroll 1
-        for (;;) {
-            if (__builtin_expect(!have, 0)) {
-                // not there when the tile before looked for them, or no tile is left
-                if (owes) {
-                    tmem_wait_st();
-                    tc_fence_before();
-                    if (lane == 0) mbar_arrive(B.p_full(sb_before));
-                    owes = false;
-                }
-                #pragma unroll 1
-                for (uint32_t i = 0; j < n_tiles; ++i) {
-                    if (__all_sync(0xffffffffu, mbar_try_wait(B.s_full(sb), s_parity))) { have = true; break; }
-                    if (__any_sync(0xffffffffu, meet_s[warp & 3] != 0)) break;
-                    if (i >= kSpinLimit) { ok = false; j = n_tiles; }
-                }
+        for (int j = 0; j < n_tiles; ++j) {
+            if (__builtin_expect(!have, 0)) {                               // not there when the tile before looked for them
+                if (owes) { hand_over(); owes = false; }
+                ok = __all_sync(0xffffffffu, mbar_wait_warp(B.s_full(sb), s_parity));
                 tc_fence_after();
-                if (have) { tmem_ld32(lane_addr + sb * 128 + sb_wg, x0); tmem_ld32(lane_addr + sb * 128 + sb_wg + 32, x1); }
-            }
-            float mx = -INFINITY;
-            if (have) {
-                tmem_wait_ld();
-                if (owes) {                                                 // the previous tile's P is in TMEM
-                    tmem_wait_st();
-                    tc_fence_before();
-                    if (lane == 0) mbar_arrive(B.p_full(sb_before));
+                if (!ok) {
+                    if (j == 0) { post(-INFINITY); pair_sync(pair_id); }
+                    break;
                 }
-                if (j >= j_tail || j < j_head) {
-                    const unsigned long long vis = vis_word(it.key_begin + j * kTile + sb_wg, anc[0], lo_row[0]);
-                    mask_chunk(x0, (uint32_t)vis);
-                    mask_chunk(x1, (uint32_t)(vis >> 32));
-                }
-                mx = fmaxf(chunk_max(x0), chunk_max(x1));
+                tmem_ld32(lane_addr + sb * 128 + sb_wg, x0);
+                tmem_ld32(lane_addr + sb * 128 + sb_wg + 32, x1);
             }
-            const bool moves = __any_sync(0xffffffffu, mx > limit) != 0;
-            if (__builtin_expect(moves || !have || j == 0, 0)) {
-                // The two warps of the pair meet: one whose row has outgrown its reference, and its partner, wherever that
-                // stands (it runs at most to the scores that wait for this warp's P), or both at their end.
+            tmem_wait_ld();
+            if (owes) hand_over();                                          // (behind the loads: 41 tiles 46.4 -> 45.1 us)
+            if (j >= j_tail || j < j_head) {
+                const unsigned long long vis = vis_word(it.key_begin + j * kTile + sb_wg, anc[0], lo_row[0]);
+                mask_chunk(x0, (uint32_t)vis);
+                mask_chunk(x1, (uint32_t)(vis >> 32));
+            }
+            const float mx = fmaxf(chunk_max(x0), chunk_max(x1));
+            // pass the tile
+            moved <<= 1;
+            if (__builtin_expect(j == 0, 0)) {
                 const float mine = mx > limit ? mx : -INFINITY;
-                xch[wg * 128 + row_local] = mine;
-                // (at the end the sums meet, behind the row as it is staged below: every Q K^T is complete, Q's place is free)
-                if (j == n_tiles) reinterpret_cast<float*>(q_sm + row_local * kRowBytes + kD * 2)[1 + wg] = l_run[0];
-                if (lane == 0) {
-                    tile_s[warp] = j;
-                    if (moves) meet_s[warp & 3] = 1;
-                }
-                if (!pair_or(pair_id, moves || j == 0)) break;              // both are through
-                const float cand = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
-                const int j_other = tile_s[warp ^ 4], j_done = min(j, j_other);
-                const bool moved = cand > -INFINITY;
-                float alpha = 1.f;
-                if (moved) {
-                    alpha = (m_ref[0] == -INFINITY) ? 0.f : ex2((m_ref[0] - cand) * c2);
-                    m_ref[0] = cand;
-                    l_run[0] *= alpha;
-                    limit = cand + thr;
-                    mc = cand * c2;
-                }
-                if (j_done > 0 || j > j_other) {
-                    // the accumulator holds the tiles before j_done (this half of it), and P of this warp's further tiles waits
-                    // for the partner's
-                    if (j_done > 0 && ok) ok = mbar_wait_warp(B.o_done(0, j_done - 1), ((j_done - 1) >> 2) & 1);
-                    tc_fence_after();
+                post(mine);
+                pair_sync(pair_id);
+                m_ref[0] = m_acc = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
+                if (m_acc > -INFINITY) { limit = m_acc + thr; mc = m_acc * c2; }
+                __syncwarp();
+            } else if (__builtin_expect(__any_sync(0xffffffffu, mx > limit), 0)) {
+                if (moved & 2u) {                                           // what this warp posted for the tile before
                     #pragma unroll 1
-                    for (int ch = 0; j_done > 0 && ch < 4; ++ch) {
-                        const uint32_t o_addr = lane_addr + kOCol + sb_wg + ch * 16;
-                        float o[16];
-                        tmem_ld16(o_addr, o);
-                        tmem_wait_ld();
-                        #pragma unroll
-                        for (int c = 0; c < 16; ++c) o[c] *= alpha;
-                        tmem_st16(o_addr, reinterpret_cast<uint32_t*>(o));
+                    for (uint32_t i = 0; ok && !pair_settled(__shfl_sync(0xffffffffu, pair_s[warp ^ 4], 0), j - 1); ++i) {
+                        if (i >= 256) __nanosleep(100);
+                        if (i >= kSpinLimit) ok = false;
                     }
-                    #pragma unroll 1
-                    for (int t = 2 * j_done; t < 2 * j; ++t) {
-                        const uint32_t p_addr = lane_addr + ((t >> 1) % NSB) * 128 + sb_wg + 16 * (t & 1);
-                        uint32_t p[16];
-                        tmem_ld16(p_addr, reinterpret_cast<float*>(p));
-                        tmem_wait_ld();
-                        #pragma unroll
-                        for (int c = 0; c < 16; ++c)
-                            p[c] = pack_bf16x2(__uint_as_float(p[c] << 16) * alpha, __uint_as_float(p[c] & 0xffff0000u) * alpha);
-                        tmem_st16(p_addr, p);
-                    }
-                    tmem_wait_st();
-                    tc_fence_before();
+                    if (!ok) break;
                 }
-                if (lane == 0) meet_s[warp & 3] = 0;
-                pair_or(pair_id + 4u, false);                               // everything is rescaled, everybody has read
-                if (!have) continue;
+                moved |= 1u;
+                const float mine = mx > limit ? mx : -INFINITY;
+                post(mine);
+                if (mine > -INFINITY) {
+                    l_run[0] *= rescale(m_ref[0], mine, c2);
+                    m_ref[0] = mine;
+                    mc = mine * c2;
+                }
             }
+            if (lane == 0) pair_s[warp] = pair_word(j + 1, false, moved);
             // p = 2^(s c2 - m c2), row sum from the unrounded p, P (bf16) over this thread's own scores
             const uint64_t neg_mc2 = pair_of(-mc, -mc);
             uint64_t sum[2] = {0ull, 0ull};
             const uint32_t x_addr = lane_addr + sb * 128 + sb_wg;           // this thread's scores, then its P
+            p_bar = B.p_full(sb);
             exp_chunk(x0, c22, neg_mc2, sum, x_addr);
-            sb_before = sb;
-            ++j;
             if (++sb == NSB) { sb = 0; s_parity ^= 1u; }
             const uint32_t s_next = lane_addr + sb * 128 + sb_wg;
-            have = j < n_tiles && __all_sync(0xffffffffu, mbar_test_wait(B.s_full(sb), s_parity));
+            have = j + 1 < n_tiles && __all_sync(0xffffffffu, mbar_test_wait(B.s_full(sb), s_parity));
             tc_fence_after();
             if (have) tmem_ld32(s_next, x0);
+            int word = pair_s[warp ^ 4];
             exp_chunk(x1, c22, neg_mc2, sum, x_addr + 16);
             if (have) tmem_ld32(s_next + 32, x1);
             l_run[0] += sum_of(sum);
+            // settle it
+            if (__builtin_expect((moved & 1u) || !__all_sync(0xffffffffu, pair_quiet(word, j)), 0)) {
+                #pragma unroll 1
+                for (uint32_t i = 0; ok; ++i) {
+                    word = __shfl_sync(0xffffffffu, pair_s[warp ^ 4], 0);
+                    if (pair_passed(word) > j) break;
+                    if (i >= 256) __nanosleep(100);
+                    if (i >= kSpinLimit) ok = false;
+                }
+                if (!ok) break;
+                const bool other = pair_moved(word, j);
+                if (other || (moved & 1u)) {
+                    float m_new = m_ref[0];
+                    if (other) {
+                        __threadfence_block();
+                        m_new = fmaxf(m_new, xch[(wg ^ 1) * 128 + row_local]);
+                        __syncwarp();
+                        if (lane == 0) pair_s[warp] = pair_word(j + 1, true, moved);
+                    }
+                    const float of_p = rescale(m_ref[0], m_new, c2), of_acc = rescale(m_acc, m_new, c2);
+                    tmem_wait_st();
+                    if (__any_sync(0xffffffffu, of_p != 1.f)) {
+                        #pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t p[16];
+                            tmem_ld16(x_addr + 16 * h, reinterpret_cast<float*>(p));
+                            tmem_wait_ld();
+                            #pragma unroll
+                            for (int c = 0; c < 16; ++c)
+                                p[c] = pack_bf16x2(__uint_as_float(p[c] << 16) * of_p, __uint_as_float(p[c] & 0xffff0000u) * of_p);
+                            tmem_st16(x_addr + 16 * h, p);
+                        }
+                    }
+                    if (j > 0 && __any_sync(0xffffffffu, of_acc != 1.f)) {  // (this half of it)
+                        ok = __all_sync(0xffffffffu, mbar_wait_warp(B.o_done(0, j - 1), ((j - 1) >> 2) & 1));
+                        if (!ok) break;
+                        tc_fence_after();
+                        #pragma unroll 1
+                        for (int ch = 0; ch < 4; ++ch) {
+                            const uint32_t o_addr = lane_addr + kOCol + sb_wg + ch * 16;
+                            float o[16];
+                            tmem_ld16(o_addr, o);
+                            tmem_wait_ld();
+                            #pragma unroll
+                            for (int c = 0; c < 16; ++c) o[c] *= of_acc;
+                            tmem_st16(o_addr, reinterpret_cast<uint32_t*>(o));
+                        }
+                    }
+                    l_run[0] *= of_p;
+                    m_ref[0] = m_acc = m_new;
+                    if (m_new > -INFINITY) { limit = m_new + thr; mc = m_new * c2; }
+                }
+            }
             owes = true;
         }
+        if (owes && ok) hand_over();
+        if (!ok && lane == 0) pair_s[warp] = pair_word(n_tiles, false, 0u);  // (the partner need not wait as well)
+        // The sums meet, behind the row as it is staged below: every Q K^T is complete, Q's place is free.
+        reinterpret_cast<float*>(q_sm + row_local * kRowBytes + kD * 2)[1 + wg] = l_run[0];
+        pair_sync(pair_id + 4u);
         }
         // ---- epilogue: normalised partial output + natural-log LSE -------------------------------
         if (tid == 0) SPARROW_STAMP(5);                                 // softmax loop left

@@ -31,9 +31,7 @@ def _profile(kind, n):
     return torch.zeros(n)
 
 
-@pytest.mark.parametrize("alone", [False, True])
-@pytest.mark.parametrize("T,hq,hkv", [(16, 28, 4), (30, 28, 4), (3, 8, 8)])
-def test_growing_scores(T, hq, hkv, alone):
+def _case(T, hq, hkv):
     kinds = ["stairs", "low", "high", "turns", "cliff", "falls", "late", "none"]
     case = W.make_verify_case(8300 + T, [KV] * len(kinds), T, "random", DEV, hq=hq, hkv=hkv)
     for b, kind in enumerate(kinds):
@@ -41,15 +39,44 @@ def test_growing_scores(T, hq, hkv, alone):
     sign = torch.tensor([8.0, 0.0, -8.0], device=DEV)
     rows = torch.arange(hq, device=DEV)[None, :] + torch.arange(T, device=DEV)[:, None]       # neighbours differ
     case.q[..., 0] = sign[rows % 3].to(torch.bfloat16)
-    ctx = B.Context.for_cache(case.k, W.SCALE, n_q_heads=hq)
-    ctx.set_plan_policy(B.PLAN_THROUGHPUT)
-    out = torch.full_like(case.q, float("nan"))
-    lse = torch.full((case.B, hq, T), float("nan"), dtype=torch.float32, device=DEV)
+    return case
+
+
+def _new(case):
+    return torch.full_like(case.q, float("nan")), torch.full((case.B, case.q.shape[2], case.T), float("nan"), dtype=torch.float32, device=DEV)
+
+
+def _call(ctx, case, outs, alone):
     if alone:
-        B.sparrow_verify_attn(ctx, case.q, case.k, case.v, case.kv_len, case.parents, T, out, lse)
+        for out, lse in outs:
+            B.sparrow_verify_attn(ctx, case.q, case.k, case.v, case.kv_len, case.parents, case.T, out, lse)
     else:                                                                  # (pieces of up to 15 tiles)
-        B.sparrow_verify_attn_batch(ctx, B.VerifyBatch([(case.q, case.k, case.v, case.kv_len, case.parents, T, out, lse)]))
+        B.sparrow_verify_attn_batch(ctx, B.VerifyBatch([(case.q, case.k, case.v, case.kv_len, case.parents, case.T, out, lse) for out, lse in outs]))
     torch.cuda.synchronize()
     assert ctx.last_device_status() == 0
+
+
+@pytest.mark.parametrize("alone", [False, True])
+@pytest.mark.parametrize("T,hq,hkv", [(16, 28, 4), (30, 28, 4), (3, 8, 8)])
+def test_growing_scores(T, hq, hkv, alone):
+    case = _case(T, hq, hkv)
+    ctx = B.Context.for_cache(case.k, W.SCALE, n_q_heads=hq)
+    ctx.set_plan_policy(B.PLAN_THROUGHPUT)
+    out, lse = _new(case)
+    _call(ctx, case, [(out, lse)], alone)
     d_out, d_lse = compare(out, lse, *oracle_verify(case))
     assert d_out <= TOL and d_lse <= TOL_LSE, (d_out, d_lse)
+
+
+@pytest.mark.parametrize("alone", [False, True])
+@pytest.mark.parametrize("T,hq,hkv", [(16, 28, 4), (3, 8, 8)])
+def test_growing_scores_repeat_bit_for_bit(T, hq, hkv, alone):
+    """The warps that share a row come to its tiles in an order that differs from call to call; the bits do not."""
+    case = _case(T, hq, hkv)
+    ctx = B.Context.for_cache(case.k, W.SCALE, n_q_heads=hq)
+    ctx.set_plan_policy(B.PLAN_THROUGHPUT)
+    outs = [_new(case) for _ in range(24)]
+    for _ in range(4):
+        _call(ctx, case, outs, alone)
+        for out, lse in outs[1:]:
+            assert torch.equal(out.view(torch.int16), outs[0][0].view(torch.int16)) and torch.equal(lse, outs[0][1])
