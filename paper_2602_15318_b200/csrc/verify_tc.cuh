@@ -21,7 +21,7 @@
 //                        tile, with its P over its own scores.  They use the same reference maximum and run apart from one
 //                        another, by a tile at most: what one does besides its exponentials is filled by the
 //                        exponentials of the other.  A reference only moves when a score exceeds it by more than
-//                        2^16; the warp that finds one says so and goes on, and its partner follows
+//                        2^8; the warp that finds one says so and goes on, and its partner follows
 //                        before it hands over P of that tile (softmax_pair.cuh: no barrier but in the first tile and at the end).
 //                        Each thread sums its own columns; the halves' sums meet once, in the epilogue.
 //                        Cycles per tile (41 tiles a CTA, 20 CTAs): 1,985 with a barrier of all softmax warps in every tile, 1,880
@@ -30,8 +30,8 @@
 //                        three or four times a tile).  Two warps that issue products, one for S and one for O, take 1,450,
 //                        but start a lone call 0.2 us later and gain nothing there.
 //                        References that move, 16,384 keys, 64 nodes, us (a barrier of all in every tile in brackets): nothing
-//                        moves 22.8 (25.1), one key in 700 stands out 23.5 (25.6), one half outgrows the reference in every
-//                        second tile 24.2 (27.2), both halves of every row in every tile 31.8 (28.6: there P of a half is
+//                        moves 22.7 (25.1), one key in 700 stands out 23.6 (25.6), one half outgrows the reference in every
+//                        second tile 26.0 (27.2), both halves of every row in every tile 31.9 (28.6: there P of a half is
 //                        rescaled as well, and each waits for what the other posts).
 //                        Two row blocks: warpgroup g owns block g, one thread per row and all 128
 //                        keys of a tile, and works through its block's tiles on its own (no
@@ -98,7 +98,10 @@ constexpr int kRowBytes = kPartRowHalves * 2;    // a partial row: 272 bytes
 constexpr int kMiscBytes = 2048;                 // barriers, flags, ancestor words, maxima exchange
 constexpr uint32_t kSpinLimit = 1u << 22;        // polls before a wait gives up
 constexpr int kPrefetchTiles = 2;                // brought into L2 ahead of the wait for the predecessor
-constexpr float kRescaleLog2 = 16.0f;             // lazy-max threshold in log2 units
+// Lazy-max threshold in log2 units.  A key that holds most of a row's weight should be the reference: its P is then 1, otherwise
+// rounded to bf16 while the row is divided by the sum of unrounded ones (one key by 2^9 ... 2^15 above the rest, |v| < 4: out is 7.8e-3
+// off at most with 8, 2.0e-2 with 16).  Where no reference moves the two are equally fast.
+constexpr float kRescaleLog2 = 8.0f;
 
 // Rows received from the CTAs of a cluster lie in the ring's last stage; with two row blocks (up to 256 rows and
 // rounded-up shares) they need a little more behind it.
