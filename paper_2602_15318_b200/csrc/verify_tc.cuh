@@ -1029,12 +1029,14 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 tmem_ld32(s_addr + 32, x1);
                 tmem_wait_st();
                 tc_fence_before();
+                __syncwarp();
                 if (lane == 0) mbar_arrive(B.p_full(blk));
                 tmem_wait_ld();
                 exp_chunk(x0, c22, neg_mc2, sum, s_addr + 64);
                 exp_chunk(x1, c22, neg_mc2, sum, s_addr + 80);
                 tmem_wait_st();
                 tc_fence_before();
+                __syncwarp();
                 if (lane == 0) mbar_arrive(B.p_full(2 + blk));
                 my_l += sum_of(sum);
             }
@@ -1058,6 +1060,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         auto hand_over = [&]() {
             tmem_wait_st();
             tc_fence_before();
+            __syncwarp();
             if (lane == 0) mbar_arrive(p_bar);
         };
         auto post = [&](float mine) {                                       // (the partner has read what was posted before)

@@ -56,6 +56,17 @@ def test_a_cluster_meets_before_its_first_push(name, start):
     assert 0 <= body.find("cluster_wait()") < push
 
 
+def test_a_warp_is_through_with_its_stores_before_one_lane_hands_them_over():
+    """P is stored by all lanes of a warp and handed over by one: every lane's wait and fence stand ahead of that arrival by
+    a barrier of the warp, not by the warp happening to be converged."""
+    softmax = _code("verify_tc.cuh")
+    softmax = softmax[softmax.index("else if (warp < 8) {"):]
+    arrivals = [m.start() for m in re.finditer(r"if \(lane == 0\) mbar_arrive\(", softmax)]
+    assert len(arrivals) == 3
+    for at in arrivals:
+        assert re.search(r"tmem_wait_st\(\);\s*tc_fence_before\(\);\s*__syncwarp\(\);\s*$", softmax[:at])
+
+
 HARNESS = r"""
 #include <cstdio>
 #include <vector>
