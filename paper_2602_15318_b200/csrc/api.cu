@@ -683,7 +683,9 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
 }
 
 // Estimates for the choice of a plan, us: a tile of 128 keys with one / two row blocks, the merges of a lone
-// call, and what an item of a call in a batch costs besides its tiles.
+// call, and what an item of a call in a batch costs besides its tiles.  They were fitted together, over forced choices, to the
+// kernels as they were when a tile took 1.0 and 1.8 us; it takes 0.85 and 1.65 since (long pieces, one call alone), and the fit
+// was not made again.
 constexpr float kTileUs[2] = {1.2f, 2.0f};
 constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 4.f, kTwoBlocksWholeUs = 1.f;
 constexpr float kItemUs[2] = {5.f, 11.f}, kWholeItemUs[2] = {6.5f, 8.5f};      // its rows are merged; it is its unit's only piece
@@ -768,7 +770,7 @@ float lone_cost_of_items(const sparrow_ctx* c, const SplitPlan& p)
 // calls of a batch: a call's bits do not depend on them.
 //
 // A draft block of more than one row block: an item with two of them reads its keys once for both and keeps the
-// tensor pipe fuller on long pieces (2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
+// tensor pipe fuller on long pieces (an estimate of 2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
 // and merge, no empty half where the blocks are odd in number, and twice as many of them fill the chip.
 // Where units are whole an item of two blocks costs less than two items of one, the more so the shorter the
 // sequences (24 sequences of 100 keys, T = 20: 96 items 6.1 us a call in a batch, 192 items 9.8), unless the blocks are odd in

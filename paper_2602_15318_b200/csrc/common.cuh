@@ -232,7 +232,7 @@ inline void piece_range(int n_keys, int ns, int split, int tile, int* begin, int
 
 // Tiles of piece `split` of `ns` over `tiles` tiles as the kernels take them: as even as whole tiles allow, the longer
 // pieces first.  The last one holds the draft block, whose masks and tables already make it the latest (26,112 keys,
-// T = 16: 0.7 us behind pieces of the same six tiles, one tile is 1.1 us).
+// T = 16: 0.7 us behind pieces of the same six tiles, about what one tile takes).
 struct TileRun {
     int first, count;
 };

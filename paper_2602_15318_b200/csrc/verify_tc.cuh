@@ -427,13 +427,14 @@ __device__ __forceinline__ float rescale(float m, float m_new, float c2) { retur
 // only after its last O += P V, so the K stream runs ahead of the V stream.
 struct Bars {
     uint32_t base;
-    // slots of 8 bytes: 0-27 here and in o_done, 30 and 31 below (28 and 29 hold the TMEM address and flags)
+    // slots of 8 bytes: 0-27 here and in o_done, 31 is p_full(3); 28 and 29 hold the TMEM address and flags, 30 is free.
+    // With one row block 31 is free as well, and 24-27 (o_done of the second block) hold the words that the softmax pairs post.
     __device__ __forceinline__ uint32_t k_full(int i) const { return base + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t k_empty(int i) const { return base + 24u + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t v_full(int i) const { return base + 48u + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t v_empty(int i) const { return base + 72u + 8u * (uint32_t)i; }
-    // (a fourth score / P slot, used with two row blocks)
-    __device__ __forceinline__ uint32_t s_full(int i) const { return i < 3 ? base + 96u + 8u * (uint32_t)i : base + 240u; }
+    __device__ __forceinline__ uint32_t s_full(int i) const { return base + 96u + 8u * (uint32_t)i; }
+    // (a fourth, with two row blocks: two halves of P for each)
     __device__ __forceinline__ uint32_t p_full(int i) const { return i < 3 ? base + 120u + 8u * (uint32_t)i : base + 248u; }
     __device__ __forceinline__ uint32_t q_full() const { return base + 144u; }
     __device__ __forceinline__ uint32_t fin() const { return base + 152u; }       // finishers' bulk copies
@@ -572,16 +573,16 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     unsigned char* q_sm = sm;
     unsigned char* kv_sm = sm + NB * kQBlockBytes;
     unsigned char* misc = kv_sm + NS * kStageBytes + recv_extra(NB);
-    uint64_t* bar_mem = reinterpret_cast<uint64_t*>(misc);                  // barriers in bytes 0-223 and 240-255 (see Bars)
+    uint64_t* bar_mem = reinterpret_cast<uint64_t*>(misc);                  // barriers in bytes 0-223 and 248-255 (see Bars)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 224);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(misc + 228);
     volatile uint32_t* write_ok = reinterpret_cast<volatile uint32_t*>(misc + 232);   // the counters allow global writes
     volatile int32_t* fin_go = reinterpret_cast<volatile int32_t*>(misc + 236);       // finishers: their waits succeeded
-    // one row block, in slots of barriers that only two blocks use: [8] what the softmax warps have posted (see pair_word)
+    // one row block, in the slots of barriers that only two blocks use: [8] what the softmax warps have posted (see pair_word)
     volatile int32_t* pair_s = reinterpret_cast<volatile int32_t*>(misc + 192);
     unsigned long long* anc_s = reinterpret_cast<unsigned long long*>(misc + kBarrierBytes);   // [64]
     int32_t* par_s = reinterpret_cast<int32_t*>(misc + 768);                          // [64]: parents in the prologue, then the rows' first visible keys
-    float* xch = reinterpret_cast<float*>(misc + 1024);                               // [2][128] maxima / sums exchange
+    float* xch = reinterpret_cast<float*>(misc + 1024);                               // [2][128] maxima that the halves of a row exchange (one row block)
 
     Bars B;
     SPARROW_TIMELINE_CALL(sync.call);
