@@ -4,13 +4,13 @@
 // whatever the timing: nobody waits for a partner that does not come, and the results do not depend on who came first.
 //
 // A warp *passes* tile j when it has looked at its scores; where one of them has outgrown its row's reference the row's maximum in this
-// half is the warp's own new reference, posted before it passes.  Then it makes P of the tile.  It *settles* the tile when its
+// half is the warp's own new reference, posted as it passes.  Then it makes P of the tile.  It *settles* the tile when its
 // partner has passed it too: the row's reference is now the larger of the two, and P, the sums and this warp's half of the
-// accumulator follow where they were made with another one.  Only then P is handed over, and only then the warp looks at the next
-// tile.  So both look at tile j + 1 with one reference, a function of the scores up to tile j, and every P and every accumulator goes
-// through the same roundings in every order of events.  Neither is ever more than one tile ahead; handing P over later costs
-// nothing, the product needs the partner's half as well; and the partner passes on its own (its scores of tile j stand behind the
-// product of tile j - 3, whose P both have handed over).
+// accumulator follow where they were made with another one.  It passes the next tile and hands P over only behind that.  So
+// both look at tile j + 1 with one reference, a function of the scores up to tile j, and every P and every accumulator goes through the
+// same roundings in every order of events.  Neither is ever more than one tile ahead, and P held back until then costs nothing: the product
+// needs the partner's half as well.  Nobody waits for what waits for him: the scores of tile j stand behind the product of tile j - 3,
+// whose P both hand over when they have passed tile j - 2, and a partner passes tile j - 1 without this warp's P of it.
 // What a warp posts lies there until its partner has read it: with a move in each of two tiles in a row it waits for that.
 // The piece's first tile, in which nearly every row gets its reference, is the exception: there both wait for one another at a
 // barrier before they pass.

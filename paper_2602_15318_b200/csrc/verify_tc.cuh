@@ -30,8 +30,8 @@
 //                        three or four times a tile).  Two warps that issue products, one for S and one for O, take 1,450,
 //                        but start a lone call 0.2 us later and gain nothing there.
 //                        References that move, 16,384 keys, 64 nodes, us (a barrier of all in every tile in brackets): nothing
-//                        moves 22.7 (25.1), one key in 700 stands out 23.6 (25.6), one half outgrows the reference in every
-//                        second tile 26.0 (27.2), both halves of every row in every tile 31.9 (28.6: there P of a half is
+//                        moves 22.2 (25.2), one key in 700 stands out 23.9 (25.7), one half outgrows the reference in every
+//                        second tile 27.2 (27.2), both halves of every row in every tile 32.2 (28.6: there P of a half is
 //                        rescaled as well, and each waits for what the other posts).
 //                        Two row blocks: warpgroup g owns block g, one thread per row and all 128
 //                        keys of a tile, and works through its block's tiles on its own (no
@@ -1055,140 +1055,145 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         float mc = 0.f;                                                     // reference in log2 units, 0 as long as there is none
         float m_acc = -INFINITY;                                            // what the accumulator is on; m_ref: what this tile's P is on
         int sb = 0;                                                         // the tile's S block
-        uint32_t s_parity = 0, moved = 0;                                   // moved: bit 0 in this tile, bit 1 in the one before
-        bool have = false, owes = false;                                    // the tile's scores are requested; P of the tile before is not handed over
-        uint32_t p_bar = 0;                                                 // (its barrier)
-        auto hand_over = [&]() {
-            tmem_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(p_bar);
-        };
+        uint32_t s_parity = 0, moved = 0;                                   // moved: bit 0 in the tile passed last, bit 1 in the one before
+        bool have = false;                                                  // the tile's scores are requested
+        uint32_t p_addr = 0, p_bar = 0;                                     // P of the tile before, which is not handed over, and its barrier
+        int word = 0;                                                       // the partner's
         auto post = [&](float mine) {                                       // (the partner has read what was posted before)
             xch[wg * 128 + row_local] = mine;
             __threadfence_block();
             __syncwarp();
         };
         #pragma unroll 1
-        for (int j = 0; j < n_tiles; ++j) {
-            if (__builtin_expect(!have, 0)) {                               // not there when the tile before looked for them
-                if (owes) { hand_over(); owes = false; }
-                ok = __all_sync(0xffffffffu, mbar_wait_warp(B.s_full(sb), s_parity));
-                tc_fence_after();
-                if (!ok) {
-                    if (j == 0) { post(-INFINITY); pair_sync(pair_id); }
-                    break;
+        for (int j = 0;; ++j) {
+            float mx = -INFINITY;
+            word = pair_s[warp ^ 4];                                        // (looked at below: the scores take longer)
+            if (j < n_tiles) {
+                if (__builtin_expect(!have, 0)) {                           // not there when the tile before looked for them
+                    ok = __all_sync(0xffffffffu, mbar_wait_warp(B.s_full(sb), s_parity));
+                    tc_fence_after();
+                    if (!ok) {
+                        if (j == 0) { post(-INFINITY); pair_sync(pair_id); }
+                        break;
+                    }
+                    tmem_ld32(lane_addr + sb * 128 + sb_wg, x0);
+                    tmem_ld32(lane_addr + sb * 128 + sb_wg + 32, x1);
                 }
-                tmem_ld32(lane_addr + sb * 128 + sb_wg, x0);
-                tmem_ld32(lane_addr + sb * 128 + sb_wg + 32, x1);
+                tmem_wait_ld();
+                if (j >= j_tail || j < j_head) {
+                    const unsigned long long vis = vis_word(it.key_begin + j * kTile + sb_wg, anc[0], lo_row[0]);
+                    mask_chunk(x0, (uint32_t)vis);
+                    mask_chunk(x1, (uint32_t)(vis >> 32));
+                }
+                mx = fmaxf(chunk_max(x0), chunk_max(x1));
             }
-            tmem_wait_ld();
-            if (owes) hand_over();                                          // (behind the loads: 41 tiles 46.4 -> 45.1 us)
-            if (j >= j_tail || j < j_head) {
-                const unsigned long long vis = vis_word(it.key_begin + j * kTile + sb_wg, anc[0], lo_row[0]);
-                mask_chunk(x0, (uint32_t)vis);
-                mask_chunk(x1, (uint32_t)(vis >> 32));
-            }
-            const float mx = fmaxf(chunk_max(x0), chunk_max(x1));
-            // pass the tile
-            moved <<= 1;
-            if (__builtin_expect(j == 0, 0)) {
-                const float mine = mx > limit ? mx : -INFINITY;
-                post(mine);
-                pair_sync(pair_id);
-                m_ref[0] = m_acc = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
-                if (m_acc > -INFINITY) { limit = m_acc + thr; mc = m_acc * c2; }
-                __syncwarp();
-            } else if (__builtin_expect(__any_sync(0xffffffffu, mx > limit), 0)) {
-                if (moved & 2u) {                                           // what this warp posted for the tile before
+            // settle the tile before, pass this one
+            if (__builtin_expect(j == 0 || (moved & 1u) || __any_sync(0xffffffffu, mx > limit || !pair_quiet(word, j - 1)), 0)) {
+                if (j > 0) {
                     #pragma unroll 1
-                    for (uint32_t i = 0; ok && !pair_settled(__shfl_sync(0xffffffffu, pair_s[warp ^ 4], 0), j - 1); ++i) {
+                    for (uint32_t i = 0; ok; ++i) {
+                        word = __shfl_sync(0xffffffffu, pair_s[warp ^ 4], 0);
+                        if (pair_passed(word) >= j) break;
                         if (i >= 256) __nanosleep(100);
                         if (i >= kSpinLimit) ok = false;
                     }
                     if (!ok) break;
+                    const bool other = pair_moved(word, j - 1);
+                    if (other || (moved & 1u)) {
+                        float m_new = m_ref[0];
+                        if (other) {
+                            __threadfence_block();
+                            m_new = fmaxf(m_new, xch[(wg ^ 1) * 128 + row_local]);
+                            __syncwarp();
+                            if (lane == 0) pair_s[warp] = pair_word(j, true, moved);
+                        }
+                        const float of_p = rescale(m_ref[0], m_new, c2), of_acc = rescale(m_acc, m_new, c2);
+                        tmem_wait_st();
+                        if (__any_sync(0xffffffffu, of_p != 1.f)) {
+                            #pragma unroll 1
+                            for (int h = 0; h < 2; ++h) {
+                                uint32_t p[16];
+                                tmem_ld16(p_addr + 16 * h, reinterpret_cast<float*>(p));
+                                tmem_wait_ld();
+                                #pragma unroll
+                                for (int c = 0; c < 16; ++c)
+                                    p[c] = pack_bf16x2(__uint_as_float(p[c] << 16) * of_p, __uint_as_float(p[c] & 0xffff0000u) * of_p);
+                                tmem_st16(p_addr + 16 * h, p);
+                            }
+                        }
+                        if (j > 1 && __any_sync(0xffffffffu, of_acc != 1.f)) {  // (this half of it)
+                            ok = __all_sync(0xffffffffu, mbar_wait_warp(B.o_done(0, j - 2), ((j - 2) >> 2) & 1));
+                            if (!ok) break;
+                            tc_fence_after();
+                            #pragma unroll 1
+                            for (int ch = 0; ch < 4; ++ch) {
+                                const uint32_t o_addr = lane_addr + kOCol + sb_wg + ch * 16;
+                                float o[16];
+                                tmem_ld16(o_addr, o);
+                                tmem_wait_ld();
+                                #pragma unroll
+                                for (int c = 0; c < 16; ++c) o[c] *= of_acc;
+                                tmem_st16(o_addr, reinterpret_cast<uint32_t*>(o));
+                            }
+                        }
+                        l_run[0] *= of_p;
+                        m_ref[0] = m_acc = m_new;
+                        if (m_new > -INFINITY) { limit = m_new + thr; mc = m_new * c2; }
+                    }
                 }
-                moved |= 1u;
+                moved <<= 1;
                 const float mine = mx > limit ? mx : -INFINITY;
-                post(mine);
-                if (mine > -INFINITY) {
-                    l_run[0] *= rescale(m_ref[0], mine, c2);
-                    m_ref[0] = mine;
-                    mc = mine * c2;
+                if (j == 0) {
+                    post(mine);
+                    pair_sync(pair_id);
+                    m_ref[0] = m_acc = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
+                    if (m_acc > -INFINITY) { limit = m_acc + thr; mc = m_acc * c2; }
+                    __syncwarp();
+                } else if (__any_sync(0xffffffffu, mine > -INFINITY)) {
+                    if (moved & 2u) {                                       // what this warp posted for the tile before
+                        #pragma unroll 1
+                        for (uint32_t i = 0; ok && !pair_settled(__shfl_sync(0xffffffffu, pair_s[warp ^ 4], 0), j - 1); ++i) {
+                            if (i >= 256) __nanosleep(100);
+                            if (i >= kSpinLimit) ok = false;
+                        }
+                        if (!ok) break;
+                    }
+                    moved |= 1u;
+                    post(mine);
+                    if (mine > -INFINITY) {
+                        l_run[0] *= rescale(m_ref[0], mine, c2);
+                        m_ref[0] = mine;
+                        mc = mine * c2;
+                    }
                 }
+            } else {
+                moved <<= 1;
             }
-            if (lane == 0) pair_s[warp] = pair_word(j + 1, false, moved);
+            // (the post first: the partner may be waiting for it.  The order and one vote for both questions: 41 tiles alone 44.3 -> 42.5 us,
+            // a call of two tiles 7.04 -> 7.20, where P of the last tile is handed over a little later.)
+            if (lane == 0 && j < n_tiles) pair_s[warp] = pair_word(j + 1, false, moved);
+            if (j > 0) {                                                    // P of the tile before is in TMEM and settled
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(p_bar);
+            }
+            if (j == n_tiles) break;
             // p = 2^(s c2 - m c2), row sum from the unrounded p, P (bf16) over this thread's own scores
             const uint64_t neg_mc2 = pair_of(-mc, -mc);
             uint64_t sum[2] = {0ull, 0ull};
-            const uint32_t x_addr = lane_addr + sb * 128 + sb_wg;           // this thread's scores, then its P
+            p_addr = lane_addr + sb * 128 + sb_wg;                          // this thread's scores, then its P
             p_bar = B.p_full(sb);
-            exp_chunk(x0, c22, neg_mc2, sum, x_addr);
+            exp_chunk(x0, c22, neg_mc2, sum, p_addr);
             if (++sb == NSB) { sb = 0; s_parity ^= 1u; }
             const uint32_t s_next = lane_addr + sb * 128 + sb_wg;
             have = j + 1 < n_tiles && __all_sync(0xffffffffu, mbar_test_wait(B.s_full(sb), s_parity));
             tc_fence_after();
             if (have) tmem_ld32(s_next, x0);
-            int word = pair_s[warp ^ 4];
-            exp_chunk(x1, c22, neg_mc2, sum, x_addr + 16);
+            exp_chunk(x1, c22, neg_mc2, sum, p_addr + 16);
             if (have) tmem_ld32(s_next + 32, x1);
             l_run[0] += sum_of(sum);
-            // settle it
-            if (__builtin_expect((moved & 1u) || !__all_sync(0xffffffffu, pair_quiet(word, j)), 0)) {
-                #pragma unroll 1
-                for (uint32_t i = 0; ok; ++i) {
-                    word = __shfl_sync(0xffffffffu, pair_s[warp ^ 4], 0);
-                    if (pair_passed(word) > j) break;
-                    if (i >= 256) __nanosleep(100);
-                    if (i >= kSpinLimit) ok = false;
-                }
-                if (!ok) break;
-                const bool other = pair_moved(word, j);
-                if (other || (moved & 1u)) {
-                    float m_new = m_ref[0];
-                    if (other) {
-                        __threadfence_block();
-                        m_new = fmaxf(m_new, xch[(wg ^ 1) * 128 + row_local]);
-                        __syncwarp();
-                        if (lane == 0) pair_s[warp] = pair_word(j + 1, true, moved);
-                    }
-                    const float of_p = rescale(m_ref[0], m_new, c2), of_acc = rescale(m_acc, m_new, c2);
-                    tmem_wait_st();
-                    if (__any_sync(0xffffffffu, of_p != 1.f)) {
-                        #pragma unroll 1
-                        for (int h = 0; h < 2; ++h) {
-                            uint32_t p[16];
-                            tmem_ld16(x_addr + 16 * h, reinterpret_cast<float*>(p));
-                            tmem_wait_ld();
-                            #pragma unroll
-                            for (int c = 0; c < 16; ++c)
-                                p[c] = pack_bf16x2(__uint_as_float(p[c] << 16) * of_p, __uint_as_float(p[c] & 0xffff0000u) * of_p);
-                            tmem_st16(x_addr + 16 * h, p);
-                        }
-                    }
-                    if (j > 0 && __any_sync(0xffffffffu, of_acc != 1.f)) {  // (this half of it)
-                        ok = __all_sync(0xffffffffu, mbar_wait_warp(B.o_done(0, j - 1), ((j - 1) >> 2) & 1));
-                        if (!ok) break;
-                        tc_fence_after();
-                        #pragma unroll 1
-                        for (int ch = 0; ch < 4; ++ch) {
-                            const uint32_t o_addr = lane_addr + kOCol + sb_wg + ch * 16;
-                            float o[16];
-                            tmem_ld16(o_addr, o);
-                            tmem_wait_ld();
-                            #pragma unroll
-                            for (int c = 0; c < 16; ++c) o[c] *= of_acc;
-                            tmem_st16(o_addr, reinterpret_cast<uint32_t*>(o));
-                        }
-                    }
-                    l_run[0] *= of_p;
-                    m_ref[0] = m_acc = m_new;
-                    if (m_new > -INFINITY) { limit = m_new + thr; mc = m_new * c2; }
-                }
-            }
-            owes = true;
         }
-        if (owes && ok) hand_over();
         if (!ok && lane == 0) pair_s[warp] = pair_word(n_tiles, false, 0u);  // (the partner need not wait as well)
         // The sums meet, behind the row as it is staged below: every Q K^T is complete, Q's place is free.
         reinterpret_cast<float*>(q_sm + row_local * kRowBytes + kD * 2)[1 + wg] = l_run[0];

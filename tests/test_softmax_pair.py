@@ -29,7 +29,7 @@ struct Overwrites : Kernel { static bool may_post(int, int) { return true; } };
 struct WaitsForPass : Kernel { static bool may_post(int j, int word) { return pair_passed(word) > j; } };
 
 constexpr int kMost = 7, kBlocks = 3;         // tiles; score blocks
-enum { POLL, LOOK, POST, WORK, SETTLE, SETTLED, FIRST, LAST, DONE };
+enum { POLL, SETTLE, LOOK, POST, HAND, WORK, FIRST, LAST, DONE };
 struct Warp { signed char pc, j, handed, ref, acc, moved, cand; };
 struct State {
     Warp w[2];
@@ -70,16 +70,32 @@ Result explore(int n, const signed char (&score)[2][kMost])
             Warp& w = x.w[i];
             const int partner = x.word[i ^ 1], j = w.j;
             switch (w.pc) {
-            case POLL:
-                if (j >= x.landed) continue;
-                w.pc = LOOK;
+            case POLL:                         // (at the end there is no tile to wait for)
+                if (j < n && j >= x.landed) continue;
+                w.pc = j > 0 ? SETTLE : LOOK;
                 break;
+            case SETTLE: {                     // the tile before
+                const int t = j - 1;
+                if (!Rule::may_settle(t, partner)) continue;
+                const bool other = pair_passed(partner) > t && pair_moved(partner, t);
+                if (pair_passed(partner) > t + 2) ++r.wrong;
+                if (!pair_quiet(partner, t) || w.moved) {
+                    signed char ref = w.ref;
+                    if (other) ref = std::max(ref, x.posted[i ^ 1]);
+                    if (ref != w.ref) x.p_ref[i][t][1] = ref + 2;
+                    w.ref = w.acc = ref;
+                    if (other) x.word[i] = pair_word(j, true, w.moved);
+                }
+                x.o_ref[i][t] = w.acc + 2;
+                w.pc = j < n ? LOOK : HAND;
+                break;
+            }
             case LOOK: {
                 const bool moves = score[i][j] > w.ref;
                 w.moved = (w.moved << 1) & 3;
                 if (j == 0) { x.posted[i] = w.cand = score[i][0]; w.pc = FIRST; break; }
                 if (moves) { w.moved |= 1; w.cand = score[i][j]; w.pc = POST; }
-                else { x.word[i] = pair_word(j + 1, false, w.moved); w.pc = WORK; }
+                else { x.word[i] = pair_word(j + 1, false, w.moved); w.pc = HAND; }
                 break;
             }
             case POST:                         // (looked at again and again)
@@ -87,30 +103,16 @@ Result explore(int n, const signed char (&score)[2][kMost])
                 x.posted[i] = w.cand;
                 w.ref = w.cand;
                 x.word[i] = pair_word(j + 1, false, w.moved);
-                w.pc = WORK;
+                w.pc = HAND;
+                break;
+            case HAND:                         // P of the tile before
+                ++w.handed;
+                w.pc = j < n ? WORK : LAST;
                 break;
             case WORK:
                 x.p_ref[i][j][0] = w.ref + 2;
-                w.pc = SETTLE;
-                break;
-            case SETTLE: {
-                if (!Rule::may_settle(j, partner)) continue;
-                const bool other = pair_passed(partner) > j && pair_moved(partner, j);
-                if (pair_passed(partner) > j + 2) ++r.wrong;
-                if (!pair_quiet(partner, j) || w.moved) {
-                    signed char ref = w.ref;
-                    if (other) ref = std::max(ref, x.posted[i ^ 1]);
-                    if (ref != w.ref) x.p_ref[i][j][1] = ref + 2;
-                    w.ref = w.acc = ref;
-                    if (other) x.word[i] = pair_word(j + 1, true, w.moved);
-                }
-                x.o_ref[i][j] = w.acc + 2;
-                w.pc = SETTLED;
-                break;
-            }
-            case SETTLED:
-                ++w.handed; ++w.j;
-                w.pc = w.j < n ? POLL : LAST;
+                ++w.j;
+                w.pc = POLL;
                 break;
             case FIRST:
                 if (i == 1 || x.w[1].pc != FIRST) continue;
