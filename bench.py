@@ -93,7 +93,7 @@ class ClockSampler:
 def kernel_sources_sha256():
     import hashlib
     h = hashlib.sha256()
-    for f in ("verify_tc.cuh", "common.cuh"):
+    for f in ("verify_tc.cuh", "softmax_pair.cuh", "common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2602_15318_b200", "csrc", f), "rb").read())
     return h.hexdigest()
 

@@ -684,7 +684,7 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
 
 // Estimates for the choice of a plan, us: a tile of 128 keys with one / two row blocks, the merges of a lone
 // call, and what an item of a call in a batch costs besides its tiles.  They were fitted together, over forced choices, to the
-// kernels as they were when a tile took 1.0 and 1.8 us; it takes 0.85 and 1.65 since (long pieces, one call alone), and the fit
+// kernels as they were when a tile took 1.0 and 1.8 us; it takes 0.8 and 1.7 since (long pieces, one call alone), and the fit
 // was not made again.
 constexpr float kTileUs[2] = {1.2f, 2.0f};
 constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 4.f, kTwoBlocksWholeUs = 1.f;

@@ -25,7 +25,7 @@
 //                        before it hands over P of that tile (softmax_pair.cuh: no barrier but in the first tile and at the end).
 //                        Each thread sums its own columns; the halves' sums meet once, in the epilogue.
 //                        Cycles per tile (41 tiles a CTA, 20 CTAs): 1,985 with a barrier of all softmax warps in every tile, 1,880
-//                        with one between the two of a pair, 1,600 without; the exponentials alone are 1,024, the
+//                        with one between the two of a pair, 1,540 like this; the exponentials alone are 1,024, the
 //                        products 1,030 (a wait at a barrier that is complete costs the issuing warp another 100,
 //                        three or four times a tile).  Two warps that issue products, one for S and one for O, take 1,450,
 //                        but start a lone call 0.2 us later and gain nothing there.
