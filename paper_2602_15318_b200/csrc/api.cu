@@ -548,8 +548,10 @@ sparrow_status launch_verify_tc(sparrow_ctx* c, const SplitPlan& plan, const Syn
     // before is this context's previous call), or, with wait_first, stream order with the launch and
     // the set-up overlapping the predecessor's end.
     cfg.numAttrs = !sy.enabled ? 0 : plan.cluster > 1 ? 2 : 1;       // (clusters only occur among these)
-    const cudaError_t e = nb == 1 ? cudaLaunchKernelEx(&cfg, tc::verify_tc_kernel<1>, a, sy, plan, mq, mk, mv)
-                                  : cudaLaunchKernelEx(&cfg, tc::verify_tc_kernel<2>, a, sy, plan, mq, mk, mv);
+    const bool clustered = plan.cluster > 1;                         // (only where sy.enabled)
+    auto* const kernel = nb == 1 ? (clustered ? tc::verify_tc_kernel<1, true> : tc::verify_tc_kernel<1, false>)
+                                 : (clustered ? tc::verify_tc_kernel<2, true> : tc::verify_tc_kernel<2, false>);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a, sy, plan, mq, mk, mv);
     if (e != cudaSuccess) return SPARROW_ERR_CUDA;
     c->launches.fetch_add(1);
     return SPARROW_OK;
@@ -653,8 +655,8 @@ const ClusterTable* cluster_table(int device)
     ClusterTable& t = tables[device];
     int expected = 0;
     if (t.state.compare_exchange_strong(expected, 1)) {
-        query_max_clusters(tc::verify_tc_kernel<1>, tc::kThreads, tc::smem_bytes(1, 3), t.n[0]);
-        query_max_clusters(tc::verify_tc_kernel<2>, tc::kThreads, tc::smem_bytes(2, 2), t.n[1]);
+        query_max_clusters(tc::verify_tc_kernel<1, true>, tc::kThreads, tc::smem_bytes(1, 3), t.n[0]);
+        query_max_clusters(tc::verify_tc_kernel<2, true>, tc::kThreads, tc::smem_bytes(2, 2), t.n[1]);
         query_max_clusters(gather::split_gather_kernel, gather::kThreads, gather::kClusterSmemBytes, t.n[2]);
         t.state.store(2);
     }
@@ -692,15 +694,14 @@ constexpr float kItemUs[2] = {5.f, 11.f}, kWholeItemUs[2] = {6.5f, 8.5f};      /
 constexpr float kWaveUs[2] = {6.f, 8.f};                                       // a further wave of a call with more units than SMs
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
-// at most 16 pieces per unit, pieces short enough to leave a stage of the K/V ring free for the rows that are
-// sent around (2 tiles with one row block, 1 with two), and whole clusters per GPC.  Rewrites the plan where
+// at most 16 pieces per unit and whole clusters per GPC.  Rewrites the plan where
 // that is estimated to pay (448 keys, T = 8 9.2 -> 7.4 us; 3,000 keys in 12 pieces of two tiles instead of 24 of one
-// 13.1 -> 9.5).  Returns the estimate.
+// 13.1 -> 9.5; longer pieces than leave a stage of the ring free: 8,000 keys, T = 8 in 16 pieces of 4 tiles
+// instead of 32 of 2 10.9 -> 9.2, 3,000 keys, T = 64 11.8 -> 10.4).  Returns the estimate.
 float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
 {
     const int nb = p->blocks_per_group, units = p->batch * p->n_kv_heads * p->n_groups;
     const float per_tile = nb == 1 ? kTileUs[0] : kTileUs[1];
-    const int free_stage_tiles = nb == 1 ? 2 : 1;
     int most = 0, least = 1 << 30;                     // tiles of the longest and the shortest sequence
     float best = 0.f;
     for (int b = 0; b < p->batch; ++b) {
@@ -715,7 +716,7 @@ float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
     for (int n = 1; may_rewrite && n <= kMaxMergeCluster && n <= least; ++n) {
         const int piece = (most + n - 1) / n;
         if (n == 1 && units > c->n_sm) continue;
-        if (n > 1 && (piece > free_stage_tiles || !c->max_clusters[nb - 1] || units > c->max_clusters[nb - 1][n])) continue;
+        if (n > 1 && (!c->max_clusters[nb - 1] || units > c->max_clusters[nb - 1][n])) continue;
         const float t = per_tile * piece + (n > 1 ? kMergeClusterUs : 0.f);
         if (t < best) { best = t; pieces = n; }
     }
@@ -955,10 +956,10 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
     if (cudaFuncSetAttribute(gather::split_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              gather::kClusterSmemBytes) != cudaSuccess)
         return SPARROW_ERR_CUDA;
-    if (cudaFuncSetAttribute(tc::verify_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::smem_bytes(1, 3)) != cudaSuccess ||
-        cudaFuncSetAttribute(tc::verify_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::smem_bytes(2, 2)) != cudaSuccess)
+    if (cudaFuncSetAttribute(tc::verify_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::smem_bytes(1, 3)) != cudaSuccess ||
+        cudaFuncSetAttribute(tc::verify_tc_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::smem_bytes(1, 3)) != cudaSuccess ||
+        cudaFuncSetAttribute(tc::verify_tc_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::smem_bytes(2, 2)) != cudaSuccess ||
+        cudaFuncSetAttribute(tc::verify_tc_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::smem_bytes(2, 2)) != cudaSuccess)
         return SPARROW_ERR_CUDA;
     if (cudaFuncSetAttribute(sample::accept_sample_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              sample::kMaxResident * (int)sizeof(uint2)) != cudaSuccess ||
@@ -1142,9 +1143,9 @@ sparrow_status sparrow_verify_attn_static(const sparrow_layout* L, const void* q
         if (prop.major != 10) return SPARROW_ERR_ARCH;
         if (cudaFuncSetAttribute(gather::split_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  gather::kClusterSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(tc::verify_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(tc::verify_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  tc::smem_bytes(1, 3)) != cudaSuccess ||
-            cudaFuncSetAttribute(tc::verify_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(tc::verify_tc_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  tc::smem_bytes(2, 2)) != cudaSuccess)
             return SPARROW_ERR_CUDA;
         void* fn = nullptr;

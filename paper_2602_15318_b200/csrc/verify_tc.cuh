@@ -558,7 +558,14 @@ struct MergeList {
 };
 static_assert(sizeof(MergeList) <= kMaxT * 8, "the list lies over the ancestor words");
 
-template <int NB>
+// NB: row blocks of an item.  CL: the call's units are thread-block clusters, which merge their pieces in shared memory;
+// otherwise a piece is final or goes through the workspace.  One kernel for both was 0.4 us slower where a call is
+// short (2,048 keys, T = 8 7.20 -> 6.85 us, 300 keys 6.53 -> 6.29): code that is not there is not fetched.
+//
+// The kernels of one row block must not spill: the stack lies in L2 behind the stream of tiles (nearly all of L1 is shared memory), and
+// 24 bytes of it between the last product and the partial rows took 0.5 us (26,112 keys, T = 16).  What an
+// edge tile needs is therefore read from the tables when it comes and not kept over the loop.
+template <int NB, bool CL>
 __global__ void __launch_bounds__(kBoundThreads, 1)
 verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ SyncArgs sync,
                  const __grid_constant__ SplitPlan plan, const __grid_constant__ CUtensorMap tmap_q,
@@ -670,7 +677,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (plan.cluster > 1) cluster_arrive_relaxed();      // (waited for ahead of the first access to a peer)
+    // (waited for ahead of the first access to a peer.  The rows that peers send come to the ring's last stage: where this piece
+    // uses it, the softmax warps arrive behind their last product.)
+    if (CL && !(warp < 8 && n_tiles >= NS)) cluster_arrive_relaxed();
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 0) SPARROW_STAMP(1);                             // set-up done
 
@@ -896,7 +905,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             // epilogue's critical path.  1 = go, 2 = a wait gave up.
             bool go = wait_counter(sync.fin_done + sync.parity, sync.fin_wait_same);
             if (!go) atomicOr(args.status, timeout_bits(kSiteWriteSame));
-            if (go && (plan.seq[it.b].n_splits == 1 || plan.cluster > 1)) {
+            if (go && (CL || plan.seq[it.b].n_splits == 1)) {
                 go = wait_counter(sync.fin_done + (sync.parity ^ 1), sync.fin_wait_other);
                 if (!go) atomicOr(args.status, timeout_bits(kSiteWriteOther));
             }
@@ -1045,11 +1054,13 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // One row block: the two warpgroups split a tile's 128 keys; thread = one row, 64 keys.  The two warps that share
         // 32 rows run apart from one another, by a tile at most (softmax_pair.cuh).
         const int sb_wg = 64 * wg;
+        auto row_anc = [&]() { return (row_ok[0] && it.key_end > kv_len) ? anc_s[plan.T_tree - T + t_row[0]] : 0ull; };
+        auto row_lo = [&]() { return row_ok[0] ? par_s[t_row[0]] : 0; };
         const uint32_t pair_id = 4u + (uint32_t)(warp & 3);
         float x0[32], x1[32];
         // tiles whose every key is visible to the warp's rows: [j_head, j_tail)
         const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
-        const int j_head = __reduce_max_sync(0xffffffffu, lo_row[0] > it.key_begin ? (lo_row[0] - it.key_begin + kTile - 1) / kTile : 0);
+        const int j_head = __reduce_max_sync(0xffffffffu, row_lo() > it.key_begin ? (row_lo() - it.key_begin + kTile - 1) / kTile : 0);
         // scores above this need a new reference.  (Rows of padding hold whatever the Q box left there: they never do.)
         float limit = row_ok[0] ? -INFINITY : INFINITY;
         float mc = 0.f;                                                     // reference in log2 units, 0 as long as there is none
@@ -1081,7 +1092,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 }
                 tmem_wait_ld();
                 if (j >= j_tail || j < j_head) {
-                    const unsigned long long vis = vis_word(it.key_begin + j * kTile + sb_wg, anc[0], lo_row[0]);
+                    const unsigned long long vis = vis_word(it.key_begin + j * kTile + sb_wg, row_anc(), row_lo());
                     mask_chunk(x0, (uint32_t)vis);
                     mask_chunk(x1, (uint32_t)(vis >> 32));
                 }
@@ -1201,8 +1212,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
         // ---- epilogue: normalised partial output + natural-log LSE -------------------------------
         if (tid == 0) SPARROW_STAMP(5);                                 // softmax loop left
-        const bool direct = plan.seq[it.b].n_splits == 1;                  // the only piece: write the final result
-        const bool clustered = plan.cluster > 1;                           // the unit's pieces meet in the cluster's shared memory
+        const bool direct = !CL && plan.seq[it.b].n_splits == 1;                  // the only piece: write the final result
+        constexpr bool clustered = CL;                           // the unit's pieces meet in the cluster's shared memory
         if (tid == 0) {
             // Global writes start below.  In overlapped mode a lane of the gate warp has been waiting,
             // since the kernel started, for the counters that allow them (see there).
@@ -1233,6 +1244,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const float lse_val = l_all > 0.f ? (m_fin * c2 + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
         if (ok) ok = mbar_wait_warp(B.o_done(blk, n_tiles - 1), ((n_tiles - 1) >> 2) & 1);    // the last product is in
         tc_fence_after();
+        if (CL && n_tiles >= NS) cluster_arrive();                     // the whole ring is idle
         if (tid == 0) SPARROW_STAMP(6);                                // last product complete
         const int h_row = it.kvh * qg + g_row;
         const bool has_lse = my_row && (wg == 0 || NB == 2);
@@ -1289,7 +1301,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         // ---- publish this item; the call's finisher CTAs merge its partials ---------------------------
         // (overlapped mode: arrival words and finisher counters as described at SyncArgs; a
         // stream-ordered call only stores its partials, and a combine kernel follows)
-        const int fin_idx = (int)blockIdx.x - (plan.n_items - sync.n_fin);     // >= 0: this CTA is a finisher
+        const int fin_idx = CL ? -1 : (int)blockIdx.x - (plan.n_items - sync.n_fin);     // >= 0: this CTA is a finisher
         const int rows_per_block = tpb * qg;                            // 126 for 7 heads x 18 tokens
         const int seq_rows = plan.n_kv_heads * qg * T;                  // query rows of a sequence
         // The call's row list: the query rows of every sequence with several pieces, (KV head, row group,
@@ -1302,7 +1314,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
         const int my_begin = fin_idx >= 0 ? min(total, fin_idx * chunk) : 0;
         int share_end = fin_idx >= 0 ? min(total, my_begin + chunk) : 0;       // end of the share being merged
-        const bool merges = my_begin < share_end;
+        const bool merges = !CL && my_begin < share_end;
         MergeList* list = reinterpret_cast<MergeList*>(anc_s);          // (the tables are no longer needed)
         // Fills the list with what one pass merges, from row `row` on: runs of rows of one unit, as many as
         // fit the K/V ring with all their pieces.
@@ -1345,13 +1357,13 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const MergeOut merge_out = {args.out, args.lse, T, args.n_q_heads, qg, plan.inv_group};
         if (clustered) {
             // Every CTA of the cluster merges a share of the unit's rows: it is sent its rows of every piece, one
-            // bulk copy from each peer, into the last stage of the K/V ring, which pieces this short never use.
+            // bulk copy from each peer, into the last stage of the K/V ring.
             const int cl = plan.cluster;
             const int unit_rows = qg * min(NB * tpb, T - block0 * tpb);
             const uint32_t recv = smem_u32(kv_sm) + (NS - 1) * kStageBytes;
             int r_begin;
             const int n = merge_share(unit_rows, it.split, plan.inv_cluster, &r_begin) - r_begin;
-            cluster_wait();                                            // every peer runs, its barriers are initialised
+            cluster_wait();                                            // every peer runs, its barriers are initialised, its last stage is free
             if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n * cl * kRowBytes));
             const int peer = warp + 8 * lane;                          // (spread over the warps: a warp's lanes issue one after the other)
             if (peer < cl) {
@@ -1386,7 +1398,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             if (tid == 0) SPARROW_STAMP(7);                            // partial rows stored
             const bool arrives = !direct && !clustered;
             if (tid == 0 && arrives) publish_counter(arrive_word);
-            if (merges || (sync.lone && arrives)) {
+            if (!CL && (merges || (sync.lone && arrives))) {
                 if (tid == 0) {
                     // every partial of the call in place, and the previous call's final results written
                     // (both words are polled in one loop: the second is usually there already, and a lone
@@ -1483,7 +1495,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     }
 
     // ---- teardown -------------------------------------------------------------------------------
-    if (plan.cluster > 1) {
+    if (CL) {
         // Nobody leaves before its peers have received what it sends them.
         if (warp >= 8) { cluster_wait(); cluster_arrive_relaxed(); }    // (the softmax warps have done both)
         cluster_wait();

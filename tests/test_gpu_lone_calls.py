@@ -41,6 +41,28 @@ def test_verify_alone(hq, hkv, kv_len, T, tree):
         check(out, lse, *ref)
 
 
+@pytest.mark.parametrize("hq,hkv,kv_len,T,tree", [
+    (28, 4, [32 * 128 - 7], 8, "chain"),      # sixteen pieces, one of them of three tiles: only its CTA uses the ring's last stage
+    (28, 4, [33 * 128], 16, "random"),        # two of three tiles
+    (28, 4, [40 * 128 + 1], 18, "random"),    # three tiles, and one with a few keys
+    (28, 4, [16 * 6 * 128 - 9], 9, "chain"),  # six tiles each: the ring goes round twice
+    (28, 4, [3000], 64, "random"),            # sixteen units
+    (28, 4, [1500, 700], 36, "random"),       # two row blocks, more tiles than their ring has stages
+    (28, 4, [2500] * 8, 33, "random"),
+    (8, 8, [6000, 900, 3000], 20, "random"),  # ragged: some pieces leave the last stage alone
+    (16, 1, [5000], 20, "random"),
+])
+def test_long_pieces_in_clusters_repeat_bit_for_bit(hq, hkv, kv_len, T, tree):
+    """Pieces that use the ring stage which their peers' rows come to."""
+    case = W.make_verify_case(7500 + hq + T + kv_len[0], kv_len, T, tree, DEV, hq=hq, hkv=hkv)
+    ctx = B.Context.for_cache(case.k, W.SCALE, n_q_heads=hq)
+    out, lse, _ = run_verify(case, ctx)
+    check(out, lse, *oracle_verify(case))
+    for _ in range(20):
+        again, lse_again, _ = run_verify(case, ctx)
+        assert torch.equal(out, again) and torch.equal(lse, lse_again)
+
+
 def test_verify_alone_back_to_back_and_in_front_of_a_batch():
     """Lone calls of different kinds (cluster, workspace, one piece) and a batch that overlaps its own calls,
     enqueued without synchronisation on one context: every result its own, in the batch bit for bit."""
