@@ -1244,7 +1244,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const float lse_val = l_all > 0.f ? (m_fin * c2 + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
         if (ok) ok = mbar_wait_warp(B.o_done(blk, n_tiles - 1), ((n_tiles - 1) >> 2) & 1);    // the last product is in
         tc_fence_after();
-        if (CL && n_tiles >= NS) cluster_arrive();                     // the whole ring is idle
+        // The whole ring is idle: what peers may write over, the tensor pipe's reads and the loads behind them, is complete by the
+        // barrier above, so there is nothing left for a releasing arrival to order (8,000 keys, T = 8 9.2 -> 9.7 us with one).
+        if (CL && n_tiles >= NS) cluster_arrive_relaxed();
         if (tid == 0) SPARROW_STAMP(6);                                // last product complete
         const int h_row = it.kvh * qg + g_row;
         const bool has_lse = my_row && (wg == 0 || NB == 2);
