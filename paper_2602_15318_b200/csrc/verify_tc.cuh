@@ -25,10 +25,11 @@
 //                        before it hands over P of that tile (softmax_pair.cuh: no barrier but in the first tile and at the end).
 //                        Each thread sums its own columns; the halves' sums meet once, in the epilogue.
 //                        Cycles per tile (41 tiles a CTA, 20 CTAs): 1,985 with a barrier of all softmax warps in every tile, 1,880
-//                        with one between the two of a pair, 1,540 like this; the exponentials alone are 1,024, the
-//                        products 1,030 (a wait at a barrier that is complete costs the issuing warp another 100,
-//                        three or four times a tile).  Two warps that issue products, one for S and one for O, take 1,450,
-//                        but start a lone call 0.2 us later and gain nothing there.
+//                        with one between the two of a pair, 1,540 without, 1,450 with half a tile between the two; the exponentials
+//                        alone are 1,024, the products 1,030 (a wait at a barrier that is complete costs the issuing warp 85 and the
+//                        pipe holds about 100 cycles of work behind the issuing lane, so V is waited for together with P).
+//                        All of it at 1.55 to 1.7 GHz: with all SMs at work the GPU is at its power cap, and a cycle saved is a third of one
+//                        in time.
 //                        References that move, 16,384 keys, 64 nodes, us (a barrier of all in every tile in brackets): nothing
 //                        moves 22.2 (25.2), one key in 700 stands out 23.9 (25.7), one half outgrows the reference in every
 //                        second tile 27.2 (27.2), both halves of every row in every tile 32.2 (28.6: there P of a half is
@@ -97,6 +98,7 @@ constexpr int kStageBytes = 4 * kSubTileBytes;   // K (32 KB) + V (32 KB)
 constexpr int kRowBytes = kPartRowHalves * 2;    // a partial row: 272 bytes
 constexpr int kMiscBytes = 2048;                 // barriers, flags, ancestor words, maxima exchange
 constexpr uint32_t kSpinLimit = 1u << 22;        // polls before a wait gives up
+constexpr uint32_t kPairLag = 512;               // cycles by which the second softmax warp of a pair lags: 64 exponentials of a warp
 constexpr int kPrefetchTiles = 2;                // brought into L2 ahead of the wait for the predecessor
 // Lazy-max threshold in log2 units.  A key that holds most of a row's weight should be the reference: its P is then 1, otherwise
 // rounded to bf16 while the row is divided by the sum of unrounded ones (one key by 2^9 ... 2^15 above the rest, |v| < 4: out is 7.8e-3
@@ -160,6 +162,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     for (uint32_t i = 0; i < kSpinLimit; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
+}
+// Bounded as well, as one piece of code for a warp whose next instruction should follow the phase at once: a wait at a
+// complete barrier costs about 85 cycles, during which the tensor pipe runs out of work.
+__device__ __forceinline__ bool mbar_wait_tight(uint32_t bar, uint32_t parity)
+{
+    uint32_t left;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .u32 i;\n\tmov.u32 i, %3;\n\t"
+        "WAIT:\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t@p bra DONE;\n\t"
+        "sub.u32 i, i, 1;\n\tsetp.ne.u32 p, i, 0;\n\t@p bra WAIT;\n\t"
+        "DONE:\n\tmov.u32 %0, i;\n\t}"
+        : "=r"(left) : "r"(bar), "r"(parity), "n"(kSpinLimit) : "memory");
+    return left != 0;
 }
 // Same for a whole warp.  Every lane polls, so that the warp stays converged and no shuffle stands
 // between the phase flip and the next instruction: a wait-issue-commit round of eight tensor-core
@@ -627,9 +642,17 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const int st = j % NS;
         const uint32_t dst = smem_u32(kv_sm + st * kStageBytes + 2 * kSubTileBytes);
         const int row = it.key_begin + j * kTile;
-        mbar_expect_tx(B.v_full(st), 2 * kSubTileBytes);
-        tma_load_4d(dst, &tmap_v, 0, row, it.kvh, it.b, B.v_full(st), stream_policy);
-        tma_load_4d(dst + kSubTileBytes, &tmap_v, 64, row, it.kvh, it.b, B.v_full(st), stream_policy);
+        uint32_t bar = B.v_full(st);
+        // One row block: V counts on the barrier of its tile's P, so that the product waits once; the last tile's has its own
+        // (its rows past the end are zeroed ahead of P).  The phase is the tile's: its stage is free, so P of the
+        // tile before in it was complete.
+        if (NB == 1) {
+            if (j < n_tiles - 1) bar = B.p_full(st);
+            else mbar_arrive(B.p_full(st));
+        }
+        mbar_expect_tx(bar, 2 * kSubTileBytes);
+        tma_load_4d(dst, &tmap_v, 0, row, it.kvh, it.b, bar, stream_policy);
+        tma_load_4d(dst + kSubTileBytes, &tmap_v, 64, row, it.kvh, it.b, bar, stream_policy);
     };
 
     // The first tiles are on their way into L2 while the kernel waits to be released behind its predecessor (1.7 us), which may
@@ -655,8 +678,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_k) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_v) : "memory");
         for (int i = 0; i < 3; ++i) { mbar_init(B.k_full(i), 1); mbar_init(B.k_empty(i), 1); mbar_init(B.v_full(i), 1); mbar_init(B.v_empty(i), 1); }      // (a tile is read by every block)
-        // one row block: a P block comes from all eight softmax warps; two: from the block's own four
-        for (int i = 0; i < 3; ++i) { mbar_init(B.s_full(i), 1); mbar_init(B.p_full(i), NB == 1 ? 8 : 4); }
+        // one row block: a P block comes from all eight softmax warps and counts its tile's V; two: from the block's own four
+        for (int i = 0; i < 3; ++i) { mbar_init(B.s_full(i), 1); mbar_init(B.p_full(i), NB == 1 ? 9 : 4); }
         for (int i = 0; i < 4; ++i) mbar_init(B.o_done(0, i), 1);
         if (NB == 2) {
             mbar_init(B.p_full(3), 4);
@@ -833,29 +856,33 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 }
                 int ring = 0;                                             // tile modulo 3
                 uint32_t parity = 0;
-                ok = ok && mbar_wait_warp(B.v_full(0), 0);
                 #pragma unroll 1
                 for (int j = 0; j < n_tiles && ok; ++j) {
-                    if (j == n_tiles - 1) zero_v_tail(j);
-                    if (!mbar_wait_warp(B.p_full(ring), parity)) { ok = false; break; }
-                    tc_fence_after();
+                    if (j == n_tiles - 1) {
+                        ok = mbar_wait_warp(B.v_full(ring), 0);
+                        if (!ok) break;
+                        zero_v_tail(j);
+                    }
                     const uint64_t vd = v_desc0 + (uint64_t)((ring * kStageBytes) >> 4);
+                    const uint32_t p_col = tmem_u + ring * 128, o_bar = B.o_done(0, j), v_bar = B.v_empty(ring), k_bar = B.k_full(ring);
+                    const int this_ring = ring;
+                    const uint32_t this_parity = parity;
+                    if (++ring == NS) { ring = 0; parity ^= 1u; }
+                    ok = mbar_wait_tight(B.p_full(this_ring), this_parity);
+                    if (!ok) break;
+                    tc_fence_after();
                     if (elect_one()) {
                         #pragma unroll
                         for (int kk = 0; kk < 8; ++kk)
-                            mma_ts(tmem_u + kOCol, tmem_u + ring * 128 + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)((kk * 2048) >> 4),
+                            mma_ts(tmem_u + kOCol, p_col + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)((kk * 2048) >> 4),
                                    idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
-                        tc_commit(B.o_done(0, j));
-                        tc_commit(B.v_empty(ring));
+                        tc_commit(o_bar);
+                        tc_commit(v_bar);
                     }
                     __syncwarp();
-                    const uint32_t parity_next = parity ^ 1u;
-                    const int this_ring = ring;
-                    if (++ring == NS) { ring = 0; parity = parity_next; }
-                    // (the next tile's V is waited for while the pipe has work)
-                    if (j + 1 < n_tiles && !mbar_wait_warp(B.v_full(ring), parity)) { ok = false; break; }
                     if (j + NS < n_tiles) {                               // the S block and the stage that have become free
-                        if (!mbar_wait_warp(B.k_full(this_ring), this_ring == NS - 1 ? parity : parity_next)) { ok = false; break; }
+                        ok = mbar_wait_tight(k_bar, this_parity ^ 1u);
+                        if (!ok) break;
                         tc_fence_after();
                         issue_qk(this_ring);
                     }
@@ -1159,6 +1186,14 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     pair_sync(pair_id);
                     m_ref[0] = m_acc = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
                     if (m_acc > -INFINITY) { limit = m_acc + thr; mc = m_acc * c2; }
+                    // The second warp of the pair starts half a tile's exponentials late and stays so: what each does besides them
+                    // falls into the other's.  In step, both wait for the exponentials together (41 tiles alone 1,560 -> 1,460
+                    // cycles a tile with the waits of the issuing warp; 8,000 keys, T = 8 9.12 -> 8.81 us, 26,112 keys 16.42 ->
+                    // 16.24, 3,000 keys, T = 64 10.42 -> 10.10).  It costs nothing: they would have shared the unit.
+                    if (wg == 1 && n_tiles > 2) {
+                        const uint32_t c0 = (uint32_t)clock();
+                        while ((uint32_t)clock() - c0 < kPairLag) {}
+                    }
                     __syncwarp();
                 } else if (__any_sync(0xffffffffu, mine > -INFINITY)) {
                     if (moved & 2u) {                                       // what this warp posted for the tile before
