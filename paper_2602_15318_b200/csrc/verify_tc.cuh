@@ -721,9 +721,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             #pragma unroll
             for (int blk = 0; blk < NB; ++blk) {
                 const uint32_t dst = smem_u32(q_sm + blk * kQBlockBytes);
-                const int tok = it.b * T + (block0 + blk) * tpb;
-                tma_load_4d(dst, &tmap_q, 0, 0, it.kvh, tok, B.q_full());
-                tma_load_4d(dst + kSubTileBytes, &tmap_q, 64, 0, it.kvh, tok, B.q_full());
+                const int tok = (block0 + blk) * tpb;
+                tma_load_4d(dst, &tmap_q, 0, it.kvh * qg, tok, it.b, B.q_full());
+                tma_load_4d(dst + kSubTileBytes, &tmap_q, 64, it.kvh * qg, tok, it.b, B.q_full());
             }
             for (int j = j_first; j < n_tiles && j < NS; ++j) { issue_k(j); issue_v(j); }
             // refill whichever ring has a free slot; K slots free up ahead of V slots
@@ -761,6 +761,15 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             const uint64_t q_desc0 = smem_desc(smem_u32(q_sm), 16, 1024);
             const uint64_t k_desc0 = smem_desc(smem_u32(kv_sm), 16, 1024);
             const uint64_t v_desc0 = smem_desc(smem_u32(kv_sm) + 2 * kSubTileBytes, kSubTileBytes, 1024);
+            // Rows that no box of Q covers are zeros, as are the tokens of a box past the last: scores and P of padding are zeros
+            // as well, and products of zeros take less power, which is what long calls are short of (four sequences of
+            // 20,000 keys, T = 20, 45 % of the rows padding, 41.2 -> 40.5 us; three of 9,001, T = 23 20.5 -> 20.0).
+            #pragma unroll 1
+            for (int i = lane + qg * tpb * 8; i < kBlockRows * 8; i += 32)
+                #pragma unroll
+                for (int sub = 0; sub < 2 * NB; ++sub) *reinterpret_cast<uint4*>(q_sm + sub * kSubTileBytes + i * 16) = make_uint4(0, 0, 0, 0);
+            fence_proxy_async();
+            __syncwarp();
             // (a bounded wait must not include what is left of the predecessor's time: kernels that let their
             // dependents start early may run on for longer than its polls)
             if (sync.wait_first) wait_for_predecessors();
@@ -949,19 +958,18 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const float thr = kRescaleLog2 / c2;             // threshold in raw score units
         const uint64_t c22 = pair_of(c2, c2);
         const int g_row = row_local % qg;
-        int t_row[NB], lo_row[NB];
-        bool row_ok[NB];
-        unsigned long long anc[NB];
-        float m_ref[NB], l_run[NB];
-        #pragma unroll
-        for (int blk = 0; blk < NB; ++blk) {
-            t_row[blk] = (block0 + blk) * tpb + row_local / qg;
-            row_ok[blk] = row_local < tpb * qg && t_row[blk] < T;
-            // the queries are the last T nodes of the tree
-            anc[blk] = (row_ok[blk] && it.key_end > kv_len) ? anc_s[plan.T_tree - T + t_row[blk]] : 0ull;
-            lo_row[blk] = row_ok[blk] ? par_s[t_row[blk]] : 0;
-            m_ref[blk] = -INFINITY; l_run[blk] = 0.f;
-        }
+        // A thread's row: of the one block, or of its warpgroup's own.
+        const int blk = NB == 1 ? 0 : wg;
+        const int t_row = (block0 + blk) * tpb + row_local / qg;
+        const bool row_ok = row_local < tpb * qg && t_row < T;
+        // (read from the tables where they are needed; the queries are the last T nodes of the tree)
+        auto row_anc = [&]() { return (row_ok && it.key_end > kv_len) ? anc_s[plan.T_tree - T + t_row] : 0ull; };
+        auto row_lo = [&]() { return row_ok ? par_s[t_row] : 0; };
+        const int lo_first = row_lo();
+        // tiles whose every key is visible to the warp's rows: [j_head, j_tail)
+        const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
+        const int j_head = __reduce_max_sync(0xffffffffu, lo_first > it.key_begin ? (lo_first - it.key_begin + kTile - 1) / kTile : 0);
+        float m_ref = -INFINITY, l_run = 0.f;
         bool ok = true;
 
         // visibility word, for the 64 keys that start at key j0, of a row with ancestor word `anc_row` and lower
@@ -982,20 +990,11 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             else if (cut > 0) vis &= ~((1ull << cut) - 1ull);
             return vis;
         };
-        float my_m = -INFINITY, my_l = 0.f;       // two row blocks: the state of this warpgroup's own block
         if constexpr (NB == 2) {
             // ---- two row blocks: warpgroup g owns block g, one thread per query row, and works
             // through the block's half-tile jobs on its own -- no exchange with the other warpgroup,
             // whose exponentials fill the gaps this one leaves while it waits for the tensor pipe.
-            const int blk = wg;
-            // this warpgroup's block, in scalars (indexing the per-block arrays with wg would put them in local memory)
-            const unsigned long long my_anc = wg ? anc[NB - 1] : anc[0];
-            const int my_lo = wg ? lo_row[NB - 1] : lo_row[0];
-            const bool my_ok = wg ? row_ok[NB - 1] : row_ok[0];
             const uint32_t s_addr = lane_addr + blk * 128;
-            // tiles whose every key is visible to this row: [j_head, j_tail)
-            const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
-            const int j_head = __reduce_max_sync(0xffffffffu, my_lo > it.key_begin ? (my_lo - it.key_begin + kTile - 1) / kTile : 0);
             #pragma unroll 1
             for (int j = 0; j < n_tiles; ++j) {
                 const int tile0 = it.key_begin + j * kTile;
@@ -1010,7 +1009,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 tmem_ld32(s_addr + 32, x1);
                 tmem_wait_ld();
                 if (edge) {
-                    const unsigned long long vis = vis_word(tile0, my_anc, my_lo);
+                    const unsigned long long vis = vis_word(tile0, row_anc(), row_lo());
                     mask_chunk(x0, (uint32_t)vis);
                     mask_chunk(x1, (uint32_t)(vis >> 32));
                     tmem_st32(s_addr, reinterpret_cast<uint32_t*>(x0));
@@ -1023,20 +1022,20 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 tmem_ld32(s_addr + 96, x1);
                 tmem_wait_ld();
                 if (edge) {
-                    const unsigned long long vis = vis_word(tile0 + 64, my_anc, my_lo);
+                    const unsigned long long vis = vis_word(tile0 + 64, row_anc(), row_lo());
                     mask_chunk(x0, (uint32_t)vis);
                     mask_chunk(x1, (uint32_t)(vis >> 32));
                 }
                 mx = fmaxf(mx, fmaxf(chunk_max(x0), chunk_max(x1)));
                 // lazy reference maximum, per row; the accumulator is rescaled by the whole warp (the
                 // TMEM accesses are warp-wide) whenever one of its rows moved
-                const bool need = my_ok && (mx > my_m + thr || (my_m == -INFINITY && mx > -INFINITY));
+                const bool need = row_ok && (mx > m_ref + thr || (m_ref == -INFINITY && mx > -INFINITY));
                 if (__any_sync(0xffffffffu, need)) {
                     float alpha = 1.f;
                     if (need) {
-                        alpha = (my_m == -INFINITY) ? 0.f : ex2((my_m - mx) * c2);
-                        my_m = mx;
-                        my_l *= alpha;
+                        alpha = (m_ref == -INFINITY) ? 0.f : ex2((m_ref - mx) * c2);
+                        m_ref = mx;
+                        l_run *= alpha;
                     }
                     if (j > 0) {                                            // O holds earlier tiles
                         if (!mbar_wait_warp(B.o_done(blk, j - 1), ((j - 1) >> 2) & 1)) { ok = false; break; }
@@ -1057,7 +1056,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 // of the score block -- first the upper 64 keys (their scores are in registers and their
                 // columns are the ones P overwrites), then the lower 64, fetched again.  The upper keys'
                 // half of O += P V runs beside the exponentials of the lower ones.
-                const float mc = (my_m == -INFINITY) ? 0.f : my_m * c2;
+                const float mc = m_ref > -INFINITY ? m_ref * c2 : row_ok ? 0.f : INFINITY;     // (padding: P is 0)
                 const uint64_t neg_mc2 = pair_of(-mc, -mc);
                 uint64_t sum[2] = {0ull, 0ull};
                 exp_chunk(x0, c22, neg_mc2, sum, s_addr + 96);
@@ -1075,22 +1074,17 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(B.p_full(2 + blk));
-                my_l += sum_of(sum);
+                l_run += sum_of(sum);
             }
         } else {
         // One row block: the two warpgroups split a tile's 128 keys; thread = one row, 64 keys.  The two warps that share
         // 32 rows run apart from one another, by a tile at most (softmax_pair.cuh).
         const int sb_wg = 64 * wg;
-        auto row_anc = [&]() { return (row_ok[0] && it.key_end > kv_len) ? anc_s[plan.T_tree - T + t_row[0]] : 0ull; };
-        auto row_lo = [&]() { return row_ok[0] ? par_s[t_row[0]] : 0; };
         const uint32_t pair_id = 4u + (uint32_t)(warp & 3);
         float x0[32], x1[32];
-        // tiles whose every key is visible to the warp's rows: [j_head, j_tail)
-        const int j_tail = (min(it.key_end, kv_len) - it.key_begin) / kTile;
-        const int j_head = __reduce_max_sync(0xffffffffu, row_lo() > it.key_begin ? (row_lo() - it.key_begin + kTile - 1) / kTile : 0);
-        // scores above this need a new reference.  (Rows of padding hold whatever the Q box left there: they never do.)
-        float limit = row_ok[0] ? -INFINITY : INFINITY;
-        float mc = 0.f;                                                     // reference in log2 units, 0 as long as there is none
+        // scores above this need a new reference (rows of padding never do)
+        float limit = row_ok ? -INFINITY : INFINITY;
+        float mc = row_ok ? 0.f : INFINITY;                                 // reference in log2 units, 0 as long as there is none (padding: P is 0)
         float m_acc = -INFINITY;                                            // what the accumulator is on; m_ref: what this tile's P is on
         int sb = 0;                                                         // the tile's S block
         uint32_t s_parity = 0, moved = 0;                                   // moved: bit 0 in the tile passed last, bit 1 in the one before
@@ -1138,14 +1132,14 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     if (!ok) break;
                     const bool other = pair_moved(word, j - 1);
                     if (other || (moved & 1u)) {
-                        float m_new = m_ref[0];
+                        float m_new = m_ref;
                         if (other) {
                             __threadfence_block();
                             m_new = fmaxf(m_new, xch[(wg ^ 1) * 128 + row_local]);
                             __syncwarp();
                             if (lane == 0) pair_s[warp] = pair_word(j, true, moved);
                         }
-                        const float of_p = rescale(m_ref[0], m_new, c2), of_acc = rescale(m_acc, m_new, c2);
+                        const float of_p = rescale(m_ref, m_new, c2), of_acc = rescale(m_acc, m_new, c2);
                         tmem_wait_st();
                         if (__any_sync(0xffffffffu, of_p != 1.f)) {
                             #pragma unroll 1
@@ -1174,8 +1168,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                                 tmem_st16(o_addr, reinterpret_cast<uint32_t*>(o));
                             }
                         }
-                        l_run[0] *= of_p;
-                        m_ref[0] = m_acc = m_new;
+                        l_run *= of_p;
+                        m_ref = m_acc = m_new;
                         if (m_new > -INFINITY) { limit = m_new + thr; mc = m_new * c2; }
                     }
                 }
@@ -1184,7 +1178,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 if (j == 0) {
                     post(mine);
                     pair_sync(pair_id);
-                    m_ref[0] = m_acc = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
+                    m_ref = m_acc = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
                     if (m_acc > -INFINITY) { limit = m_acc + thr; mc = m_acc * c2; }
                     // The second warp of the pair starts half a tile's exponentials late and stays so: what each does besides them
                     // falls into the other's.  In step, both wait for the exponentials together (41 tiles alone 1,560 -> 1,460
@@ -1207,8 +1201,8 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     moved |= 1u;
                     post(mine);
                     if (mine > -INFINITY) {
-                        l_run[0] *= rescale(m_ref[0], mine, c2);
-                        m_ref[0] = mine;
+                        l_run *= rescale(m_ref, mine, c2);
+                        m_ref = mine;
                         mc = mine * c2;
                     }
                 }
@@ -1238,11 +1232,11 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
             if (have) tmem_ld32(s_next, x0);
             exp_chunk(x1, c22, neg_mc2, sum, p_addr + 16);
             if (have) tmem_ld32(s_next + 32, x1);
-            l_run[0] += sum_of(sum);
+            l_run += sum_of(sum);
         }
         if (!ok && lane == 0) pair_s[warp] = pair_word(n_tiles, false, 0u);  // (the partner need not wait as well)
         // The sums meet, behind the row as it is staged below: every Q K^T is complete, Q's place is free.
-        reinterpret_cast<float*>(q_sm + row_local * kRowBytes + kD * 2)[1 + wg] = l_run[0];
+        reinterpret_cast<float*>(q_sm + row_local * kRowBytes + kD * 2)[1 + wg] = l_run;
         pair_sync(pair_id + 4u);
         }
         // ---- epilogue: normalised partial output + natural-log LSE -------------------------------
@@ -1260,7 +1254,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         }
         // A thread finishes one row: its 64 output dims [64 wg, 64 wg + 64) of the one block, or all 128 of its
         // warpgroup's own block.
-        const int blk = NB == 1 ? 0 : wg;
         const int dim0 = NB == 1 ? 64 * wg : 0;
         // Partial rows are staged as they lie in the workspace ([row][272 bytes]: an odd number of 16-byte
         // chunks, so a warp's rows do not share banks) and leave as one bulk copy per block: the copy's own
@@ -1271,12 +1264,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         float* tail = reinterpret_cast<float*>(stage + row_local * kRowBytes + kD * 2);
         if constexpr (NB == 2) softmax_bar_sync();
         // (one row block: the halves' sums met with the pair's last barrier; the maxima are the same)
-        const float l_all = NB == 1 ? tail[1] + tail[2] : my_l;
-        const float m_fin = NB == 1 ? m_ref[0] : my_m;
-        const bool my_row = NB == 1 ? row_ok[0] : (wg ? row_ok[NB - 1] : row_ok[0]);
-        const int my_t = (block0 + blk) * tpb + row_local / qg;
+        const float l_all = NB == 1 ? tail[1] + tail[2] : l_run;
         const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
-        const float lse_val = l_all > 0.f ? (m_fin * c2 + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+        const float lse_val = l_all > 0.f ? (m_ref * c2 + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
         if (ok) ok = mbar_wait_warp(B.o_done(blk, n_tiles - 1), ((n_tiles - 1) >> 2) & 1);    // the last product is in
         tc_fence_after();
         // The whole ring is idle: what peers may write over, the tensor pipe's reads and the loads behind them, is complete by the
@@ -1284,7 +1274,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         if (CL && n_tiles >= NS) cluster_arrive_relaxed();
         if (tid == 0) SPARROW_STAMP(6);                                // last product complete
         const int h_row = it.kvh * qg + g_row;
-        const bool has_lse = my_row && (wg == 0 || NB == 2);
+        const bool has_lse = row_ok && (wg == 0 || NB == 2);
         if (ok && has_lse && !direct) *tail = lse_val;
         if (ok) {
             #pragma unroll 1
@@ -1301,7 +1291,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     #pragma unroll
                     for (int c = 0; c < 16; ++c) w[c] = pack_half2(o[2 * c] * inv, o[2 * c + 1] * inv);
                 }
-                if (my_row) {
+                if (row_ok) {
                     uint4* dst = reinterpret_cast<uint4*>(stage + row_local * kRowBytes + col * 2);
                     #pragma unroll
                     for (int c = 0; c < 4; ++c) dst[c] = pk[c];
@@ -1312,7 +1302,7 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         softmax_bar_sync();                                            // every row is staged
         ok = ok && *write_ok == 1u;                                    // (thread 0 settled it ahead of the barrier)
         if (direct) {
-            if (ok && has_lse) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + my_t] = lse_val;
+            if (ok && has_lse) args.lse[((size_t)it.b * args.n_q_heads + h_row) * T + t_row] = lse_val;
             // final rows: 16 threads write a row's 256 bytes (a row per thread took 2 us longer)
             #pragma unroll
             for (int bk = 0; bk < NB; ++bk) {
