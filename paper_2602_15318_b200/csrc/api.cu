@@ -685,14 +685,20 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
     return SPARROW_OK;
 }
 
-// Estimates for the choice of a plan, us: a tile of 128 keys with one / two row blocks, the merges of a lone
-// call, and what an item of a call in a batch costs besides its tiles.  They were fitted together, over forced choices, to the
-// kernels as they were when a tile took 1.0 and 1.8 us; it takes 0.8 and 1.7 since (long pieces, one call alone), and the fit
-// was not made again.
-constexpr float kTileUs[2] = {1.2f, 2.0f};
-constexpr float kMergeWorkspaceUs = 5.f, kMergeClusterUs = 2.f, kTwoBlocksUs = 4.f, kTwoBlocksWholeUs = 1.f;
-constexpr float kItemUs[2] = {5.f, 11.f}, kWholeItemUs[2] = {6.5f, 8.5f};      // its rows are merged; it is its unit's only piece
+// Estimates for the choice of a plan, us.  A lone call: a tile of 128 keys with one / two row blocks, a merge through the
+// workspace (of one sequence, of several: uneven pieces, more and shorter runs of rows), a merge in a cluster (by the rows that a CTA of it finishes and the pieces that it folds), and what items of two row
+// blocks cost besides.  Fitted to 170 shapes with every cluster size, the workspace and whole units forced (1 to 8 sequences of
+// 300 to 32,768 keys, T = 1 to 64, six head geometries).  The two kernels' tiles take 0.75 to 0.95 and 1.65, by the load; two row blocks
+// win where the GPU is full and at its power cap: pieces of more than about 40 tiles of one block (six sequences
+// of 27,000 keys, T = 19 62 and 55 us; two of 30,000, T = 36 36 and 41).
+constexpr float kTileUs[2] = {0.8f, 1.4f};
+constexpr float kMergeWorkspaceUs[2] = {3.7f, 5.3f}, kMergeClusterUs = 0.1f, kMergeRowUs = 0.03f, kMergePieceUs = 0.02f;
+constexpr float kTwoBlocksUs = 4.f, kTwoBlocksWholeUs = 1.f;
 constexpr float kWaveUs[2] = {6.f, 8.f};                                       // a further wave of a call with more units than SMs
+// A call in a batch: a tile, and what an item costs besides its tiles where its rows are merged and where it is its unit's only
+// piece.  Fitted together, over forced choices, to the kernels as they were when a tile took 1.0 and 1.8 us; it takes 0.75 and
+// 1.65 since (long pieces, one call alone), and the fit was not made again.
+constexpr float kBatchTileUs[2] = {1.2f, 2.0f}, kItemUs[2] = {5.f, 11.f}, kWholeItemUs[2] = {6.5f, 8.5f};
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
 // at most 16 pieces per unit and whole clusters per GPC.  Rewrites the plan where
@@ -702,6 +708,7 @@ constexpr float kWaveUs[2] = {6.f, 8.f};                                       /
 float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
 {
     const int nb = p->blocks_per_group, units = p->batch * p->n_kv_heads * p->n_groups;
+    const int unit_rows = p->group * std::min(nb * p->tok_per_block, p->T);
     const float per_tile = nb == 1 ? kTileUs[0] : kTileUs[1];
     int most = 0, least = 1 << 30;                     // tiles of the longest and the shortest sequence
     float best = 0.f;
@@ -710,7 +717,7 @@ float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
         const int piece = (tiles + p->seq[b].n_splits - 1) / p->seq[b].n_splits;
         if (tiles > most) most = tiles;
         if (tiles < least) least = tiles;
-        const float t = per_tile * piece + (p->seq[b].n_splits > 1 ? kMergeWorkspaceUs : 0.f);
+        const float t = per_tile * piece + (p->seq[b].n_splits > 1 ? kMergeWorkspaceUs[p->batch > 1] : 0.f);
         if (t > best) best = t;
     }
     int pieces = 0;
@@ -718,7 +725,8 @@ float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
         const int piece = (most + n - 1) / n;
         if (n == 1 && units > c->n_sm) continue;
         if (n > 1 && (!c->max_clusters[nb - 1] || units > c->max_clusters[nb - 1][n])) continue;
-        const float t = per_tile * piece + (n > 1 ? kMergeClusterUs : 0.f);
+        const float merge = kMergeClusterUs + kMergeRowUs * (float)((unit_rows + n - 1) / n) + kMergePieceUs * (float)n;
+        const float t = per_tile * piece + (n > 1 ? merge : 0.f);
         if (t < best) { best = t; pieces = n; }
     }
     if (pieces == 0) return best;
@@ -741,7 +749,7 @@ float batch_cost(const SplitPlan& p)
     float cost = 0.f;
     for (int b = 0; b < p.batch; ++b) {
         const int tiles = (p.seq[b].n_keys - p.seq[b].key0 + kKeyTile - 1) / kKeyTile, ns = p.seq[b].n_splits;
-        cost += (float)units * ((float)ns * (ns > 1 ? kItemUs[nb] : kWholeItemUs[nb]) + kTileUs[nb] * (float)tiles);
+        cost += (float)units * ((float)ns * (ns > 1 ? kItemUs[nb] : kWholeItemUs[nb]) + kBatchTileUs[nb] * (float)tiles);
     }
     return cost;
 }
