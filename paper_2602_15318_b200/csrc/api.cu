@@ -452,8 +452,10 @@ sparrow_status launch_split_gather(sparrow_ctx* c, const SplitPlan& plan, const 
     a.lse = lse;
     a.status = reinterpret_cast<unsigned*>(c->ws);
     other_kernel_enqueued();
-    return launch_behind(c, gather::split_gather_kernel, (unsigned)plan.n_items, gather::kThreads,
-                         plan.cluster > 1 ? gather::kClusterSmemBytes : gather::kSmemBytes, st, plan.cluster > 1 ? (unsigned)plan.cluster : 0u, plan, a);
+    if (plan.cluster > 1)
+        return launch_behind(c, gather::split_gather_kernel<true>, (unsigned)plan.n_items, gather::kThreads, gather::kClusterSmemBytes, st,
+                             (unsigned)plan.cluster, plan, a);
+    return launch_behind(c, gather::split_gather_kernel<false>, (unsigned)plan.n_items, gather::kThreads, gather::kSmemBytes, st, 0u, plan, a);
 }
 
 // Cached tensor maps.  tag == 0: one K or V buffer, dims (128 dims, capacity rows, KV heads,
@@ -658,7 +660,7 @@ const ClusterTable* cluster_table(int device)
     if (t.state.compare_exchange_strong(expected, 1)) {
         query_max_clusters(tc::verify_tc_kernel<1, true>, tc::kThreads, tc::smem_bytes(1, 3), t.n[0]);
         query_max_clusters(tc::verify_tc_kernel<2, true>, tc::kThreads, tc::smem_bytes(2, 2), t.n[1]);
-        query_max_clusters(gather::split_gather_kernel, gather::kThreads, gather::kClusterSmemBytes, t.n[2]);
+        query_max_clusters(gather::split_gather_kernel<true>, gather::kThreads, gather::kClusterSmemBytes, t.n[2]);
         t.state.store(2);
     }
     while (t.state.load() != 2) std::this_thread::yield();      // another thread is asking
@@ -962,8 +964,8 @@ sparrow_status sparrow_create(sparrow_ctx** out, const sparrow_layout* L, int de
     if (major != 10) return SPARROW_ERR_ARCH;
     DeviceGuard guard(device);
     if (!guard.ok) return SPARROW_ERR_CUDA;
-    if (cudaFuncSetAttribute(gather::split_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             gather::kClusterSmemBytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(gather::split_gather_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gather::kClusterSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(gather::split_gather_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, gather::kSmemBytes) != cudaSuccess)
         return SPARROW_ERR_CUDA;
     if (cudaFuncSetAttribute(tc::verify_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::smem_bytes(1, 3)) != cudaSuccess ||
         cudaFuncSetAttribute(tc::verify_tc_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::smem_bytes(1, 3)) != cudaSuccess ||
@@ -1150,9 +1152,7 @@ sparrow_status sparrow_verify_attn_static(const sparrow_layout* L, const void* q
         cudaDeviceProp prop;
         if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return SPARROW_ERR_CUDA;
         if (prop.major != 10) return SPARROW_ERR_ARCH;
-        if (cudaFuncSetAttribute(gather::split_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 gather::kClusterSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(tc::verify_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(tc::verify_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  tc::smem_bytes(1, 3)) != cudaSuccess ||
             cudaFuncSetAttribute(tc::verify_tc_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  tc::smem_bytes(2, 2)) != cudaSuccess)

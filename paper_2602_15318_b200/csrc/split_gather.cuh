@@ -1,11 +1,11 @@
 // Split-KV pass with row-gathered K/V loads: the kernel behind the text-anchored window mode
-// (Eq. 2: keys/values restricted to the anchor list) and a general path for any key layout.
+// (Eq. 2: keys/values restricted to the anchor list).
 //
 // One CTA = one work item (sequence, KV head, one 128-row block of packed query rows, key-range
 // piece).  The g query heads of the GQA group times p = 128 / g draft tokens form one block (row
 // r = (t % p) g + head; g = 7: 18 tokens, two rows of padding), so every gathered K/V row is loaded once per KV head
 // and block.  K/V rows are fetched
-// with 16-byte cp.async (row index = key index, or anchor_idx[key] when gathering) into a
+// with 16-byte cp.async (row index = anchor_idx[key]) into a
 // two-stage XOR-swizzled shared-memory ring; S = QK^T and O += PV run on mma.sync m16n8k16 bf16
 // with fp32 accumulation; the online softmax is fp32 with quad shuffles.  A piece's result is a
 // normalised fp16 partial output and a natural-log LSE per row: where the unit's pieces share a
@@ -23,11 +23,11 @@ struct SplitArgs {
     const __nv_bfloat16* q;
     const __nv_bfloat16* k;
     const __nv_bfloat16* v;
-    const int32_t* parents;      // verification: DEV [B][T]; anchored: DEV [B][tree_nodes] or nullptr (chain)
-    const int32_t* anchor_idx;   // anchored: DEV [B][n_anchor]; nullptr in verification mode
+    const int32_t* parents;      // DEV [B][tree_nodes] or nullptr (chain)
+    const int32_t* anchor_idx;   // DEV [B][n_anchor]
     int32_t n_anchor;
     int32_t window;
-    int32_t tree_nodes;          // anchored mode with a draft tree: its nodes are the last tree_nodes anchors, the
+    int32_t tree_nodes;          // with a draft tree: its nodes are the last tree_nodes anchors, the
                                  // queries the last T of them; 0 = chain rule for every anchor
     int32_t n_q_heads;
     int32_t kv_capacity;
@@ -87,6 +87,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 // byte offset of 16-byte chunk c of row r inside a [rows][128] bf16 tile (XOR swizzle)
 __device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 256 + ((c ^ (r & 7)) << 4)); }
 
+// CL: the pieces of a unit are a thread-block cluster and merge in shared memory; otherwise a piece is final or leaves its
+// partial rows to the combine kernel.
+template <bool CL>
 __global__ void __launch_bounds__(kThreads, 1)
 split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constant__ SplitArgs args)
 {
@@ -99,7 +102,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
 
     // The combine kernel may be scheduled now: it waits for this grid as a whole before it reads.
     __shared__ uint64_t merge_bar;
-    if (plan.cluster > 1) {
+    if (CL) {
         if (threadIdx.x == 0) {
             tc::mbar_init(smem_u32(&merge_bar), 1);
             tc::fence_barrier_init();
@@ -112,28 +115,26 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
     const int g4 = lane >> 2, c4 = lane & 3;
     const Item it = decode_item(plan, blockIdx.x);
     const int T = plan.T;
-    const bool anchored = args.anchor_idx != nullptr;
-    const int kv_len = anchored ? 0 : plan.seq[it.b].kv_len;
-    const int32_t* aidx = anchored ? args.anchor_idx + (size_t)it.b * args.n_anchor : nullptr;
+    const int32_t* aidx = args.anchor_idx + (size_t)it.b * args.n_anchor;
 
     const __nv_bfloat16* kbase = args.k + (size_t)it.b * args.kv_stride_batch + (size_t)it.kvh * args.kv_stride_head;
     const __nv_bfloat16* vbase = args.v + (size_t)it.b * args.kv_stride_batch + (size_t)it.kvh * args.kv_stride_head;
     const int n_tiles = (it.key_end - it.key_begin + kTile - 1) / kTile;
 
-    // Row indices of a tile, four per thread (one per 16-byte chunk this thread copies).  In anchored
-    // mode they come from the anchor list: a memory round trip that the row copies depend on, so
-    // the indices of a tile are fetched one whole tile ahead of its copies.
+    // Row indices of a tile, four per thread (one per 16-byte chunk this thread copies).  They come from the
+    // anchor list: a memory round trip that the row copies depend on, so the indices of a tile are fetched one
+    // whole tile ahead of its copies.
     constexpr int kAbsent = -2147483647 - 1;                 // key past the end of the piece
     constexpr int kPerThread = (kTile * 16) / kThreads;      // 4
     // The thread that owns chunk 0 of a row also fetches the anchor before it: the list must be
     // strictly increasing (the window rule and the position of the tree nodes rely on it).
-    const bool checks_order = anchored && (tid & 15) == 0;
+    const bool checks_order = (tid & 15) == 0;
     auto fetch_rows = [&](int tile, int (&rows)[kPerThread], int (&before)[kPerThread]) {
         #pragma unroll
         for (int i = 0; i < kPerThread; ++i) {
             const int r = (tid + i * kThreads) >> 4;
             const int j = it.key_begin + tile * kTile + r;
-            rows[i] = j < it.key_end ? (anchored ? ld_behind(aidx + j) : j) : kAbsent;
+            rows[i] = j < it.key_end ? ld_behind(aidx + j) : kAbsent;
             before[i] = (checks_order && j > 0 && j < it.key_end) ? ld_behind(aidx + j - 1) : kAbsent;
         }
     };
@@ -152,7 +153,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
                 atomicOr(args.status, kStatAnchor);
                 row = -1;
             }
-            if (anchored && c == 0) apos_s[stage * kTile + r] = row;
+            if (c == 0) apos_s[stage * kTile + r] = row;
             const size_t off = (size_t)(row < 0 ? 0 : row) * kD + c * 8;
             const int bytes = row < 0 ? 0 : 16;          // 0 -> the 16 bytes are zero-filled
             cp_async16(smem_u32(ks + swz(r, c)), kbase + off, bytes);
@@ -184,15 +185,14 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
     // tile 0, which wait for their indices, are then the only second round trip.  (Q behind the positions and the
     // positions behind the indices, one round trip after the other: 448 anchors 8.25 us, like this 8.21.)
     if (n_tiles > 0) fetch_rows(0, rows_next, before_next);
-    const int tree_nodes = anchored ? args.tree_nodes : 0;
-    const int n_par = anchored ? tree_nodes : T;
+    const int tree_nodes = args.tree_nodes;
     int par[2] = {-1, -1}, qpos = -1;
     if (warp == 0) {
         #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if (lane + 32 * k < n_par) par[k] = ld_behind(args.parents + (size_t)it.b * n_par + lane + 32 * k);
+            if (lane + 32 * k < tree_nodes) par[k] = ld_behind(args.parents + (size_t)it.b * tree_nodes + lane + 32 * k);
     }
-    if (anchored && tid < T) qpos = ld_behind(aidx + args.n_anchor - T + tid);
+    if (tid < T) qpos = ld_behind(aidx + args.n_anchor - T + tid);
     #pragma unroll
     for (int u = 0; u < kChunksPerThread; ++u) {
         const int i = tid + u * kThreads;
@@ -204,11 +204,11 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
     if (n_tiles > 1) fetch_rows(1, rows_next, before_next);
 
     // ---- prologue: masks / query positions, packed Q block -> registers --------------------
-    if (anchored && tid < T) {
+    if (tid < T) {
         if (qpos < 0 || qpos >= args.kv_capacity) { atomicOr(args.status, kStatAnchor); qpos = -1; }
         qpos_s[tid] = qpos;
     }
-    if (warp == 0) build_ancestor_words(par[0], par[1], anc_s, n_par, args.status);
+    if (warp == 0) build_ancestor_words(par[0], par[1], anc_s, tree_nodes, args.status);
     cp_async_wait<1>();                                          // (this thread's chunks of Q; tile 0 may be on its way)
     __syncthreads();
     uint32_t qf[8][4];
@@ -219,15 +219,17 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
             ldsm_x4(smem_u32(q_stage + swz(r, ks * 2 + (lane >> 4))), qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3]);
     }
     // per-thread row state: rows lr0 = warp*16+g4 and lr0+8
-    int row_t[2]; bool row_ok[2]; unsigned long long row_anc[2]; int row_qpos[2];
+    // A row sees an anchor at position p behind row_lo, up to row_hi (its own; a row without a valid one sees none).
+    int row_t[2]; bool row_ok[2]; unsigned long long row_anc[2]; int row_lo[2], row_hi[2];
     #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
         const int lr = warp * 16 + g4 + rr * 8;
         row_t[rr] = it.group * plan.tok_per_block + ((lr * plan.inv_group) >> 16);
         row_ok[rr] = lr < plan.tok_per_block * plan.group && row_t[rr] < T;
         const int t = row_ok[rr] ? row_t[rr] : 0;
-        row_anc[rr] = anchored ? (tree_nodes > 0 ? anc_s[tree_nodes - T + t] : 0ull) : anc_s[t];
-        row_qpos[rr] = anchored ? qpos_s[t] : 0;
+        row_hi[rr] = qpos_s[t];
+        row_lo[rr] = args.window > 0 ? max(row_hi[rr] - args.window, -1) : -1;
+        row_anc[rr] = tree_nodes > 0 && row_hi[rr] >= 0 ? anc_s[tree_nodes - T + t] : 0ull;
     }
     const bool warp_has_rows = __any_sync(0xffffffffu, row_ok[0] || row_ok[1]);
     __syncthreads();                      // Q staging area is reused by the K/V ring from here on
@@ -268,31 +270,35 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
                 mma_bf16(s[2 * np + 1], qf[kstep], b2, b3);
             }
         }
-        // visibility
-        const int j0 = it.key_begin + tile * kTile;
-        const bool need_mask = anchored || (j0 + kTile > it.key_end) || (j0 + kTile > kv_len);
-        if (need_mask) {
+        // Visibility: by position, and by ancestors from the column of the tree's first node on.  (An anchor that is not
+        // there or not valid has position -1.)  What bounds this kernel is how much code a CTA fetches for its one or two
+        // tiles: two comparisons an element, where every element had been asked for its kind, took 448 anchors from 8.05
+        // to 5.96 us and 6,000 from 21.0 to 15.6, together with one kernel per way of merging.
+        const int col0 = args.n_anchor - tree_nodes - (it.key_begin + tile * kTile);
+        const int2* pos = reinterpret_cast<const int2*>(apos_s + stage * kTile) + c4;
+        if (tree_nodes == 0 || col0 >= kTile) {
             #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
+                const int2 p = pos[nt * 4];
                 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int rr = e >> 1;
-                    const int col = nt * 8 + 2 * c4 + (e & 1);
-                    const int j = j0 + col;
-                    bool vis = j < it.key_end;
-                    if (vis) {
-                        if (anchored) {
-                            const int p = apos_s[stage * kTile + col];
-                            const int qp = row_qpos[rr];
-                            const int node = j - (args.n_anchor - tree_nodes);     // >= 0: a node of the draft tree
-                            if (tree_nodes > 0 && node >= 0)
-                                vis = p >= 0 && qp >= 0 && ((row_anc[rr] >> node) & 1ull);
-                            else
-                                vis = p >= 0 && qp >= 0 && p <= qp && (args.window <= 0 || qp - args.window < p);
-                        } else if (j >= kv_len) {
-                            vis = (row_anc[rr] >> (j - kv_len)) & 1ull;
-                        }
-                    }
+                    const int pe = e & 1 ? p.y : p.x;
+                    if (pe <= row_lo[e >> 1] || pe > row_hi[e >> 1]) s[nt][e] = -INFINITY;
+                }
+            }
+        } else {
+            unsigned long long word[2];                  // the tree's visible columns, this thread's first one in bit 0
+            #pragma unroll
+            for (int rr = 0; rr < 2; ++rr)
+                word[rr] = (col0 >= 0 ? row_anc[rr] << col0 : col0 > -64 ? row_anc[rr] >> -col0 : 0ull) >> (2 * c4);
+            #pragma unroll
+            for (int nt = 0; nt < 8; ++nt) {
+                const int2 p = pos[nt * 4];
+                #pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int pe = e & 1 ? p.y : p.x, rr = e >> 1;
+                    const bool in_tree = nt * 8 + (e & 1) + 2 * c4 >= col0;
+                    const bool vis = in_tree ? pe >= 0 && ((word[rr] >> (nt * 8 + (e & 1))) & 1ull) : pe > row_lo[rr] && pe <= row_hi[rr];
                     if (!vis) s[nt][e] = -INFINITY;
                 }
             }
@@ -351,7 +357,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
     // ---- epilogue: normalised partial output + natural-log LSE ------------------------------
     // Where the unit's pieces share a cluster a partial row is staged in shared memory (over the K/V ring) and
     // sent to the CTA that finishes it.
-    const bool clustered = plan.cluster > 1;
+    constexpr bool clustered = CL;
     #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
         float l = l_run[rr];
@@ -361,7 +367,7 @@ split_gather_kernel(const __grid_constant__ SplitPlan plan, const __grid_constan
         const int lr = warp * 16 + g4 + rr * 8;
         const float inv = l > 0.f ? 1.f / l : 0.f;
         const float lse_val = l > 0.f ? (m_run[rr] * c2 + log2f(l)) * 0.6931471805599453f : -INFINITY;
-        if (plan.seq[it.b].n_splits == 1) {                 // the only piece: write the final result
+        if (!CL && plan.seq[it.b].n_splits == 1) {          // the only piece: write the final result
             const int t = row_t[rr], h = it.kvh * plan.group + lr - (t - it.group * plan.tok_per_block) * plan.group;
             __nv_bfloat16* dst = args.out + (((size_t)it.b * T + t) * args.n_q_heads + h) * kD;
             #pragma unroll
