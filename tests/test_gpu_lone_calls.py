@@ -106,6 +106,31 @@ def test_anchored_pieces(n_text, T, batch):
     check(out, lse, *oracle_anchor(case))
 
 
+@pytest.mark.parametrize("n_text,T_tree,T_new,window", [
+    (0, 1, 1, 0),                           # a tile that is a tree of one node
+    (63, 1, 1, 0),                          # a node in a tile's last column
+    (64, 64, 64, 0),                        # a whole tile of nodes, from its first column
+    (65, 64, 64, 0),                        # 63 nodes in one tile, one in the next
+    (127, 64, 9, 40),                       # one node in a tile, 63 in the next; text of the tile before outside the window
+    (100, 64, 33, 70),                      # nodes in two tiles, the window's end beside them
+    (16 * 64 - 32, 64, 20, 300),            # seventeen tiles, merged by the combine kernel
+    (30, 33, 2, 1),                         # a window that leaves no text
+])
+def test_gathered_trees_across_tiles(n_text, T_tree, T_new, window):
+    """Gathered keys are masked by position in front of the draft tree and by ancestors from the column of its first node on."""
+    idx = list(range(40, 40 + n_text)) + list(range(2000, 2000 + T_tree))
+    case = W.make_anchor_case(7600 + n_text + T_tree, idx, window + 2000 - 40 - n_text if window else 0, T_tree, 2, DEV)
+    parents = torch.tensor([W.random_tree_parents(7650 + b + n_text, 99, T_tree) for b in range(2)], dtype=torch.int32, device=DEV)
+    q = case.q[:, T_tree - T_new:].contiguous()
+    ctx = B.Context.for_cache(case.k, W.SCALE)
+    out, lse = torch.full_like(q, float("nan")), torch.full((2, W.HQ, T_new), float("nan"), dtype=torch.float32, device=DEV)
+    B.sparrow_anchor_attn_tree(ctx, q, case.k, case.v, case.anchor_idx, case.n_anchor, case.window, parents, T_tree, T_new, out, lse)
+    torch.cuda.synchronize()
+    assert ctx.last_device_status() == 0
+    check(out, lse, *oracle.anchor_attn_tree(W.bf16_bits(q), W.bf16_bits(case.k), W.bf16_bits(case.v), case.anchor_idx.cpu().numpy(),
+                                             case.window, parents.cpu().numpy(), W.SCALE))
+
+
 @pytest.mark.parametrize("hq,hkv,kv_len,T", [
     (32, 8, [48 * 128 - 12] * 3, 12),       # one piece of 48 tiles a unit
     (32, 8, [48 * 128 - 11, 300, 6000], 12),  # ragged lengths, 49 tiles the longest
