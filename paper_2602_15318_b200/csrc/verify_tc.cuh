@@ -105,9 +105,12 @@ constexpr int kPrefetchTiles = 2;                // brought into L2 ahead of the
 // off at most with 8, 2.0e-2 with 16).  Where no reference moves the two are equally fast.
 constexpr float kRescaleLog2 = 8.0f;
 
-// Rows received from the CTAs of a cluster lie in the ring's last stage; with two row blocks (up to 256 rows and
-// rounded-up shares) they need a little more behind it.
+// Rows received from the CTAs of a cluster lie in one stage of the ring (see recv_stage).  One row block: behind the start of it, where in the
+// first stage the end of the staged rows lies.  Two row blocks (up to 256 rows and rounded-up shares): in the last
+// stage and a little more behind it.
 constexpr int kMaxMergeCluster = 16;
+constexpr int kRecvSkip = 4096;
+static_assert(kBlockRows * kRowBytes - kQBlockBytes <= kRecvSkip && kRecvSkip + (kBlockRows + kMaxMergeCluster) * kRowBytes <= kStageBytes, "");
 __host__ __device__ constexpr int recv_extra(int n_blocks)
 {
     return n_blocks == 1 ? 0 : ((2 * kBlockRows + kMaxMergeCluster) * kRowBytes - kStageBytes + 1023) / 1024 * 1024;
@@ -437,6 +440,13 @@ __device__ __forceinline__ void pair_sync(uint32_t id) { asm volatile("bar.sync 
 // What is on reference m, brought to reference m_new >= m (raw scores; none yet: -inf).
 __device__ __forceinline__ float rescale(float m, float m_new, float c2) { return m == m_new ? 1.f : m == -INFINITY ? 0.f : ex2((m - m_new) * c2); }
 
+// The stage of the ring that a CTA of a cluster receives its rows in, for a piece of n tiles: with one row block the one whose last tile
+// is furthest back (of a piece that does not fill the ring: an unused one), which is idle two tiles before the product of
+// the last.  With two row blocks only the last stage has the room.
+__host__ __device__ constexpr int recv_stage(int n_blocks, int n) { return n_blocks == 1 ? n % 3 : 1; }
+// The last tile in that stage, of n >= the ring's depth.
+__host__ __device__ constexpr int recv_last_tile(int n_blocks, int n) { return n_blocks == 1 ? n - 3 : (n & ~1) - 1; }
+
 // Shared-memory addresses of the mbarriers (8-byte slots).  K and V tiles have their own full /
 // empty pairs: a K tile is released as soon as its last S = Q K^T has been computed, a V tile
 // only after its last O += P V, so the K stream runs ahead of the V stream.
@@ -700,9 +710,9 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // (waited for ahead of the first access to a peer.  The rows that peers send come to the ring's last stage: where this piece
-    // uses it, the softmax warps arrive behind their last product.)
-    if (CL && !(warp < 8 && n_tiles >= NS)) cluster_arrive_relaxed();
+    // (waited for ahead of the first access to a peer.  The rows that peers send come to a stage of the ring: where this piece
+    // uses it, the producer's warp arrives once it is idle.)
+    if (CL && !(warp == kProducerWarp && n_tiles >= NS)) cluster_arrive_relaxed();
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 0) SPARROW_STAMP(1);                             // set-up done
 
@@ -737,6 +747,17 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                 if (progress) idle = 0;
                 else if (++idle > kSpinLimit) { atomicOr(args.status, timeout_bits(kSiteProducer)); *abort_flag = 1; break; }
             }
+            if (CL && n_tiles >= NS) {
+                const int last = recv_last_tile(NB, n_tiles);           // (its phase is the one in progress or just completed: see issue_v)
+                if (!mbar_wait(B.v_empty(recv_stage(NB, n_tiles)), (last / NS) & 1)) { atomicOr(args.status, timeout_bits(kSiteProducer)); *abort_flag = 1; }
+            }
+        }
+        // Peers may write over the stage now.  What was written to it and read from it, by the loads, by zero_v_tail and by the
+        // products, is ordered ahead of this by the products' barrier, and the arrival releases it.  The fence in a releasing
+        // arrival takes 0.4 us: here it runs beside the last two tiles, behind the last product it took 8,000 keys, T = 8 from 9.2 to 9.6.
+        if (CL && n_tiles >= NS) {
+            __syncwarp();
+            cluster_arrive();
         }
     } else if (warp == kMmaWarp) {
         // ================= MMA issuer =================
@@ -1269,9 +1290,6 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const float lse_val = l_all > 0.f ? (m_ref * c2 + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
         if (ok) ok = mbar_wait_warp(B.o_done(blk, n_tiles - 1), ((n_tiles - 1) >> 2) & 1);    // the last product is in
         tc_fence_after();
-        // The whole ring is idle: what peers may write over, the tensor pipe's reads and the loads behind them, is complete by the
-        // barrier above, so there is nothing left for a releasing arrival to order (8,000 keys, T = 8 9.2 -> 9.7 us with one).
-        if (CL && n_tiles >= NS) cluster_arrive_relaxed();
         if (tid == 0) SPARROW_STAMP(6);                                // last product complete
         const int h_row = it.kvh * qg + g_row;
         const bool has_lse = row_ok && (wg == 0 || NB == 2);
@@ -1384,19 +1402,21 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
         const MergeOut merge_out = {args.out, args.lse, T, args.n_q_heads, qg, plan.inv_group};
         if (clustered) {
             // Every CTA of the cluster merges a share of the unit's rows: it is sent its rows of every piece, one
-            // bulk copy from each peer, into the last stage of the K/V ring.
+            // bulk copy from each peer, into a stage of the K/V ring.
             const int cl = plan.cluster;
             const int unit_rows = qg * min(NB * tpb, T - block0 * tpb);
-            const uint32_t recv = smem_u32(kv_sm) + (NS - 1) * kStageBytes;
+            auto recv_at = [&](int tiles) { return smem_u32(kv_sm) + (uint32_t)(recv_stage(NB, tiles) * kStageBytes + (NB == 1 ? kRecvSkip : 0)); };
+            const uint32_t recv = recv_at(n_tiles);
             int r_begin;
             const int n = merge_share(unit_rows, it.split, plan.inv_cluster, &r_begin) - r_begin;
-            cluster_wait();                                            // every peer runs, its barriers are initialised, its last stage is free
-            if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n * cl * kRowBytes));
             const int peer = warp + 8 * lane;                          // (spread over the warps: a warp's lanes issue one after the other)
+            const uint32_t peer_recv = recv_at(piece_tiles((n_keys_seq - plan.seq[it.b].key0 + kTile - 1) / kTile, cl, peer).count);
+            cluster_wait();                                            // every peer runs, its barriers are initialised, the stage is free
+            if (tid == 0) mbar_expect_tx(B.fin(), (uint32_t)(n * cl * kRowBytes));
             if (peer < cl) {
                 int r0;
                 const int r1 = merge_share(unit_rows, peer, plan.inv_cluster, &r0);      // the peer's share
-                const uint32_t dst = map_to_rank(recv + (uint32_t)(it.split * (r1 - r0) * kRowBytes), (uint32_t)peer);
+                const uint32_t dst = map_to_rank(peer_recv + (uint32_t)(it.split * (r1 - r0) * kRowBytes), (uint32_t)peer);
                 const uint32_t bar = map_to_rank(B.fin(), (uint32_t)peer);
                 // (staged block by block: the share may straddle the two)
                 const int mid = min(max(rows_per_block, r0), r1);

@@ -112,3 +112,53 @@ def test_the_kernels_pieces_tile_the_key_range(tmp_path):
     subprocess.run([build.nvcc(), *build.NVCC_FLAGS[:2], "-std=c++17", "-I" + CSRC, "-o", str(exe), str(src)], check=True, timeout=600)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
+
+
+def _one_program(tmp_path, name, text, *flags):
+    src, exe = tmp_path / (name + ".cu"), tmp_path / name
+    src.write_text(text)
+    subprocess.run([build.nvcc(), *build.NVCC_FLAGS[:2], "-std=c++17", "-I" + CSRC, "-I" + os.path.join(build.ROOT, "include"), *flags,
+                    "-o", str(exe), str(src)], check=True, timeout=600)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
+
+
+STAGES = r"""
+#include <cstdio>
+#include "verify_tc.cuh"
+using namespace sparrow::tc;
+int main()
+{
+    for (int nb = 1; nb <= 2; ++nb)
+        for (int n = 1; n <= 200; ++n) {
+            const int depth = nb == 1 ? 3 : 2, stage = recv_stage(nb, n);
+            int last = -1;
+            for (int j = 0; j < n; ++j)
+                if (j % depth == stage) last = j;
+            if (stage < 0 || stage >= depth) { std::printf("no stage: %d blocks, %d tiles\n", nb, n); return 1; }
+            if (n < depth ? last != -1 : last != recv_last_tile(nb, n)) { std::printf("%d blocks, %d tiles: last tile %d\n", nb, n, last); return 1; }
+            if (nb == 1 && n >= depth && last > n - depth) { std::printf("%d tiles: stage busy until tile %d\n", n, last); return 1; }
+        }
+    std::puts("ok");
+    return 0;
+}
+"""
+
+
+def test_rows_of_a_cluster_come_to_a_stage_that_is_idle(tmp_path):
+    """The stage that peers write to: unused where the piece does not fill the ring, else free once the tile that the producer
+    waits for is through; with one row block that tile is never one of the last two."""
+    _one_program(tmp_path, "stages", STAGES)
+
+
+def test_the_stage_is_released_to_the_peers_behind_its_last_use():
+    """The only arrival that makes a used stage of the ring writable for peers orders what was done to it ahead of their
+    copies: it stands behind the wait for the stage's last product, and releases."""
+    code = _code("verify_tc.cuh")
+    kernel = code[code.index("verify_tc_kernel(const"):]
+    producer = _between(kernel, "if (warp == kProducerWarp) {", "else if (warp == kMmaWarp)")
+    at = producer.index("cluster_arrive();")
+    assert 0 <= producer.find("mbar_wait(B.v_empty(recv_stage(NB, n_tiles))") < at
+    late = [m.start() for m in re.finditer(r"n_tiles >= NS\)[^;]*cluster_arrive_relaxed\(\)", kernel)]
+    assert len(late) == 1 and "!(warp == kProducerWarp && n_tiles >= NS)" in kernel[late[0] - 60:late[0] + 20]       # (everybody else's, at the start)
+    assert kernel.count("cluster_arrive();") == 1
