@@ -162,3 +162,16 @@ def test_the_stage_is_released_to_the_peers_behind_its_last_use():
     late = [m.start() for m in re.finditer(r"n_tiles >= NS\)[^;]*cluster_arrive_relaxed\(\)", kernel)]
     assert len(late) == 1 and "!(warp == kProducerWarp && n_tiles >= NS)" in kernel[late[0] - 60:late[0] + 20]       # (everybody else's, at the start)
     assert kernel.count("cluster_arrive();") == 1
+
+
+def test_no_kind_of_bounded_wait_in_front_of_the_wait_for_the_predecessor():
+    """As above, for every wait that the sources define (by name: a function that returns whether it succeeded)."""
+    names = sorted(set(re.findall(r"__forceinline__ bool (\w*wait\w*)\(", _code("verify_tc.cuh") + _code("common.cuh"))))
+    assert {"mbar_wait", "mbar_wait_tight", "mbar_wait_warp", "mbar_try_wait", "mbar_test_wait", "wait_counter"} <= set(names)
+    kernel = _code("verify_tc.cuh")
+    kernel = kernel[kernel.index("verify_tc_kernel(const"):]
+    for start, end in (("if (warp == kProducerWarp) {", "else if (warp == kMmaWarp)"), ("else if (warp == kMmaWarp) {", "else if (warp == kGateWarp)"),
+                       ("else if (warp == kGateWarp) {", "else if (warp < 8)")):
+        part = _between(kernel, start, end)
+        first = re.search(r"\b(" + "|".join(names) + r"|ld_acquire)\(", part)
+        assert first and 0 <= part.find("wait_for_predecessors()") < first.start()
