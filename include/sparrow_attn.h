@@ -97,7 +97,9 @@ sparrow_status sparrow_destroy(sparrow_ctx* ctx);
  * share the GPU with no other call of the context (single calls without sparrow_set_call_overlap(), graph
  * capture, SPARROW_NO_PDL, sparrow_anchor_attn, sparrow_verify_attn_static) always use one wave
  * over all SMs.  They do not need that wave to be resident as a whole: kernels of other streams and
- * contexts may hold SMs at the same time.  Calls that may overlap (batches, the opt-in) do need SMs for
+ * contexts may hold SMs at the same time.  Where such a call merges its pieces in thread-block clusters (of 2 to 16 CTAs; SPARROW_LOG=1
+ * says so), a cluster starts once that many SMs of one GPC are free: beside a kernel that leaves fewer in every GPC, when that
+ * kernel ends.  Calls that may overlap (batches, the opt-in) do need SMs for
  * the CTAs that merge them -- the last 32, under LATENCY all of them -- at one time: keep calls
  * of several contexts that overlap under LATENCY from running concurrently. */
 typedef enum {

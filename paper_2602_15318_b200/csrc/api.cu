@@ -35,7 +35,7 @@ typedef CUresult (*TensorMapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint3
 
 struct TensorMapEntry {
     const void* base;        // nullptr: free slot
-    int tag;                 // 0: K/V cache map; n > 0: Q map for n = batch * T tokens
+    int tag;                 // 0: K/V cache map; T > 0: map of q with T tokens a sequence
     CUtensorMap map;
 };
 // Hashed by (base pointer, tag), a bucket being kMapWays consecutive slots: room for the q / K / V
@@ -689,10 +689,14 @@ sparrow_status check_tree_host(const int32_t* parents, int T)
 
 // Estimates for the choice of a plan, us.  A lone call: a tile of 128 keys with one / two row blocks, a merge through the
 // workspace (of one sequence, of several: uneven pieces, more and shorter runs of rows), a merge in a cluster (by the rows that a CTA of it finishes and the pieces that it folds), and what items of two row
-// blocks cost besides.  Fitted to 170 shapes with every cluster size, the workspace and whole units forced (1 to 8 sequences of
+// blocks cost besides.  Fitted with every cluster size, the workspace and whole units forced (1 to 8 sequences of
 // 300 to 32,768 keys, T = 1 to 64, six head geometries).  The two kernels' tiles take 0.75 to 0.95 and 1.65, by the load; two row blocks
 // win where the GPU is full and at its power cap: pieces of more than about 40 tiles of one block (six sequences
 // of 27,000 keys, T = 19 62 and 55 us; two of 30,000, T = 36 36 and 41).
+// Calls in plain stream order (captured into a graph, programmatic launch off, no workspace of their own) choose between one and two row blocks
+// by the same figures, although combine_kernel merges their pieces.  Against the figures for a tile of 1.2 and 2.0 us, which
+// took two blocks there, 36 of 40 captured calls whose choice differs are faster, by 6 % in the median (two of 24,411, T = 60 51.5 ->
+// 47.1 us, eight of 4,142, 8 KV heads, T = 64 50.2 -> 40.5), three are slower, by 6 % at most (seven of 9,632, T = 25 37.6 -> 39.9).
 constexpr float kTileUs[2] = {0.8f, 1.4f};
 constexpr float kMergeWorkspaceUs[2] = {3.7f, 5.3f}, kMergeClusterUs = 0.1f, kMergeRowUs = 0.03f, kMergePieceUs = 0.02f;
 constexpr float kTwoBlocksUs = 4.f, kTwoBlocksWholeUs = 1.f;
@@ -704,9 +708,13 @@ constexpr float kBatchTileUs[2] = {1.2f, 2.0f}, kItemUs[2] = {5.f, 11.f}, kWhole
 // A lone call's pieces can meet in a thread-block cluster per unit instead of in the workspace, or a unit can
 // be one piece: cheaper by the round trips through L2 (partial rows out, arrival words, rows back in), but with
 // at most 16 pieces per unit and whole clusters per GPC.  Rewrites the plan where
-// that is estimated to pay (448 keys, T = 8 9.2 -> 7.4 us; 3,000 keys in 12 pieces of two tiles instead of 24 of one
-// 13.1 -> 9.5; longer pieces than leave a stage of the ring free: 8,000 keys, T = 8 in 16 pieces of 4 tiles
-// instead of 32 of 2 10.9 -> 9.2, 3,000 keys, T = 64 11.8 -> 10.4).  Returns the estimate.
+// that is estimated to pay.  Workspace and cluster, us, caches in L2: 1,500 keys, T = 16 9.8 and 7.1; 4,000 keys, T = 8 9.9 and 7.9;
+// 8,000 keys in 37 pieces and in 16 of four tiles 11.1 and 9.1; 12,000 keys 12.3 and 10.7; 3,000 keys, T = 64 11.9 and 10.3; of several
+// sequences four of 6,400, T = 6 16.1 and 14.2.  Caches in DRAM, where clusters leave SMs
+// without work: 8,000 keys 12.0 and 9.7, 10,500 keys, T = 16 13.1 and 11.7, 12,000 keys 13.6 and 11.7.
+// A cluster starts once one GPC has room for it, which is asked of an idle GPU.  Beside calls of other contexts it waits for that
+// room, a merge through the workspace for SMs for its last CTAs and for its own patience: 55 SMs held for 0.26 ms, 8,000 keys, T = 8
+// 0.44 ms through the workspace, 0.05 in clusters; 110 SMs for 0.6 ms: 0.64 and 0.49.  Returns the estimate.
 float plan_lone_call(const sparrow_ctx* c, bool may_rewrite, SplitPlan* p)
 {
     const int nb = p->blocks_per_group, units = p->batch * p->n_kv_heads * p->n_groups;
@@ -782,7 +790,7 @@ float lone_cost_of_items(const sparrow_ctx* c, const SplitPlan& p)
 // calls of a batch: a call's bits do not depend on them.
 //
 // A draft block of more than one row block: an item with two of them reads its keys once for both and keeps the
-// tensor pipe fuller on long pieces (an estimate of 2.0 us a tile instead of 2 x 1.2); items with one have the shorter prologue
+// tensor pipe fuller on long pieces (an estimate of 2.0 us a tile instead of 2 x 1.2 in a batch, 1.4 instead of 2 x 0.8 alone); items with one have the shorter prologue
 // and merge, no empty half where the blocks are odd in number, and twice as many of them fill the chip.
 // Where units are whole an item of two blocks costs less than two items of one, the more so the shorter the
 // sequences (24 sequences of 100 keys, T = 20: 96 items 6.1 us a call in a batch, 192 items 9.8), unless the blocks are odd in
@@ -825,9 +833,10 @@ sparrow_status plan_verify(const sparrow_ctx* c, bool may_share, bool may_cluste
 }
 
 // The gathered pass cut so that a unit's pieces share a cluster and merge there instead of through the
-// workspace and a second kernel, as long as no piece gets longer by it (a gathered tile of 64 keys takes about
-// 2.7 us): 448 anchors, T = 8 11.7 -> 9.9 us; four sequences of 448 anchors, T = 60 32.4 -> 25.6; with longer
-// pieces it lost (6,000 anchors in 16 pieces of 6 tiles instead of 37 of 3: 24.1 -> 32.4).
+// workspace and a second kernel, as long as no piece gets longer by it: 448 anchors, T = 8 9.3 -> 6.9 us; 1,500, T = 40 16.7 ->
+// 13.3; four sequences of 448 anchors, T = 60 25.1 -> 17.7.  The line lies where it lay when a tile took about 2.7 us; the present kernel's
+// pays with some longer pieces too (workspace and cluster: 1,017 anchors, T = 8 10.3 and 9.1, 2,500, T = 16 15.8 and 13.1, 6,000 16.0
+// and 15.8), not with all (two sequences of 6,000, T = 30 37.9 and 47.9).
 void plan_gather_cluster(const sparrow_ctx* c, int n_anchor, SplitPlan* p)
 {
     const int units = p->batch * p->n_kv_heads * p->n_groups;

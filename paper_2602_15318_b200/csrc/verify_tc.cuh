@@ -25,11 +25,11 @@
 //                        before it hands over P of that tile (softmax_pair.cuh: no barrier but in the first tile and at the end).
 //                        Each thread sums its own columns; the halves' sums meet once, in the epilogue.
 //                        Cycles per tile (41 tiles a CTA, 20 CTAs): 1,985 with a barrier of all softmax warps in every tile, 1,880
-//                        with one between the two of a pair, 1,540 without, 1,450 with half a tile between the two; the exponentials
-//                        alone are 1,024, the products 1,030 (a wait at a barrier that is complete costs the issuing warp 85 and the
-//                        pipe holds about 100 cycles of work behind the issuing lane, so V is waited for together with P).
-//                        All of it at 1.55 to 1.7 GHz: with all SMs at work the GPU is at its power cap, and a cycle saved is a third of one
-//                        in time.
+//                        with one between the two of a pair, 1,520 to 1,550 without (0.77 to 0.79 us at 1,965 MHz, in step or half a
+//                        tile apart); the exponentials alone are 1,024, the products 1,030 (a wait at a barrier that is complete costs
+//                        the issuing warp 85 and the pipe holds about 100 cycles of work behind the issuing lane, so V is waited for
+//                        together with P).  With all SMs at work the GPU is at its power cap, 1.55 to 1.7 GHz, and a cycle saved is a
+//                        third of one in time.
 //                        References that move, 16,384 keys, 64 nodes, us (a barrier of all in every tile in brackets): nothing
 //                        moves 22.2 (25.2), one key in 700 stands out 23.9 (25.7), one half outgrows the reference in every
 //                        second tile 27.2 (27.2), both halves of every row in every tile 32.2 (28.6: there P of a half is
@@ -447,9 +447,10 @@ __host__ __device__ constexpr int recv_stage(int n_blocks, int n) { return n_blo
 // The last tile in that stage, of n >= the ring's depth.
 __host__ __device__ constexpr int recv_last_tile(int n_blocks, int n) { return n_blocks == 1 ? n - 3 : (n & ~1) - 1; }
 
-// Shared-memory addresses of the mbarriers (8-byte slots).  K and V tiles have their own full /
-// empty pairs: a K tile is released as soon as its last S = Q K^T has been computed, a V tile
-// only after its last O += P V, so the K stream runs ahead of the V stream.
+// Shared-memory addresses of the mbarriers (8-byte slots).  K and V tiles have their own empty
+// barriers: a K tile is released as soon as its last S = Q K^T has been computed, a V tile
+// only after its last O += P V, so the K stream runs ahead of the V stream.  They have their own full barriers as
+// well, except that with one row block V counts on the barrier of its tile's P, the last tile's on its own.
 struct Bars {
     uint32_t base;
     // slots of 8 bytes: 0-27 here and in o_done, 31 is p_full(3); 28 and 29 hold the TMEM address and flags, 30 is free.
@@ -1202,9 +1203,11 @@ verify_tc_kernel(const __grid_constant__ TcArgs args, const __grid_constant__ Sy
                     m_ref = m_acc = fmaxf(mine, xch[(wg ^ 1) * 128 + row_local]);
                     if (m_acc > -INFINITY) { limit = m_acc + thr; mc = m_acc * c2; }
                     // The second warp of the pair starts half a tile's exponentials late and stays so: what each does besides them
-                    // falls into the other's.  In step, both wait for the exponentials together (41 tiles alone 1,560 -> 1,460
-                    // cycles a tile with the waits of the issuing warp; 8,000 keys, T = 8 9.12 -> 8.81 us, 26,112 keys 16.42 ->
-                    // 16.24, 3,000 keys, T = 64 10.42 -> 10.10).  It costs nothing: they would have shared the unit.
+                    // falls into the other's; in step, both wait for the exponentials together.  Lone calls, caches in L2, in step
+                    // -> like this, us: three tiles a CTA (4,089 keys, T = 8) 8.26 -> 8.00, four (8,000 keys, T = 8) 9.46 -> 9.05,
+                    // (3,000 keys, T = 64) 10.63 -> 10.30, five or six (26,112 keys) 16.49 -> 16.28, 14 or 15 (64 nodes on
+                    // 16,384 keys) 22.63 -> 22.32.  41 tiles a CTA on 20 CTAs, 0.77 to 0.79 us each: 42.4 and 42.4.  One and two
+                    // tiles: alike (1,500 keys, T = 16 7.03 and 7.08, 4,000 keys, T = 8 7.88 and 7.86).
                     if (wg == 1 && n_tiles > 2) {
                         const uint32_t c0 = (uint32_t)clock();
                         while ((uint32_t)clock() - c0 < kPairLag) {}
